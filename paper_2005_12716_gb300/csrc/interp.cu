@@ -10,6 +10,7 @@
 // points arrive in mesh order, so neighbouring threads share most of their stencil lines.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <mutex>
 #include <vector>
@@ -124,17 +125,25 @@ struct LevelTables {
   alignas(4) unsigned char lut[ZLUT];
   float z0, inv_h;
 };
+static_assert(sizeof(LevelTables) == sizeof(Levels) && sizeof(Levels) % 16 == 0 &&
+                  offsetof(LevelTables, inv) == offsetof(Levels, inv) && offsetof(LevelTables, lut) == offsetof(Levels, lut4) &&
+                  offsetof(LevelTables, z0) == offsetof(Levels, z0),
+              "the same layout");
 
-// Copy of the level tables in shared memory (per-thread indices would serialise on the
-// parameter bank).
-__device__ __forceinline__ void fill_level_tables(LevelTables& T, const Levels& L, int nz) {
-  if (threadIdx.x == 0) {
-    T.z0 = L.z0;
-    T.inv_h = L.inv_h;
-  }
-  for (int i = threadIdx.x; i < ZLUT / 4; i += blockDim.x) reinterpret_cast<unsigned*>(T.lut)[i] = L.lut4[i];
-  for (int i = threadIdx.x; i < nz; i += blockDim.x) T.z[i] = L.z[i];
-  for (int j = threadIdx.x; j <= nz - 4; j += blockDim.x) T.inv[j] = L.inv[j];
+// The level tables of a kernel parameter by a generic pointer: loads through it are ordinary cached
+// loads, where per-thread indices into the parameter itself serialise on the constant bank, a lane
+// at a time.
+__device__ __forceinline__ const LevelTables* level_tables(const Levels& L) {
+  const LevelTables* p = reinterpret_cast<const LevelTables*>(&L);
+  asm volatile("" : "+l"(p));
+  return p;
+}
+
+// Copy of the level tables in shared memory.
+__device__ __forceinline__ void fill_level_tables(LevelTables& T, const Levels& L) {
+  const uint4* src = reinterpret_cast<const uint4*>(level_tables(L));
+  uint4* dst = reinterpret_cast<uint4*>(&T);
+  for (int i = threadIdx.x; i < int(sizeof(LevelTables) / 16); i += blockDim.x) dst[i] = src[i];
 }
 
 struct PointCell {
@@ -184,57 +193,6 @@ __device__ __forceinline__ PointCell point_cell(const InterpArgs& a, const Level
   point_xy<P2>(a, x, y, c);
   point_level(a, T, z, c);
   return c;
-}
-
-// Stencil sums straight from global memory (L1/L2), all time levels.
-template <bool P2 = true>
-__device__ __forceinline__ void gather_global(const InterpArgs& a, const PointCell& c, float4& acc,
-                                              float& acc_eta) {
-  const size_t plane = size_t(a.Nyr) * a.Nxr;
-  const int nys = a.Nyr > 1 ? 4 : 1;
-  int xi[4], yi[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    xi[q] = wrapi<P2>(c.ix - 1 + q, a.Nxr);
-    yi[q] = a.Nyr > 1 ? wrapi<P2>(c.iy - 1 + q, a.Nyr) : 0;
-  }
-  acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  acc_eta = 0.f;
-  for (int tl = 0; tl < a.n_tl; ++tl) {
-    const float wtl = a.wt[tl];
-    const float4* base_t = a.nodes + size_t(tl) * a.nz * plane;
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
-      const float4* lev = base_t + size_t(c.j0 + q) * plane;
-      // select instead of a dynamic index so the weights stay in registers
-      const float wzq = wtl * (q == 0 ? c.wz[0] : q == 1 ? c.wz[1] : q == 2 ? c.wz[2] : c.wz[3]);
-#pragma unroll 1
-      for (int b = 0; b < nys; ++b) {
-        const int yb = b == 0 ? yi[0] : b == 1 ? yi[1] : b == 2 ? yi[2] : yi[3];
-        const float wyb = b == 0 ? c.wy[0] : b == 1 ? c.wy[1] : b == 2 ? c.wy[2] : c.wy[3];
-        const float4* row = lev + size_t(yb) * a.Nxr;
-        const float wzy = wzq * wyb;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float4 gv = __ldg(&row[xi[k]]);
-          const float ww = wzy * c.wx[k];
-          acc.x = fmaf(ww, gv.x, acc.x);
-          acc.y = fmaf(ww, gv.y, acc.y);
-          acc.z = fmaf(ww, gv.z, acc.z);
-          acc.w = fmaf(ww, gv.w, acc.w);
-        }
-      }
-    }
-    const float* et = a.eta + size_t(tl) * plane;
-#pragma unroll 1
-    for (int b = 0; b < nys; ++b) {
-      const int yb = b == 0 ? yi[0] : b == 1 ? yi[1] : b == 2 ? yi[2] : yi[3];
-      const float wyb = b == 0 ? c.wy[0] : b == 1 ? c.wy[1] : b == 2 ? c.wy[2] : c.wy[3];
-      const float* row = et + size_t(yb) * a.Nxr;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) acc_eta = fmaf(wtl * wyb * c.wx[k], __ldg(&row[xi[k]]), acc_eta);
-    }
-  }
 }
 
 __device__ __forceinline__ void store_point(const InterpArgs& a, int64_t i, float4 acc,
@@ -357,6 +315,111 @@ __device__ __forceinline__ void row_sum(const float4* row, const float* erow,
   re = 0.f;
 #pragma unroll
   for (int kx = 0; kx < 4; ++kx) re = fmaf(wx[kx], erow[kx], re);
+}
+
+// Points whose stencils are gathered straight from global memory (L1/L2): one record per point,
+// 80 bytes so that the eight records a warp reads at once lie in different banks.
+struct alignas(16) GatherRec {
+  int4 cell;             // first stencil node in x and y (before the -1 shift), first level, inside
+  float4 wy, wz;
+  float wx[4];           // the four gathered fields overwrite the x weights
+  float eta, pad_[3];
+};
+static_assert(sizeof(GatherRec) == 80, "GatherRec layout");
+
+// Stencil sums of points p0 .. p0 + WPTS - 1 by one warp, four lanes a point, lane k the stencil's x
+// node k. A warp load then covers the 64-byte stencil rows of eight points (8 to 16 L1 lines), where
+// one point a lane touches 32 lines with every load: the L1's line rate is what bounds scattered
+// points (74 % of its data pipe on the first workload below, 87 % on the second). Each lane sums its
+// column over y, z and time; the quad's x sum is a shuffle reduction that leaves field k with lane k.
+// 16 M scattered points on the 8.6 GB grid of 2048 x 1024 modes and 128 levels: 5.17 -> 3.28 ms; 8.2 M
+// mesh points on the four-fold padded 512 x 256-mode grid: 1.45 -> 1.02 ms (one point a lane before).
+template <bool P2, int WPTS>
+__device__ __forceinline__ void gather_warp(const InterpArgs& a, const LevelTables& zs, int64_t p0, GatherRec* rec) {
+  const size_t plane = size_t(a.Nyr) * a.Nxr;
+  const size_t tl_stride = size_t(a.nz) * plane;
+  const int lane = threadIdx.x & 31, k = lane & 3;
+  const bool two_d = a.Nyr == 1;
+  const int64_t i = p0 + lane;
+  float z = 0.f;
+  if (WPTS == 32 || lane < WPTS) {
+    const int64_t ic = i < a.np ? i : a.np - 1;    // lanes past the end repeat the last point
+    z = __ldg(&a.pts[3 * ic + 2]);
+    const PointCell c = point_cell<P2>(a, zs, __ldg(&a.pts[3 * ic]), __ldg(&a.pts[3 * ic + 1]), z);
+    GatherRec& r = rec[lane];
+    r.cell = make_int4(c.ix, c.iy, c.j0, c.inside);
+    r.wy = make_float4(c.wy[0], c.wy[1], c.wy[2], c.wy[3]);
+    r.wz = make_float4(c.wz[0], c.wz[1], c.wz[2], c.wz[3]);
+    *reinterpret_cast<float4*>(r.wx) = make_float4(c.wx[0], c.wx[1], c.wx[2], c.wx[3]);
+  }
+  __syncwarp();
+#pragma unroll 1
+  for (int s = 0; s < WPTS / 8; ++s) {
+    GatherRec& r = rec[8 * s + (lane >> 2)];
+    const int4 c = r.cell;
+    const float4 wy = r.wy, wz = r.wz;
+    const float wxk = r.wx[k];
+    const int xk = wrapi<P2>(c.x - 1 + k, a.Nxr);
+    int row[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) row[b] = xk + (two_d ? 0 : wrapi<P2>(c.y - 1 + b, a.Nyr) * a.Nxr);
+    const float wyb[4] = {wy.x, wy.y, wy.z, wy.w}, wzq[4] = {wz.x, wz.y, wz.z, wz.w};
+    unsigned long long uv = 0ull, wt = 0ull;       // (u, v) and (w, dphi/dt)
+    float e = 0.f;
+    for (int tl = 0; tl < a.n_tl; ++tl) {
+      const float wtl = a.wt[tl];
+      const float4* base = a.nodes + size_t(tl) * tl_stride + size_t(c.z) * plane;
+      const float* et = a.eta + size_t(tl) * plane;
+      if (two_d) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float4 g = __ldg(&base[q * plane + row[0]]);
+          const float w = wtl * wzq[q];
+          fma2(uv, pack2(w, w), pack2(g.x, g.y));
+          fma2(wt, pack2(w, w), pack2(g.z, g.w));
+        }
+        e = fmaf(wtl, __ldg(&et[row[0]]), e);
+        continue;
+      }
+#pragma unroll 1
+      for (int q = 0; q < 4; ++q) {
+        unsigned long long ruv = 0ull, rwt = 0ull;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const float4 g = __ldg(&base[q * plane + row[b]]);
+          const unsigned long long w2 = pack2(wyb[b], wyb[b]);
+          fma2(ruv, w2, pack2(g.x, g.y));
+          fma2(rwt, w2, pack2(g.z, g.w));
+        }
+        const float w = wtl * (q == 0 ? wz.x : q == 1 ? wz.y : q == 2 ? wz.z : wz.w);
+        fma2(uv, pack2(w, w), ruv);
+        fma2(wt, pack2(w, w), rwt);
+      }
+      float re = 0.f;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) re = fmaf(wyb[b], __ldg(&et[row[b]]), re);
+      e = fmaf(wtl, re, e);
+    }
+    float f0 = wxk * lo2(uv), f1 = wxk * hi2(uv), f2 = wxk * lo2(wt), f3 = wxk * hi2(wt);
+    e *= wxk;
+    e += __shfl_xor_sync(0xffffffffu, e, 1);
+    e += __shfl_xor_sync(0xffffffffu, e, 2);
+    // transposing reduction: lanes k and k ^ 1 swap the halves they do not keep, then k and k ^ 2
+    const bool odd = k & 1, high = k & 2;
+    float g0 = odd ? f1 : f0, g1 = odd ? f3 : f2;
+    g0 += __shfl_xor_sync(0xffffffffu, odd ? f0 : f1, 1);
+    g1 += __shfl_xor_sync(0xffffffffu, odd ? f2 : f3, 1);
+    const float h = (high ? g1 : g0) + __shfl_xor_sync(0xffffffffu, high ? g0 : g1, 2);
+    __syncwarp();                                  // every lane of the quad has read the record
+    r.wx[k] = h;
+    if (k == 0) r.eta = e;
+  }
+  __syncwarp();
+  if ((WPTS == 32 || lane < WPTS) && i < a.np) {
+    const float4 f = *reinterpret_cast<const float4*>(rec[lane].wx);
+    store_point(a, i, f, rec[lane].eta, z, rec[lane].cell.w != 0);
+  }
+  __syncwarp();                                    // the records are rewritten by the next call
 }
 
 // Time-blended box of grid nodes x0..x0+bx-1, y0..y0+by-1 (wrapped), levels l0..l0+bz-1 into
@@ -539,9 +602,9 @@ __device__ __forceinline__ void plan_chunk(const InterpArgs& a, const LevelTable
 }
 
 template <bool P2>
-__global__ void __launch_bounds__(BOX_THREADS) k_interp_plan(InterpArgs a, Levels L, int4* __restrict__ plan) {
+__global__ void __launch_bounds__(BOX_THREADS) k_interp_plan(const __grid_constant__ InterpArgs a, const __grid_constant__ Levels L, int4* __restrict__ plan) {
   __shared__ LevelTables zs;
-  fill_level_tables(zs, L, a.nz);
+  fill_level_tables(zs, L);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   plan_chunk<P2>(a, zs, int64_t(blockIdx.x) * PLAN_WARPS + warp, plan, lane);
@@ -555,19 +618,16 @@ __device__ __forceinline__ bool plan_is_global(const int4 pl, int nz) {
   return bp.l0 + bp.bz > nz;
 }
 
-// Points p0 + k * BOX_THREADS + threadIdx.x (k < BOX_PPT) gathered from global memory.
+// The chunk's points gathered from global memory, 32 at a time by each warp; rec: 32 records per warp.
+static_assert(BOX_THREADS * sizeof(GatherRec) <= BOX_SMEM, "the records fit the tile's shared memory");
 template <bool P2>
-__device__ __forceinline__ void global_points(const InterpArgs& a, const LevelTables& zs, int64_t p0) {
+__device__ __forceinline__ void global_points(const InterpArgs& a, const LevelTables& zs, int64_t p0,
+                                              GatherRec* rec) {
 #pragma unroll 1
   for (int k = 0; k < BOX_PPT; ++k) {
-    const int64_t i = p0 + k * BOX_THREADS + threadIdx.x;
-    if (i >= a.np) break;                           // later points of this thread are past np too
-    const float pz = __ldg(&a.pts[3 * i + 2]);
-    const PointCell c = point_cell<P2>(a, zs, __ldg(&a.pts[3 * i]), __ldg(&a.pts[3 * i + 1]), pz);
-    float4 acc;
-    float acc_eta;
-    gather_global<P2>(a, c, acc, acc_eta);
-    store_point(a, i, acc, acc_eta, pz, c.inside);
+    const int64_t i0 = p0 + k * BOX_THREADS + (threadIdx.x & ~31);
+    if (i0 >= a.np) break;                         // uniform over the warp
+    gather_warp<P2, 32>(a, zs, i0, rec + (threadIdx.x & ~31));
   }
 }
 
@@ -592,7 +652,7 @@ __device__ __forceinline__ void box_chunk(const InterpArgs& a, const LevelTables
   const BoxPlan bp = decode_plan(pl);
   if (plan_is_global(pl, a.nz)) {                  // no tile, or a plan of another level list
     __syncthreads();
-    if (kGlobal) global_points<P2>(a, zs, p0);
+    if (kGlobal) global_points<P2>(a, zs, p0, reinterpret_cast<GatherRec*>(sbox));
     return;
   }
   const int bx = bp.bx, by = bp.by, bz = bp.bz;
@@ -717,14 +777,14 @@ __device__ __forceinline__ void box_chunk(const InterpArgs& a, const LevelTables
 // The chunks with a staged tile (box, plane or two planes); kSplit: k_interp_global takes the
 // others, else this kernel gathers them too (from global memory, with L1 reduced by the tile).
 template <bool P2, bool kSplit>
-__global__ void __launch_bounds__(BOX_THREADS, 3) k_interp_box(InterpArgs a, Levels L,
+__global__ void __launch_bounds__(BOX_THREADS, 3) k_interp_box(const __grid_constant__ InterpArgs a, const __grid_constant__ Levels L,
                                                                 const int4* __restrict__ plan) {
   extern __shared__ float4 sbox[];
   float* seta = reinterpret_cast<float*>(sbox + BOX_NODES);
   __shared__ LevelTables zs;
   const int4 pl = plan[blockIdx.x];
   if (kSplit && plan_is_global(pl, a.nz)) return;   // uniform over the CTA
-  fill_level_tables(zs, L, a.nz);
+  fill_level_tables(zs, L);
   box_chunk<P2, !kSplit>(a, zs, blockIdx.x, pl, sbox, seta);
 }
 
@@ -732,27 +792,22 @@ __global__ void __launch_bounds__(BOX_THREADS, 3) k_interp_box(InterpArgs a, Lev
 // more nodes than shared memory holds). No dynamic shared memory, so that L1 keeps the rows
 // neighbouring points share: launched apart from k_interp_box, whose 68 KB tile per CTA would
 // leave L1 a fifth of its size.
-// One quarter of a chunk (256 points, one a thread) per CTA, in point order: the CTAs in flight
-// then cover consecutive points, whose stencils share rows in L2, over a quarter of the span that
-// whole chunks per CTA would (3 % faster on the large sea); the quarters of chunks with a staged
-// tile exit at once.
+// A warp per GLOBAL_WPTS points, CTAs in point order and without a block barrier: with 16 points a
+// warp the points in flight span half the grid that 32 would (their shared rows stay in L2 until both
+// have read them: 3.5 -> 3.3 ms on the scattered points above), with 8 the idle lanes of the cell
+// search cost more than that gives (3.4 ms). Four loads in flight a lane (a rolled level loop, 48
+// registers, five CTAs per SM): more of them evict each other's lines from L1 (5.8 ms with sixteen).
+constexpr int GLOBAL_WPTS = 16;
+constexpr int GLOBAL_PTS = GLOBAL_WPTS * (BOX_THREADS / 32);     // points per CTA
 template <bool P2>
-__global__ void __launch_bounds__(BOX_THREADS, 4) k_interp_global(InterpArgs a, Levels L,
-                                                                   const int4* __restrict__ plan) {
-  __shared__ LevelTables zs;
-  const int64_t sub = blockIdx.x, chunk = sub / BOX_PPT;
-  const int4 pl = plan[chunk];
-  if (!plan_is_global(pl, a.nz)) return;            // uniform over the CTA
-  fill_level_tables(zs, L, a.nz);
-  __syncthreads();
-  const int64_t i = chunk * BOX_PTS + (sub % BOX_PPT) * BOX_THREADS + threadIdx.x;
-  if (i >= a.np) return;
-  const float pz = __ldg(&a.pts[3 * i + 2]);
-  const PointCell c = point_cell<P2>(a, zs, __ldg(&a.pts[3 * i]), __ldg(&a.pts[3 * i + 1]), pz);
-  float4 acc;
-  float acc_eta;
-  gather_global<P2>(a, c, acc, acc_eta);
-  store_point(a, i, acc, acc_eta, pz, c.inside);
+__global__ void __launch_bounds__(BOX_THREADS, 5) k_interp_global(const __grid_constant__ InterpArgs a,
+                                                                       const __grid_constant__ Levels L,
+                                                                       const int4* __restrict__ plan) {
+  __shared__ GatherRec rec[GLOBAL_PTS];
+  const int warp = threadIdx.x >> 5;
+  const int64_t p0 = int64_t(blockIdx.x) * GLOBAL_PTS + warp * GLOBAL_WPTS;
+  if (p0 >= a.np || !plan_is_global(plan[p0 / BOX_PTS], a.nz)) return;   // uniform over the warp
+  gather_warp<P2, GLOBAL_WPTS>(a, *level_tables(L), p0, rec + warp * GLOBAL_WPTS);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -793,15 +848,7 @@ __global__ void __launch_bounds__(BOX_THREADS) k_interp_plan_batch(const BatchIn
   if (c >= chunk0[n]) return;                       // no block barrier in this kernel
   const int i = batch_instance(chunk0, n, c);
   copy_words(sa, &inst[i].a, int(sizeof(InterpArgs)), lane, 32);
-  const Levels& L = inst[i].L;
-  const int nz = inst[i].a.nz;
-  if (lane == 0) {
-    zs->z0 = L.z0;
-    zs->inv_h = L.inv_h;
-  }
-  for (int k = lane; k < ZLUT / 4; k += 32) reinterpret_cast<unsigned*>(zs->lut)[k] = L.lut4[k];
-  for (int k = lane; k < nz; k += 32) zs->z[k] = L.z[k];
-  for (int j = lane; j <= nz - 4; j += 32) zs->inv[j] = L.inv[j];
+  copy_words(zs, &inst[i].L, int(sizeof(LevelTables)), lane, 32);
   __syncwarp();
   plan_chunk<true>(*sa, *zs, c - chunk0[i], plan + chunk0[i], lane);
 }
@@ -825,7 +872,7 @@ __global__ void __launch_bounds__(BOX_THREADS, 3) k_interp_box_batch(const Batch
     const int i = batch_instance(chunk0, n, c);
     if (i != cur) {
       copy_words(&sa, &inst[i].a, int(sizeof(InterpArgs)), threadIdx.x, blockDim.x);
-      fill_level_tables(zs, inst[i].L, inst[i].a.nz);
+      fill_level_tables(zs, inst[i].L);
       cur = i;
     }
     __syncthreads();                                // arguments and tables in place
@@ -950,7 +997,7 @@ __device__ __forceinline__ void learned_tiles(const float4* nodes, int SY, int S
   }
 }
 
-__global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(InterpArgs a, Levels L,
+__global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_constant__ InterpArgs a, const __grid_constant__ Levels L,
                                                                     const int4* __restrict__ plan,
                                                                     const PackedFwd* __restrict__ Wg) {
   extern __shared__ float4 sbox[];
@@ -958,7 +1005,7 @@ __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(InterpArgs a,
   LPoint* rec = reinterpret_cast<LPoint*>(seta + BOX_COLS);
   WeightsSmem& W = *reinterpret_cast<WeightsSmem*>(rec + LRN_SB);
   __shared__ LevelTables zs;
-  fill_level_tables(zs, L, a.nz);
+  fill_level_tables(zs, L);
   {
     // rows re-strided into the padded layout, 16 bytes (8 bf16) at a time
     using namespace mlpnet;
@@ -1140,10 +1187,10 @@ struct FeatArgs {
   float* eta_out;        // [np] or NULL
 };
 
-__global__ void __launch_bounds__(128) k_mlp_features(FeatArgs f, Levels L) {
+__global__ void __launch_bounds__(128) k_mlp_features(FeatArgs f, const __grid_constant__ Levels L) {
   __shared__ LevelTables zs;
   const InterpArgs& a = f.a;
-  fill_level_tables(zs, L, a.nz);
+  fill_level_tables(zs, L);
   __syncthreads();
   const size_t plane = size_t(a.Nyr) * a.Nxr;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < a.np;
@@ -1414,8 +1461,9 @@ int interp_impl(const swense_grid* g, double t, const float* pts, const int32_t*
     if (split) {
       if (a.p2) k_interp_box<true, true><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
       else k_interp_box<false, true><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
-      if (a.p2) k_interp_global<true><<<unsigned(blocks * BOX_PPT), BOX_THREADS, 0, stream>>>(a, lev, plan);
-      else k_interp_global<false><<<unsigned(blocks * BOX_PPT), BOX_THREADS, 0, stream>>>(a, lev, plan);
+      const unsigned gctas = unsigned((np + GLOBAL_PTS - 1) / GLOBAL_PTS);
+      if (a.p2) k_interp_global<true><<<gctas, BOX_THREADS, 0, stream>>>(a, lev, plan);
+      else k_interp_global<false><<<gctas, BOX_THREADS, 0, stream>>>(a, lev, plan);
       count_launches(2);
     } else {
       if (a.p2) k_interp_box<true, false><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
