@@ -333,8 +333,10 @@ enum swense_direct_precision {
  *   (A e^{-i omega (t - t_ref)}, phase reduced in FP64), otherwise t is ignored.
  * pts: device float [np][3]; outputs device float [np] each, any may be NULL.
  * precision:
- *   SWENSE_DIRECT_FP32: one thread per point, every mode in FP32 (the phase m x/Lx + n y/Ly is
- *     an exact 32-bit fraction of a turn, so accuracy does not degrade with |k x|).
+ *   SWENSE_DIRECT_FP32: every mode in FP32 (the phases m x/Lx and n y/Ly are exact 32-bit
+ *     fractions of a turn, so accuracy does not degrade with |k x|); rows n and -n, which share
+ *     |k|, are summed together, four points a thread, and few points split the modes over blocks
+ *     whose partial sums are added in a fixed order.
  *   SWENSE_DIRECT_SPLIT_BF16: the sums as a dense contraction on the tcgen05 tensor cores. The
  *     points are sorted by z (a counting sort into 65536 buckets between their min and max z)
  *     and cut into tiles of 128, two tiles per cluster of two CTAs (cta_group::2); the phase
@@ -353,7 +355,8 @@ enum swense_direct_precision {
  *   SWENSE_DIRECT_SPLIT_BF16_PAIRWISE: per (point, mode) pair the operand e^{i k.x} f(z) is
  *     generated in registers and split into BF16 hi + lo for legacy mma.sync m16n8k16 products
  *     (the same accuracy; kept for comparison and for tiles the tensor-core path leaves).
- * Uses the scratch workspace (FP32: 64 B per mode slot; SPLIT_BF16: 32 B per mode slot, 20 B
+ * Uses the scratch workspace (FP32: 48 B per mode slot, rows padded to 64 modes, and at most
+ * 20 B per point and block of modes; SPLIT_BF16: 32 B per mode slot, 20 B
  * per point and 256 KB; PAIRWISE: 80 B per mode). Errors: ARG, SIZE, UNSUPPORTED, OOM, CUDA;
  * the tensor-core kernel's bounded waits report through swense_async_status.
  */

@@ -6,11 +6,14 @@
 // and whatIsSpectralMethod and Bernoulli for the pressure. Used for small mode counts and for
 // near-body points that must not carry interpolation error.
 //
-// FP32 path: one thread per point, modes streamed through shared memory in tiles (every lane
-// reads the same mode: broadcast). The phase k.x is carried as an exact 32-bit fraction of a
-// turn: per point X = frac(x / Lx) * 2^32 and Y = frac(y / Ly) * 2^32 (formed in FP64 once per
-// point), per mode the integer product m X + n Y (mod 2^32), so the argument error does not grow
-// with |k x|. Depth factors use a compensated |k| z product. Sums are accumulated per tile and
+// FP32 path: rows n and -n of the one-sided spectrum share |k|, so they are summed together. With
+// theta = kx_m x and phi = ky_n y the two modes' contribution to a field is
+//   cos(phi) F (P cos(theta) + Q sin(theta)) + sin(phi) F (R cos(theta) + S sin(theta))
+// with P, Q, R, S made from the two amplitudes, so the inner loop over m needs one depth factor, one
+// rotation of theta and four products per field for two modes. The phase is carried as an exact
+// 32-bit fraction of a turn: per point X = frac(x / Lx) * 2^32 and Y = frac(y / Ly) * 2^32 (formed in
+// FP64 once per point), per mode the integer product m X (mod 2^32), so the argument error does not
+// grow with |k x|. Depth factors use a compensated |k| z product. Sums are accumulated per tile and
 // then added to the running totals to limit FP32 round-off growth over many modes.
 #include <algorithm>
 #include <cmath>
@@ -21,15 +24,6 @@
 
 namespace swense {
 namespace {
-
-// Coefficients of one mode, 64 bytes:
-//   c0 = (m, n as int bits, |k|, 1 / (1 + e^{-2|k|h}) or 1 in deep water)
-//   c1 = (W_eta, W_u), c2 = (W_v, W_w), c3 = (W_t, 0, 0)
-// with W_eta = c A^eta, W_u = c i kx A^phi, W_v = c i ky A^phi, W_w = c |k| A^phi,
-// W_t = c A^phit and c = 1 for m = 0, 2 otherwise (one-sided spectrum weights).
-struct ModeCoef {
-  float4 c0, c1, c2, c3;
-};
 
 // Weighted coefficients of slot i = r (nx/2 + 1) + m of the one-sided spectrum at time offset dt
 // (linear propagation e^{-i omega dt} when omega is given). Nyquist slots return live = false.
@@ -76,36 +70,67 @@ __device__ __forceinline__ SlotCoef slot_coef(int i, const float2* __restrict__ 
   return sc;
 }
 
-__global__ void k_direct_prep(const float2* __restrict__ Ae, const float2* __restrict__ Ap,
-                              const float2* __restrict__ At, const double* __restrict__ omega,
-                              double dt, int nx, int ny, float kxs, float kys, float depth,
-                              ModeCoef* __restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= ny * (nx / 2 + 1)) return;
-  const SlotCoef sc = slot_coef(i, Ae, Ap, At, omega, dt, nx, ny, kxs, kys, depth);
-  ModeCoef mc;
-  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (!sc.live) {
-    mc.c0 = make_float4(__int_as_float(0), __int_as_float(0), 0.f, 1.f);
-    mc.c1 = mc.c2 = mc.c3 = zero;
-    out[i] = mc;
+// Depth factors as depth_factors (fft.cuh) with 1 / (1 + e^{-2 k h}) given.
+template <bool FINITE>
+__device__ __forceinline__ void direct_depth(float k, float z, float h, float invd, float& F, float& S) {
+  const float kz = k * z;
+  const float kz_lo = fmaf(k, z, -kz);
+  float e1 = expf(kz);
+  e1 = fmaf(e1, kz_lo, e1);
+  if (!FINITE) {
+    F = S = e1;
     return;
   }
-  mc.c0 = make_float4(__int_as_float(sc.m), __int_as_float(sc.n), sc.k, sc.invd);
-  mc.c1 = make_float4(sc.we.x, sc.we.y, sc.wu.x, sc.wu.y);
-  mc.c2 = make_float4(sc.wv.x, sc.wv.y, sc.ww.x, sc.ww.y);
-  mc.c3 = make_float4(sc.wt.x, sc.wt.y, 0.f, 0.f);
-  out[i] = mc;
+  const float e2 = expf(-k * (z + 2.f * h));
+  F = (e1 + e2) * invd;
+  S = (e1 - e2) * invd;
 }
 
-constexpr int kDirThreads = 256;
-constexpr int kDirTile = 256;   // modes per shared-memory tile
+// One (m, |n|) pair of modes, 96 bytes: per field the factors of (cos, sin)(phi) x (cos, sin)(theta),
+//   q = (P, R, Q, S): C += F (P cos(theta) + Q sin(theta)), S += F (R cos(theta) + S sin(theta)),
+// for eta (F = 1), u, v, w (F = the vertical factor S(z)), dphi/dt; then |k| and, in finite depth,
+// 1 / (1 + e^{-2 |k| h}).
+struct PairCoef {
+  float4 q[5];
+  float k, invd, pad_[2];
+};
+static_assert(sizeof(PairCoef) == 96, "pair record");
+
+constexpr int kDirTile = 64;    // pairs of one row |n| per tile
+constexpr int kDirAnchor = 16;  // exact phase of theta every this many modes
+
+// Pairs in tiles: entry ((|n| tpr + m / kDirTile) kDirTile + m % kDirTile), zero past nx/2 - 1.
+__global__ void k_direct_prep(const float2* __restrict__ Ae, const float2* __restrict__ Ap,
+                              const float2* __restrict__ At, const double* __restrict__ omega,
+                              double dt, int nx, int ny, float kxs, float kys, float depth, int tpr, int64_t n,
+                              PairCoef* __restrict__ out) {
+  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int m = int(i % (tpr * kDirTile)), row = int(i / (tpr * kDirTile));
+  PairCoef pc{};
+  pc.invd = 1.f;
+  if (m < nx / 2) {
+    const int nxh1 = nx / 2 + 1;
+    const SlotCoef p = slot_coef(row * nxh1 + m, Ae, Ap, At, omega, dt, nx, ny, kxs, kys, depth);
+    SlotCoef o{};                                  // the partner row -n (none for n = 0)
+    if (row > 0) o = slot_coef((ny - row) * nxh1 + m, Ae, Ap, At, omega, dt, nx, ny, kxs, kys, depth);
+    const float2 a[5] = {p.we, p.wu, p.wv, p.ww, p.wt}, b[5] = {o.we, o.wu, o.wv, o.ww, o.wt};
+#pragma unroll
+    for (int f = 0; f < 5; ++f)
+      pc.q[f] = make_float4(a[f].x + b[f].x, b[f].y - a[f].y, -(a[f].y + b[f].y), b[f].x - a[f].x);
+    pc.k = p.k;
+    pc.invd = p.invd;
+  }
+  out[i] = pc;
+}
 
 struct DirectArgs {
-  const ModeCoef* modes;
-  unsigned n_modes;
+  const PairCoef* pairs;
+  int n_tiles, tpr;          // tiles; tiles per row |n|
+  int tps;                   // tiles per split (blockIdx.y)
   const float* pts;
   float *o_eta, *o_u, *o_v, *o_w, *o_p;
+  float* part;               // [splits][5][np] partial sums, or NULL: one split writes the outputs
   int64_t np;
   double inv_lx, inv_ly;
   float depth;
@@ -113,80 +138,137 @@ struct DirectArgs {
   float rho, g;
 };
 
-
-__global__ void __launch_bounds__(kDirThreads) k_direct_fp32(DirectArgs a) {
-  __shared__ ModeCoef tile[kDirTile];
-  const unsigned nm = a.n_modes;
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const bool live = i < a.np;
-  float x = 0.f, y = 0.f, z = 0.f;
-  if (live) {
-    x = a.pts[3 * i];
-    y = a.pts[3 * i + 1];
-    z = a.pts[3 * i + 2];
-  }
-  const unsigned X = turn_fraction(x, a.inv_lx), Y = turn_fraction(y, a.inv_ly);
-  const float h = a.depth;
-  // e^{i 2 pi x / Lx}: the phase step from mode m to m + 1 along a row (same n)
-  float sstep, cstep;
-  sincospif(2.f * (float(int(X)) * 2.3283064365386963e-10f), &sstep, &cstep);
-  int prev_m = -2, prev_n = 0, run = 0;
-  float sn = 0.f, cs = 1.f;
-  float s_eta = 0.f, s_u = 0.f, s_v = 0.f, s_w = 0.f, s_t = 0.f;
-  for (unsigned base = 0; base < nm; base += kDirTile) {
-    const unsigned cnt = min(unsigned(kDirTile), nm - base);
-    __syncthreads();
-    for (unsigned j = threadIdx.x; j < cnt; j += blockDim.x) tile[j] = a.modes[base + j];
-    __syncthreads();
-    float t_eta = 0.f, t_u = 0.f, t_v = 0.f, t_w = 0.f, t_t = 0.f;
-    for (unsigned j = 0; j < cnt; ++j) {
-      const float4 c0 = tile[j].c0, c1 = tile[j].c1, c2 = tile[j].c2, c3 = tile[j].c3;
-      const int m = __float_as_int(c0.x), n = __float_as_int(c0.y);
-      if (m == prev_m + 1 && n == prev_n && run < 15) {
-        // consecutive mode of the same row: advance the phase by the per-point step
-        const float c2 = fmaf(cs, cstep, -sn * sstep);
-        sn = fmaf(sn, cstep, cs * sstep);
-        cs = c2;
-        ++run;
-      } else {
-        // exact phase m X + n Y (mod 2^32) every 16 modes and at row starts
-        const unsigned ph = unsigned(m) * X + unsigned(n) * Y;
-        const float turns = float(int(ph)) * 2.3283064365386963e-10f;   // 2^-32, in [-0.5, 0.5)
-        sincospif(2.f * turns, &sn, &cs);
-        run = 0;
-      }
-      prev_m = m;
-      prev_n = n;
-      const float k = c0.z;
-      float F, S;
-      depth_factors(k, z, h, F, S);
-      t_eta = fmaf(c1.x, cs, fmaf(-c1.y, sn, t_eta));
-      t_u = fmaf(F, fmaf(c1.z, cs, -c1.w * sn), t_u);
-      t_v = fmaf(F, fmaf(c2.x, cs, -c2.y * sn), t_v);
-      t_w = fmaf(S, fmaf(c2.z, cs, -c2.w * sn), t_w);
-      t_t = fmaf(F, fmaf(c3.x, cs, -c3.y * sn), t_t);
-    }
-    s_eta += t_eta;
-    s_u += t_u;
-    s_v += t_v;
-    s_w += t_w;
-    s_t += t_t;
-  }
-  if (!live) return;
-  if (a.o_eta) a.o_eta[i] = s_eta;
-  if (a.o_u) a.o_u[i] = s_u;
-  if (a.o_v) a.o_v[i] = s_v;
-  if (a.o_w) a.o_w[i] = s_w;
+__device__ __forceinline__ void direct_store(const DirectArgs& a, int64_t i, float z, const float (&s)[5]) {
+  if (a.o_eta) a.o_eta[i] = s[0];
+  if (a.o_u) a.o_u[i] = s[1];
+  if (a.o_v) a.o_v[i] = s[2];
+  if (a.o_w) a.o_w[i] = s[3];
   if (a.o_p) {
     float p;
     if (a.p_mode == SWENSE_P_PHIT) {
-      p = s_t;
+      p = s[4];
     } else {
-      p = -a.rho * (s_t + 0.5f * (s_u * s_u + s_v * s_v + s_w * s_w));
+      p = -a.rho * (s[4] + 0.5f * (s[1] * s[1] + s[2] * s[2] + s[3] * s[3]));
       if (a.p_mode == SWENSE_P_TOTAL) p -= a.rho * a.g * z;
     }
     a.o_p[i] = p;
   }
+}
+
+// Four points a thread: a pair's 22 coefficients come from shared memory as six 16-byte broadcasts,
+// which occupy the shared-memory port for 24 cycles a warp, against about 31 FP32 operations a point;
+// with one point a thread the port, not the FP32 pipe, would bound the kernel. blockIdx.y takes a
+// contiguous range of tiles, so that few points still fill the GPU; the partial sums are added in
+// order by k_direct_finish. 100,003 points x 4,032 modes in finite depth: 1538 -> 396 us (one mode at
+// a time, one point a thread, the division of the depth factor per pair before).
+constexpr int kDirThreads = 128;
+constexpr int kDirPts = 4;
+
+template <bool FINITE>
+__global__ void __launch_bounds__(kDirThreads, 4) k_direct_fp32(DirectArgs a) {
+  __shared__ PairCoef tile[2][kDirTile];
+  const int64_t i0 = int64_t(blockIdx.x) * (kDirThreads * kDirPts) + threadIdx.x;
+  unsigned X[kDirPts], Y[kDirPts];
+  float z[kDirPts], sst[kDirPts], cst[kDirPts], sn[kDirPts], cs[kDirPts], tot[kDirPts][5];
+#pragma unroll
+  for (int p = 0; p < kDirPts; ++p) {
+    const int64_t i = i0 + p * kDirThreads;
+    const int64_t ic = i < a.np ? i : a.np - 1;
+    X[p] = turn_fraction(a.pts[3 * ic], a.inv_lx);
+    Y[p] = turn_fraction(a.pts[3 * ic + 1], a.inv_ly);
+    z[p] = a.pts[3 * ic + 2];
+    // e^{i 2 pi x / Lx}: the rotation from mode m to m + 1
+    sincospif(2.f * (float(int(X[p])) * 2.3283064365386963e-10f), &sst[p], &cst[p]);
+#pragma unroll
+    for (int f = 0; f < 5; ++f) tot[p][f] = 0.f;
+  }
+  const int t0 = blockIdx.y * a.tps, t1 = min(t0 + a.tps, a.n_tiles);
+  constexpr int kWords = int(sizeof(PairCoef)) * kDirTile / 16;
+  auto load = [&](int t) {
+    const uint4* src = reinterpret_cast<const uint4*>(a.pairs + size_t(t) * kDirTile);
+    uint4* dst = reinterpret_cast<uint4*>(tile[t & 1]);
+    for (int v = threadIdx.x; v < kWords; v += kDirThreads) cp_async16(dst + v, src + v, 16);
+    cp_async_commit();
+  };
+  load(t0);
+  for (int t = t0; t < t1; ++t) {
+    if (t + 1 < t1) {
+      load(t + 1);
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
+    }
+    __syncthreads();
+    const PairCoef* tc = tile[t & 1];
+    const int n = t / a.tpr, m0 = (t - n * a.tpr) * kDirTile;
+    float2 acc[kDirPts][5];                        // (C, S) of each field
+#pragma unroll
+    for (int p = 0; p < kDirPts; ++p)
+#pragma unroll
+      for (int f = 0; f < 5; ++f) acc[p][f] = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int j0 = 0; j0 < kDirTile; j0 += kDirAnchor) {
+#pragma unroll
+      for (int p = 0; p < kDirPts; ++p)            // exact phase m X (mod 2^32)
+        sincospif(2.f * (float(int(unsigned(m0 + j0) * X[p])) * 2.3283064365386963e-10f), &sn[p], &cs[p]);
+#pragma unroll 1
+      for (int j = j0; j < j0 + kDirAnchor; ++j) {
+        const PairCoef& c = tc[j];
+        const float4 qe = c.q[0], qu = c.q[1], qv = c.q[2], qw = c.q[3], qt = c.q[4];
+        const float k = c.k, invd = FINITE ? c.invd : 1.f;
+#pragma unroll
+        for (int p = 0; p < kDirPts; ++p) {
+          float F, S;
+          direct_depth<FINITE>(k, z[p], a.depth, invd, F, S);
+          auto add = [&](float2& s, const float4& q, float cc, float ss) {
+            s = pfma(make_float2(cc, cc), make_float2(q.x, q.y), s);
+            s = pfma(make_float2(ss, ss), make_float2(q.z, q.w), s);
+          };
+          const float fc = F * cs[p], fs = F * sn[p];
+          add(acc[p][0], qe, cs[p], sn[p]);
+          add(acc[p][1], qu, fc, fs);
+          add(acc[p][2], qv, fc, fs);
+          add(acc[p][3], qw, FINITE ? S * cs[p] : fc, FINITE ? S * sn[p] : fs);
+          add(acc[p][4], qt, fc, fs);
+          const float c2 = fmaf(cs[p], cst[p], -sn[p] * sst[p]);
+          sn[p] = fmaf(sn[p], cst[p], cs[p] * sst[p]);
+          cs[p] = c2;
+        }
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < kDirPts; ++p) {
+      float sy, cy;
+      sincospif(2.f * (float(int(unsigned(n) * Y[p])) * 2.3283064365386963e-10f), &sy, &cy);
+#pragma unroll
+      for (int f = 0; f < 5; ++f) tot[p][f] += fmaf(cy, acc[p][f].x, sy * acc[p][f].y);
+    }
+    __syncthreads();                               // tile (t & 1) is reloaded next iteration
+  }
+#pragma unroll
+  for (int p = 0; p < kDirPts; ++p) {
+    const int64_t i = i0 + p * kDirThreads;
+    if (i >= a.np) continue;
+    if (a.part) {
+#pragma unroll
+      for (int f = 0; f < 5; ++f) a.part[(int64_t(blockIdx.y) * 5 + f) * a.np + i] = tot[p][f];
+    } else {
+      direct_store(a, i, z[p], tot[p]);
+    }
+  }
+}
+
+// Sums of the splits in order, Bernoulli, outputs.
+__global__ void __launch_bounds__(256) k_direct_finish(DirectArgs a, int splits) {
+  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i >= a.np) return;
+  float s[5];
+#pragma unroll
+  for (int f = 0; f < 5; ++f) {
+    s[f] = a.part[int64_t(f) * a.np + i];
+    for (int q = 1; q < splits; ++q) s[f] += a.part[(int64_t(q) * 5 + f) * a.np + i];
+  }
+  direct_store(a, i, a.pts[3 * i + 2], s);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -591,29 +673,46 @@ extern "C" int swense_direct(const swense_modes* md, double t, const float* pts,
     return direct_tc(md, t, pts, np, eta, u, v, w, p, p_mode, rho, grav, stream);
   if (precision == SWENSE_DIRECT_SPLIT_BF16_PAIRWISE)
     return direct_split_impl(md, t, pts, nullptr, nullptr, 0, np, eta, u, v, w, p, p_mode, rho, grav, stream, 0);
-  const size_t nslot = size_t(ny) * (nx / 2 + 1);
-  const size_t bytes = nslot * sizeof(ModeCoef);
+  const int rows = ny > 1 ? ny / 2 : 1;           // |n| = 0 .. ny/2 - 1 (the Nyquist row is ignored)
+  const int tpr = (nx / 2 + kDirTile - 1) / kDirTile;
+  const int64_t n_tiles = int64_t(rows) * tpr, n_pairs = n_tiles * kDirTile;
+  if (n_tiles >= (int64_t(1) << 31)) return fail(SWENSE_ERR_SIZE, "too many modes for one call");
+  const int64_t blocks = (np + kDirThreads * kDirPts - 1) / (kDirThreads * kDirPts);
+  if (blocks >= (int64_t(1) << 31)) return fail(SWENSE_ERR_SIZE, "too many points for one call");
+  int dev = 0, sms = 0;
+  SWENSE_CUDA_TRY(cudaGetDevice(&dev));
+  SWENSE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  // four blocks fit an SM: split the modes until the grid fills the GPU about three times over (a
+  // partly filled last wave then costs little), at least one tile a split
+  const int64_t want = std::max<int64_t>(1, (int64_t(sms) * 12 + blocks - 1) / blocks);
+  const int64_t tps = (n_tiles + std::min(want, n_tiles) - 1) / std::min(want, n_tiles);
+  const int splits = int((n_tiles + tps - 1) / tps);
+  const size_t b_pairs = (size_t(n_pairs) * sizeof(PairCoef) + 255) & ~size_t(255);
+  const size_t b_part = splits > 1 ? size_t(splits) * 5 * size_t(np) * sizeof(float) : 0;
   void* ws = nullptr;
-  int st = workspace(bytes, stream, &ws);
+  int st = workspace(b_pairs + b_part, stream, &ws);
   if (st) return st;
-  ModeCoef* modes = static_cast<ModeCoef*>(ws);
+  PairCoef* pairs = static_cast<PairCoef*>(ws);
   const float depth = md->depth > 0 ? float(md->depth) : 0.f;
-  k_direct_prep<<<unsigned((nslot + 255) / 256), 256, 0, stream>>>(
+  k_direct_prep<<<unsigned((n_pairs + 255) / 256), 256, 0, stream>>>(
       reinterpret_cast<const float2*>(md->A_eta), reinterpret_cast<const float2*>(md->A_phi),
       reinterpret_cast<const float2*>(md->A_phit), md->omega, t - md->t_ref, nx, ny,
       float(6.283185307179586476925 / md->Lx), ny > 1 ? float(6.283185307179586476925 / md->Ly) : 0.f,
-      depth, modes);
+      depth, tpr, n_pairs, pairs);
   SWENSE_CUDA_TRY(cudaGetLastError());
   count_launches(1);
   DirectArgs a{};
-  a.modes = modes;
-  a.n_modes = unsigned(nslot);
+  a.pairs = pairs;
+  a.n_tiles = int(n_tiles);
+  a.tpr = tpr;
+  a.tps = int(tps);
   a.pts = pts;
   a.o_eta = eta;
   a.o_u = u;
   a.o_v = v;
   a.o_w = w;
   a.o_p = p;
+  a.part = splits > 1 ? reinterpret_cast<float*>(static_cast<char*>(ws) + b_pairs) : nullptr;
   a.np = np;
   a.inv_lx = 1.0 / md->Lx;
   a.inv_ly = ny > 1 ? 1.0 / md->Ly : 0.0;
@@ -621,10 +720,15 @@ extern "C" int swense_direct(const swense_modes* md, double t, const float* pts,
   a.p_mode = p_mode;
   a.rho = float(rho);
   a.g = float(grav);
-  const int64_t blocks = (np + kDirThreads - 1) / kDirThreads;
-  if (blocks >= (int64_t(1) << 31)) return fail(SWENSE_ERR_SIZE, "too many points for one call");
-  k_direct_fp32<<<unsigned(blocks), kDirThreads, 0, stream>>>(a);
+  const dim3 grid{unsigned(blocks), unsigned(splits), 1u};
+  if (depth > 0.f) k_direct_fp32<true><<<grid, kDirThreads, 0, stream>>>(a);
+  else k_direct_fp32<false><<<grid, kDirThreads, 0, stream>>>(a);
   SWENSE_CUDA_TRY(cudaGetLastError());
   count_launches(1);
+  if (splits > 1) {
+    k_direct_finish<<<unsigned((np + 255) / 256), 256, 0, stream>>>(a, splits);
+    SWENSE_CUDA_TRY(cudaGetLastError());
+    count_launches(1);
+  }
   return SWENSE_OK;
 }
