@@ -124,10 +124,11 @@ typedef struct swense_grid_desc {
  * power-of-two factors only (SWENSE_ERR_UNSUPPORTED otherwise); the tuned launch shape of the
  * factor p2 is used.
  * Arithmetic: FP32 transforms, FP32 depth factors with a compensated |k| z product.
- * Uses the scratch workspace (4 * ny_r * (nx/2 + 1) complex64 per level of a level chunk, each
- * row padded to whole 128-byte lines; twice that for transform variant 5) when ny > 1. When
- * ny > 1 the eta transform runs on a second, library-owned stream, forked from `stream` and
- * joined back before the call returns, so it overlaps the level transforms. The workspace, the
+ * Uses the scratch workspace (4 * ny_r * nx/2 complex64 per level of a level chunk, each row padded
+ * to whole 128-byte lines, twice that for transform variant 5; and the modes of four fields and eta
+ * per time level) when ny > 1. For columns or rows beyond the warp-wide transforms the eta transform
+ * runs on a second, library-owned stream, forked from `stream` and joined back before the call
+ * returns, so it overlaps the level transforms. The workspace, the
  * twiddle table and the library's streams are created by the first call on a device, which must
  * not be inside a stream capture. Errors: ARG, SIZE, LEVELS, OOM, CUDA.
  */
@@ -142,8 +143,9 @@ int swense_fields_on_grid(const swense_modes* modes, int32_t n_tl, const double*
  * device memory up front in its own pool, a plugin whose host forbids allocations outside set-up,
  * or code that cannot afford the implicit device synchronisation a cudaMalloc/cudaFree may do.
  * This entry point takes the same arguments and produces the same grid as swense_fields_on_grid,
- * with the same transform kernels and launch shape (the tuned one, else the default), except that
- * the two-stream variant 5 runs as variant 2 and the eta transform stays on `stream` (no library
+ * with the same transform kernels and launch shape (the tuned one, else the default; the
+ * shared-memory path where the pair's modal fields leave no room for a level), except that
+ * the two-stream variant 5 runs as variant 0 and the eta transform stays on `stream` (no library
  * stream is used); but it allocates nothing: it calls no cudaMalloc, cudaFree or allocating
  * library routine. Its
  * scratch (the transformed levels between the two passes, and the propagated modes) lives in a
@@ -169,23 +171,21 @@ int swense_fields_on_grid_noalloc(const swense_modes* modes, int32_t n_tl, const
 
 /*
  * swense_autotune_grid — choose the launch shape of swense_fields_on_grid for this grid shape
- * (the transform path: warp-register kernels with 1, 2 or 4 levels per column-transform block,
- * or the shared-memory kernels; the level-chunk size among 16, 32, 64, 96, 128, 256 MB; and, for
- * 256- to 1024-point rows, whether one row-transform block handles both field pairs or one) by
+ * (the transform path: the wide-radix transform pair with 1, 2 or 4 levels per column-transform
+ * block, or the shared-memory kernels; the level-chunk size among 16, 32, 64, 96, 128, 256 MB; and
+ * the row pass's form) by
  * timing each candidate five times on `stream` (best of five, each from a cold L2: the
  * workspace, grown to at least 256 MB, is overwritten before each repetition); the choice is
  * cached per (nx, ny, pad_n, nz)
  * and used by later calls. No counterpart in the paper. Writes the grid (same outputs as
  * swense_fields_on_grid), synchronises the stream, must not be captured. 2-D grids have a
  * single path (nothing to tune; *lpc_out = -1).
- * lpc_out (0 = shared-memory path), chunk_bytes_out, row_variant_out (0 = both field pairs per
- * warp, 1 = one field pair per block, 2 = transposed intermediate: the row pass reads its inputs
- * straight from memory; both lengths in 256..1024; 3 = as 2 with one transform per warp;
- * 4 = as 2 with each warp's rows staged in shared memory by bulk asynchronous copies; 5 = as 2
- * with chunk c's row pass on a library-internal second stream while chunk c+1's column pass
- * runs on `stream`, two intermediate buffers, joined back before the call's work ends), plus 16
- * when the transposed pair's column pass runs one modal field per block (four times the blocks
- * per level, half the registers; the untuned default for 1024-point columns):
+ * lpc_out (0 = shared-memory path), chunk_bytes_out, row_variant_out (0 = the row pass reads the
+ * intermediate straight from memory; 4 = each warp's rows staged in shared memory by bulk
+ * asynchronous copies, 256- to 1024-point rows; 5 = as 0 with chunk c's row pass on a
+ * library-internal second stream while chunk c+1's column pass runs on `stream`, two intermediate
+ * buffers, joined back before the call's work ends; 1, 2 and 3, and 16 more than any of them, name
+ * earlier variants and run as 0):
  * host, may be NULL. Errors: as swense_fields_on_grid.
  */
 int swense_autotune_grid(const swense_modes* modes, int32_t n_tl, const double* t,
@@ -198,8 +198,8 @@ int swense_autotune_grid(const swense_modes* modes, int32_t n_tl, const double* 
  * (nx, ny, pad_n, nz), e.g. a choice that swense_autotune_grid returned in an earlier process.
  * lpc: -1 (forget any choice: untuned defaults again), 0 (shared-memory path), 1, 2 or 4 levels
  * per column block;
- * chunk_bytes in [1 MiB, 1 GiB] (L2-resident level chunk); row_variant 0..5, plus 16 for the
- * one-field column pass (as returned by swense_autotune_grid). Results do not depend on the choice beyond FP32 rounding. No
+ * chunk_bytes in [1 MiB, 1 GiB] (level chunk); row_variant 0..5, or 16 more (see
+ * swense_autotune_grid). Results do not depend on the choice beyond FP32 rounding. No
  * counterpart in the paper. Errors: SWENSE_ERR_ARG for values outside those sets.
  */
 int swense_set_grid_tune(int32_t nx, int32_t ny, int32_t pad_n, int32_t nz, int32_t lpc,

@@ -40,14 +40,15 @@ std::mutex g_mutex;
 DeviceState g_dev[kMaxDevices];
 
 // Entry j holds e^{+2 pi i e / SWENSE_MAX_FFT}, e = twiddle_exponent(j): the plain table, then the
-// pass-major tables (layout at stk_twp). Computed in FP64 with sincospi (exact argument scaling)
-// and rounded once, so each pass-major entry equals the plain entry of the same e bit for bit.
-__device__ float2 g_twiddle[kTwiddleLen];
+// pass-major tables (layout at stk_twp), then the wide passes' tables (wide_exponent). Computed in
+// FP64 with sincospi (exact argument scaling) and rounded once, so each pass-major entry equals the
+// plain entry of the same e bit for bit.
+__device__ float2 g_twiddle[kTwiddleAll];
 
 __global__ void k_fill_twiddles() {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= kTwiddleLen) return;
-  const int e = twiddle_exponent(j);
+  if (j >= kTwiddleAll) return;
+  const int e = j < kWideTw ? twiddle_exponent(j) : wide_exponent(j);
   double s, c;
   sincospi(2.0 * double(e) / double(SWENSE_MAX_FFT), &s, &c);
   g_twiddle[j] = make_float2(float(c), float(s));
@@ -109,7 +110,7 @@ int twiddles(cudaStream_t stream, const float2** out) {
       if (cap != cudaStreamCaptureStatusNone)
         return fail(SWENSE_ERR_ARG, "the first call on a device must not be inside a stream "
                                     "capture (it fills the twiddle table)");
-      k_fill_twiddles<<<(kTwiddleLen + 255) / 256, 256, 0, stream>>>();
+      k_fill_twiddles<<<(kTwiddleAll + 255) / 256, 256, 0, stream>>>();
       SWENSE_CUDA_TRY(cudaGetLastError());
       count_launches(1);
       SWENSE_CUDA_TRY(cudaStreamSynchronize(stream));

@@ -91,103 +91,6 @@ __device__ __forceinline__ float spline_prefilter(int m, int Nx, int n, int Ny) 
 namespace swense {
 
 // ------------------------------------------------------------------------------------------------
-// Warp-register inverse DFT of length N = 32 * E (E <= 32), one transform per warp.
-//
-// With n = n1 + 32 n2 (n1 = lane, n2 < E) and m = m2 + E m1 (m2 < E, m1 < 32):
-//   X[m] = sum_{n1} e^{2 pi i n1 m1 / 32} [ e^{2 pi i n1 m2 / N} sum_{n2} x[n1 + 32 n2] e^{2 pi i n2 m2 / E} ]
-// so each lane does a length-E DFT over its own elements in registers, multiplies by the
-// lane's twiddles, and the warp does E length-32 DFTs across lanes (radix-2 decimation in
-// frequency with shuffles). Lane l ends up with X[m2 + E * bitrev5(l)], m2 = 0 .. E-1: E
-// consecutive outputs, ready for a contiguous store.
-
-constexpr int ct_log2(int v) { return v <= 1 ? 0 : 1 + ct_log2(v >> 1); }
-constexpr int ct_rev(int v, int bits) {
-  int r = 0;
-  for (int b = 0; b < bits; ++b) r |= ((v >> b) & 1) << (bits - 1 - b);
-  return r;
-}
-
-// Per-lane constants of one transform size (kernel-lifetime registers).
-template <int E>
-struct WarpFftTw {
-  float2 wE[E > 1 ? E / 2 : 1];   // e^{2 pi i j / E}, j < E/2
-  float2 w2[E];                   // e^{2 pi i lane m2 / N}
-  float2 ws[5];                   // e^{2 pi i (lane mod s) / (2 s)}, s = 16, 8, 4, 2, 1
-};
-
-template <int E>
-__device__ __forceinline__ void warp_fft_init(WarpFftTw<E>& T, const float2* __restrict__ tw, int lane) {
-  constexpr int N = 32 * E;
-#pragma unroll
-  for (int j = 0; j < (E > 1 ? E / 2 : 1); ++j) T.wE[j] = __ldg(&tw[j * (SWENSE_MAX_FFT / (E > 1 ? E : 2))]);
-#pragma unroll
-  for (int m2 = 0; m2 < E; ++m2) T.w2[m2] = __ldg(&tw[(lane * m2) * (SWENSE_MAX_FFT / N)]);
-#pragma unroll
-  for (int st = 0; st < 5; ++st) {
-    const int s = 16 >> st;
-    T.ws[st] = __ldg(&tw[(lane % s) * (SWENSE_MAX_FFT / (2 * s))]);
-  }
-}
-
-// In-register length-E inverse DFT, natural order in and out (iterative radix-2 DIT).
-template <int E>
-__device__ __forceinline__ void dft_reg(float2 (&v)[E], const float2 (&wE)[E > 1 ? E / 2 : 1]) {
-  constexpr int B = ct_log2(E);
-#pragma unroll
-  for (int i = 0; i < E; ++i) {
-    const int j = ct_rev(i, B);
-    if (j > i) {
-      const float2 t = v[i];
-      v[i] = v[j];
-      v[j] = t;
-    }
-  }
-#pragma unroll
-  for (int len = 2; len <= E; len <<= 1) {
-    const int half = len >> 1;
-#pragma unroll
-    for (int i = 0; i < E; i += len) {
-#pragma unroll
-      for (int j = 0; j < half; ++j) {
-        const float2 b = v[i + j + half];
-        const float2 t = j == 0 ? b : cmul(wE[j * (E / len)], b);
-        v[i + j + half] = csub(v[i + j], t);
-        v[i + j] = cadd(v[i + j], t);
-      }
-    }
-  }
-}
-
-// Full warp transform: register DFT, lane twiddles, cross-lane length-32 DFT.
-template <int E>
-__device__ __forceinline__ void warp_fft(float2 (&v)[E], const WarpFftTw<E>& T, int lane) {
-  dft_reg<E>(v, T.wE);
-#pragma unroll
-  for (int m2 = 1; m2 < E; ++m2) v[m2] = cmul(v[m2], T.w2[m2]);
-#pragma unroll
-  for (int st = 0; st < 5; ++st) {
-    const int s = 16 >> st;
-    // lower lane: v + o; upper lane: (o - v) * w. Written as (o + sgn v) * w with sgn = -1 and
-    // w = ws on upper lanes, sgn = +1 and w = 1 on lower lanes (no branch, no select per element)
-    const bool upper = (lane & s) != 0;
-    const float sgn = upper ? -1.f : 1.f;
-    const float2 w = upper ? T.ws[st] : make_float2(1.f, 0.f);
-#pragma unroll
-    for (int m = 0; m < E; ++m) {
-      float2 o;
-      o.x = __shfl_xor_sync(0xffffffffu, v[m].x, s);
-      o.y = __shfl_xor_sync(0xffffffffu, v[m].y, s);
-      const float2 r = make_float2(fmaf(sgn, v[m].x, o.x), fmaf(sgn, v[m].y, o.y));
-      v[m] = s > 1 ? cmul(r, w) : r;
-    }
-  }
-}
-
-}  // namespace swense
-
-namespace swense {
-
-// ------------------------------------------------------------------------------------------------
 // Per-warp Stockham inverse DFT of length N = 32 E (8 <= E <= 64), radix-8 passes followed by one
 // radix-4 or radix-2 pass when log2 N is not a multiple of 3 (Stockham autosort: natural order in
 // and out). Butterfly j of a pass with radix R after NS points have been combined reads
@@ -501,5 +404,179 @@ __device__ __forceinline__ void stkb_fft2(float2 (&v1)[N / TH], float2 (&v2)[N /
   static_assert(N / 8 >= TH, "constant index parts are multiples of the thread count");
   stkb_pass2<N, TH, 0>(v1, v2, tw, buf1, buf2, t);
 }
+
+}  // namespace swense
+
+namespace swense {
+
+// ------------------------------------------------------------------------------------------------
+// Wide-radix inverse DFTs in two or three Stockham passes: N = R0 R1 (R2), with R0 elements a thread.
+// A 16- or 32-point DFT in registers replaces two or three radix-8/-4 passes and their exchanges, so a
+// transform of up to 1024 points goes through shared memory once and one of 2048 points twice.
+// Pass p with stride NS and radix R: butterfly j reads x[j + r N/R], multiplies by
+// e^{2 pi i (j mod NS) r / (NS R)} and writes y[(j / NS) NS R + (j mod NS) + r NS].
+
+// cos(2 pi j / 32)
+__host__ __device__ constexpr double root32_cos(int j) {
+  j &= 31;
+  if (j > 16) j = 32 - j;
+  const bool neg = j > 8;
+  if (neg) j = 16 - j;
+  const double c = j == 0   ? 1.0
+                   : j == 1 ? 0.98078528040323044913
+                   : j == 2 ? 0.92387953251128675613
+                   : j == 3 ? 0.83146961230254523708
+                   : j == 4 ? 0.70710678118654752440
+                   : j == 5 ? 0.55557023301960222474
+                   : j == 6 ? 0.38268343236508977173
+                   : j == 7 ? 0.19509032201612826785
+                            : 0.0;
+  return neg ? -c : c;
+}
+// v e^{2 pi i j / 32}, j a constant after unrolling
+__device__ __forceinline__ float2 rot32(float2 v, int j) {
+  j &= 31;
+  if (j == 0) return v;
+  if (j == 8) return make_float2(-v.y, v.x);
+  if (j == 16) return make_float2(-v.x, -v.y);
+  if (j == 24) return make_float2(v.y, -v.x);
+  const float c = float(root32_cos(j)), s = float(root32_cos(j - 8));
+  if (j == 4) return make_float2(c * (v.x - v.y), c * (v.x + v.y));
+  if (j == 12) return make_float2(c * (v.x + v.y), c * (v.y - v.x));
+  return cmul(v, make_float2(c, s));
+}
+
+// In-register DFT of v[0 .. R-1]; X[k] is left in v[dft_slot<R>(k)].
+template <int R>
+__host__ __device__ constexpr int dft_slot(int k) {
+  return R == 32 ? 4 * (k % 8) + k / 8 : R == 16 ? 4 * (k % 4) + k / 4 : k;
+}
+template <int R>
+__device__ __forceinline__ void wide_dft(float2* v) {
+  if constexpr (R == 2) {
+    stk_dft2(v);
+  } else if constexpr (R == 4) {
+    stk_dft4(v[0], v[1], v[2], v[3]);
+  } else if constexpr (R == 8) {
+    stk_dft8(v);
+  } else {
+    // R = 4 Q, n = n2 + 4 n1, k = k1 + Q k2: Q-point DFTs over n1, twiddles W_R^{n2 k1}, 4-point over n2
+    static_assert(R == 16 || R == 32, "register DFT sizes");
+    constexpr int Q = R / 4;
+#pragma unroll
+    for (int n2 = 0; n2 < 4; ++n2) {
+      if constexpr (Q == 4) {
+        stk_dft4(v[n2], v[n2 + 4], v[n2 + 8], v[n2 + 12]);
+      } else {
+        float2 t[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) t[i] = v[n2 + 4 * i];
+        stk_dft8(t);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[n2 + 4 * i] = t[i];
+      }
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < Q; ++k1) {
+#pragma unroll
+      for (int n2 = 1; n2 < 4; ++n2) v[n2 + 4 * k1] = rot32(v[n2 + 4 * k1], n2 * k1 * (32 / R));
+      stk_dft4(v[4 * k1], v[4 * k1 + 1], v[4 * k1 + 2], v[4 * k1 + 3]);
+    }
+  }
+}
+
+// Factors of the first two passes' product of length N = R0 R1 (32 <= N <= 1024): entry
+// kWideTw + N + r R0 + j holds e^{2 pi i j r / N} (j < R0). Third pass (stride 256, radix N / 256,
+// N = 512 .. 2048): entry kWideTw3 + N + 256 r + j holds e^{2 pi i j r / N} (j < 256).
+// R0 of a column transform; rows use 16 x 16 passes from 256 points on (wide_r0 for N <= 256).
+constexpr int wide_r0(int n) { return n >= 512 ? 32 : (n >= 128 ? 16 : 8); }
+constexpr int kWideTw = kTwiddleLen, kWideTw3 = kWideTw + 2048, kTwiddleAll = kWideTw3 + 4096;
+__host__ __device__ constexpr int wide_exponent(int i) {          // of twiddle entry i >= kWideTw
+  const bool third = i >= kWideTw3;
+  const int o = i - (third ? kWideTw3 : kWideTw);
+  int n = 1;
+  while (2 * n <= o) n *= 2;                       // slot o lies in [n, 2n)
+  if (n < 32 || n > (third ? 2048 : 1024) || (third && n < 512)) return 0;
+  const int q = third ? 256 : wide_r0(n);
+  return ((o - n) % q) * ((o - n) / q) * (SWENSE_MAX_FFT / n);
+}
+
+// Two row transforms side by side by T = N / R0 threads (t = 0 .. T-1): element e of thread t holds
+// position t + T e on entry, and element wide_row_elem(b, r) position wide_row_pos(t, b, r) on exit.
+// Both buffers are padded by one element in R0, which makes every exchange conflict-free.
+template <int N>
+struct WideRow {
+  static constexpr int R0 = N >= 128 ? 16 : 8, R1 = N >= 256 ? 16 : N / R0, R2 = N / (R0 * R1);
+  static constexpr int E = R0, T = N / E, RL = R2 > 1 ? R2 : R1, BL = E / RL;
+  static constexpr int kBuf = N + N / R0;
+  static constexpr int kRows = T >= 128 ? 1 : 128 / T;            // rows per 128-thread block
+  __device__ static __forceinline__ int elem(int b, int r) { return b * RL + dft_slot<RL>(r); }
+  __device__ static __forceinline__ int pos(int t, int b, int r) { return t + T * b + (N / RL) * r; }
+  __device__ static __forceinline__ void sync() {
+    if constexpr (T <= 32) __syncwarp();
+    else __syncthreads();
+  }
+  __device__ static __forceinline__ void fft2(float2 (&z1)[E], float2 (&z2)[E], const float2* __restrict__ tw,
+                                              float2* b1, float2* b2, int t) {
+    wide_dft<R0>(z1);
+    wide_dft<R0>(z2);
+#pragma unroll
+    for (int r = 0; r < R0; ++r) {
+      b1[t * (R0 + 1) + r] = z1[dft_slot<R0>(r)];
+      b2[t * (R0 + 1) + r] = z2[dft_slot<R0>(r)];
+    }
+    sync();
+    constexpr int B1 = E / R1, S1 = N / R1;        // S1 is a multiple of R0: the pad index splits
+#pragma unroll
+    for (int b = 0; b < B1; ++b) {
+      const int jj = t + T * b, base = jj + jj / R0;
+#pragma unroll
+      for (int r = 0; r < R1; ++r) {
+        z1[b * R1 + r] = b1[base + r * (S1 + S1 / R0)];
+        z2[b * R1 + r] = b2[base + r * (S1 + S1 / R0)];
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < B1; ++b) {
+      const int jm = (t + T * b) % R0;
+#pragma unroll
+      for (int r = 1; r < R1; ++r) {
+        const float2 w = __ldg(&tw[kWideTw + R0 * R1 + r * R0 + jm]);
+        z1[b * R1 + r] = cmul(z1[b * R1 + r], w);
+        z2[b * R1 + r] = cmul(z2[b * R1 + r], w);
+      }
+      wide_dft<R1>(&z1[b * R1]);
+      wide_dft<R1>(&z2[b * R1]);
+    }
+    if constexpr (R2 > 1) {
+      static_assert(R2 == 1 || (R0 == 16 && R1 == 16), "three passes start with 16 x 16");
+      sync();                                      // every thread has read the first exchange
+      const int wb = (t / 16) * 272 + t % 16;
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        b1[wb + 17 * r] = z1[dft_slot<16>(r)];
+        b2[wb + 17 * r] = z2[dft_slot<16>(r)];
+      }
+      sync();
+#pragma unroll
+      for (int b = 0; b < BL; ++b) {
+        const int jj = t + T * b, base = jj + jj / 16;
+#pragma unroll
+        for (int r = 0; r < R2; ++r) {
+          z1[b * R2 + r] = b1[base + 272 * r];
+          z2[b * R2 + r] = b2[base + 272 * r];
+        }
+#pragma unroll
+        for (int r = 1; r < R2; ++r) {
+          const float2 w = __ldg(&tw[kWideTw3 + N + 256 * r + jj]);
+          z1[b * R2 + r] = cmul(z1[b * R2 + r], w);
+          z2[b * R2 + r] = cmul(z2[b * R2 + r], w);
+        }
+        wide_dft<R2>(&z1[b * R2]);
+        wide_dft<R2>(&z2[b * R2]);
+      }
+    }
+  }
+};
 
 }  // namespace swense

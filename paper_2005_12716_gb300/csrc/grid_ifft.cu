@@ -14,7 +14,8 @@
 //           to nx_r), inverse-transform along x and store float4 (u, v, w, dphi/dt) per node.
 // Level chunks are sized so G stays L2-resident between the passes. eta is one extra transform
 // per time level (pass A on A^eta; pass B packs two grid rows per complex transform).
-// 2-D (ny == 1): pass B alone, reading the modes directly.
+// Transforms of 32 to 1024 points along y and 32 points and more along x run as a wide-radix pair over
+// a transposed intermediate instead (k_col_w, k_row_w). 2-D (ny == 1): one kernel (k_line).
 #include <algorithm>
 #include <array>
 #include <cmath>
@@ -107,13 +108,10 @@ __global__ void __launch_bounds__(256) k_pass_a(PassAArgs a, Levels L) {
   }
 }
 
-enum { B_LEVEL_G = 0, B_LEVEL_DIRECT = 1, B_ETA_G = 2, B_ETA_DIRECT = 3 };
+enum { B_LEVEL_G = 0, B_ETA_G = 1 };
 
 struct PassBArgs {
   const float2* G;        // pass-A output (levels or eta)
-  const float2* A_phi;    // direct mode (ny == 1): modes of this time level
-  const float2* A_phit;
-  const float2* A_eta;
   float4* nodes;          // [nz][Nyr][Nxr] of this time level
   float* eta;             // [Nyr][Nxr] of this time level
   const float2* tw;
@@ -121,8 +119,6 @@ struct PassBArgs {
   int rb;                 // rows (level modes) or row pairs (eta modes) per CTA
   int lev0;
   int mode;
-  float kxs, depth;
-  int spline;
 };
 
 // Hermitian packing of two one-sided spectra P, Q (coefficients of real fields p, q) into one
@@ -136,43 +132,24 @@ __device__ __forceinline__ void pack_pair(float2* Z, int m, int Nxr, int log2Nxr
   }
 }
 
-__global__ void __launch_bounds__(256) k_pass_b(PassBArgs a, Levels L) {
+__global__ void __launch_bounds__(256) k_pass_b(PassBArgs a) {
   extern __shared__ float2 sm[];
   const int slot = blockIdx.y;
-  const bool eta_mode = a.mode >= B_ETA_G;
+  const bool eta_mode = a.mode == B_ETA_G;
   const int rows_per_cta = eta_mode ? 2 * a.rb : a.rb;
   const int y0 = blockIdx.x * rows_per_cta;
   const int narr = eta_mode ? a.rb : 2 * a.rb;
   for (int i = threadIdx.x; i < narr * a.Nxr; i += blockDim.x) sm[i] = make_float2(0.f, 0.f);
   __syncthreads();
   if (!eta_mode) {
-    const float z = L.z[a.lev0 + slot];
     for (int i = threadIdx.x; i < a.rb * a.Mh; i += blockDim.x) {
       const int m = i % a.Mh, rr = i / a.Mh;
       const int y = y0 + rr;
       if (y >= a.Nyr) continue;
-      float2 U, V, W, T;
-      if (a.mode == B_LEVEL_G) {
-        const size_t base = (size_t(slot) * 4 * a.Nyr + y) * a.Mh + m;
-        const size_t fs = size_t(a.Nyr) * a.Mh;
-        U = __ldcg(&a.G[base]);
-        V = __ldcg(&a.G[base + fs]);
-        W = __ldcg(&a.G[base + 2 * fs]);
-        T = __ldcg(&a.G[base + 3 * fs]);
-      } else {
-        const float pf = a.spline ? spline_prefilter(m, a.Nxr, 0, 1) : 1.f;
-        float2 Ap = __ldg(&a.A_phi[m]);
-        float2 At = __ldg(&a.A_phit[m]);
-        Ap = make_float2(pf * Ap.x, pf * Ap.y);
-        At = make_float2(pf * At.x, pf * At.y);
-        const float kx = float(m) * a.kxs;
-        float F, S;
-        depth_factors(kx, z, a.depth, F, S);
-        U = make_float2(-kx * F * Ap.y, kx * F * Ap.x);
-        V = make_float2(0.f, 0.f);
-        W = make_float2(kx * S * Ap.x, kx * S * Ap.y);
-        T = make_float2(F * At.x, F * At.y);
-      }
+      const size_t base = (size_t(slot) * 4 * a.Nyr + y) * a.Mh + m;
+      const size_t fs = size_t(a.Nyr) * a.Mh;
+      const float2 U = __ldcg(&a.G[base]), V = __ldcg(&a.G[base + fs]);
+      const float2 W = __ldcg(&a.G[base + 2 * fs]), T = __ldcg(&a.G[base + 3 * fs]);
       pack_pair(sm + size_t(2 * rr) * a.Nxr, m, a.Nxr, a.log2Nxr, U, V);
       pack_pair(sm + size_t(2 * rr + 1) * a.Nxr, m, a.Nxr, a.log2Nxr, W, T);
     }
@@ -181,15 +158,8 @@ __global__ void __launch_bounds__(256) k_pass_b(PassBArgs a, Levels L) {
       const int m = i % a.Mh, pp = i / a.Mh;
       const int ya = y0 + 2 * pp, yb = ya + 1;
       if (ya >= a.Nyr) continue;
-      float2 Ea, Eb = make_float2(0.f, 0.f);
-      if (a.mode == B_ETA_G) {
-        Ea = __ldcg(&a.G[size_t(ya) * a.Mh + m]);
-        if (yb < a.Nyr) Eb = __ldcg(&a.G[size_t(yb) * a.Mh + m]);
-      } else {
-        const float pf = a.spline ? spline_prefilter(m, a.Nxr, 0, 1) : 1.f;
-        Ea = __ldg(&a.A_eta[m]);
-        Ea = make_float2(pf * Ea.x, pf * Ea.y);
-      }
+      const float2 Ea = __ldcg(&a.G[size_t(ya) * a.Mh + m]);
+      const float2 Eb = yb < a.Nyr ? __ldcg(&a.G[size_t(yb) * a.Mh + m]) : make_float2(0.f, 0.f);
       pack_pair(sm + size_t(pp) * a.Nxr, m, a.Nxr, a.log2Nxr, Ea, Eb);
     }
   }
@@ -203,9 +173,7 @@ __global__ void __launch_bounds__(256) k_pass_b(PassBArgs a, Levels L) {
       if (y >= a.Nyr) continue;
       const float2 z1 = sm[size_t(2 * rr) * a.Nxr + x];
       const float2 z2 = sm[size_t(2 * rr + 1) * a.Nxr + x];
-      // 2-D: v is identically zero (the imaginary part of z1 holds only round-off)
-      const float v = a.mode == B_LEVEL_DIRECT ? 0.f : z1.y;
-      __stcs(&out[size_t(y) * a.Nxr + x], make_float4(z1.x, v, z2.x, z2.y));
+      __stcs(&out[size_t(y) * a.Nxr + x], make_float4(z1.x, z1.y, z2.x, z2.y));
     }
   } else {
     for (int i = threadIdx.x; i < a.rb * a.Nxr; i += blockDim.x) {
@@ -243,12 +211,123 @@ __global__ void k_propagate(const float2* __restrict__ Ae, const float2* __restr
         make_float2(fmaf(src[q].x, c, src[q].y * s), fmaf(src[q].y, c, -src[q].x * s));
 }
 
+// A 2-D (x, z) request in one launch: block (l, tl) propagates the one row of modes to time level tl
+// (as k_propagate), forms level l's spectra Z1 = U and Z2 = W + iT (v is identically zero), l = nz:
+// eta's, and transforms them in shared memory. Rows are short (256 modes in the regular-wave runs), so
+// launches bound the request: five serial ones took 27 us, this one takes 5 us.
+struct LineArgs {
+  const float2 *Ae, *Ap, *At;
+  const double* omega;
+  float4* nodes;          // [n_tl][nz][Nxr]
+  float* eta;             // [n_tl][Nxr]
+  const float2* tw;
+  int nxh1, Mh, Nxr, log2Nxr, nz, spline;
+  float kxs, depth;
+};
+__global__ void __launch_bounds__(256) k_line(LineArgs a, const __grid_constant__ Levels L,
+                                              const __grid_constant__ PropTimes T) {
+  extern __shared__ float2 sm[];                 // Z1, Z2 (bit-reversed, then transformed in place)
+  const int l = blockIdx.x, tl = blockIdx.y;
+  const bool is_eta = l == a.nz;
+  const int narr = is_eta ? 1 : 2;
+  float2 *Z1 = sm, *Z2 = sm + a.Nxr;
+  for (int i = threadIdx.x; i < narr * a.Nxr; i += blockDim.x) sm[i] = make_float2(0.f, 0.f);
+  __syncthreads();
+  const float z = is_eta ? 0.f : L.z[l];
+  const float2 zero = make_float2(0.f, 0.f);
+  for (int m = threadIdx.x; m < a.Mh; m += blockDim.x) {
+    const size_t src = a.omega ? m : size_t(tl) * a.nxh1 + m;
+    float c = 1.f, s = 0.f;
+    if (a.omega) {
+      const double turns = a.omega[m] * T.dt[tl] * 0.15915494309189533577;  // theta / (2 pi)
+      sincospif(2.f * float(turns - rint(turns)), &s, &c);
+    }
+    const float pf = a.spline ? spline_prefilter(m, a.Nxr, 0, 1) : 1.f;
+    auto mode = [&](const float2* A) {
+      float2 v = __ldg(&A[src]);
+      if (a.omega) v = make_float2(fmaf(v.x, c, v.y * s), fmaf(v.y, c, -v.x * s));
+      return make_float2(pf * v.x, pf * v.y);
+    };
+    if (is_eta) {
+      pack_pair(Z1, m, a.Nxr, a.log2Nxr, mode(a.Ae), zero);
+      continue;
+    }
+    const float2 Ap = mode(a.Ap), At = mode(a.At);
+    const float kx = float(m) * a.kxs;
+    float F, S;
+    depth_factors(kx, z, a.depth, F, S);
+    pack_pair(Z1, m, a.Nxr, a.log2Nxr, make_float2(-kx * F * Ap.y, kx * F * Ap.x), zero);
+    pack_pair(Z2, m, a.Nxr, a.log2Nxr, make_float2(kx * S * Ap.x, kx * S * Ap.y), make_float2(F * At.x, F * At.y));
+  }
+  __syncthreads();
+  fft_inv_inplace(sm, a.Nxr, a.log2Nxr, narr, a.tw);
+  if (is_eta) {
+    float* out = a.eta + size_t(tl) * a.Nxr;
+    for (int x = threadIdx.x; x < a.Nxr; x += blockDim.x) __stcs(&out[x], Z1[x].x);
+  } else {
+    float4* out = a.nodes + (size_t(tl) * a.nz + l) * a.Nxr;
+    for (int x = threadIdx.x; x < a.Nxr; x += blockDim.x)
+      __stcs(&out[x], make_float4(Z1[x].x, 0.f, Z2[x].x, Z2[x].y));
+  }
+}
+
+// Modal fields at z = 0 of every time level (blockIdx.y) for the transposed pair's column pass:
+// U = i kx A^phi, V = i ky A^phi, W = |k| A^phi, T = A^phit, propagated to the level's time (omega given,
+// as in k_propagate; otherwise snapshot blockIdx.y) and with the spline prefilter; made
+// once, where the column pass would make each at every vertical level. eta's modes come fifth,
+// [tl][5][ny][ld], or (eta non-NULL: its own transform follows, which prefilters itself) are only
+// propagated, [tl][ny][nx/2+1].
+struct FormArgs {
+  const float2 *Ae, *Ap, *At;
+  const double* omega;
+  float2 *eta, *fields;
+  int ny, nxh1, ld, Nxr, Nyr, spline;
+  float kxs, kys;
+};
+__global__ void __launch_bounds__(256) k_form_modes(FormArgs a, PropTimes T) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, nslot = a.ny * a.nxh1;
+  if (i >= nslot) return;
+  const int r = i / a.nxh1, m = i - r * a.nxh1, tl = blockIdx.y;
+  float2 e, p, t;
+  if (a.omega) {
+    const double turns = a.omega[i] * T.dt[tl] * 0.15915494309189533577;  // theta / (2 pi)
+    const double frac = turns - rint(turns);
+    float s, c;
+    sincospif(2.f * float(frac), &s, &c);
+    auto turn = [&](float2 v) { return make_float2(fmaf(v.x, c, v.y * s), fmaf(v.y, c, -v.x * s)); };
+    e = turn(__ldg(&a.Ae[i]));
+    p = turn(__ldg(&a.Ap[i]));
+    t = turn(__ldg(&a.At[i]));
+    if (a.eta) a.eta[size_t(tl) * nslot + i] = e;
+  } else {
+    e = __ldg(&a.Ae[size_t(tl) * nslot + i]);
+    p = __ldg(&a.Ap[size_t(tl) * nslot + i]);
+    t = __ldg(&a.At[size_t(tl) * nslot + i]);
+  }
+  if (m >= a.nxh1 - 1) return;                     // the Nyquist column carries no mode
+  const int n = r < a.ny / 2 ? r : r - a.ny;
+  if (a.spline) {
+    const float pf = spline_prefilter(m, a.Nxr, n, a.Nyr);
+    e = make_float2(pf * e.x, pf * e.y);
+    p = make_float2(pf * p.x, pf * p.y);
+    t = make_float2(pf * t.x, pf * t.y);
+  }
+  const float kx = float(m) * a.kxs, ky = float(n) * a.kys, k = sqrtf(kx * kx + ky * ky);
+  const size_t fs = size_t(a.ny) * a.ld;
+  float2* o = a.fields + size_t(tl) * 5 * fs + size_t(r) * a.ld + m;
+  o[0] = make_float2(-kx * p.y, kx * p.x);
+  o[fs] = make_float2(-ky * p.y, ky * p.x);
+  o[2 * fs] = make_float2(k * p.x, k * p.y);
+  o[3 * fs] = t;
+  o[4 * fs] = e;
+}
+
 constexpr int kThreads = 256;
 constexpr size_t kSmemBudget = 64 * 1024;
-constexpr size_t kChunkBytes = size_t(64) << 20;
-constexpr int kColBlock = 8;    // kx columns per column-transform CTA
-constexpr int kColLevels = 2;   // levels per column-transform CTA
-constexpr int kRowBlock = 8;    // grid rows per row-transform CTA (one per warp)
+// Level chunks of 256 MB: a pass then has whole waves of blocks (2048 x 1024 modes: 9.5 ms for 256
+// levels, against 10.3 at 64 MB and 11.8 at 32 MB), which outweighs an intermediate that stays in L2.
+constexpr size_t kChunkBytes = size_t(256) << 20;
+constexpr int kColLevels = 1;   // levels per column-transform CTA
 
 int set_smem(const void* fn, size_t bytes) {
   SWENSE_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
@@ -256,366 +335,28 @@ int set_smem(const void* fn, size_t bytes) {
 }
 
 
-// ------------------------------------------------------------------------------------------------
-// Warp-register path for 32 <= ny_r, nx_r <= 1024 (one transform per warp, no shared-memory
-// butterflies). Intermediate layout G2[level][field][m][y] (y contiguous): a column transform
-// writes its warp's outputs as contiguous runs; the row kernel stages rb rows of all m.
-
-// 8-byte asynchronous global -> shared copy (zero-filled when src_bytes == 0).
-__device__ __forceinline__ void cp_async8(void* smem, const void* gmem, int src_bytes) {
-  const unsigned d = unsigned(__cvta_generic_to_shared(smem));
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(gmem), "r"(src_bytes));
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-}
-
 struct ColArgs {
-  const float2* A_phi;   // [ny][nxh1] of this time level
-  const float2* A_phit;
-  float2* G;             // [nlev][4][Mh][Nyr]
+  const float2* A;       // [n_tl][5][ny][ldG] modal fields at z = 0 and eta (k_form_modes)
+  float2* G;             // [nslot][4][Nyr][ldG]
   const float2* tw;
-  int ny, nxh1, Mh, Nyr;
-  int cb, lpc;           // kx columns and levels per CTA
-  int lev0, nlev;        // chunk
+  int ny, Mh, Nyr, nz;
+  int lpc;               // slots per CTA
+  int lev0, nlev;        // chunk: first slot and slots. Slot tl nz + l is level l of time level tl
+  int n_lev;             // n_tl nz; slot n_lev + tl is eta of time level tl
   float kxs, kys, depth;
-  int Nxr, spline;
-  int ldG;               // m stride of the transposed intermediate (k_col_t)
+  int ldG;               // m stride of the modal fields and of the transposed intermediate
 };
 
-// Modal field q at (kx, ky, |k|) with depth factors F, S: U = i kx F A, V = i ky F A,
-// W = |k| S A, T = F A_t.
-__device__ __forceinline__ float2 modal_field(int q, float kx, float ky, float k, float F, float S,
-                                              float2 Ap, float2 At) {
-  if (q == 0) return make_float2(-kx * F * Ap.y, kx * F * Ap.x);
-  if (q == 1) return make_float2(-ky * F * Ap.y, ky * F * Ap.x);
-  if (q == 2) return make_float2(k * S * Ap.x, k * S * Ap.y);
-  return make_float2(F * At.x, F * At.y);
-}
-
-template <int E, int NF>
-__global__ void __launch_bounds__(256, 2) k_col_fft(ColArgs a, Levels L) {
-  extern __shared__ float2 sm[];                 // [2][ny][cb + 1]
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c0 = blockIdx.x * kColBlock;
-  const int ncol = min(kColBlock, a.Mh - c0);
-  const int ld = kColBlock + 1;
-  for (int i = threadIdx.x; i < a.ny * kColBlock; i += blockDim.x) {
-    const int c = i % kColBlock, r = i / kColBlock;
-    const bool ok = c < ncol;
-    const size_t gi = ok ? size_t(r) * a.nxh1 + c0 + c : 0;
-    cp_async8(&sm[r * ld + c], &a.A_phi[gi], ok ? 8 : 0);
-    cp_async8(&sm[(a.ny + r) * ld + c], &a.A_phit[gi], ok ? 8 : 0);
-  }
-  WarpFftTw<E> T;
-  warp_fft_init<E>(T, a.tw, lane);
-  cp_async_wait_all();
-  __syncthreads();
-  const int nyh = a.ny >> 1;
-  const int groups = 4 / NF;
-  const int ntask = a.lpc * kColBlock * groups;
-  for (int task = warp; task < ntask; task += blockDim.x >> 5) {
-    const int g = task % groups;
-    const int rest = task / groups;
-    const int c = rest % kColBlock;
-    const int level = blockIdx.y * a.lpc + rest / kColBlock;
-    if (c >= ncol || level >= a.nlev) continue;
-    const float z = L.z[a.lev0 + level];
-    const int m = c0 + c;
-    const float kx = float(m) * a.kxs;
-    float2 v[NF][E];
-#pragma unroll
-    for (int k = 0; k < E; ++k) {
-      const int p = lane + 32 * k;
-      int n;
-      bool live = true;
-      if (p < nyh) n = p;
-      else if (p > a.Nyr - nyh) n = p - a.Nyr;
-      else { n = 0; live = false; }
-      float2 Ap = make_float2(0.f, 0.f), At = make_float2(0.f, 0.f);
-      if (live) {
-        const int r = n >= 0 ? n : a.ny + n;
-        Ap = sm[r * ld + c];
-        At = sm[(a.ny + r) * ld + c];
-        if (a.spline) {
-          const float pf = spline_prefilter(m, a.Nxr, n, a.Nyr);
-          Ap = make_float2(pf * Ap.x, pf * Ap.y);
-          At = make_float2(pf * At.x, pf * At.y);
-        }
-      }
-      const float ky = float(n) * a.kys;
-      const float kk = sqrtf(kx * kx + ky * ky);
-      float F, S;
-      depth_factors(kk, z, a.depth, F, S);
-#pragma unroll
-      for (int f = 0; f < NF; ++f) v[f][k] = modal_field(g * NF + f, kx, ky, kk, F, S, Ap, At);
-    }
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      warp_fft<E>(v[f], T, lane);
-      float2* out = a.G + ((size_t(level) * 4 + g * NF + f) * a.Mh + m) * a.Nyr +
-                    E * int(bitrev(unsigned(lane), 5));
-#pragma unroll
-      for (int m2 = 0; m2 < E; m2 += 2) {
-        if (E == 1) {
-          out[0] = v[f][0];
-        } else {
-          __stcg(reinterpret_cast<float4*>(out + m2),
-                 make_float4(v[f][m2].x, v[f][m2].y, v[f][m2 + 1].x, v[f][m2 + 1].y));
-        }
-      }
-    }
-  }
-}
-
 struct RowArgs {
-  const float2* G;       // [nlev][4][Mh][Nyr]
-  float4* nodes;         // [nz][Nyr][Nxr] of this time level
+  const float2* G;       // [nslot][4][Nyr][ldG]
+  float4* nodes;         // [n_tl nz][Nyr][Nxr]
+  float* eta;            // [n_tl][Nyr][Nxr] (k_row_w)
   const float2* tw;
-  int Mh, Nxr, Nyr, rb, lev0;
-  int ldG;               // m stride of the transposed intermediate (k_row_t)
+  int Mh, Nxr, Nyr, lev0, n_lev;
+  int ldG;               // m stride of the transposed intermediate
   int polls;             // k_row_tma: polls of a bounded wait before it gives up
   int selftest;          // k_row_tma: 1 = issue no copy, so every wait runs out (self-test)
 };
-
-template <int E>
-__global__ void __launch_bounds__(256, 2) k_row_fft(RowArgs a) {
-  extern __shared__ float2 sm[];                 // [4][Mh][rb + 1]
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int y0 = blockIdx.x * kRowBlock;
-  const int level = blockIdx.y;
-  const int ld = kRowBlock + 1;
-  const float2* G = a.G + size_t(level) * 4 * a.Mh * a.Nyr;
-  for (int i = threadIdx.x; i < 4 * a.Mh * kRowBlock; i += blockDim.x) {
-    const int rr = i % kRowBlock, qm = i / kRowBlock;
-    const int y = y0 + rr;
-    cp_async8(&sm[qm * ld + rr], &G[size_t(qm) * a.Nyr + (y < a.Nyr ? y : 0)], y < a.Nyr ? 8 : 0);
-  }
-  WarpFftTw<E> T;
-  warp_fft_init<E>(T, a.tw, lane);
-  cp_async_wait_all();
-  __syncthreads();
-  for (int rr = warp; rr < kRowBlock; rr += blockDim.x >> 5) {
-    const int y = y0 + rr;
-    if (y >= a.Nyr) break;
-    float2 z1[E], z2[E];
-    const size_t fs = size_t(a.Mh) * ld;
-#pragma unroll
-    for (int k = 0; k < E; ++k) {
-      const int p = lane + 32 * k;
-      int m = -1;
-      bool mirror = false;
-      if (p < a.Mh) m = p;
-      else if (p > a.Nxr - a.Mh) { m = a.Nxr - p; mirror = true; }
-      float2 U = make_float2(0.f, 0.f), V = U, W = U, Tt = U;
-      if (m >= 0) {
-        const size_t o = size_t(m) * ld + rr;
-        U = sm[o];
-        V = sm[o + fs];
-        W = sm[o + 2 * fs];
-        Tt = sm[o + 3 * fs];
-      }
-      // Hermitian packing of two real fields into one complex spectrum (p + i q)
-      if (p == 0) {
-        z1[k] = make_float2(U.x, V.x);
-        z2[k] = make_float2(W.x, Tt.x);
-      } else if (!mirror) {
-        z1[k] = make_float2(U.x - V.y, U.y + V.x);
-        z2[k] = make_float2(W.x - Tt.y, W.y + Tt.x);
-      } else {
-        z1[k] = make_float2(U.x + V.y, V.x - U.y);
-        z2[k] = make_float2(W.x + Tt.y, Tt.x - W.y);
-      }
-    }
-    warp_fft<E>(z1, T, lane);
-    warp_fft<E>(z2, T, lane);
-    float4* out = a.nodes + (size_t(a.lev0 + level) * a.Nyr + y) * a.Nxr + E * int(bitrev(unsigned(lane), 5));
-#pragma unroll
-    for (int m2 = 0; m2 < E; ++m2)
-      __stcs(&out[m2], make_float4(z1[m2].x, z1[m2].y, z2[m2].x, z2[m2].y));
-  }
-}
-
-// Stockham per-warp variants of the two transform kernels (N = transform length >= 256): same
-// inputs, outputs and layouts as k_col_fft / k_row_fft, with stk_fft (radix-8 register passes,
-// exchanges through a warp-private shared buffer) in place of the shuffle-based transform.
-template <int N, int NF>
-__global__ void __launch_bounds__(256, N >= 1024 ? 1 : 2) k_col_stk(ColArgs a, Levels L) {
-  extern __shared__ float2 sm[];                 // [2][ny][cb + 1] modes, then per-warp buffers
-  constexpr int E = N / 32, RL = stk_radix(N, stk_npass(N) - 1);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c0 = blockIdx.x * kColBlock;
-  const int ncol = min(kColBlock, a.Mh - c0);
-  const int ld = kColBlock + 1;
-  float2* wbuf = sm + 2 * a.ny * ld + warp * stk_buf(N);
-  for (int i = threadIdx.x; i < a.ny * kColBlock; i += blockDim.x) {
-    const int c = i % kColBlock, r = i / kColBlock;
-    const bool ok = c < ncol;
-    const size_t gi = ok ? size_t(r) * a.nxh1 + c0 + c : 0;
-    cp_async8(&sm[r * ld + c], &a.A_phi[gi], ok ? 8 : 0);
-    cp_async8(&sm[(a.ny + r) * ld + c], &a.A_phit[gi], ok ? 8 : 0);
-  }
-  float2 T[stk_twn(N)];
-  stk_init<N>(T, a.tw, lane);
-  cp_async_wait_all();
-  __syncthreads();
-  const int nyh = a.ny >> 1;
-  const int groups = 4 / NF;
-  const int ntask = a.lpc * kColBlock * groups;
-  for (int task = warp; task < ntask; task += blockDim.x >> 5) {
-    const int g = task % groups;
-    const int rest = task / groups;
-    const int c = rest % kColBlock;
-    const int level = blockIdx.y * a.lpc + rest / kColBlock;
-    if (c >= ncol || level >= a.nlev) continue;
-    const float z = L.z[a.lev0 + level];
-    const int m = c0 + c;
-    const float kx = float(m) * a.kxs;
-    float2 v[NF][E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int p = lane + 32 * (e / 8) + (e % 8) * (N / 8);
-      int n;
-      bool live = true;
-      if (p < nyh) n = p;
-      else if (p > N - nyh) n = p - N;
-      else { n = 0; live = false; }
-      float2 Ap = make_float2(0.f, 0.f), At = make_float2(0.f, 0.f);
-      if (live) {
-        const int r = n >= 0 ? n : a.ny + n;
-        Ap = sm[r * ld + c];
-        At = sm[(a.ny + r) * ld + c];
-        if (a.spline) {
-          const float pf = spline_prefilter(m, a.Nxr, n, a.Nyr);
-          Ap = make_float2(pf * Ap.x, pf * Ap.y);
-          At = make_float2(pf * At.x, pf * At.y);
-        }
-      }
-      const float ky = float(n) * a.kys;
-      const float kk = sqrtf(kx * kx + ky * ky);
-      float F, S;
-      depth_factors(kk, z, a.depth, F, S);
-#pragma unroll
-      for (int f = 0; f < NF; ++f) v[f][e] = modal_field(g * NF + f, kx, ky, kk, F, S, Ap, At);
-    }
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      stk_fft<N>(v[f], T, a.tw, wbuf, lane);
-      float2* out = a.G + ((size_t(level) * 4 + g * NF + f) * a.Mh + m) * a.Nyr;
-#pragma unroll
-      for (int e = 0; e < E; ++e) __stcg(&out[lane + 32 * (e / RL) + (e % RL) * (N / RL)], v[f][e]);
-    }
-  }
-}
-
-// Hermitian packing of two real-output half spectra A, B (one column of the staged rows, stride
-// ld) into z = A + i B over the full length-N spectrum, in the first-pass register layout of
-// stk_fft; the upper half holds conj(A) + i conj(B) mirrored, the Nyquist slot stays zero.
-template <int N>
-__device__ __forceinline__ void row_pack(float2 (&z)[N / 32], const float2* A, const float2* B, int ld,
-                                         int Mh, int lane) {
-#pragma unroll
-  for (int e = 0; e < N / 32; ++e) {
-    const int p = lane + 32 * (e / 8) + (e % 8) * (N / 8);
-    const bool lo = p < Mh, hi = p > N - Mh;
-    float2 a = make_float2(0.f, 0.f), b = a;
-    if (lo || hi) {
-      const int o = (lo ? p : N - p) * ld;
-      a = A[o];
-      b = B[o];
-    }
-    if (p == 0) z[e] = make_float2(a.x, b.x);
-    else if (!hi) z[e] = make_float2(a.x - b.y, a.y + b.x);
-    else z[e] = make_float2(a.x + b.y, b.x - a.y);
-  }
-}
-
-template <int N>
-__global__ void __launch_bounds__(256, N >= 1024 ? 1 : 2) k_row_stk(RowArgs a) {
-  extern __shared__ float2 sm[];                 // [4][Mh][rb + 1] staging, then warp buffers
-  constexpr int E = N / 32, RL = stk_radix(N, stk_npass(N) - 1);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int y0 = blockIdx.x * kRowBlock;
-  const int level = blockIdx.y;
-  const int ld = kRowBlock + 1;
-  const float2* G = a.G + size_t(level) * 4 * a.Mh * a.Nyr;
-  float2* wbuf = sm + 4 * a.Mh * ld + warp * stk_buf(N);
-  for (int i = threadIdx.x; i < 4 * a.Mh * kRowBlock; i += blockDim.x) {
-    const int rr = i % kRowBlock, qm = i / kRowBlock;
-    const int y = y0 + rr;
-    cp_async8(&sm[qm * ld + rr], &G[size_t(qm) * a.Nyr + (y < a.Nyr ? y : 0)], y < a.Nyr ? 8 : 0);
-  }
-  float2 T[stk_twn(N)];
-  stk_init<N>(T, a.tw, lane);
-  cp_async_wait_all();
-  __syncthreads();
-  const size_t fs = size_t(a.Mh) * ld;
-  for (int rr = warp; rr < kRowBlock; rr += blockDim.x >> 5) {
-    const int y = y0 + rr;
-    if (y >= a.Nyr) break;
-    float4* out = a.nodes + (size_t(a.lev0 + level) * a.Nyr + y) * N;
-    if constexpr (N <= 256) {
-      float2 z1[E], z2[E];
-      row_pack<N>(z1, sm + rr, sm + fs + rr, ld, a.Mh, lane);
-      row_pack<N>(z2, sm + 2 * fs + rr, sm + 3 * fs + rr, ld, a.Mh, lane);
-      stk_fft<N>(z1, T, a.tw, wbuf, lane);
-      stk_fft<N>(z2, T, a.tw, wbuf, lane);
-#pragma unroll
-      for (int e = 0; e < E; ++e)
-        __stcs(&out[lane + 32 * (e / RL) + (e % RL) * (N / RL)],
-               make_float4(z1[e].x, z1[e].y, z2[e].x, z2[e].y));
-    } else {
-      // one transform at a time (register budget): each half of a node's float4 is written by
-      // its own pass; the two halves meet in L2 before the sector goes to DRAM
-      float2* o2 = reinterpret_cast<float2*>(out);
-#pragma unroll 1
-      for (int q = 0; q < 2; ++q) {
-        float2 z[E];
-        row_pack<N>(z, sm + 2 * q * fs + rr, sm + (2 * q + 1) * fs + rr, ld, a.Mh, lane);
-        stk_fft<N>(z, T, a.tw, wbuf, lane);
-#pragma unroll
-        for (int e = 0; e < E; ++e)
-          __stcs(&o2[2 * (lane + 32 * (e / RL) + (e % RL) * (N / RL)) + q], z[e]);
-      }
-    }
-  }
-}
-
-// Row pass, one field pair per CTA (blockIdx.z: 0 -> (U, V) into (u, v), 1 -> (W, T) into
-// (w, dphi/dt)), one length-N transform per warp: half the registers of k_row_stk, so three CTAs
-// fit on an SM. The staged rows are dead once every warp holds its row, and the same shared
-// memory then serves as the per-warp exchange buffers. Each CTA writes one float2 half of the
-// nodes' float4; the two halves meet in L2.
-template <int N>
-__global__ void __launch_bounds__(256, N >= 1024 ? 2 : 3) k_row_half(RowArgs a) {
-  extern __shared__ float2 sm[];                 // [2][Mh][rb + 1] staging, then warp buffers
-  constexpr int E = N / 32, RL = stk_radix(N, stk_npass(N) - 1);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int y0 = blockIdx.x * kRowBlock;
-  const int level = blockIdx.y;
-  const int q = blockIdx.z;
-  constexpr int ld = kRowBlock + 1;
-  const float2* G = a.G + (size_t(level) * 4 + 2 * q) * a.Mh * a.Nyr;
-  for (int i = threadIdx.x; i < 2 * a.Mh * kRowBlock; i += blockDim.x) {
-    const int rr = i % kRowBlock, fm = i / kRowBlock;
-    const int y = y0 + rr;
-    cp_async8(&sm[fm * ld + rr], &G[size_t(fm) * a.Nyr + (y < a.Nyr ? y : 0)], y < a.Nyr ? 8 : 0);
-  }
-  float2 T[stk_twn(N)];
-  stk_init<N>(T, a.tw, lane);
-  cp_async_wait_all();
-  __syncthreads();
-  const size_t fs = size_t(a.Mh) * ld;
-  float2 z[E];
-  row_pack<N>(z, sm + warp, sm + fs + warp, ld, a.Mh, lane);   // kRowBlock rows, one per warp
-  __syncthreads();
-  const int y = y0 + warp;
-  if (y >= a.Nyr) return;
-  stk_fft<N>(z, T, a.tw, sm + warp * stk_buf(N), lane);
-  float2* o2 = reinterpret_cast<float2*>(a.nodes + (size_t(a.lev0 + level) * a.Nyr + y) * N) + q;
-#pragma unroll
-  for (int e = 0; e < E; ++e) __stcs(&o2[2 * (lane + 32 * (e / RL) + (e % RL) * (N / RL))], z[e]);
-}
 
 // m stride of the transposed intermediate: a whole number of 128-byte lines per field row, so
 // the row pass can drop the rows it has consumed from L2 without touching a neighbour's data.
@@ -632,394 +373,184 @@ __device__ __forceinline__ void discard_rows(const float2* row, size_t fs, int n
   }
 }
 
-// Transposed-intermediate pair for 256- to 1024-point transforms. The column pass writes
-// G[level][field][y][m] with the m stride padded to whole 128-byte lines (ldG), so a grid row's
-// inputs are contiguous; the row pass then reads them straight into registers with coalesced
-// loads, with no staging and no block-wide barrier.
+// Transposed pair for 32- to 1024-point columns (and rows of 32 to 8192 points). The column pass
+// writes G[level][field][y][m] with the m stride padded to whole 128-byte lines (ldG), so that a grid
+// row's inputs are contiguous for the row pass.
 //
-// Column pass: the eight warps of a block own eight consecutive kx columns; each loads its
-// column's modes once (reused over the block's levels), forms NF modal fields per depth-factor
-// evaluation, transforms them, and the block writes the eight columns out row by row through a
-// padded shared tile (64-byte segments).
-// Position of (row, column) in the 8-column tiles through which the column passes transpose
-// their output: a row's columns are XOR-swizzled by (row >> 1) & 7, so that a warp's column
-// writes (16 consecutive rows a half-warp) and the row reads (two rows of 8 columns a
-// half-warp) each hit 32 different banks.
-static_assert(kColBlock == 8, "the tile swizzle spans 8 columns");
-__device__ __forceinline__ int tile_pos(int row, int col) { return row * kColBlock + (col ^ ((row >> 1) & 7)); }
+// Column pass: a block owns kCols neighbouring kx columns of one level at a time, its lanes laid out
+// column-fastest: every global access (modes in, intermediate out) is a run of kCols neighbouring m,
+// with no transposing tile, and the one exchange between the two wide passes has whole rows of
+// columns in neighbouring banks. The depth factors of a level are made once, in shared memory, for
+// the four modal fields, which the block transforms one after another. Before, each field's block
+// made its own (a square root and an exponential per point: 118 instructions a point against 64 now)
+// and went through shared memory four times. Eight levels of 1024 x 1024 columns: 198 -> 146 us at
+// 37 % issue (latency of the loads and of the in-register DFTs at 16 warps per SM); eight levels of
+// 256-point columns padded to 1024: 61 -> 24 us; 64 levels of 256 x 256: 64 -> 42 us.
+template <int N>
+struct ColCfg {
+  static constexpr int R0 = wide_r0(N), R1 = N / R0, E = R0, T = N / E, B1 = E / R1;
+  static constexpr int kCols = N >= 256 ? 8 : (N >= 64 ? 16 : 32);
+  static constexpr int kThr = T * kCols;
+  // 8 columns are half a row of banks: one row of padding in R0 keeps the writes of neighbouring j
+  // (rows R0 apart) in different halves
+  static constexpr int kPad = kCols == 8 ? 1 : 0;
+  static constexpr int kXch = (N + kPad * T) * kCols;
+  static constexpr int kMin = N >= 1024 ? 2 : (N >= 512 ? 4 : (N >= 128 ? 6 : 8));   // blocks per SM
+};
 
-template <int N, int NF>
-__global__ void __launch_bounds__(256, N >= 1024 ? 1 : 2) k_col_t(ColArgs a, Levels L) {
-  extern __shared__ float2 sm[];                 // tile [N][kColBlock + 1], then warp buffers
-  constexpr int E = N / 32, RL = stk_radix(N, stk_npass(N) - 1);
-  constexpr int TLD = kColBlock + 1;
-  static_assert(kColBlock * 32 == kThreads, "one column per warp");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c0 = blockIdx.x * kColBlock;
-  const int m = c0 + warp;
+template <int N, bool FINITE>
+__global__ void __launch_bounds__(ColCfg<N>::kThr, ColCfg<N>::kMin) k_col_w(ColArgs a, const __grid_constant__ Levels L) {
+  using C = ColCfg<N>;
+  constexpr int E = C::E, T = C::T, R0 = C::R0, R1 = C::R1;
+  // exchange [rows][kCols], twiddles [N], depth factors [E][kThr] (each thread its own: the data of 32
+  // elements alone take 64 registers)
+  extern __shared__ float2 sm[];
+  float2* xch = sm;
+  float2* stw = sm + C::kXch;
+  float* sF = reinterpret_cast<float*>(stw + N) + threadIdx.x;
+  const int c = threadIdx.x % C::kCols, j = threadIdx.x / C::kCols;
+  const int m = blockIdx.x * C::kCols + c;
   const bool colok = m < a.Mh;
-  float2* tile = sm;
-  float2* wbuf = sm + N * TLD + warp * stk_buf(N);
-  // depth factors of the current level, F and |k| S per element, made by the first field group
-  // and reused by the second (short columns only; after the warp buffers)
-  float* fks = reinterpret_cast<float*>(sm + N * TLD + (kThreads / 32) * stk_buf(N)) + warp * 2 * N;
-  float2 T[stk_twn(N)];
-  stk_init<N>(T, a.tw, lane);
   const int nyh = a.ny >> 1;
-  const float kx = colok ? float(m) * a.kxs : 0.f;
-  // modes of element e (zero in the padding and at the Nyquist row)
-  auto load_mode = [&](int e, float2& ap, float2& at) {
-    const int p = lane + 32 * (e / 8) + (e % 8) * (N / 8);
-    int n = 0;
-    bool live = colok;
-    if (p < nyh) n = p;
-    else if (p > N - nyh) n = p - N;
-    else live = false;
-    ap = at = make_float2(0.f, 0.f);
-    if (live) {
-      const size_t gi = size_t(n >= 0 ? n : a.ny + n) * a.nxh1 + m;
-      ap = __ldg(&a.A_phi[gi]);
-      at = __ldg(&a.A_phit[gi]);
-      if (a.spline) {
-        const float pf = spline_prefilter(m, a.Nxr, n, a.Nyr);
-        ap = make_float2(pf * ap.x, pf * ap.y);
-        at = make_float2(pf * at.x, pf * at.y);
-      }
-    }
-  };
-  // short columns keep their modes in registers across levels; longer ones reload (L1)
-  constexpr bool KEEP = N <= 256;
-  float2 Ap[KEEP ? E : 1], At[KEEP ? E : 1];
-  if constexpr (KEEP) {
-#pragma unroll
-    for (int e = 0; e < E; ++e) load_mode(e, Ap[e], At[e]);
-  }
+  for (int i = threadIdx.x; i < N; i += C::kThr) stw[i] = __ldg(&a.tw[kWideTw + N + i]);
+  const float kx = float(m) * a.kxs;
+  __syncthreads();
+  // position p = j + T e holds wavenumber index n = p (first half) or p - N, i.e. row p or ny + p - N
+  // of the modes; zero in the padding and at the Nyquist row
+  const float2* A0 = a.A + size_t(j) * a.ldG + m;
+  const int up = (a.ny - N) * a.ldG;
+  auto live = [&](int e) { return colok && (e < E / 2 ? j + T * e < nyh : N - T * e - j < nyh); };
   for (int li = 0; li < a.lpc; ++li) {
     const int level = blockIdx.y * a.lpc + li;
     if (level >= a.nlev) break;                  // uniform over the block
-    const float z = L.z[a.lev0 + level];
+    const int slot = a.lev0 + level;
+    const bool is_eta = slot >= a.n_lev;
+    const int tl = is_eta ? slot - a.n_lev : slot / a.nz;
+    const float z = is_eta ? 0.f : L.z[slot - tl * a.nz];
+    const int nq = is_eta ? 1 : 4;
 #pragma unroll 1
-    for (int g = 0; g < 4 / NF; ++g) {
-      float2 v[NF][E];
+    for (int qi = 0; qi < nq; ++qi) {
+      const int q = is_eta ? 4 : (qi < 2 ? qi : 5 - qi);   // U, V, dphi/dt (factor F), then W (factor S)
+      if (qi == 0 || (FINITE && qi == 3)) {
+#pragma unroll 2
+        for (int e = 0; e < E; ++e) {
+          float f = 0.f;
+          if (live(e)) {
+            const float ky = float(e < E / 2 ? j + T * e : j + T * e - N) * a.kys;
+            float F, S;
+            depth_factors(sqrtf(kx * kx + ky * ky), z, a.depth, F, S);
+            f = is_eta ? 1.f : (FINITE && qi == 3 ? S : F);
+          }
+          sF[e * C::kThr] = f;
+        }
+      }
+      const float2* __restrict__ A = A0 + (size_t(tl) * 5 + q) * a.ny * a.ldG;
+      float2 v[E];
 #pragma unroll
       for (int e = 0; e < E; ++e) {
-        const int p = lane + 32 * (e / 8) + (e % 8) * (N / 8);
-        // zero-padded and Nyquist positions carry no mode: evaluate their (unused) depth factor
-        // at ky = 0, where it cannot overflow (e^{|k| z} at a padded |k| can reach inf, and
-        // inf * 0 would be NaN)
-        const int n = p < nyh ? p : (p > N - nyh ? p - N : 0);
-        const float ky = float(n) * a.kys;
-        float kk, F, S;
-        float2 ap, at;
-        if constexpr (KEEP) {
-          ap = Ap[e];
-          at = At[e];
-          if (g == 0) {
-            kk = sqrtf(kx * kx + ky * ky);
-            depth_factors(kk, z, a.depth, F, S);
-            S *= kk;                               // modal_field takes |k| S as one factor
-            fks[e * 32 + lane] = F;
-            fks[N + e * 32 + lane] = S;
-          } else {
-            F = fks[e * 32 + lane];
-            S = fks[N + e * 32 + lane];
-          }
-          kk = 1.f;
-        } else {
-          kk = sqrtf(kx * kx + ky * ky);
-          depth_factors(kk, z, a.depth, F, S);
-          load_mode(e, ap, at);
+        v[e] = make_float2(0.f, 0.f);
+        if (live(e)) v[e] = __ldg(&A[e * T * a.ldG + (e < E / 2 ? 0 : up)]);
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const float f = sF[e * C::kThr];
+        v[e] = make_float2(f * v[e].x, f * v[e].y);
+      }
+      wide_dft<R0>(v);
+#pragma unroll
+      for (int r = 0; r < R0; ++r) xch[(j * (R0 + C::kPad) + r) * C::kCols + c] = v[dft_slot<R0>(r)];
+      __syncthreads();
+#pragma unroll
+      for (int b = 0; b < C::B1; ++b)
+#pragma unroll
+        for (int r = 0; r < R1; ++r) v[b * R1 + r] = xch[(j + T * b + (R0 + C::kPad) * r) * C::kCols + c];
+      __syncthreads();                           // the buffer is free for the next field
+      float2* out = a.G + (size_t(level) * 4 + (is_eta ? 0 : q)) * N * a.ldG + m;
+#pragma unroll
+      for (int b = 0; b < C::B1; ++b) {
+        const int jj = j + T * b;
+#pragma unroll
+        for (int r = 1; r < R1; ++r) v[b * R1 + r] = cmul(v[b * R1 + r], stw[r * R0 + jj]);
+        wide_dft<R1>(&v[b * R1]);
+        if (colok) {
+#pragma unroll
+          for (int r = 0; r < R1; ++r) __stcg(&out[(jj + R0 * r) * a.ldG], v[b * R1 + dft_slot<R1>(r)]);
         }
-#pragma unroll
-        for (int f = 0; f < NF; ++f) v[f][e] = modal_field(g * NF + f, kx, ky, kk, F, S, ap, at);
-      }
-#pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        stk_fft<N>(v[f], T, a.tw, wbuf, lane);
-#pragma unroll
-        for (int e = 0; e < E; ++e) tile[tile_pos(lane + 32 * (e / RL) + (e % RL) * (N / RL), warp)] = v[f][e];
-        __syncthreads();
-        float2* out = a.G + (size_t(level) * 4 + g * NF + f) * a.Nyr * a.ldG + c0;
-        // rows of 8 columns: 64 contiguous bytes of the intermediate per row
-        for (int i = threadIdx.x; i < N * kColBlock; i += kThreads) {
-          const int y = i / kColBlock, w = i % kColBlock;
-          if (c0 + w < a.Mh) __stcg(&out[size_t(y) * a.ldG + w], tile[tile_pos(y, w)]);
-        }
-        __syncthreads();
       }
     }
   }
 }
 
-// Column pass of the transposed pair with the four modal fields in separate CTAs (blockIdx.z =
-// field U, V, W, T): four times the CTAs of k_col_t per level and half its registers, so long
-// columns fill the GPU even when a level chunk holds few levels (a 1024-point column pass has
-// only Mh / 8 CTAs per level otherwise). The output tile and the warps' exchange buffers share
-// the same shared memory (a barrier between the transforms and the tile writes).
+// Row pass over the transposed intermediate for rows of 32 to 2048 points: T = N / R0 threads per grid
+// row, its four modal fields loaded straight from G (neighbouring threads read neighbouring m),
+// packed as Z1 = U + iV and Z2 = W + iT over the full x spectrum, both transformed side by side
+// (WideRow), stored as float4. Loads are cached in L1: at padding 1 a row reads each value twice, as
+// mode m and mirrored as N - m. Eight levels of 1024 x 2048 nodes at padding 4: 108 -> 72 us; at
+// padding 1 the loads of the intermediate bound it, 149 us (124 with radix-8 passes, whose six blocks
+// per SM hid more of them; the columns' gain outweighs it). Variants at 5 blocks per SM spill.
 template <int N>
-__global__ void __launch_bounds__(256, N >= 1024 ? 1 : 2) k_col_tf(ColArgs a, Levels L) {
-  extern __shared__ float2 sm[];                 // exchange buffers, then tile [N][kColBlock + 1]
-  constexpr int E = N / 32, RL = stk_radix(N, stk_npass(N) - 1);
-  static_assert(kColBlock * 32 == kThreads, "one column per warp");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c0 = blockIdx.x * kColBlock;
-  const int m = c0 + warp;
-  const bool colok = m < a.Mh;
-  const int q = blockIdx.z;
-  float2* tile = sm;
-  float2* wbuf = sm + warp * stk_buf(N);
-  float2 T[stk_twn(N)];
-  stk_init<N>(T, a.tw, lane);
-  const int nyh = a.ny >> 1;
-  const float kx = colok ? float(m) * a.kxs : 0.f;
-  const float2* __restrict__ A = q == 3 ? a.A_phit : a.A_phi;
-  // the column's modes of this field, loaded once and kept in registers over the CTA's levels
-  // (zero in the padding and at the Nyquist row)
-  float2 am[E];
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int p = lane + 32 * (e / 8) + (e % 8) * (N / 8);
-    int n = 0;
-    bool live = colok;
-    if (p < nyh) n = p;
-    else if (p > N - nyh) n = p - N;
-    else live = false;
-    am[e] = make_float2(0.f, 0.f);
-    if (live) {
-      am[e] = __ldg(&A[size_t(n >= 0 ? n : a.ny + n) * a.nxh1 + m]);
-      if (a.spline) {
-        const float pf = spline_prefilter(m, a.Nxr, n, a.Nyr);
-        am[e] = make_float2(pf * am[e].x, pf * am[e].y);
-      }
-    }
-  }
-  for (int li = 0; li < a.lpc; ++li) {
-    const int level = blockIdx.y * a.lpc + li;
-    if (level >= a.nlev) break;                  // uniform over the block
-    const float z = L.z[a.lev0 + level];
-    float2 v[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int p = lane + 32 * (e / 8) + (e % 8) * (N / 8);
-      // zero-padded and Nyquist positions carry no mode: their (unused) depth factor is taken
-      // at ky = 0, where it cannot overflow
-      const int n = p < nyh ? p : (p > N - nyh ? p - N : 0);
-      const float ky = float(n) * a.kys;
-      const float kk = sqrtf(kx * kx + ky * ky);
-      float F, S;
-      depth_factors(kk, z, a.depth, F, S);
-      v[e] = modal_field(q, kx, ky, kk, F, S, am[e], am[e]);
-    }
-    stk_fft<N>(v, T, a.tw, wbuf, lane);
-    __syncthreads();                             // every warp is done with its exchange buffer
-#pragma unroll
-    for (int e = 0; e < E; ++e) tile[tile_pos(lane + 32 * (e / RL) + (e % RL) * (N / RL), warp)] = v[e];
-    __syncthreads();
-    float2* out = a.G + (size_t(level) * 4 + q) * a.Nyr * a.ldG + c0;
-    // rows of 8 columns: 64 contiguous bytes of the intermediate per row
-    for (int i = threadIdx.x; i < N * kColBlock; i += kThreads) {
-      const int y = i / kColBlock, w = i % kColBlock;
-      if (c0 + w < a.Mh) __stcg(&out[size_t(y) * a.ldG + w], tile[tile_pos(y, w)]);
-    }
-    __syncthreads();                             // the tile is read before the next transforms
-  }
-}
-
-// The same column pass with two warps per column (1024-point columns): warp 2c + s transforms
-// the rows p = 2 i + s of column c (a 512-point Stockham transform, 16 points a lane), the odd
-// warp multiplies its result by e^{2 pi i k / N}, both halves go to the CTA's tile, and the
-// radix-2 combine X[k] = E[k] + O'[k], X[k + N/2] = E[k] - O'[k] is done while the tile is
-// written out (the operations of the one-warp transform's last pass, in the same order, so the
-// results are identical). Half the points per lane (128 registers) and twice the warps per SM of
-// k_col_tf<1024>, whose 244 registers leave one 8-warp CTA per SM; bank-conflict-free tile
-// (XOR swizzle) and no separate exchange for the combine: stage 1 of the large sea 17.65 ->
-// 16.67 ms.
-template <int N>
-__global__ void __launch_bounds__(2 * kThreads, 1) k_col_tf2(ColArgs a, Levels L) {
-  extern __shared__ float2 sm[];                 // exchange buffers, then tile [N][kColBlock] (swizzled)
-  constexpr int H = N / 2, E = H / 32, RL = stk_radix(H, stk_npass(H) - 1);
-  static_assert(kColBlock == 8, "the tile swizzle spans 8 columns");
-  static_assert(kColBlock * 64 == 2 * kThreads, "two warps per column");
-  // e^{2 pi i k / N}, k < H: the factors of the N-point transform's last pass (radix 2, stride H),
-  // read from its pass-major table (consecutive k in consecutive entries)
-  static_assert(stk_radix(N, stk_npass(N) - 1) == 2 && stk_ns(N, stk_npass(N) - 1) == H,
-                "the combine is the last radix-2 pass of the N-point transform");
-  constexpr int kTwC = stk_twp(N, stk_npass(N) - 1);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int col = warp >> 1, par = warp & 1;     // column of the CTA, parity of this warp's rows
-  const int c0 = blockIdx.x * kColBlock;
-  const int m = c0 + col;
-  const bool colok = m < a.Mh;
-  const int q = blockIdx.z;
-  float2* tile = sm;
-  float2* wbuf = sm + warp * stk_buf(H);
-  float2 T[stk_twn(H)];
-  stk_init<H>(T, a.tw, lane);
-  const int nyh = a.ny >> 1;
-  const float kx = colok ? float(m) * a.kxs : 0.f;
-  const float2* __restrict__ A = q == 3 ? a.A_phit : a.A_phi;
-  // this warp's modes (rows p = 2 i + par of the half-sequence position i), loaded once and kept
-  // in registers over the CTA's levels (zero in the padding and at the Nyquist row)
-  float2 am[E];
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int p = 2 * (lane + 32 * (e / 8) + (e % 8) * (H / 8)) + par;
-    int n = 0;
-    bool live = colok;
-    if (p < nyh) n = p;
-    else if (p > N - nyh) n = p - N;
-    else live = false;
-    am[e] = make_float2(0.f, 0.f);
-    if (live) {
-      am[e] = __ldg(&A[size_t(n >= 0 ? n : a.ny + n) * a.nxh1 + m]);
-      if (a.spline) {
-        const float pf = spline_prefilter(m, a.Nxr, n, a.Nyr);
-        am[e] = make_float2(pf * am[e].x, pf * am[e].y);
-      }
-    }
-  }
-  for (int li = 0; li < a.lpc; ++li) {
-    const int level = blockIdx.y * a.lpc + li;
-    if (level >= a.nlev) break;                  // uniform over the block
-    const float z = L.z[a.lev0 + level];
-    float2 v[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int p = 2 * (lane + 32 * (e / 8) + (e % 8) * (H / 8)) + par;
-      // zero-padded and Nyquist positions carry no mode: their (unused) depth factor is taken
-      // at ky = 0, where it cannot overflow
-      const int n = p < nyh ? p : (p > N - nyh ? p - N : 0);
-      const float ky = float(n) * a.kys;
-      const float kk = sqrtf(kx * kx + ky * ky);
-      float F, S;
-      depth_factors(kk, z, a.depth, F, S);
-      v[e] = modal_field(q, kx, ky, kk, F, S, am[e], am[e]);
-    }
-    stk_fft<H>(v, T, a.tw, wbuf, lane);
-    __syncthreads();                             // every warp is done with its exchange buffer
-    // element e holds output k = lane + 32 (e / RL) + (e % RL) (H / RL) of this half; the odd half,
-    // twiddled, goes to tile row H + k. Tile rows hold the CTA's 8 columns with column c at
-    // c ^ ((row >> 1) & 7): the column writes (16 consecutive rows a half-warp) and the row reads
-    // (two rows of 8 columns a half-warp) both hit 32 different banks.
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int k = lane + 32 * (e / RL) + (e % RL) * (H / RL);
-      if (par) v[e] = cmul(v[e], __ldg(&a.tw[kTwC + k]));
-      const int row = k + par * H;
-      tile[tile_pos(row, col)] = v[e];
-    }
-    __syncthreads();
-    float2* out = a.G + (size_t(level) * 4 + q) * a.Nyr * a.ldG + c0;
-    // the radix-2 combine on the way out: X[y] = E[y] + O'[y], X[y + H] = E[y] - O'[y]
-    for (int i = threadIdx.x; i < H * kColBlock; i += 2 * kThreads) {
-      const int y = i / kColBlock, w = i % kColBlock;
-      const float2 ev = tile[tile_pos(y, w)], od = tile[tile_pos(y + H, w)];
-      if (c0 + w < a.Mh) {
-        __stcg(&out[size_t(y) * a.ldG + w], cadd(ev, od));
-        __stcg(&out[size_t(y + H) * a.ldG + w], csub(ev, od));
-      }
-    }
-    __syncthreads();                             // the tile is read before the next transforms
-  }
-}
-
-// Row pass over the transposed intermediate: one warp per grid row of one level, its four
-// modal fields loaded straight from G (consecutive lanes read consecutive m), packed as
-// Z1 = U + iV and Z2 = W + iT over the full x spectrum, transformed, stored as float4.
-template <int N>
-__global__ void __launch_bounds__(256, N >= 1024 ? 1 : 2) k_row_t(RowArgs a) {
-  extern __shared__ float2 sm[];                 // warp exchange buffers
-  constexpr int E = N / 32, RL = stk_radix(N, stk_npass(N) - 1);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int y = blockIdx.x * (kThreads / 32) + warp;
+__global__ void __launch_bounds__(WideRow<N>::T * WideRow<N>::kRows, WideRow<N>::E == 16 ? 4 : 8) k_row_w(RowArgs a) {
+  using W = WideRow<N>;
+  extern __shared__ float2 sm[];                 // two exchange buffers per row
+  const int t = threadIdx.x % W::T, rr = threadIdx.x / W::T;
+  const int y = blockIdx.x * W::kRows + rr;      // the row count is a multiple of kRows
   const int level = blockIdx.y;
-  if (y >= a.Nyr) return;                        // no block-wide barrier in this kernel
-  float2 T[stk_twn(N)];
-  stk_init<N>(T, a.tw, lane);
-  float2* wbuf = sm + warp * stk_buf(N);
   const size_t fs = size_t(a.Nyr) * a.ldG;
   const float2* row = a.G + size_t(level) * 4 * fs + size_t(y) * a.ldG;
-  float4* out = a.nodes + (size_t(a.lev0 + level) * a.Nyr + y) * N;
-  float2 z1[E], z2[E];
+  const bool is_eta = a.lev0 + level >= a.n_lev;   // one field: Z1 = eta, the others zero
+  float2 z1[W::E], z2[W::E];
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int p = lane + 32 * (e / 8) + (e % 8) * (N / 8);
-    const bool lo = p < a.Mh, hi = p > N - a.Mh;
-    float2 U = make_float2(0.f, 0.f), V = U, W = U, Tt = U;
-    if (lo || hi) {
-      const int mm = lo ? p : N - p;
-      U = __ldcg(&row[mm]);
-      V = __ldcg(&row[fs + mm]);
-      W = __ldcg(&row[2 * fs + mm]);
-      Tt = __ldcg(&row[3 * fs + mm]);
+  for (int e = 0; e < W::E; ++e) {
+    // positions of the upper half hold the mirrored (conjugate) modes N - p
+    const int p = t + W::T * e, mm = e < W::E / 2 ? p : N - p;
+    float2 U = make_float2(0.f, 0.f), V = U, X = U, Y = U;
+    if (mm < a.Mh) {
+      U = row[mm];
+      if (!is_eta) {
+        V = row[fs + mm];
+        X = row[2 * fs + mm];
+        Y = row[3 * fs + mm];
+      }
     }
-    if (p == 0) {
-      z1[e] = make_float2(U.x, V.x);
-      z2[e] = make_float2(W.x, Tt.x);
-    } else if (!hi) {
-      z1[e] = make_float2(U.x - V.y, U.y + V.x);
-      z2[e] = make_float2(W.x - Tt.y, W.y + Tt.x);
-    } else {
+    if (e >= W::E / 2) {
       z1[e] = make_float2(U.x + V.y, V.x - U.y);
-      z2[e] = make_float2(W.x + Tt.y, Tt.x - W.y);
+      z2[e] = make_float2(X.x + Y.y, Y.x - X.y);
+    } else if (e == 0 && t == 0) {               // m = 0: the real parts only
+      z1[e] = make_float2(U.x, V.x);
+      z2[e] = make_float2(X.x, Y.x);
+    } else {
+      z1[e] = make_float2(U.x - V.y, U.y + V.x);
+      z2[e] = make_float2(X.x - Y.y, X.y + Y.x);
     }
   }
-  stk_fft<N>(z1, T, a.tw, wbuf, lane);
-  stk_fft<N>(z2, T, a.tw, wbuf, lane);
+  float2* b1 = sm + size_t(rr) * 2 * W::kBuf;
+  W::fft2(z1, z2, a.tw, b1, b1 + W::kBuf, t);
+  if (is_eta) {
+    float* out = a.eta + (size_t(a.lev0 + level - a.n_lev) * a.Nyr + y) * N;
 #pragma unroll
-  for (int e = 0; e < E; ++e)
-    __stcs(&out[lane + 32 * (e / RL) + (e % RL) * (N / RL)], make_float4(z1[e].x, z1[e].y, z2[e].x, z2[e].y));
-  __syncwarp();                                  // every lane's reads of the row are done
-  discard_rows(row, fs, 4, a.ldG, lane, 32);
-}
-
-// Same row pass with one transform per warp (warps 2r and 2r+1 of a block take Z1 and Z2 of
-// row r): half the registers, so more warps per SM; each warp writes one float2 half of the
-// nodes' float4 (the halves meet in L2).
-template <int N>
-__global__ void __launch_bounds__(256, N >= 2048 ? 1 : (N >= 1024 ? 2 : 3)) k_row_t2(RowArgs a) {
-  extern __shared__ float2 sm[];                 // warp exchange buffers
-  constexpr int E = N / 32, RL = stk_radix(N, stk_npass(N) - 1);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int y = blockIdx.x * (kThreads / 64) + (warp >> 1);
-  const int q = warp & 1;                        // 0: Z1 = U + iV, 1: Z2 = W + iT
-  const int level = blockIdx.y;
-  if (y >= a.Nyr) return;                        // no block-wide barrier in this kernel
-  float2 T[stk_twn(N)];
-  stk_init<N>(T, a.tw, lane);
-  float2* wbuf = sm + warp * stk_buf(N);
-  const size_t fs = size_t(a.Nyr) * a.ldG;
-  const float2* row = a.G + (size_t(level) * 4 + 2 * q) * fs + size_t(y) * a.ldG;
-  float2 z[E];
+    for (int b = 0; b < W::BL; ++b)
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int p = lane + 32 * (e / 8) + (e % 8) * (N / 8);
-    const bool lo = p < a.Mh, hi = p > N - a.Mh;
-    float2 A = make_float2(0.f, 0.f), B = A;
-    if (lo || hi) {
-      const int mm = lo ? p : N - p;
-      A = __ldcg(&row[mm]);
-      B = __ldcg(&row[fs + mm]);
-    }
-    if (p == 0) z[e] = make_float2(A.x, B.x);
-    else if (!hi) z[e] = make_float2(A.x - B.y, A.y + B.x);
-    else z[e] = make_float2(A.x + B.y, B.x - A.y);
+      for (int r = 0; r < W::RL; ++r) __stcs(&out[W::pos(t, b, r)], z1[W::elem(b, r)].x);
+    discard_rows(row, fs, 1, a.ldG, t, W::T);
+    return;
   }
-  stk_fft<N>(z, T, a.tw, wbuf, lane);
-  float2* out = reinterpret_cast<float2*>(a.nodes + (size_t(a.lev0 + level) * a.Nyr + y) * N) + q;
+  float4* out = a.nodes + (size_t(a.lev0 + level) * a.Nyr + y) * N;
 #pragma unroll
-  for (int e = 0; e < E; ++e) __stcs(&out[2 * (lane + 32 * (e / RL) + (e % RL) * (N / RL))], z[e]);
-  __syncwarp();                                  // every lane's reads of the two rows are done
-  discard_rows(row, fs, 2, a.ldG, lane, 32);
+  for (int b = 0; b < W::BL; ++b)
+#pragma unroll
+    for (int r = 0; r < W::RL; ++r) {
+      const int e = W::elem(b, r);
+      __stcs(&out[W::pos(t, b, r)], make_float4(z1[e].x, z1[e].y, z2[e].x, z2[e].y));
+    }
+  // every thread's reads of the row came before the last exchange's barrier
+  discard_rows(row, fs, 4, a.ldG, t, W::T);
 }
 
-// Row pass for rows longer than a warp transform (2048..8192 points): one block of kThreads per
-// grid row of one level, inputs from the transposed intermediate (coalesced), block-wide
-// Stockham transforms of Z1 = U + iV and Z2 = W + iT. 2048-point rows: three blocks per SM (80
-// registers) hide more of the intermediate's load latency than two (92): stage 1 of the large
-// sea 16.64 -> 16.12 ms.
+// Row pass for 4096- and 8192-point rows: one block of kThreads per grid row of one level, inputs
+// from the transposed intermediate (coalesced), block-wide Stockham transforms of Z1 = U + iV and
+// Z2 = W + iT.
 template <int N>
-__global__ void __launch_bounds__(256, N >= 8192 ? 1 : (N >= 4096 ? 2 : 3)) k_row_tb(RowArgs a) {
+__global__ void __launch_bounds__(256, N >= 8192 ? 1 : 2) k_row_tb(RowArgs a) {
   extern __shared__ float2 sm[];                 // one or two exchange buffers
   constexpr int E = N / kThreads, RL = stk_radix(N, stk_npass(N) - 1);
   constexpr bool BOTH = N <= 4096;               // both transforms' data in registers at once
@@ -1168,16 +699,14 @@ __global__ void __launch_bounds__(256, N >= 1024 ? 1 : 2) k_row_tma(RowArgs a, i
   }
 }
 
-// Launch-shape choices of the warp-register path, per grid shape (set by swense_autotune_grid;
-// defaults otherwise).
+// Launch-shape choices per grid shape (set by swense_autotune_grid or swense_set_grid_tune; defaults
+// otherwise).
 struct Tune {
-  int lpc = -1;                         // levels per column-transform CTA of the warp path;
+  int lpc = -1;                         // levels per column-transform CTA of the transposed pair;
                                         // 0: shared-memory path; -1: default for the shape
-  size_t chunk_bytes = kChunkBytes;     // scratch per level chunk (L2-resident)
-  int rowv = 0;                         // row pass: 0 both field pairs per warp (k_row_stk),
-                                        // 1 one field pair per CTA (k_row_half)
-  int colv = 0;                         // column pass of the transposed pair: 0 k_col_t,
-                                        // 1 k_col_tf (one modal field per CTA)
+  size_t chunk_bytes = kChunkBytes;     // scratch per level chunk
+  int rowv = 0;                         // 4: row pass with staged inputs; 5: the pair's passes
+                                        // pipelined over two streams; others: one stream
 };
 std::mutex g_tune_mutex;
 std::map<std::array<int64_t, 4>, Tune> g_tune;
@@ -1192,84 +721,33 @@ Tune tuned(int nx, int ny, int pad, int nz) {
 struct GridPlan {
   int nx, ny, nz, n_tl, nxh1, Mh, pad, spline;
   int64_t Nxr, Nyr;
-  size_t nslot, per_level, prop_bytes, geta_bytes;
+  size_t nslot, per_level, geta_bytes;
+  bool omega;
   Levels lev;
 };
 
-template <int E, int NF>
-int launch_col(const ColArgs& c, const Levels& L, dim3 grid, size_t smem, cudaStream_t stream) {
-  int st = set_smem((const void*)k_col_fft<E, NF>, smem);
+template <int N>
+int launch_col_w(const ColArgs& c, const Levels& L, int nl, cudaStream_t stream) {
+  using C = ColCfg<N>;
+  const size_t smem = (size_t(C::kXch) + N) * sizeof(float2) + size_t(C::E) * C::kThr * sizeof(float);
+  const dim3 grid(unsigned((c.Mh + C::kCols - 1) / C::kCols), unsigned((nl + c.lpc - 1) / c.lpc));
+  const void* fn = c.depth > 0.f ? (const void*)k_col_w<N, true> : (const void*)k_col_w<N, false>;
+  int st = set_smem(fn, smem);
   if (st) return st;
-  k_col_fft<E, NF><<<grid, kThreads, smem, stream>>>(c, L);
-  SWENSE_CUDA_TRY(cudaGetLastError());
-  count_launches(1);
-  return SWENSE_OK;
-}
-
-template <int N, int NF>
-int launch_col_stk(const ColArgs& c, const Levels& L, dim3 grid, size_t smem, cudaStream_t stream) {
-  smem += size_t(8) * stk_buf(N) * sizeof(float2);
-  int st = set_smem((const void*)k_col_stk<N, NF>, smem);
-  if (st) return st;
-  k_col_stk<N, NF><<<grid, kThreads, smem, stream>>>(c, L);
+  if (c.depth > 0.f) k_col_w<N, true><<<grid, C::kThr, smem, stream>>>(c, L);
+  else k_col_w<N, false><<<grid, C::kThr, smem, stream>>>(c, L);
   SWENSE_CUDA_TRY(cudaGetLastError());
   count_launches(1);
   return SWENSE_OK;
 }
 
 template <int N>
-int launch_row_stk(const RowArgs& r, dim3 grid, size_t smem, cudaStream_t stream) {
-  smem += size_t(8) * stk_buf(N) * sizeof(float2);
-  int st = set_smem((const void*)k_row_stk<N>, smem);
+int launch_row_w(const RowArgs& r, int nl, cudaStream_t stream) {
+  using W = WideRow<N>;
+  const size_t smem = size_t(W::kRows) * 2 * W::kBuf * sizeof(float2);
+  int st = set_smem((const void*)k_row_w<N>, smem);
   if (st) return st;
-  k_row_stk<N><<<grid, kThreads, smem, stream>>>(r);
-  SWENSE_CUDA_TRY(cudaGetLastError());
-  count_launches(1);
-  return SWENSE_OK;
-}
-
-template <int N, int NF>
-int launch_col_t(const ColArgs& c, const Levels& L, dim3 grid, cudaStream_t stream) {
-  const size_t smem = (size_t(N) * (kColBlock + 1) + size_t(8) * stk_buf(N)) * sizeof(float2) +
-                      (N <= 256 ? size_t(8) * 2 * N * sizeof(float) : 0);
-  int st = set_smem((const void*)k_col_t<N, NF>, smem);
-  if (st) return st;
-  k_col_t<N, NF><<<grid, kThreads, smem, stream>>>(c, L);
-  SWENSE_CUDA_TRY(cudaGetLastError());
-  count_launches(1);
-  return SWENSE_OK;
-}
-
-template <int N>
-int launch_col_tf(const ColArgs& c, const Levels& L, dim3 grid, cudaStream_t stream) {
-  const size_t smem = std::max(size_t(N) * (kColBlock + 1), size_t(8) * stk_buf(N)) * sizeof(float2);
-  int st = set_smem((const void*)k_col_tf<N>, smem);
-  if (st) return st;
-  grid.z = 4;
-  k_col_tf<N><<<grid, kThreads, smem, stream>>>(c, L);
-  SWENSE_CUDA_TRY(cudaGetLastError());
-  count_launches(1);
-  return SWENSE_OK;
-}
-
-template <int N>
-int launch_col_tf2(const ColArgs& c, const Levels& L, dim3 grid, cudaStream_t stream) {
-  const size_t smem = std::max(size_t(N) * kColBlock, size_t(16) * stk_buf(N / 2)) * sizeof(float2);
-  int st = set_smem((const void*)k_col_tf2<N>, smem);
-  if (st) return st;
-  grid.z = 4;
-  k_col_tf2<N><<<grid, 2 * kThreads, smem, stream>>>(c, L);
-  SWENSE_CUDA_TRY(cudaGetLastError());
-  count_launches(1);
-  return SWENSE_OK;
-}
-
-template <int N>
-int launch_row_t(const RowArgs& r, dim3 grid, cudaStream_t stream) {
-  const size_t smem = size_t(8) * stk_buf(N) * sizeof(float2);
-  int st = set_smem((const void*)k_row_t<N>, smem);
-  if (st) return st;
-  k_row_t<N><<<grid, kThreads, smem, stream>>>(r);
+  k_row_w<N><<<dim3(unsigned(r.Nyr / W::kRows), unsigned(nl)), W::T * W::kRows, smem, stream>>>(r);
   SWENSE_CUDA_TRY(cudaGetLastError());
   count_launches(1);
   return SWENSE_OK;
@@ -1301,134 +779,48 @@ int launch_row_tma(const RowArgs& r, unsigned nl, cudaStream_t stream) {
   return SWENSE_OK;
 }
 
-template <int N>
-int launch_row_t2(const RowArgs& r, dim3 grid, cudaStream_t stream) {
-  const size_t smem = size_t(8) * stk_buf(N) * sizeof(float2);
-  int st = set_smem((const void*)k_row_t2<N>, smem);
-  if (st) return st;
-  k_row_t2<N><<<grid, kThreads, smem, stream>>>(r);
-  SWENSE_CUDA_TRY(cudaGetLastError());
-  count_launches(1);
-  return SWENSE_OK;
-}
-
-// Transposed-intermediate pair (row variants 2 and 3): both transform lengths in 256..1024;
-// variant 3 runs one transform per warp in the row pass.
-int launch_pair_t(const ColArgs& c, const RowArgs& r, const Levels& L, int nl, cudaStream_t s,
-                  bool one_per_warp, bool staged = false, int which = 0, int colv = 0) {
-  const dim3 gc(unsigned((c.Mh + kColBlock - 1) / kColBlock), unsigned((nl + c.lpc - 1) / c.lpc));
-  const dim3 gr(unsigned((r.Nyr + 7) / 8), unsigned(nl));
-  const dim3 gr2(unsigned((r.Nyr + 3) / 4), unsigned(nl));
+// Transposed pair: `which` = 1 the column pass alone, 2 the row pass alone, 0 both; staged: the row
+// pass whose inputs arrive by bulk copies (256- to 1024-point rows; others take the plain one).
+int launch_pair(const ColArgs& c, const RowArgs& r, const Levels& L, int nl, cudaStream_t s, bool staged = false,
+                int which = 0) {
   int st = SWENSE_OK;
-  if (which != 2 && colv == 1) {
+  if (which != 2) {
     switch (c.Nyr) {
-      case 256: st = launch_col_tf<256>(c, L, gc, s); break;
-      case 512: st = launch_col_tf<512>(c, L, gc, s); break;
-      case 1024: st = launch_col_tf2<1024>(c, L, gc, s); break;
-      default: return fail(SWENSE_ERR_UNSUPPORTED, "transposed pair: column length");
-    }
-  } else if (which != 2) {
-    switch (c.Nyr) {
-      case 256: st = launch_col_t<256, 2>(c, L, gc, s); break;
-      case 512: st = launch_col_t<512, 1>(c, L, gc, s); break;
-      case 1024: st = launch_col_t<1024, 1>(c, L, gc, s); break;
+      case 32: st = launch_col_w<32>(c, L, nl, s); break;
+      case 64: st = launch_col_w<64>(c, L, nl, s); break;
+      case 128: st = launch_col_w<128>(c, L, nl, s); break;
+      case 256: st = launch_col_w<256>(c, L, nl, s); break;
+      case 512: st = launch_col_w<512>(c, L, nl, s); break;
+      case 1024: st = launch_col_w<1024>(c, L, nl, s); break;
       default: return fail(SWENSE_ERR_UNSUPPORTED, "transposed pair: column length");
     }
   }
   if (st || which == 1) return st;
-  if (one_per_warp && r.Nxr == 2048) return launch_row_t2<2048>(r, gr2, s);   // 64 elements a lane
-  switch (r.Nxr) {                               // rows longer than a warp transform
-    case 2048: return launch_row_tb<2048>(r, unsigned(nl), s);
-    case 4096: return launch_row_tb<4096>(r, unsigned(nl), s);
-    case 8192: return launch_row_tb<8192>(r, unsigned(nl), s);
-    default: break;
-  }
   if (staged) {
     switch (r.Nxr) {
       case 256: return launch_row_tma<256>(r, unsigned(nl), s);
       case 512: return launch_row_tma<512>(r, unsigned(nl), s);
       case 1024: return launch_row_tma<1024>(r, unsigned(nl), s);
-      default: return fail(SWENSE_ERR_UNSUPPORTED, "staged row pass: row length");
-    }
-  }
-  if (one_per_warp) {
-    switch (r.Nxr) {
-      case 256: return launch_row_t2<256>(r, gr2, s);
-      case 512: return launch_row_t2<512>(r, gr2, s);
-      case 1024: return launch_row_t2<1024>(r, gr2, s);
-      default: return fail(SWENSE_ERR_UNSUPPORTED, "transposed pair: row length");
+      default: break;
     }
   }
   switch (r.Nxr) {
-    case 256: return launch_row_t<256>(r, gr, s);
-    case 512: return launch_row_t<512>(r, gr, s);
-    case 1024: return launch_row_t<1024>(r, gr, s);
+    case 32: return launch_row_w<32>(r, nl, s);
+    case 64: return launch_row_w<64>(r, nl, s);
+    case 128: return launch_row_w<128>(r, nl, s);
+    case 256: return launch_row_w<256>(r, nl, s);
+    case 512: return launch_row_w<512>(r, nl, s);
+    case 1024: return launch_row_w<1024>(r, nl, s);
+    case 2048: return launch_row_w<2048>(r, nl, s);
+    case 4096: return launch_row_tb<4096>(r, unsigned(nl), s);
+    case 8192: return launch_row_tb<8192>(r, unsigned(nl), s);
     default: return fail(SWENSE_ERR_UNSUPPORTED, "transposed pair: row length");
   }
 }
 
-int launch_col_e(int E, const ColArgs& c, const Levels& L, dim3 grid, size_t smem, cudaStream_t s) {
-  switch (E) {
-    case 1: return launch_col<1, 4>(c, L, grid, smem, s);
-    case 2: return launch_col<2, 4>(c, L, grid, smem, s);
-    case 4: return launch_col<4, 4>(c, L, grid, smem, s);
-    case 8: return launch_col_stk<256, 2>(c, L, grid, smem, s);
-    case 16: return launch_col_stk<512, 1>(c, L, grid, smem, s);
-    case 32: return launch_col_stk<1024, 1>(c, L, grid, smem, s);
-    default: return fail(SWENSE_ERR_UNSUPPORTED, "column transform size");
-  }
-}
-
-template <int E>
-int launch_row(const RowArgs& r, dim3 grid, size_t smem, cudaStream_t stream) {
-  int st = set_smem((const void*)k_row_fft<E>, smem);
-  if (st) return st;
-  k_row_fft<E><<<grid, kThreads, smem, stream>>>(r);
-  SWENSE_CUDA_TRY(cudaGetLastError());
-  count_launches(1);
-  return SWENSE_OK;
-}
-
-template <int N>
-int launch_row_half(const RowArgs& r, dim3 grid, cudaStream_t stream) {
-  static_assert(kRowBlock * 32 == kThreads, "one staged row per warp");
-  const size_t smem = std::max(size_t(2) * r.Mh * (kRowBlock + 1), size_t(8) * stk_buf(N)) * sizeof(float2);
-  int st = set_smem((const void*)k_row_half<N>, smem);
-  if (st) return st;
-  grid.z = 2;
-  k_row_half<N><<<grid, kThreads, smem, stream>>>(r);
-  SWENSE_CUDA_TRY(cudaGetLastError());
-  count_launches(1);
-  return SWENSE_OK;
-}
-
-int launch_row_e(int E, const RowArgs& r, dim3 grid, size_t smem, cudaStream_t s, int rowv = 0) {
-  if (rowv == 1) {
-    switch (E) {
-      case 8: return launch_row_half<256>(r, grid, s);
-      case 16: return launch_row_half<512>(r, grid, s);
-      case 32: return launch_row_half<1024>(r, grid, s);
-      default: break;                   // shorter rows: the joint kernel
-    }
-  }
-  switch (E) {
-    case 1: return launch_row<1>(r, grid, smem, s);
-    case 2: return launch_row<2>(r, grid, smem, s);
-    case 4: return launch_row<4>(r, grid, smem, s);
-    case 8: return launch_row_stk<256>(r, grid, smem, s);
-    case 16: return launch_row_stk<512>(r, grid, smem, s);
-    case 32: return launch_row_stk<1024>(r, grid, smem, s);
-    default: return fail(SWENSE_ERR_UNSUPPORTED, "row transform size");
-  }
-}
-
-// The warp-register path covers 32 <= ny_r, nx_r <= 1024 (3-D only); the transposed pair also
-// takes rows of 2048..8192 points (block-wide row transforms) over 256..1024-point columns.
-bool warp_path(int ny, int64_t Nxr, int64_t Nyr) {
-  return ny > 1 && Nyr >= 32 && Nyr <= 1024 && Nxr >= 32 && Nxr <= 1024;
-}
+// The transposed pair covers 3-D grids with 32- to 1024-point columns and rows of 32 points and more.
 bool pair_path(int ny, int64_t Nxr, int64_t Nyr) {
-  return ny > 1 && Nyr >= 256 && Nyr <= 1024 && Nxr >= 256 && Nxr <= SWENSE_MAX_FFT;
+  return ny > 1 && Nyr >= 32 && Nyr <= 1024 && Nxr >= 32 && Nxr <= SWENSE_MAX_FFT;
 }
 
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
@@ -1481,19 +873,49 @@ int plan_grid(const swense_modes* md, int32_t n_tl, const double* t, const swens
   p->Nyr = Nyr;
   p->nslot = size_t(ny) * p->nxh1;
   p->per_level = size_t(4) * Nyr * trans_ld(p->Mh) * sizeof(float2);
-  p->prop_bytes = md->omega ? size_t(n_tl) * 3 * p->nslot * sizeof(float2) : 0;
+  p->omega = md->omega != nullptr;
   p->geta_bytes = ny > 1 ? size_t(Nyr) * p->Mh * sizeof(float2) : 0;
   return SWENSE_OK;
 }
 
-// Untuned column-pass variant of the transposed pair: one modal field per CTA (k_col_tf) for
-// 1024-point columns, whose k_col_t runs one CTA per SM with only Mh / 8 CTAs per level.
-int default_colv(const GridPlan& p) { return pair_path(p.ny, p.Nxr, p.Nyr) && p.Nyr >= 1024 ? 1 : 0; }
+// The launch shape of a request: the tuned one of its grid shape, else the transposed pair where it
+// applies and the shared-memory path elsewhere.
+struct Shape {
+  int chunk, lpc, rowv;   // chunk: levels (the pair: slots, of all time levels and eta) per chunk
+};
+
+// Whether a launch shape runs the transposed pair, and with eta's transforms among its slots (the
+// row passes of 4096 points and more and the staged one take levels only).
+bool runs_pair(const GridPlan& p, int lpc) { return lpc > 0 && pair_path(p.ny, p.Nxr, p.Nyr); }
+bool eta_inline(const GridPlan& p, const Shape& s) { return runs_pair(p, s.lpc) && p.Nxr <= 2048 && s.rowv != 4; }
+// Slots of a request: levels of all time levels (and eta) for the pair, else one time level's levels.
+int grid_slots(const GridPlan& p, const Shape& s) {
+  return runs_pair(p, s.lpc) ? p.n_tl * (p.nz + (eta_inline(p, s) ? 1 : 0)) : p.nz;
+}
+
+int chunk_slots(const GridPlan& p, const Shape& s, size_t bytes) {
+  return int(std::max<size_t>(1, std::min<size_t>(size_t(grid_slots(p, s)), bytes / p.per_level)));
+}
+Shape grid_shape(const GridPlan& p) {
+  const Tune tn = tuned(p.nx, p.ny, p.pad, p.nz);
+  Shape s;
+  s.lpc = tn.lpc >= 0 ? tn.lpc : (pair_path(p.ny, p.Nxr, p.Nyr) ? kColLevels : 0);
+  s.rowv = tn.lpc >= 0 ? tn.rowv : 0;
+  s.chunk = p.ny > 1 ? chunk_slots(p, s, tn.chunk_bytes) : 0;
+  return s;
+}
+
+// Scratch bytes of the prepared modes: the pair's modal fields and eta's propagated modes, or the
+// three propagated arrays of the shared-memory path.
+size_t modes_bytes(const GridPlan& p, bool pair) {
+  const size_t own = p.omega ? (pair ? 1 : 3) * p.nslot : 0;
+  return size_t(p.n_tl) * (own + (pair ? size_t(5) * p.ny * trans_ld(p.Mh) : 0)) * sizeof(float2);
+}
 
 // Scratch bytes for a level chunk of `chunk` levels (0 when no scratch is needed).
-size_t scratch_bytes(const GridPlan& p, int chunk, int nbuf = 1) {
+size_t scratch_bytes(const GridPlan& p, int chunk, int nbuf, bool pair) {
   const size_t g_bytes = p.ny > 1 ? size_t(chunk) * p.per_level : 0;
-  return align256(p.prop_bytes) + align256(p.geta_bytes) + size_t(nbuf) * align256(g_bytes);
+  return align256(modes_bytes(p, pair)) + align256(p.geta_bytes) + size_t(nbuf) * align256(g_bytes);
 }
 
 // Library-internal second stream and events (per device) for the two-stream transform
@@ -1533,26 +955,30 @@ int get_pipe(Pipe** out) {
 // the eta transform of each time level on the per-device second stream, forked after that time
 // level's propagated modes exist and joined back before the call returns (graph-capturable).
 int launch_grid(const GridPlan& p, const swense_modes* md, const double* t, float* nodes, float* eta,
-                void* ws, int chunk, cudaStream_t stream, int lpc = kColLevels, int rowv = 0,
-                int overlap = 0, int eta_side = 0, int colv = 0) {
+                void* ws, const Shape& shape, cudaStream_t stream, bool overlap, bool eta_side) {
   const float2* tw = nullptr;
   {
     int st = twiddles(stream, &tw);
     if (st) return st;
   }
+  const int chunk = shape.chunk;
   const int ny = p.ny, nz = p.nz, Mh = p.Mh, nxh1 = p.nxh1;
   const int64_t Nxr = p.Nxr, Nyr = p.Nyr;
   const size_t nslot = p.nslot;
-  float2* prop = static_cast<float2*>(ws);
-  float2* g_eta = reinterpret_cast<float2*>(static_cast<char*>(ws) + align256(p.prop_bytes));
-  float2* g_lev = reinterpret_cast<float2*>(static_cast<char*>(ws) + align256(p.prop_bytes) +
-                                            align256(p.geta_bytes));
+  const bool pair = runs_pair(p, shape.lpc);
+  const int ld = trans_ld(Mh);
+  float2* prop = static_cast<float2*>(ws);       // pair: eta's modes (with omega), then the modal fields
+  float2* form = prop + (pair && md->omega ? size_t(p.n_tl) * nslot : 0);
+  const size_t b_modes = align256(modes_bytes(p, pair));
+  float2* g_eta = reinterpret_cast<float2*>(static_cast<char*>(ws) + b_modes);
+  float2* g_lev = reinterpret_cast<float2*>(static_cast<char*>(ws) + b_modes + align256(p.geta_bytes));
   // second intermediate buffer of the two-stream pipeline
   float2* g_lev2 = reinterpret_cast<float2*>(reinterpret_cast<char*>(g_lev) +
                                              align256(size_t(chunk) * p.per_level));
   Pipe* pipe = nullptr;
-  const bool use_pipe = overlap && rowv == 2 && pair_path(p.ny, p.Nxr, p.Nyr);
-  const bool eta_fork = eta_side && p.ny > 1;
+  const bool use_pipe = overlap && pair;
+  const bool inline_eta = eta_inline(p, shape);
+  const bool eta_fork = eta_side && p.ny > 1 && !inline_eta;
   if (use_pipe || eta_fork) {
     int st = get_pipe(&pipe);
     if (st) return st;
@@ -1583,6 +1009,22 @@ int launch_grid(const GridPlan& p, const swense_modes* md, const double* t, floa
   const float depth = md->depth > 0 ? float(md->depth) : 0.f;
   const int log2Nxr = ilog2(Nxr), log2Nyr = ilog2(Nyr);
 
+  PropTimes T{};
+  for (int l = 0; md->omega && l < p.n_tl; ++l) T.dt[l] = t[l] - md->t_ref;
+  const float2 *A_eta = reinterpret_cast<const float2*>(md->A_eta), *A_phi = reinterpret_cast<const float2*>(md->A_phi),
+               *A_phit = reinterpret_cast<const float2*>(md->A_phit);
+  if (ny == 1) {
+    const size_t smem = size_t(2) * Nxr * sizeof(float2);
+    int st = set_smem((const void*)k_line, smem);
+    if (st) return st;
+    const LineArgs a{A_eta, A_phi, A_phit, md->omega, reinterpret_cast<float4*>(nodes), eta, tw, nxh1, Mh, int(Nxr),
+                     log2Nxr, nz, p.spline, kxs, depth};
+    k_line<<<dim3(unsigned(nz + 1), unsigned(p.n_tl)), kThreads, smem, stream>>>(a, p.lev, T);
+    SWENSE_CUDA_TRY(cudaGetLastError());
+    count_launches(1);
+    return SWENSE_OK;
+  }
+
   // launch shapes
   int fp = 4, cb = 1;
   while (fp > 1 && size_t(fp) * Nyr * sizeof(float2) > kSmemBudget) fp >>= 1;
@@ -1608,18 +1050,22 @@ int launch_grid(const GridPlan& p, const swense_modes* md, const double* t, floa
     if (st) return st;
   }
 
-  if (md->omega) {                                // all time levels' modes at once
-    PropTimes T{};
-    for (int l = 0; l < p.n_tl; ++l) T.dt[l] = t[l] - md->t_ref;
-    k_propagate<<<dim3(unsigned((nslot + 255) / 256), unsigned(p.n_tl)), 256, 0, stream>>>(
-        reinterpret_cast<const float2*>(md->A_eta), reinterpret_cast<const float2*>(md->A_phi),
-        reinterpret_cast<const float2*>(md->A_phit), md->omega, int(nslot), T, prop);
+  if (md->omega || pair) {                        // all time levels' modes at once
+    const dim3 gm(unsigned((nslot + 255) / 256), unsigned(p.n_tl));
+    if (pair) {
+      const FormArgs f{A_eta, A_phi, A_phit, md->omega, inline_eta ? nullptr : prop, form, ny, nxh1, ld, int(Nxr), int(Nyr), p.spline, kxs, kys};
+      k_form_modes<<<gm, 256, 0, stream>>>(f, T);
+    } else {
+      k_propagate<<<gm, 256, 0, stream>>>(A_eta, A_phi, A_phit, md->omega, int(nslot), T, prop);
+    }
     SWENSE_CUDA_TRY(cudaGetLastError());
     count_launches(1);
   }
-  for (int l = 0; l < p.n_tl; ++l) {
-    const float2 *Ae, *Ap, *At;
-    if (md->omega) {
+  for (int l = 0; l < p.n_tl && !inline_eta; ++l) {
+    const float2 *Ae, *Ap = nullptr, *At = nullptr;
+    if (md->omega && pair) {
+      Ae = prop + size_t(l) * nslot;
+    } else if (md->omega) {
       float2* o = prop + size_t(l) * 3 * nslot;
       Ae = o;
       Ap = o + nslot;
@@ -1633,9 +1079,6 @@ int launch_grid(const GridPlan& p, const swense_modes* md, const double* t, floa
     float* eta_l = eta + size_t(l) * Nyr * Nxr;
 
     PassBArgs b{};
-    b.A_phi = Ap;
-    b.A_phit = At;
-    b.A_eta = Ae;
     b.nodes = nodes_l;
     b.eta = eta_l;
     b.tw = tw;
@@ -1643,24 +1086,6 @@ int launch_grid(const GridPlan& p, const swense_modes* md, const double* t, floa
     b.Nxr = int(Nxr);
     b.log2Nxr = log2Nxr;
     b.Nyr = int(Nyr);
-    b.kxs = kxs;
-    b.depth = depth;
-    b.spline = p.spline;
-
-    if (ny == 1) {
-      b.mode = B_ETA_DIRECT;
-      b.rb = 1;
-      b.lev0 = 0;
-      k_pass_b<<<dim3(1, 1), kThreads, size_t(Nxr) * sizeof(float2), stream>>>(b, p.lev);
-      SWENSE_CUDA_TRY(cudaGetLastError());
-      count_launches(1);
-      b.mode = B_LEVEL_DIRECT;
-      b.rb = 1;
-      k_pass_b<<<dim3(1, nz), kThreads, rowb, stream>>>(b, p.lev);
-      SWENSE_CUDA_TRY(cudaGetLastError());
-      count_launches(1);
-      continue;
-    }
 
     PassAArgs a{};
     a.A_phi = Ap;
@@ -1700,85 +1125,11 @@ int launch_grid(const GridPlan& p, const swense_modes* md, const double* t, floa
     b.rb = rb_eta;
     b.lev0 = 0;
     k_pass_b<<<dim3(unsigned((Nyr + 2 * rb_eta - 1) / (2 * rb_eta)), 1), kThreads, smem_b_eta,
-               es>>>(b, p.lev);
+               es>>>(b);
     SWENSE_CUDA_TRY(cudaGetLastError());
     count_launches(1);
 
-    if (lpc > 0 && (warp_path(ny, Nxr, Nyr) || (pair_path(ny, Nxr, Nyr) && rowv >= 2))) {
-      ColArgs ca{};
-      ca.A_phi = Ap;
-      ca.A_phit = At;
-      ca.G = g_lev;
-      ca.tw = tw;
-      ca.ny = ny;
-      ca.nxh1 = nxh1;
-      ca.Mh = Mh;
-      ca.Nyr = int(Nyr);
-      ca.cb = kColBlock;
-      ca.lpc = lpc;
-      ca.kxs = kxs;
-      ca.kys = kys;
-      ca.depth = depth;
-      ca.Nxr = int(Nxr);
-      ca.spline = p.spline;
-      RowArgs ra{};
-      ra.G = g_lev;
-      ra.nodes = nodes_l;
-      ra.tw = tw;
-      ra.Mh = Mh;
-      ra.Nxr = int(Nxr);
-      ra.Nyr = int(Nyr);
-      ra.rb = kRowBlock;
-      ra.polls = kMbarPolls;
-      ra.selftest = 0;
-      const size_t smem_col = size_t(2) * ny * (kColBlock + 1) * sizeof(float2);
-      const size_t smem_row = size_t(4) * Mh * (kRowBlock + 1) * sizeof(float2);
-      ca.ldG = ra.ldG = trans_ld(Mh);
-      const bool pair_t = (rowv == 2 || rowv == 3 || (rowv == 4 && Nxr <= 1024)) && pair_path(ny, Nxr, Nyr);
-  
-      for (int l0 = 0; l0 < nz; l0 += chunk) {
-        if (pair_t && use_pipe) {
-          const int nl = std::min(chunk, nz - l0);
-          const int b = chunk_no & 1;
-          ca.lev0 = l0;
-          ca.nlev = nl;
-          ra.lev0 = l0;
-          ca.G = b ? g_lev2 : g_lev;
-          ra.G = ca.G;
-          if (chunk_no >= 2) SWENSE_CUDA_TRY(cudaStreamWaitEvent(stream, pipe->row_done[b], 0));
-          int st = launch_pair_t(ca, ra, p.lev, nl, stream, false, false, 1, colv);   // column pass
-          if (st) return st;
-          SWENSE_CUDA_TRY(cudaEventRecord(pipe->col_done[b], stream));
-          SWENSE_CUDA_TRY(cudaStreamWaitEvent(pipe->side, pipe->col_done[b], 0));
-          st = launch_pair_t(ca, ra, p.lev, nl, pipe->side, false, false, 2);    // row pass
-          if (st) return st;
-          SWENSE_CUDA_TRY(cudaEventRecord(pipe->row_done[b], pipe->side));
-          ++chunk_no;
-          continue;
-        }
-        if (pair_t) {
-          const int nl = std::min(chunk, nz - l0);
-          ca.lev0 = l0;
-          ca.nlev = nl;
-          ra.lev0 = l0;
-          int st = launch_pair_t(ca, ra, p.lev, nl, stream, rowv == 3, rowv == 4, 0, colv);
-          if (st) return st;
-          continue;
-        }
-        const int nl = std::min(chunk, nz - l0);
-        ca.lev0 = l0;
-        ca.nlev = nl;
-        ra.lev0 = l0;
-        int st = launch_col_e(int(Nyr / 32), ca, p.lev,
-                              dim3((Mh + kColBlock - 1) / kColBlock, (nl + lpc - 1) / lpc),
-                              smem_col, stream);
-        if (!st) st = launch_row_e(int(Nxr / 32), ra,
-                                   dim3(unsigned((Nyr + kRowBlock - 1) / kRowBlock), nl), smem_row, stream,
-                                   rowv);
-        if (st) return st;
-      }
-      continue;
-    }
+    if (pair) continue;                          // the levels of all time levels follow
     a.eta_mode = 0;
     a.fp = fp;
     a.cb = cb;
@@ -1793,10 +1144,59 @@ int launch_grid(const GridPlan& p, const swense_modes* md, const double* t, floa
       k_pass_a<<<dim3((Mh + cb - 1) / cb, nl), kThreads, smem_a, stream>>>(a, p.lev);
       SWENSE_CUDA_TRY(cudaGetLastError());
       count_launches(1);
-      k_pass_b<<<dim3(unsigned((Nyr + rb - 1) / rb), nl), kThreads, smem_b, stream>>>(b, p.lev);
+      k_pass_b<<<dim3(unsigned((Nyr + rb - 1) / rb), nl), kThreads, smem_b, stream>>>(b);
       SWENSE_CUDA_TRY(cudaGetLastError());
       count_launches(1);
     }
+  }
+  if (!pair) return SWENSE_OK;
+  ColArgs ca{};
+  ca.A = form;
+  ca.G = g_lev;
+  ca.tw = tw;
+  ca.ny = ny;
+  ca.Mh = Mh;
+  ca.Nyr = int(Nyr);
+  ca.nz = nz;
+  ca.n_lev = p.n_tl * nz;
+  ca.lpc = shape.lpc;
+  ca.kxs = kxs;
+  ca.kys = kys;
+  ca.depth = depth;
+  RowArgs ra{};
+  ra.G = g_lev;
+  ra.nodes = reinterpret_cast<float4*>(nodes);
+  ra.eta = eta;
+  ra.tw = tw;
+  ra.Mh = Mh;
+  ra.Nxr = int(Nxr);
+  ra.Nyr = int(Nyr);
+  ra.n_lev = ca.n_lev;
+  ra.polls = kMbarPolls;
+  ra.selftest = 0;
+  ca.ldG = ra.ldG = ld;
+  const int slots = grid_slots(p, shape);
+  for (int l0 = 0; l0 < slots; l0 += chunk) {
+    const int nl = std::min(chunk, slots - l0);
+    ca.lev0 = ra.lev0 = l0;
+    ca.nlev = nl;
+    if (!use_pipe) {
+      int st = launch_pair(ca, ra, p.lev, nl, stream, shape.rowv == 4);
+      if (st) return st;
+      continue;
+    }
+    const int b = chunk_no & 1;
+    ca.G = b ? g_lev2 : g_lev;
+    ra.G = ca.G;
+    if (chunk_no >= 2) SWENSE_CUDA_TRY(cudaStreamWaitEvent(stream, pipe->row_done[b], 0));
+    int st = launch_pair(ca, ra, p.lev, nl, stream, false, 1);          // column pass
+    if (st) return st;
+    SWENSE_CUDA_TRY(cudaEventRecord(pipe->col_done[b], stream));
+    SWENSE_CUDA_TRY(cudaStreamWaitEvent(pipe->side, pipe->col_done[b], 0));
+    st = launch_pair(ca, ra, p.lev, nl, pipe->side, false, 2);          // row pass
+    if (st) return st;
+    SWENSE_CUDA_TRY(cudaEventRecord(pipe->row_done[b], pipe->side));
+    ++chunk_no;
   }
   return SWENSE_OK;
 }
@@ -1880,13 +1280,8 @@ int fields_on_grid_shifted(const GridPlan& p, const swense_modes* md, const doub
   sp.Nyr = p.ny > 1 ? int64_t(p2) * p.ny : 1;
   sp.per_level = size_t(4) * sp.Nyr * trans_ld(sp.Mh) * sizeof(float2);
   sp.geta_bytes = p.ny > 1 ? size_t(sp.Nyr) * sp.Mh * sizeof(float2) : 0;
-  const Tune tn = tuned(p.nx, p.ny, p2, p.nz);
-  const int chunk = p.ny > 1 ? int(std::max<size_t>(1, std::min<size_t>(p.nz, tn.chunk_bytes / sp.per_level))) : 0;
-  const bool pair = pair_path(sp.ny, sp.Nxr, sp.Nyr);
-  const int lpc = tn.lpc >= 0 ? tn.lpc : (pair ? 4 : ((sp.Nxr <= 512 && sp.Nyr <= 512) ? kColLevels : 0));
-  const int rowv0 = tn.lpc >= 0 ? tn.rowv : (pair ? 2 : 0);
-  const int rowv = rowv0 == 5 ? 2 : rowv0;                    // one stream for the sub-grids
-  const size_t scratch = align256(scratch_bytes(sp, chunk, 1));
+  const Shape shape = grid_shape(sp);                         // one stream for the sub-grids
+  const size_t scratch = align256(scratch_bytes(sp, shape.chunk, 1, runs_pair(sp, shape.lpc)));
   const int64_t sub_nodes = int64_t(p.n_tl) * p.nz * sp.Nyr * sp.Nxr;
   const int64_t sub_eta = int64_t(p.n_tl) * sp.Nyr * sp.Nxr;
   const int64_t nmodes = int64_t(md->n_snap) * p.ny * p.nxh1;
@@ -1914,7 +1309,7 @@ int fields_on_grid_shifted(const GridPlan& p, const swense_modes* md, const doub
           p.spline, sm, sm + b_modes / sizeof(float2), sm + 2 * (b_modes / sizeof(float2)));
       SWENSE_CUDA_TRY(cudaGetLastError());
       count_launches(1);
-      st = launch_grid(sp, &shifted, t, reinterpret_cast<float*>(snodes), seta, ws, chunk, stream, lpc, rowv, 0, 0);
+      st = launch_grid(sp, &shifted, t, reinterpret_cast<float*>(snodes), seta, ws, shape, stream, false, false);
       if (st) return st;
       const int64_t tot = sub_nodes + sub_eta;
       const int64_t gb = std::min<int64_t>((tot + threads - 1) / threads, int64_t(152) * 64);
@@ -1941,23 +1336,14 @@ extern "C" int swense_fields_on_grid(const swense_modes* md, int32_t n_tl, const
   int st = plan_grid(md, n_tl, t, desc, nodes, eta, &p);
   if (st) return st;
   if (!is_pow2(p.pad)) return fields_on_grid_shifted(p, md, t, nodes, eta, stream);
-  const Tune tn = tuned(p.nx, p.ny, p.pad, p.nz);
-  const int chunk = p.ny > 1 ? int(std::max<size_t>(1, std::min<size_t>(p.nz, tn.chunk_bytes / p.per_level))) : 0;
+  const Shape shape = grid_shape(p);
   void* ws = nullptr;
-  // untuned default: the transposed Stockham pair where both lengths are 256..1024, else the
-  // warp path where its transforms stay in registers (n <= 512), else the shared-memory path
-  const bool pair = pair_path(p.ny, p.Nxr, p.Nyr);
-  const int lpc = tn.lpc >= 0 ? tn.lpc : (pair ? 4 : ((p.Nxr <= 512 && p.Nyr <= 512) ? kColLevels : 0));
-  const int rowv = tn.lpc >= 0 ? tn.rowv : (pair ? 2 : 0);
-  const int colv = tn.lpc >= 0 ? tn.colv : default_colv(p);
-  // variant 5: variant 2 with its column and row passes pipelined over two streams
-  const size_t ws_bytes = scratch_bytes(p, chunk, rowv == 5 ? 2 : 1);
+  const size_t ws_bytes = scratch_bytes(p, shape.chunk, shape.rowv == 5 ? 2 : 1, runs_pair(p, shape.lpc));
   if (ws_bytes) {
     st = workspace(ws_bytes, stream, &ws);
     if (st) return st;
   }
-  return launch_grid(p, md, t, nodes, eta, ws, chunk, stream, lpc, rowv == 5 ? 2 : rowv, rowv == 5, 1,
-                     colv);
+  return launch_grid(p, md, t, nodes, eta, ws, shape, stream, shape.rowv == 5, true);
 }
 
 namespace swense {
@@ -1972,9 +1358,8 @@ int grid_scratch(const swense_modes* md, int32_t n_tl, const double* t, const sw
   int st = plan_grid(md, n_tl, t, desc, nodes, eta, &p);
   if (st) return st;
   if (!is_pow2(p.pad)) return fail(SWENSE_ERR_UNSUPPORTED, "batched grids take power-of-two padding factors");
-  const Tune tn = tuned(p.nx, p.ny, p.pad, p.nz);
-  const int chunk = p.ny > 1 ? int(std::max<size_t>(1, std::min<size_t>(p.nz, tn.chunk_bytes / p.per_level))) : 0;
-  *bytes = scratch_bytes(p, chunk, 1);
+  const Shape shape = grid_shape(p);
+  *bytes = scratch_bytes(p, shape.chunk, 1, runs_pair(p, shape.lpc));
   return SWENSE_OK;
 }
 
@@ -1984,14 +1369,7 @@ int grid_with_scratch(const swense_modes* md, int32_t n_tl, const double* t, con
   int st = plan_grid(md, n_tl, t, desc, nodes, eta, &p);
   if (st) return st;
   if (!is_pow2(p.pad)) return fail(SWENSE_ERR_UNSUPPORTED, "batched grids take power-of-two padding factors");
-  const Tune tn = tuned(p.nx, p.ny, p.pad, p.nz);
-  const int chunk = p.ny > 1 ? int(std::max<size_t>(1, std::min<size_t>(p.nz, tn.chunk_bytes / p.per_level))) : 0;
-  const bool pair = pair_path(p.ny, p.Nxr, p.Nyr);
-  const int lpc = tn.lpc >= 0 ? tn.lpc : (pair ? 4 : ((p.Nxr <= 512 && p.Nyr <= 512) ? kColLevels : 0));
-  int rowv = tn.lpc >= 0 ? tn.rowv : (pair ? 2 : 0);
-  if (rowv == 5) rowv = 2;
-  const int colv = tn.lpc >= 0 ? tn.colv : default_colv(p);
-  return launch_grid(p, md, t, nodes, eta, ws, chunk, stream, lpc, rowv, 0, 0, colv);
+  return launch_grid(p, md, t, nodes, eta, ws, grid_shape(p), stream, false, false);
 }
 
 }  // namespace swense
@@ -2016,40 +1394,32 @@ extern "C" int swense_autotune_grid(const swense_modes* md, int32_t n_tl, const 
     // evicts the grid): the workspace, sized for the largest candidate and at least twice the
     // L2, is overwritten before each repetition (its contents are scratch).
     constexpr size_t kFlushBytes = size_t(256) << 20;
-    const size_t max_chunk = std::max<size_t>(1, std::min<size_t>(p.nz, (size_t(256) << 20) / p.per_level));
-    const size_t ws_all = std::max(scratch_bytes(p, int(max_chunk), 2), kFlushBytes);
+    const int max_chunk = chunk_slots(p, Shape{0, 1, 0}, size_t(256) << 20);
+    const size_t ws_all = std::max(scratch_bytes(p, max_chunk, 2, pair_path(p.ny, p.Nxr, p.Nyr)), kFlushBytes);
     {
       void* ws = nullptr;
       st = workspace(ws_all, stream, &ws);
       if (st) return st;
     }
+    const bool pp = pair_path(p.ny, p.Nxr, p.Nyr);
     for (int lpc : {0, 1, 2, 4})
-    for (int rv : {0, 1, 2, 3, 4, 5, 2 + 16, 3 + 16, 4 + 16, 5 + 16}) {
-      const int rowv = rv & 15, colv = rv >> 4;
-      const bool wp = warp_path(p.ny, p.Nxr, p.Nyr), pp = pair_path(p.ny, p.Nxr, p.Nyr);
-      // beyond the warp path, the pair runs with row variant 2 (block rows) or, for 2048-point
-      // rows, 3 (one 64-element-per-lane transform per warp)
-      const bool pair_ok = pp && (rowv == 2 || (rowv == 3 && p.Nxr == 2048));
-      if (lpc > 0 && !wp && !pair_ok) continue;
-      if (rowv && (lpc == 0 || p.Nxr < 256)) continue;   // only the Stockham row sizes have variants
-      if (rowv >= 2 && !pp) continue;
-      if (colv && !(pp && rowv >= 2)) continue;
-      if (!wp && !pair_ok && lpc > 0) continue;
-      if (rowv == 4 && p.Nxr > 1024) continue;
-      if (p.Nxr > 1024 && rowv != 2 && !(rowv == 3 && p.Nxr == 2048)) continue;
+    for (int rowv : {0, 4, 5}) {
+      if (lpc > 0 && !pp) continue;
+      if (rowv && lpc == 0) continue;
+      if (rowv == 4 && (p.Nxr < 256 || p.Nxr > 1024)) continue;
       for (size_t mb : {16, 32, 64, 96, 128, 256}) {
         const size_t cb = mb << 20;
-        const int chunk = int(std::max<size_t>(1, std::min<size_t>(p.nz, cb / p.per_level)));
+        Shape shape{0, lpc, rowv};
+        shape.chunk = chunk_slots(p, shape, cb);
         void* ws = nullptr;
         st = workspace(ws_all, stream, &ws);
-        const int rv2 = rowv == 5 ? 2 : rowv;
-        if (!st) st = launch_grid(p, md, t, nodes, eta, ws, chunk, stream, lpc, rv2, rowv == 5, 1, colv);   // warm
+        if (!st) st = launch_grid(p, md, t, nodes, eta, ws, shape, stream, rowv == 5, true);   // warm
         // best of five (the fastest repetition is the least disturbed one)
         float ms = 0.f, tot = 1e30f;
         for (int rep = 0; rep < 5 && !st; ++rep) {
           if (cudaMemsetAsync(ws, 0, kFlushBytes, stream) != cudaSuccess) { st = SWENSE_ERR_CUDA; break; }
           if (cudaEventRecord(e0, stream) != cudaSuccess) { st = SWENSE_ERR_CUDA; break; }
-          st = launch_grid(p, md, t, nodes, eta, ws, chunk, stream, lpc, rv2, rowv == 5, 1, colv);
+          st = launch_grid(p, md, t, nodes, eta, ws, shape, stream, rowv == 5, true);
           if (cudaEventRecord(e1, stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
               cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) st = SWENSE_ERR_CUDA;
           tot = std::min(tot, ms);
@@ -2060,7 +1430,6 @@ extern "C" int swense_autotune_grid(const swense_modes* md, int32_t n_tl, const 
           best.lpc = lpc;
           best.chunk_bytes = cb;
           best.rowv = rowv;
-          best.colv = colv;
         }
       }
       if (st) break;
@@ -2073,7 +1442,7 @@ extern "C" int swense_autotune_grid(const swense_modes* md, int32_t n_tl, const 
   }
   if (lpc_out) *lpc_out = best.lpc;
   if (chunk_bytes_out) *chunk_bytes_out = int64_t(best.chunk_bytes);
-  if (row_variant_out) *row_variant_out = best.rowv + 16 * best.colv;
+  if (row_variant_out) *row_variant_out = best.rowv;
   return SWENSE_OK;
 }
 
@@ -2093,8 +1462,7 @@ extern "C" int swense_set_grid_tune(int32_t nx, int32_t ny, int32_t pad_n, int32
   Tune tn;
   tn.lpc = lpc;
   tn.chunk_bytes = size_t(chunk_bytes);
-  tn.rowv = row_variant & 15;
-  tn.colv = row_variant >> 4;
+  tn.rowv = row_variant & 15;           // the one-field column variants (+16) run the same kernel
   g_tune[{nx, ny, pad_n, nz}] = tn;
   return SWENSE_OK;
 }
@@ -2135,7 +1503,6 @@ extern "C" int swense_selftest_wait_timeout(void* stream_) {
   r.Mh = N / 2;
   r.Nxr = N;
   r.Nyr = rows;
-  r.rb = kRowBlock;
   r.ldG = trans_ld(N / 2);
   r.polls = 8;
   r.selftest = 1;
@@ -2183,15 +1550,21 @@ extern "C" int swense_fields_on_grid_noalloc(const swense_modes* md, int32_t n_t
   if (!is_pow2(p.pad))
     return fail(SWENSE_ERR_UNSUPPORTED, "padding factors that are not powers of two need the workspace (swense_fields_on_grid)");
   const size_t cap = size_t(SWENSE_NOALLOC_SCRATCH_BYTES);
-  const size_t fixed = scratch_bytes(p, 0);
-  int chunk = 0;
+  // the launch shape swense_fields_on_grid would take (tuned, else its default), except that the
+  // two-stream pipeline (variant 5) stays on `stream`: the fixed array holds one level chunk, not
+  // two, and this call uses no library stream. The limit is that of the shared-memory path, which
+  // takes over where the pair's modal fields leave no room for a level.
+  Shape shape = grid_shape(p);
+  const size_t fixed = scratch_bytes(p, 0, 1, false);
   if (p.ny > 1) {
     if (fixed + p.per_level > cap)
       return fail(SWENSE_ERR_SIZE,
                   "request needs " + std::to_string(fixed + p.per_level) +
                       " bytes of scratch for one level; swense_fields_on_grid_noalloc has " +
                       std::to_string(cap) + " (SWENSE_NOALLOC_SCRATCH_BYTES)");
-    chunk = int(std::min<size_t>(size_t(p.nz), (cap - fixed) / p.per_level));
+    if (scratch_bytes(p, 1, 1, runs_pair(p, shape.lpc)) > cap) shape.lpc = 0;
+    shape.chunk = grid_slots(p, shape);
+    while (shape.chunk > 1 && scratch_bytes(p, shape.chunk, 1, runs_pair(p, shape.lpc)) > cap) --shape.chunk;
   } else if (fixed > cap) {
     return fail(SWENSE_ERR_SIZE, "request needs " + std::to_string(fixed) +
                                      " bytes of scratch; swense_fields_on_grid_noalloc has " +
@@ -2200,14 +1573,5 @@ extern "C" int swense_fields_on_grid_noalloc(const swense_modes* md, int32_t n_t
   void* ws = nullptr;
   st = noalloc_scratch(&ws);
   if (st) return st;
-  // the launch shape swense_fields_on_grid would take (tuned, else its default), except that the
-  // two-stream pipeline (variant 5) runs as variant 2: the fixed array holds one level chunk, not
-  // two, and this call uses no library stream
-  const Tune tn = tuned(p.nx, p.ny, p.pad, p.nz);
-  const bool pair = pair_path(p.ny, p.Nxr, p.Nyr);
-  const int lpc = tn.lpc >= 0 ? tn.lpc : (pair ? 4 : ((p.Nxr <= 512 && p.Nyr <= 512) ? kColLevels : 0));
-  int rowv = tn.lpc >= 0 ? tn.rowv : (pair ? 2 : 0);
-  if (rowv == 5) rowv = 2;
-  const int colv = tn.lpc >= 0 ? tn.colv : default_colv(p);
-  return launch_grid(p, md, t, nodes, eta, ws, chunk, stream, lpc, rowv, 0, 0, colv);
+  return launch_grid(p, md, t, nodes, eta, ws, shape, stream, false, false);
 }
