@@ -806,7 +806,8 @@ __global__ void __launch_bounds__(BOX_THREADS, 5) k_interp_global(const __grid_c
   __shared__ GatherRec rec[GLOBAL_PTS];
   const int warp = threadIdx.x >> 5;
   const int64_t p0 = int64_t(blockIdx.x) * GLOBAL_PTS + warp * GLOBAL_WPTS;
-  if (p0 >= a.np || !plan_is_global(plan[p0 / BOX_PTS], a.nz)) return;   // uniform over the warp
+  // uniform over the warp; no plan: every point is gathered here
+  if (p0 >= a.np || (plan && !plan_is_global(plan[p0 / BOX_PTS], a.nz))) return;
   gather_warp<P2, GLOBAL_WPTS>(a, *level_tables(L), p0, rec + warp * GLOBAL_WPTS);
 }
 
@@ -1441,8 +1442,15 @@ int interp_impl(const swense_grid* g, double t, const float* pts, const int32_t*
     a.perm = perm;
     const int64_t blocks = (np + BOX_PTS - 1) / BOX_PTS;
     if (blocks >= (int64_t(1) << 31)) return fail(SWENSE_ERR_SIZE, "too many points for one call");
-    const int4* plan = plan_in;
-    if (!plan) {
+    // Fewer chunks than SMs: planning and staging would be two launches of a few blocks each, bound by
+    // latency (18 + 25 us for 50,000 points of a 2-D wave); the gather without tiles fills the GPU from
+    // a few thousand points on (50,000 points: 7 us). Above that, the tiles' reuse wins on meshes.
+    int dev = 0, sms = 0;
+    SWENSE_CUDA_TRY(cudaGetDevice(&dev));
+    SWENSE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const bool small = blocks < sms;
+    const int4* plan = small ? nullptr : plan_in;
+    if (!plan && !small) {
       int4* pw = reinterpret_cast<int4*>(static_cast<char*>(ws) + 256);
       if (a.p2) k_interp_plan<true><<<unsigned(plan_blocks(np)), BOX_THREADS, 0, stream>>>(a, lev, pw);
       else k_interp_plan<false><<<unsigned(plan_blocks(np)), BOX_THREADS, 0, stream>>>(a, lev, pw);
@@ -1454,17 +1462,20 @@ int interp_impl(const swense_grid* g, double t, const float* pts, const int32_t*
     // stencils then rarely fit a tile) send the chunks without a tile to k_interp_global, where
     // L1 is not reduced by the tile; dense ones (meshes at their grid's resolution) gather the
     // rare such chunks inside k_interp_box and skip the second launch.
-    const bool split = double(np) < 0.25 * double(a.Nxr) * double(a.Nyr) * double(a.nz);
+    const bool split = small || double(np) < 0.25 * double(a.Nxr) * double(a.Nyr) * double(a.nz);
     const void* kbox = a.p2 ? (split ? (const void*)k_interp_box<true, true> : (const void*)k_interp_box<true, false>)
                             : (split ? (const void*)k_interp_box<false, true> : (const void*)k_interp_box<false, false>);
     SWENSE_CUDA_TRY(cudaFuncSetAttribute(kbox, cudaFuncAttributeMaxDynamicSharedMemorySize, int(BOX_SMEM)));
     if (split) {
-      if (a.p2) k_interp_box<true, true><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
-      else k_interp_box<false, true><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
+      if (!small) {
+        if (a.p2) k_interp_box<true, true><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
+        else k_interp_box<false, true><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
+        count_launches(1);
+      }
       const unsigned gctas = unsigned((np + GLOBAL_PTS - 1) / GLOBAL_PTS);
       if (a.p2) k_interp_global<true><<<gctas, BOX_THREADS, 0, stream>>>(a, lev, plan);
       else k_interp_global<false><<<gctas, BOX_THREADS, 0, stream>>>(a, lev, plan);
-      count_launches(2);
+      count_launches(1);
     } else {
       if (a.p2) k_interp_box<true, false><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
       else k_interp_box<false, false><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
