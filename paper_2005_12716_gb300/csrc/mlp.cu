@@ -10,7 +10,8 @@
 // layer's accumulator fragments become the next layer's A fragments in registers. Inference
 // splits inputs and activations into BF16 hi + lo (two MMAs per step) so the result tracks an
 // FP64 evaluation of the same BF16 weights to ~1e-5; training uses plain BF16 operands.
-// Weight gradients (sums over the batch) are reduced on the CUDA cores in FP32, then Adam.
+// Weight gradients (sums over the batch) are formed on the CUDA cores in FP32 by the block that made
+// the rows' activations, reduced over the blocks in a fixed order, then Adam.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -56,19 +57,13 @@ __global__ void k_mlp_pack(const float* __restrict__ P, Packed* __restrict__ out
 }
 
 // A fragments of 16 rows of x (FP32, leading dimension XLD, columns >= NIN read as 0).
-template <bool SPLIT>
 __device__ __forceinline__ void load_x(const float* __restrict__ x, int64_t row0, int64_t rows,
-                                       const int32_t* __restrict__ idx, unsigned (&ahi)[5][4],
-                                       unsigned (&alo)[5][4], int lane) {
+                                       unsigned (&ahi)[5][4], unsigned (&alo)[5][4], int lane) {
   const int g = lane >> 2, t = lane & 3;
-  int64_t r[2] = {row0 + g, row0 + g + 8};
+  const int64_t r[2] = {row0 + g, row0 + g + 8};
   const float* xr[2];
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const bool ok = r[h] < rows;
-    const int64_t rr = ok ? (idx ? int64_t(idx[r[h]]) : r[h]) : 0;
-    xr[h] = ok ? x + rr * XLD : nullptr;
-  }
+  for (int h = 0; h < 2; ++h) xr[h] = r[h] < rows ? x + r[h] * XLD : nullptr;
 #pragma unroll
   for (int kk = 0; kk < 5; ++kk) {
 #pragma unroll
@@ -80,8 +75,7 @@ __device__ __forceinline__ void load_x(const float* __restrict__ x, int64_t row0
         if (col < NIN) v0 = __ldg(&xr[h][col]);
         if (col + 1 < NIN) v1 = __ldg(&xr[h][col + 1]);
       }
-      if (SPLIT) bf2_split(v0, v1, ahi[kk][q], alo[kk][q]);
-      else ahi[kk][q] = bf2(v0, v1);
+      bf2_split(v0, v1, ahi[kk][q], alo[kk][q]);
     }
   }
 }
@@ -101,7 +95,7 @@ __global__ void __launch_bounds__(128) k_mlp_forward(const Packed* __restrict__ 
   for (int64_t row0 = (int64_t(blockIdx.x) * 4 + warp) * 16; row0 < rows;
        row0 += int64_t(gridDim.x) * 64) {
     unsigned xh[5][4], xl[5][4];
-    load_x<true>(x, row0, rows, nullptr, xh, xl, lane);
+    load_x(x, row0, rows, xh, xl, lane);
     float z1[8][4];
     layer<5, 8, true>(z1, xh, xl, &s.w1[0][0], KIN, s.b1, lane);
     unsigned h1h[4][4], h1l[4][4];
@@ -124,6 +118,22 @@ __global__ void __launch_bounds__(128) k_mlp_forward(const Packed* __restrict__ 
 }
 
 // ------------------------------------------------------------------------------ training
+// One block takes TROWS rows of the batch at a time: its warps 0..3 run forward and backward on 16 rows
+// each (tensor cores) and leave the rows' activations and gradients in shared memory, from which its
+// eight other warps add the rows' contribution to every weight gradient, a 4 x 8 tile of one matrix a
+// thread (three 16-byte shared loads per 32 products); separate warps, so that neither part's registers
+// burden the other (twelve warps in all: three per scheduler leave 168 registers a thread). The sums stay in registers over the block's rows and
+// go to the block's own row of `part`. With the activations written out to memory and one thread per
+// parameter summing 256 rows, the gradients took 47 us of a 62 us step (batch 8192); this kernel does
+// both passes in 21 us (a latency chain of three layers forward and back on one wave of blocks).
+constexpr int TROWS = 64, TFB = 128, TTHR = TFB + 256, XS = 72, HS = NH + 4;
+struct TrainSmem {
+  Packed p;
+  float x[TROWS][XS];              // columns >= NIN zero
+  float h1[TROWS][HS], h2[TROWS][HS], dz1[TROWS][HS], dz2[TROWS][HS];
+  float dy[TROWS][4];
+  float loss[4];
+};
 struct TrainArgs {
   const Packed* P;
   const float* x;          // [N][XLD] features
@@ -131,168 +141,260 @@ struct TrainArgs {
   const float* target;     // [N]
   const int32_t* batch;    // [B] row indices into x
   int B;
-  float* h1;               // [B][64] saved activations (FP32)
-  float* h2;
-  float* dz1;
-  float* dz2;
-  float* dy;               // [B][4]
+  float* part;             // [gridDim.x][NPARAM] per-block gradient sums
   float* loss_part;        // [gridDim.x] per-block sums of squared residuals / B
   float tscale;            // targets are multiplied by this on reading
 };
 
-__global__ void __launch_bounds__(128) k_mlp_train_fb(TrainArgs a) {
-  __shared__ Packed s;
+__global__ void __launch_bounds__(TTHR, 1) k_mlp_train(TrainArgs a) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  TrainSmem& s = *reinterpret_cast<TrainSmem*>(smraw);
+  const int tid = threadIdx.x;
   {
     const int4* src = reinterpret_cast<const int4*>(a.P);
-    int4* dst = reinterpret_cast<int4*>(&s);
-    for (int i = threadIdx.x; i < int(sizeof(Packed) / 16); i += blockDim.x) dst[i] = src[i];
+    int4* dst = reinterpret_cast<int4*>(&s.p);
+    for (int i = tid; i < int(sizeof(Packed) / 16); i += TTHR) dst[i] = src[i];
   }
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
   const float invB = 1.f / float(a.B);
-  float lsum = 0.f;
-  for (int64_t row0 = (int64_t(blockIdx.x) * 4 + warp) * 16; row0 < a.B;
-       row0 += int64_t(gridDim.x) * 64) {
-    unsigned xh[5][4], xl[5][4];
-    load_x<false>(a.x, row0, a.B, a.batch, xh, xl, lane);
-    float z1[8][4];
-    layer<5, 8, false>(z1, xh, xl, &s.w1[0][0], KIN, s.b1, lane);
-    unsigned h1[4][4], unused1[4][4];
-    to_a<8, false>(z1, h1, unused1);
-    float z2[8][4];
-    layer<4, 8, false>(z2, h1, unused1, &s.w2[0][0], NH, s.b2, lane);
-    unsigned h2[4][4], unused2[4][4];
-    to_a<8, false>(z2, h2, unused2);
-    float o[1][4];
-    layer<4, 1, false>(o, h2, unused2, &s.w3[0][0], NH, s.b3, lane);
-    // dY: only the row's own output column carries 2 (y - target) / B
-    float dyf[4];
-    int64_t rr[2];
+  const int step = int(gridDim.x) * TROWS;
+  // both halves of the block pass the same barriers, three per tile of rows, from their own loops
+  auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(TTHR) : "memory"); };
+  __syncthreads();                                 // the weights are in place
+  if (warp < 4) {
+    float lsum = 0.f;
+    for (int r0 = blockIdx.x * TROWS; r0 < a.B; r0 += step) {
+      sync();                                      // the tile's x rows are in place
+      const int w0 = 16 * warp;
+      unsigned xh[5][4], unused0[5][4];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      rr[h] = row0 + g + 8 * h;
-      const bool ok = rr[h] < a.B;
-      const int src = ok ? a.batch[rr[h]] : 0;
-      const int f = ok ? a.field[src] : -1;
-      const float tg = ok ? a.target[src] * a.tscale : 0.f;
+      for (int kk = 0; kk < 5; ++kk)
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const int col = 2 * t + c;
-        float d = 0.f;
-        if (col == f) {
-          const float res = o[0][2 * h + c] - tg;
-          lsum = fmaf(res, res, lsum);
-          d = 2.f * res * invB;
+        for (int q = 0; q < 4; ++q) {
+          const int r = w0 + g + 8 * (q & 1), col = 16 * kk + 2 * t + (q >= 2 ? 8 : 0);
+          xh[kk][q] = col < XS ? bf2(s.x[r][col], s.x[r][col + 1]) : 0u;
         }
-        dyf[2 * h + c] = d;
+      float z1[8][4];
+      layer<5, 8, false>(z1, xh, unused0, &s.p.w1[0][0], KIN, s.p.b1, lane);
+      unsigned h1[4][4], unused1[4][4];
+      to_a<8, false>(z1, h1, unused1);
+      float z2[8][4];
+      layer<4, 8, false>(z2, h1, unused1, &s.p.w2[0][0], NH, s.p.b2, lane);
+      unsigned h2[4][4], unused2[4][4];
+      to_a<8, false>(z2, h2, unused2);
+      float o[1][4];
+      layer<4, 1, false>(o, h2, unused2, &s.p.w3[0][0], NH, s.p.b3, lane);
+      // dY: only the row's own output column carries 2 (y - target) / B
+      float dyf[4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int64_t rr = int64_t(r0) + w0 + g + 8 * h;
+        const bool ok = rr < a.B;
+        const int src = ok ? a.batch[rr] : 0;
+        const int f = ok ? a.field[src] : -1;
+        const float tg = ok ? a.target[src] * a.tscale : 0.f;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const int col = 2 * t + c;
+          float d = 0.f;
+          if (col == f) {
+            const float res = o[0][2 * h + c] - tg;
+            lsum = fmaf(res, res, lsum);
+            d = 2.f * res * invB;
+          }
+          dyf[2 * h + c] = d;
+        }
       }
-    }
-    // dH2 = dY W3  (K = 8 padded to 16)
-    unsigned ady[4] = {bf2(dyf[0], dyf[1]), bf2(dyf[2], dyf[3]), 0u, 0u};
-    float dh2[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      dh2[nt][0] = dh2[nt][1] = dh2[nt][2] = dh2[nt][3] = 0.f;
-      const __nv_bfloat16* wr = &s.w3t[8 * nt + g][2 * t];
-      mma16816(dh2[nt], ady, ld_u32(wr), ld_u32(wr + 8));
-    }
-    // dZ2 = dH2 * gelu'(Z2); dH1 = dZ2 W2
-    float dz2[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) dz2[nt][q] = dh2[nt][q] * gelu_grad(z2[nt][q]);
-    unsigned adz2[4][4];
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-      adz2[kk][0] = bf2(dz2[2 * kk][0], dz2[2 * kk][1]);
-      adz2[kk][1] = bf2(dz2[2 * kk][2], dz2[2 * kk][3]);
-      adz2[kk][2] = bf2(dz2[2 * kk + 1][0], dz2[2 * kk + 1][1]);
-      adz2[kk][3] = bf2(dz2[2 * kk + 1][2], dz2[2 * kk + 1][3]);
-    }
-    float dh1[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      dh1[nt][0] = dh1[nt][1] = dh1[nt][2] = dh1[nt][3] = 0.f;
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const __nv_bfloat16* wr = &s.w2t[8 * nt + g][16 * kk + 2 * t];
-        mma16816(dh1[nt], adz2[kk], ld_u32(wr), ld_u32(wr + 8));
-      }
-    }
-    // save per-row activations and gradients for the weight-gradient reduction
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (rr[h] >= a.B) continue;
-      const int64_t r = rr[h];
+      // dH2 = dY W3  (K = 8 padded to 16)
+      unsigned ady[4] = {bf2(dyf[0], dyf[1]), bf2(dyf[2], dyf[3]), 0u, 0u};
+      float dz2[8][4];
 #pragma unroll
       for (int nt = 0; nt < 8; ++nt) {
-        const int col = 8 * nt + 2 * t;
-        const float e0 = z1[nt][2 * h], e1 = z1[nt][2 * h + 1];
-        const float f0 = z2[nt][2 * h], f1 = z2[nt][2 * h + 1];
-        *reinterpret_cast<float2*>(&a.h1[r * NH + col]) = make_float2(gelu(e0), gelu(e1));
-        *reinterpret_cast<float2*>(&a.h2[r * NH + col]) = make_float2(gelu(f0), gelu(f1));
-        *reinterpret_cast<float2*>(&a.dz2[r * NH + col]) = make_float2(dz2[nt][2 * h], dz2[nt][2 * h + 1]);
-        *reinterpret_cast<float2*>(&a.dz1[r * NH + col]) =
-            make_float2(dh1[nt][2 * h] * gelu_grad(e0), dh1[nt][2 * h + 1] * gelu_grad(e1));
+        dz2[nt][0] = dz2[nt][1] = dz2[nt][2] = dz2[nt][3] = 0.f;
+        const __nv_bfloat16* wr = &s.p.w3t[8 * nt + g][2 * t];
+        mma16816(dz2[nt], ady, ld_u32(wr), ld_u32(wr + 8));
       }
-      if (t < 2) *reinterpret_cast<float2*>(&a.dy[r * 4 + 2 * t]) = make_float2(dyf[2 * h], dyf[2 * h + 1]);
+      // dZ2 = dH2 * gelu'(Z2); dH1 = dZ2 W2
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dz2[nt][q] *= gelu_grad(z2[nt][q]);
+      unsigned adz2[4][4];
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        adz2[kk][0] = bf2(dz2[2 * kk][0], dz2[2 * kk][1]);
+        adz2[kk][1] = bf2(dz2[2 * kk][2], dz2[2 * kk][3]);
+        adz2[kk][2] = bf2(dz2[2 * kk + 1][0], dz2[2 * kk + 1][1]);
+        adz2[kk][3] = bf2(dz2[2 * kk + 1][2], dz2[2 * kk + 1][3]);
+      }
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt) {
+        float dh1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+          const __nv_bfloat16* wr = &s.p.w2t[8 * nt + g][16 * kk + 2 * t];
+          mma16816(dh1, adz2[kk], ld_u32(wr), ld_u32(wr + 8));
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int r = w0 + g + 8 * h, col = 8 * nt + 2 * t;
+          const float e0 = z1[nt][2 * h], e1 = z1[nt][2 * h + 1];
+          *reinterpret_cast<float2*>(&s.h1[r][col]) = make_float2(gelu(e0), gelu(e1));
+          *reinterpret_cast<float2*>(&s.h2[r][col]) = make_float2(gelu(z2[nt][2 * h]), gelu(z2[nt][2 * h + 1]));
+          *reinterpret_cast<float2*>(&s.dz2[r][col]) = make_float2(dz2[nt][2 * h], dz2[nt][2 * h + 1]);
+          *reinterpret_cast<float2*>(&s.dz1[r][col]) =
+              make_float2(dh1[2 * h] * gelu_grad(e0), dh1[2 * h + 1] * gelu_grad(e1));
+        }
+      }
+      if (t < 2) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          *reinterpret_cast<float2*>(&s.dy[w0 + g + 8 * h][2 * t]) = make_float2(dyf[2 * h], dyf[2 * h + 1]);
+      }
+      sync();                                      // activations and gradients are in place
+      sync();                                      // and have been read
     }
+    // per-block loss in a fixed order (no atomics: training is reproducible bit for bit)
+    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+    if (lane == 0) s.loss[warp] = lsum;
+    sync();
+    if (tid == 0) a.loss_part[blockIdx.x] = ((s.loss[0] + s.loss[1]) + (s.loss[2] + s.loss[3])) * invB;
+    return;
   }
-  // per-block loss in a fixed order (no atomics: training is reproducible bit for bit)
-  for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-  __shared__ float wl[4];
-  if (lane == 0) wl[warp] = lsum;
-  __syncthreads();
-  if (threadIdx.x == 0) a.loss_part[blockIdx.x] = ((wl[0] + wl[1]) + (wl[2] + wl[3])) * invB;
+  // this thread's tile of the gradients: rows of L (dz1, dz2 or dy) times rows of R (x, h1 or h2)
+  const int v = tid - TFB;
+  const bool first = v < 128;                      // dW1, columns 0..63, or dW2: 16 x 8 tiles of 4 x 8
+  const int ig = (v & 127) >> 3, kg = v & 7;
+  const float* Lp = first ? &s.dz1[0][4 * ig] : &s.dz2[0][4 * ig];
+  const float* Rp = first ? &s.x[0][8 * kg] : &s.h1[0][8 * kg];
+  const int ldr = first ? XS : HS;
+  // four more sums: dW1's columns 64..66 (threads 0..47) and dW3's columns (threads 48..111)
+  const bool extra = v < 112, w1x = v < 48;
+  const float* Lx = w1x ? &s.dz1[0][4 * (v / 3)] : &s.dy[0][0];
+  const float* Rx = w1x ? &s.x[0][64 + v % 3] : &s.h2[0][(v - 48) & 63];
+  const int ldlx = w1x ? HS : 4, ldrx = w1x ? XS : HS;
+  const float* bp = v < NH ? &s.dz1[0][v] : (v < 2 * NH ? &s.dz2[0][v - NH] : &s.dy[0][v & 3]);
+  const int ldb = v < 2 * NH ? HS : 4;
+  float acc[4][8], accx[4] = {0.f, 0.f, 0.f, 0.f}, bacc = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[i][k] = 0.f;
+  for (int r0 = blockIdx.x * TROWS; r0 < a.B; r0 += step) {
+#pragma unroll 4
+    for (int i = v; i < TROWS * XS; i += TTHR - TFB) {
+      const int r = i / XS, c = i % XS;
+      s.x[r][c] = r0 + r < a.B && c < NIN ? __ldg(&a.x[int64_t(__ldg(&a.batch[r0 + r])) * XLD + c]) : 0.f;
+    }
+    sync();
+    sync();
+    // rows past the batch carry dy = 0, so dz1 and dz2 are zero and they add nothing
+#pragma unroll 4
+    for (int r = 0; r < TROWS; ++r) {
+      const float4 l = *reinterpret_cast<const float4*>(Lp + r * HS);
+      const float4 x0 = *reinterpret_cast<const float4*>(Rp + r * ldr);
+      const float4 x1 = *reinterpret_cast<const float4*>(Rp + r * ldr + 4);
+      const float lv[4] = {l.x, l.y, l.z, l.w}, xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc[i][k] = fmaf(lv[i], xv[k], acc[i][k]);
+    }
+    if (extra) {
+#pragma unroll 8
+      for (int r = 0; r < TROWS; ++r) {
+        const float4 l = *reinterpret_cast<const float4*>(Lx + r * ldlx);
+        const float xv = Rx[r * ldrx];
+        accx[0] = fmaf(l.x, xv, accx[0]);
+        accx[1] = fmaf(l.y, xv, accx[1]);
+        accx[2] = fmaf(l.z, xv, accx[2]);
+        accx[3] = fmaf(l.w, xv, accx[3]);
+      }
+    }
+    if (v < 2 * NH + NOUT) {
+#pragma unroll 8
+      for (int r = 0; r < TROWS; ++r) bacc += bp[r * ldb];
+    }
+    sync();
+  }
+  float* part = a.part + size_t(blockIdx.x) * NPARAM;
+  const int off = first ? OFF_W1 : OFF_W2, ld = first ? NIN : NH;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int k = 0; k < 8; ++k) part[off + (4 * ig + i) * ld + 8 * kg + k] = acc[i][k];
+  if (extra) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      part[w1x ? OFF_W1 + (4 * (v / 3) + i) * NIN + 64 + v % 3 : OFF_W3 + i * NH + v - 48] = accx[i];
+  }
+  if (v < 2 * NH + NOUT)
+    part[v < NH ? OFF_B1 + v : (v < 2 * NH ? OFF_B2 + v - NH : OFF_B3 + v - 2 * NH)] = bacc;
+  sync();                                          // pairs with the loss's barrier
 }
 
-// Weight gradients: one thread per parameter, a slice of the batch per grid row, FP32 sums;
-// each slice's sum goes to its own row of `part` (summed in order by k_mlp_reduce).
-__global__ void k_mlp_wgrad(const float* __restrict__ x, const int32_t* __restrict__ batch, int B,
-                            const float* __restrict__ h1, const float* __restrict__ h2,
-                            const float* __restrict__ dz1, const float* __restrict__ dz2,
-                            const float* __restrict__ dy, int slice, float* __restrict__ part) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= NPARAM) return;
-  const int r0 = blockIdx.y * slice, r1 = min(B, r0 + slice);
+// grad = sum over the blocks' parts in a fixed order (eight interleaved runs, then the runs), loss
+// likewise; with params given, one Adam step and the refreshed BF16 copies of the parameter (the
+// padding of the packed layout never changes).
+struct UpdateArgs {
+  const float* part;
+  int nparts;
+  float* grad;                     // NULL: not wanted
+  const float* loss_part;
+  float* loss;                     // NULL: not wanted
+  float *P, *m, *v;                // NULL: gradient only
+  Packed* out;
+  float lr, b1, b2, eps, bc1, bc2;
+};
+constexpr int UPD_RUNS = 8;
+__global__ void __launch_bounds__(32 * UPD_RUNS) k_mlp_update(UpdateArgs a) {
+  __shared__ float run[UPD_RUNS][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int p = blockIdx.x * 32 + lane;
   float acc = 0.f;
-  if (p < OFF_B1) {
-    const int i = p / NIN, k = p % NIN;
-    for (int r = r0; r < r1; ++r) acc = fmaf(dz1[r * NH + i], __ldg(&x[int64_t(batch[r]) * XLD + k]), acc);
-  } else if (p < OFF_W2) {
-    const int i = p - OFF_B1;
-    for (int r = r0; r < r1; ++r) acc += dz1[r * NH + i];
-  } else if (p < OFF_B2) {
-    const int i = (p - OFF_W2) / NH, j = (p - OFF_W2) % NH;
-    for (int r = r0; r < r1; ++r) acc = fmaf(dz2[r * NH + i], h1[r * NH + j], acc);
-  } else if (p < OFF_W3) {
-    const int i = p - OFF_B2;
-    for (int r = r0; r < r1; ++r) acc += dz2[r * NH + i];
-  } else if (p < OFF_B3) {
-    const int o = (p - OFF_W3) / NH, j = (p - OFF_W3) % NH;
-    for (int r = r0; r < r1; ++r) acc = fmaf(dy[r * 4 + o], h2[r * NH + j], acc);
-  } else {
-    const int o = p - OFF_B3;
-    for (int r = r0; r < r1; ++r) acc += dy[r * 4 + o];
-  }
-  part[size_t(blockIdx.y) * NPARAM + p] = acc;
-}
-
-// grad = sum over the slices in order; loss = sum of the per-block losses in order.
-__global__ void k_mlp_reduce(const float* __restrict__ part, int nslices, float* __restrict__ grad,
-                             const float* __restrict__ loss_part, int nblocks, float* __restrict__ loss) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < NPARAM) {
-    float acc = 0.f;
-    for (int s = 0; s < nslices; ++s) acc += part[size_t(s) * NPARAM + p];
-    grad[p] = acc;
+#pragma unroll 8
+    for (int q = w; q < a.nparts; q += UPD_RUNS) acc += a.part[size_t(q) * NPARAM + p];
   }
-  if (p == 0 && loss) {
+  run[w][lane] = acc;
+  if (blockIdx.x == 0 && w == 1 && a.loss) {
     float l = 0.f;
-    for (int b = 0; b < nblocks; ++b) l += loss_part[b];
-    *loss = l;
+    for (int q = lane; q < a.nparts; q += 32) l += a.loss_part[q];
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (lane == 0) *a.loss = l;
+  }
+  __syncthreads();
+  if (w != 0 || p >= NPARAM) return;
+  float gr = 0.f;
+#pragma unroll
+  for (int q = 0; q < UPD_RUNS; ++q) gr += run[q][lane];
+  if (a.grad) a.grad[p] = gr;
+  if (!a.P) return;
+  const float mm = fmaf(a.b1, a.m[p], (1.f - a.b1) * gr);
+  const float vv = fmaf(a.b2, a.v[p], (1.f - a.b2) * gr * gr);
+  a.m[p] = mm;
+  a.v[p] = vv;
+  const float np = a.P[p] - a.lr * (mm / a.bc1) / (sqrtf(vv / a.bc2) + a.eps);
+  a.P[p] = np;
+  Packed& o = *a.out;
+  const __nv_bfloat16 b = __float2bfloat16_rn(np);
+  if (p < OFF_B1) {
+    o.w1[p / NIN][p % NIN] = b;
+  } else if (p < OFF_W2) {
+    o.b1[p - OFF_B1] = np;
+  } else if (p < OFF_B2) {
+    const int i = (p - OFF_W2) / NH, k = (p - OFF_W2) % NH;
+    o.w2[i][k] = b;
+    o.w2t[k][i] = b;
+  } else if (p < OFF_W3) {
+    o.b2[p - OFF_B2] = np;
+  } else if (p < OFF_B3) {
+    const int i = (p - OFF_W3) / NH, k = (p - OFF_W3) % NH;
+    o.w3[i][k] = b;
+    o.w3t[k][i] = b;
+  } else {
+    o.b3[p - OFF_B3] = np;
   }
 }
 
@@ -333,19 +435,6 @@ __global__ void k_mlp_targets(const float* __restrict__ eu, const float* __restr
   field[r] = f;
 }
 
-__global__ void k_mlp_adam(float* __restrict__ P, float* __restrict__ m, float* __restrict__ v,
-                           const float* __restrict__ grad, float lr, float b1, float b2, float eps,
-                           float bc1, float bc2) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= NPARAM) return;
-  const float gr = grad[p];
-  const float mm = fmaf(b1, m[p], (1.f - b1) * gr);
-  const float vv = fmaf(b2, v[p], (1.f - b2) * gr * gr);
-  m[p] = mm;
-  v[p] = vv;
-  P[p] -= lr * (mm / bc1) / (sqrtf(vv / bc2) + eps);
-}
-
 }  // namespace
 }  // namespace swense
 
@@ -382,77 +471,64 @@ extern "C" int swense_mlp_forward(const void* packed, const float* x, int64_t ro
 
 namespace {
 
-constexpr int kWgradSlice = 256;
-
 // Workspace layout of one training step for batch B (after `base` bytes the caller keeps).
 struct StepWs {
-  float *grad, *h1, *h2, *dz1, *dz2, *dy, *part, *loss_part;
+  float *part, *loss_part;
   int32_t* idx;
   unsigned blocks;
-  int nslices;
 };
+size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
+unsigned step_blocks(int B) { return unsigned(std::min<int64_t>((int64_t(B) + TROWS - 1) / TROWS, 152)); }
 size_t step_ws_bytes(int B) {
-  const unsigned blocks = unsigned(std::min<int64_t>((int64_t(B) + 63) / 64, 152 * 16));
-  const int nslices = (B + kWgradSlice - 1) / kWgradSlice;
-  auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
-  return al(NPARAM * sizeof(float)) + 4 * al(size_t(B) * NH * sizeof(float)) + al(size_t(B) * 4 * sizeof(float)) +
-         al(size_t(nslices) * NPARAM * sizeof(float)) + al(blocks * sizeof(float)) + al(size_t(B) * sizeof(int32_t));
+  const unsigned blocks = step_blocks(B);
+  return al256(size_t(blocks) * NPARAM * sizeof(float)) + al256(blocks * sizeof(float)) + al256(size_t(B) * sizeof(int32_t));
 }
 StepWs step_ws(void* ws, int B) {
   StepWs w{};
-  w.blocks = unsigned(std::min<int64_t>((int64_t(B) + 63) / 64, 152 * 16));
-  w.nslices = (B + kWgradSlice - 1) / kWgradSlice;
-  auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
+  w.blocks = step_blocks(B);
   char* c = static_cast<char*>(ws);
-  w.grad = reinterpret_cast<float*>(c);
-  c += al(NPARAM * sizeof(float));
-  w.h1 = reinterpret_cast<float*>(c);
-  c += al(size_t(B) * NH * sizeof(float));
-  w.h2 = reinterpret_cast<float*>(c);
-  c += al(size_t(B) * NH * sizeof(float));
-  w.dz1 = reinterpret_cast<float*>(c);
-  c += al(size_t(B) * NH * sizeof(float));
-  w.dz2 = reinterpret_cast<float*>(c);
-  c += al(size_t(B) * NH * sizeof(float));
-  w.dy = reinterpret_cast<float*>(c);
-  c += al(size_t(B) * 4 * sizeof(float));
   w.part = reinterpret_cast<float*>(c);
-  c += al(size_t(w.nslices) * NPARAM * sizeof(float));
+  c += al256(size_t(w.blocks) * NPARAM * sizeof(float));
   w.loss_part = reinterpret_cast<float*>(c);
-  c += al(w.blocks * sizeof(float));
+  c += al256(w.blocks * sizeof(float));
   w.idx = reinterpret_cast<int32_t*>(c);
   return w;
 }
 
-// Forward + backward of batch rows `batch` into w.grad (and *loss if non-NULL), in a fixed order.
-int grad_into(const StepWs& w, const void* packed, const float* x, const int32_t* field, const float* target,
-              float tscale, const int32_t* batch, int B, float* loss, cudaStream_t stream) {
-  TrainArgs a{static_cast<const Packed*>(packed), x, field, target, batch, B, w.h1, w.h2, w.dz1, w.dz2, w.dy,
-              w.loss_part, tscale};
-  k_mlp_train_fb<<<w.blocks, 128, 0, stream>>>(a);
+// Forward + backward of batch rows `batch`, in a fixed order, then `u`: the gradient and loss into its
+// buffers, and the Adam step where it names parameters.
+int train_into(const StepWs& w, const void* packed, const float* x, const int32_t* field, const float* target,
+               float tscale, const int32_t* batch, int B, UpdateArgs u, cudaStream_t stream) {
+  const TrainArgs a{static_cast<const Packed*>(packed), x, field, target, batch, B, w.part, w.loss_part, tscale};
+  SWENSE_CUDA_TRY(cudaFuncSetAttribute((const void*)k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       int(sizeof(TrainSmem))));
+  k_mlp_train<<<w.blocks, TTHR, sizeof(TrainSmem), stream>>>(a);
   SWENSE_CUDA_TRY(cudaGetLastError());
-  k_mlp_wgrad<<<dim3((NPARAM + 255) / 256, w.nslices), 256, 0, stream>>>(x, batch, B, w.h1, w.h2, w.dz1, w.dz2,
-                                                                        w.dy, kWgradSlice, w.part);
-  SWENSE_CUDA_TRY(cudaGetLastError());
-  k_mlp_reduce<<<(NPARAM + 255) / 256, 256, 0, stream>>>(w.part, w.nslices, w.grad, w.loss_part, int(w.blocks),
-                                                         loss);
-  SWENSE_CUDA_TRY(cudaGetLastError());
-  count_launches(3);
-  return SWENSE_OK;
-}
-
-// One Adam step (1-based `step`) on the gradient in w.grad, then the packed copy.
-int adam_and_pack(const StepWs& w, float* params, float* adam_m, float* adam_v, void* packed, int64_t step,
-                  float lr, float beta1, float beta2, float eps, cudaStream_t stream) {
-  const double t = double(step);
-  k_mlp_adam<<<(NPARAM + 255) / 256, 256, 0, stream>>>(params, adam_m, adam_v, w.grad, lr, beta1, beta2, eps,
-                                                        float(1.0 - std::pow(double(beta1), t)),
-                                                        float(1.0 - std::pow(double(beta2), t)));
-  SWENSE_CUDA_TRY(cudaGetLastError());
-  k_mlp_pack<<<(NH * KIN + 255) / 256, 256, 0, stream>>>(params, static_cast<Packed*>(packed));
+  u.part = w.part;
+  u.nparts = int(w.blocks);
+  u.loss_part = w.loss_part;
+  k_mlp_update<<<(NPARAM + 31) / 32, 32 * UPD_RUNS, 0, stream>>>(u);
   SWENSE_CUDA_TRY(cudaGetLastError());
   count_launches(2);
   return SWENSE_OK;
+}
+
+// Adam step (1-based `step`) of params and their packed copy.
+UpdateArgs adam_args(float* params, float* adam_m, float* adam_v, void* packed, int64_t step, float lr, float beta1,
+                     float beta2, float eps, float* loss) {
+  UpdateArgs u{};
+  u.loss = loss;
+  u.P = params;
+  u.m = adam_m;
+  u.v = adam_v;
+  u.out = static_cast<Packed*>(packed);
+  u.lr = lr;
+  u.b1 = beta1;
+  u.b2 = beta2;
+  u.eps = eps;
+  u.bc1 = float(1.0 - std::pow(double(beta1), double(step)));
+  u.bc2 = float(1.0 - std::pow(double(beta2), double(step)));
+  return u;
 }
 
 }  // namespace
@@ -471,10 +547,8 @@ extern "C" int swense_mlp_train_step(float* params, float* adam_m, float* adam_v
   void* ws = nullptr;
   int st = workspace(step_ws_bytes(B), stream, &ws);
   if (st) return st;
-  const StepWs w = step_ws(ws, B);
-  st = grad_into(w, packed, x, field, target, 1.f, batch, B, loss, stream);
-  if (!st) st = adam_and_pack(w, params, adam_m, adam_v, packed, step, lr, beta1, beta2, eps, stream);
-  return st;
+  return train_into(step_ws(ws, B), packed, x, field, target, 1.f, batch, B,
+                    adam_args(params, adam_m, adam_v, packed, step, lr, beta1, beta2, eps, loss), stream);
 }
 
 extern "C" int swense_mlp_grad(const void* packed, const float* x, const int32_t* field,
@@ -486,9 +560,10 @@ extern "C" int swense_mlp_grad(const void* packed, const float* x, const int32_t
   void* ws = nullptr;
   int st = workspace(step_ws_bytes(B), stream, &ws);
   if (st) return st;
-  StepWs w = step_ws(ws, B);
-  w.grad = grad;                                 // the caller's buffer receives the sums
-  return grad_into(w, packed, x, field, target, 1.f, batch, B, loss, stream);
+  UpdateArgs u{};
+  u.grad = grad;
+  u.loss = loss;
+  return train_into(step_ws(ws, B), packed, x, field, target, 1.f, batch, B, u, stream);
 }
 
 extern "C" int swense_mlp_targets(const float* exact_u, const float* exact_v, const float* exact_w,
@@ -546,9 +621,9 @@ extern "C" int swense_mlp_train(swense_mlp* mlp, const float* x, const int32_t* 
     if (schedule_steps > 0)
       lr_s = lr * 0.5 * (1.0 + std::cos(3.14159265358979323846 * double(std::min(s, schedule_steps)) /
                                         double(schedule_steps)));
-    st = grad_into(w, mlp->packed, x, field, target, tscale, w.idx, B, losses ? losses + i : nullptr, stream);
-    if (!st) st = adam_and_pack(w, mlp->params, mlp->adam_m, mlp->adam_v, mlp->packed, s + 1,
-                                float(std::max(lr_s, 1e-30)), beta1, beta2, eps, stream);
+    st = train_into(w, mlp->packed, x, field, target, tscale, w.idx, B,
+                    adam_args(mlp->params, mlp->adam_m, mlp->adam_v, mlp->packed, s + 1, float(std::max(lr_s, 1e-30)),
+                              beta1, beta2, eps, losses ? losses + i : nullptr), stream);
     if (st) return st;
     mlp->step = s + 1;
   }
