@@ -231,7 +231,10 @@ typedef struct swense_grid {
  * stores the count. p_mode: enum swense_p_mode; rho, g used by P_DYN / P_TOTAL.
  * Points are taken in 1024-point chunks; a chunk whose points all have the same z (bitwise; a
  * layer of cell or face centres of an extruded mesh) is interpolated in z once per grid column
- * and then in x and y per point, which is the same tensor-product sum in another order.
+ * and then in x and y per point, which is the same tensor-product sum in another order. Few points
+ * (fewer chunks than SMs) are taken straight from the grid. From 2^21 points on, on a grid of more
+ * than four times as many nodes, the layers of equal z share such planes in the scratch workspace
+ * (40 B per point, at most 1.3 GB, and 32 B per chunk; without it where it cannot be had).
  * Errors: ARG, SIZE, LEVELS, CUDA.
  */
 int swense_interp(const swense_grid* grid, double t, const float* pts, int64_t np,

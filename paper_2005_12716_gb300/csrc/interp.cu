@@ -245,7 +245,8 @@ static_assert(size_t(FLAT2_COLS) * (2 * sizeof(float4) + sizeof(float)) <= BOX_S
 //   flat:     w = bx | by << 12 (4 levels from l0), z = l0 | FLAT_BIT
 //   two z:    w = bx | by << 12, z = FLAT_BIT | FLAT2_BIT (the z values are those of the chunk's
 //             first and last points; their level windows are looked up by the gather)
-//   neither fits the tile: w = -1 (global gathers)
+//   neither fits the tile: w < 0 (global gathers): -1, or for one or two z values the extents all the
+//             same, w = 1 << 31 | bx | by << 14, z = FLAT_BIT (| FLAT2_BIT)
 constexpr int FLAT_BIT = 1 << 30;
 constexpr int FLAT2_BIT = 1 << 29;
 struct BoxPlan {
@@ -327,6 +328,25 @@ struct alignas(16) GatherRec {
 };
 static_assert(sizeof(GatherRec) == 80, "GatherRec layout");
 
+// A quad's sum over its four columns (lane k's sums (u, v), (w, dphi/dt), eta times its x weight) into
+// the point's record: field k from lane k.
+__device__ __forceinline__ void quad_sum(unsigned long long uv, unsigned long long wt, float e, float wxk, int k,
+                                         GatherRec& r) {
+  const float f0 = wxk * lo2(uv), f1 = wxk * hi2(uv), f2 = wxk * lo2(wt), f3 = wxk * hi2(wt);
+  e *= wxk;
+  e += __shfl_xor_sync(0xffffffffu, e, 1);
+  e += __shfl_xor_sync(0xffffffffu, e, 2);
+  // transposing reduction: lanes k and k ^ 1 swap the halves they do not keep, then k and k ^ 2
+  const bool odd = k & 1, high = k & 2;
+  float g0 = odd ? f1 : f0, g1 = odd ? f3 : f2;
+  g0 += __shfl_xor_sync(0xffffffffu, odd ? f0 : f1, 1);
+  g1 += __shfl_xor_sync(0xffffffffu, odd ? f2 : f3, 1);
+  const float h = (high ? g1 : g0) + __shfl_xor_sync(0xffffffffu, high ? g0 : g1, 2);
+  __syncwarp();                                    // every lane of the quad has read the record
+  r.wx[k] = h;
+  if (k == 0) r.eta = e;
+}
+
 // Stencil sums of points p0 .. p0 + WPTS - 1 by one warp, four lanes a point, lane k the stencil's x
 // node k. A warp load then covers the 64-byte stencil rows of eight points (8 to 16 L1 lines), where
 // one point a lane touches 32 lines with every load: the L1's line rate is what bounds scattered
@@ -400,19 +420,7 @@ __device__ __forceinline__ void gather_warp(const InterpArgs& a, const LevelTabl
       for (int b = 0; b < 4; ++b) re = fmaf(wyb[b], __ldg(&et[row[b]]), re);
       e = fmaf(wtl, re, e);
     }
-    float f0 = wxk * lo2(uv), f1 = wxk * hi2(uv), f2 = wxk * lo2(wt), f3 = wxk * hi2(wt);
-    e *= wxk;
-    e += __shfl_xor_sync(0xffffffffu, e, 1);
-    e += __shfl_xor_sync(0xffffffffu, e, 2);
-    // transposing reduction: lanes k and k ^ 1 swap the halves they do not keep, then k and k ^ 2
-    const bool odd = k & 1, high = k & 2;
-    float g0 = odd ? f1 : f0, g1 = odd ? f3 : f2;
-    g0 += __shfl_xor_sync(0xffffffffu, odd ? f0 : f1, 1);
-    g1 += __shfl_xor_sync(0xffffffffu, odd ? f2 : f3, 1);
-    const float h = (high ? g1 : g0) + __shfl_xor_sync(0xffffffffu, high ? g0 : g1, 2);
-    __syncwarp();                                  // every lane of the quad has read the record
-    r.wx[k] = h;
-    if (k == 0) r.eta = e;
+    quad_sum(uv, wt, e, wxk, k, r);
   }
   __syncwarp();
   if ((WPTS == 32 || lane < WPTS) && i < a.np) {
@@ -598,7 +606,10 @@ __device__ __forceinline__ void plan_chunk(const InterpArgs& a, const LevelTable
   const int y0 = a.Nyr > 1 ? wrapi<P2>(refy + mn[1] - 1, a.Nyr) : 0;
   plan[chunk] = fits_flat  ? make_int4(x0, y0, mn[2] | FLAT_BIT, bx | (by << 12))
               : fits_two   ? make_int4(x0, y0, FLAT_BIT | FLAT2_BIT, bx | (by << 12))
-                           : make_int4(x0, y0, mn[2], fits ? (bx | (by << 11) | (bz << 22)) : -1);
+              : fits       ? make_int4(x0, y0, mn[2], bx | (by << 11) | (bz << 22))
+              : (flat || flat2) && inside_grid
+                  ? make_int4(x0, y0, flat ? FLAT_BIT : FLAT_BIT | FLAT2_BIT, int(0x80000000u | unsigned(bx) | unsigned(by) << 14))
+                  : make_int4(x0, y0, mn[2], -1);
 }
 
 template <bool P2>
@@ -802,13 +813,429 @@ constexpr int GLOBAL_PTS = GLOBAL_WPTS * (BOX_THREADS / 32);     // points per C
 template <bool P2>
 __global__ void __launch_bounds__(BOX_THREADS, 5) k_interp_global(const __grid_constant__ InterpArgs a,
                                                                        const __grid_constant__ Levels L,
-                                                                       const int4* __restrict__ plan) {
+                                                                       const int4* __restrict__ plan,
+                                                                       const int* __restrict__ n_global,
+                                                                       const int2* __restrict__ chunk_slot) {
   __shared__ GatherRec rec[GLOBAL_PTS];
   const int warp = threadIdx.x >> 5;
   const int64_t p0 = int64_t(blockIdx.x) * GLOBAL_PTS + warp * GLOBAL_WPTS;
-  // uniform over the warp; no plan: every point is gathered here
+  // uniform over the warp; no plan: every point is gathered here. n_global, chunk_slot: of the gather
+  // by kinds (NULL otherwise), whose other kernels took the chunks with a plane
+  if (n_global && *n_global == 0) return;
   if (p0 >= a.np || (plan && !plan_is_global(plan[p0 / BOX_PTS], a.nz))) return;
+  if (chunk_slot && chunk_slot[p0 / BOX_PTS].x >= 0) return;
   gather_warp<P2, GLOBAL_WPTS>(a, *level_tables(L), p0, rec + warp * GLOBAL_WPTS);
+}
+
+// ---------------------------------------------------------------------------------------------
+// Gather of many points on a grid much finer than they are (LAYER_POINTS and more; the rule of `split`):
+// the layers of an extruded mesh put many chunks at one z, and their stencil boxes are too wide for a
+// tile. All chunks of a z share one z-collapsed, time-blended plane of the columns that their stencils
+// cover, made once in scratch memory (k_plane_collapse), and a point then reads 16 of its nodes where
+// the grid itself would be 64 n_tl. k_gather_register enters each such chunk's z and box in a hash
+// table; k_gather_lists sizes the planes (those that pay, within the scratch given), groups them by
+// their levels and lists the chunks that read planes and those with a staged tile, for persistent
+// kernels, so that an empty list costs a launch; k_interp_global takes the rest in point order.
+// 8.2 M mesh points on the four-fold padded 512 x 256 grid: 1.02 ms straight from the grid, 0.48 ms so (planes 0.13, gather 0.24 of it).
+constexpr int64_t LAYER_POINTS = int64_t(1) << 21;
+constexpr int PLANE_SLOTS = 4096;                  // planes at most (hash table entries)
+constexpr int PLANE_UNIT = BOX_THREADS;            // a plane's columns are padded to whole units
+constexpr unsigned PLANE_BIAS = 0x40000000u;
+struct PlaneSlot {
+  unsigned key;          // ~(bits of z); 0: free (NaN is never entered)
+  unsigned cnt;          // points
+  unsigned x0, x1, y0, y1;   // box relative to chunk 0's: BIAS - first, BIAS + one past the last (maxima)
+  int off;               // first column of the plane, -1: none
+  int pad_;
+};
+struct GatherCounts {
+  unsigned long long oor;
+  int groups, units, n_plane, n_tile, n_global;
+};
+static_assert(sizeof(GatherCounts) <= 256, "the counters' part of the workspace");
+// Planes whose z has the same four levels and whose boxes lie close (their union no larger than their
+// sum) are made together: a column's nodes are loaded once for all. Others form groups of one.
+struct PlaneGroup {
+  int unit0, first, n, pad_;     // first unit of the group's box; its planes in `members`
+  int rx, ry, bx, by;            // union of their boxes
+};
+struct GatherLists {
+  GatherCounts* n;
+  PlaneSlot* slots;      // [PLANE_SLOTS]
+  PlaneGroup* groups;    // [PLANE_SLOTS]
+  int* members;          // [PLANE_SLOTS] slots, group by group
+  int2* chunk_slot;      // [chunks] slots of the chunk's first and last z, x = -1: not from planes
+  int *l_plane, *l_tile; // [chunks] chunks from planes, and of the others those with a staged tile
+  float4* cols;          // [max_units * PLANE_UNIT]
+  float* etas;
+  int max_units;
+};
+
+__device__ __forceinline__ int plane_enter(PlaneSlot* slots, float z, int cnt, int rx, int bx, int ry, int by) {
+  const unsigned key = ~__float_as_uint(z);
+  if (z != z) return -1;
+  unsigned h = (key * 2654435761u) >> 20;          // 12 bits
+  for (int probe = 0; probe < 32; ++probe, h = (h + 1) & (PLANE_SLOTS - 1)) {
+    const unsigned old = atomicCAS(&slots[h].key, 0u, key);
+    if (old != 0u && old != key) continue;
+    atomicAdd(&slots[h].cnt, unsigned(cnt));
+    atomicMax(&slots[h].x0, PLANE_BIAS - unsigned(rx));
+    atomicMax(&slots[h].x1, PLANE_BIAS + unsigned(rx + bx));
+    atomicMax(&slots[h].y0, PLANE_BIAS - unsigned(ry));
+    atomicMax(&slots[h].y1, PLANE_BIAS + unsigned(ry + by));
+    return int(h);
+  }
+  return -1;
+}
+
+template <bool P2>
+__global__ void __launch_bounds__(256) k_gather_register(const __grid_constant__ InterpArgs a,
+                                                         const int4* __restrict__ plan, int chunks, GatherLists g) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= chunks) return;
+  const int4 pl = plan[c];
+  int2 sl = make_int2(-1, -1);
+  const int bx = pl.w >= 0 ? pl.w & 4095 : pl.w & 16383, by = pl.w >= 0 ? (pl.w >> 12) & 4095 : (pl.w >> 14) & 16383;
+  // (a plan of another grid may hold boxes that no stencil of this one fits)
+  if (pl.w != -1 && (pl.z & FLAT_BIT) && bx >= 4 && (a.Nyr > 1 ? by >= 4 : by == 1)) {
+    const int rx = wrap_rel<P2>(pl.x, plan[0].x, a.Nxr), ry = a.Nyr > 1 ? wrap_rel<P2>(pl.y, plan[0].y, a.Nyr) : 0;
+    const int64_t p0 = int64_t(c) * BOX_PTS, p1 = p0 + BOX_PTS < a.np ? p0 + BOX_PTS : a.np;
+    const int n = int(p1 - p0);
+    const bool two = pl.z & FLAT2_BIT;
+    sl.x = plane_enter(g.slots, __ldg(&a.pts[3 * p0 + 2]), two ? n / 2 : n, rx, bx, ry, by);
+    sl.y = two ? plane_enter(g.slots, __ldg(&a.pts[3 * (p1 - 1) + 2]), n / 2, rx, bx, ry, by) : sl.x;
+  }
+  g.chunk_slot[c] = sl;
+}
+
+// Extents of a plane's box; none when it laps the periodic grid.
+__device__ __forceinline__ bool plane_box(const InterpArgs& a, const PlaneSlot& s, int& rx, int& ry, int& bx, int& by) {
+  rx = -int(s.x0 - PLANE_BIAS);
+  ry = -int(s.y0 - PLANE_BIAS);
+  bx = int(s.x1 - PLANE_BIAS) - rx;
+  by = int(s.y1 - PLANE_BIAS) - ry;
+  return bx <= a.Nxr && by <= a.Nyr;
+}
+
+// Exclusive prefix sum of v over the block of 1024 threads; total returned in `sum`.
+__device__ __forceinline__ long long block_scan(long long v, long long* warp_sums, long long& sum) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  long long x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  __syncthreads();                                 // the previous scan's sums have been read
+  if (lane == 31) warp_sums[w] = x;
+  __syncthreads();
+  if (w == 0) {
+    long long y = warp_sums[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long q = __shfl_up_sync(0xffffffffu, y, o);
+      if (lane >= o) y += q;
+    }
+    warp_sums[lane] = y;
+  }
+  __syncthreads();
+  sum = warp_sums[31];
+  return x - v + (w ? warp_sums[w - 1] : 0);
+}
+
+// One block. A plane pays when its columns (4 n_tl coalesced loads, shared within its group) are at most
+// four times its points (each 16 loads instead of 64 n_tl).
+__global__ void __launch_bounds__(1024) k_gather_lists(const __grid_constant__ InterpArgs a,
+                                                       const __grid_constant__ Levels L,
+                                                       const int4* __restrict__ plan, int chunks, GatherLists g) {
+  __shared__ long long ws[32];
+  __shared__ int gcnt[SWENSE_MAX_LEVELS], gx0[SWENSE_MAX_LEVELS], gx1[SWENSE_MAX_LEVELS], gy0[SWENSE_MAX_LEVELS],
+      gy1[SWENSE_MAX_LEVELS], gsum[SWENSE_MAX_LEVELS], gpos[SWENSE_MAX_LEVELS];
+  constexpr int PER = PLANE_SLOTS / 1024;
+  long long mine[PER], units = 0, sum;
+  int lev[PER];
+  if (threadIdx.x < SWENSE_MAX_LEVELS) {
+    gcnt[threadIdx.x] = gsum[threadIdx.x] = 0;
+    gx0[threadIdx.x] = gy0[threadIdx.x] = 1 << 30;
+    gx1[threadIdx.x] = gy1[threadIdx.x] = -(1 << 30);
+  }
+  for (int k = 0; k < PER; ++k) {
+    const PlaneSlot s = g.slots[threadIdx.x * PER + k];
+    int rx, ry, bx, by;
+    mine[k] = 0;
+    if (s.key && plane_box(a, s, rx, ry, bx, by)) {
+      const long long cols = (long long)bx * by;
+      if (cols <= 4ll * s.cnt) mine[k] = (cols + PLANE_UNIT - 1) / PLANE_UNIT;
+    }
+    units += mine[k];
+  }
+  long long u = block_scan(units, ws, sum);        // (its barriers also order the group tables above)
+  for (int k = 0; k < PER; ++k) {                  // planes that pass the scratch's end are left out
+    if (u + mine[k] > g.max_units) mine[k] = 0;
+    const int i = threadIdx.x * PER + k;
+    g.slots[i].off = mine[k] ? int(u) * PLANE_UNIT : -1;
+    u += mine[k];
+    if (!mine[k]) continue;
+    const PlaneSlot s = g.slots[i];
+    int rx, ry, bx, by;
+    plane_box(a, s, rx, ry, bx, by);
+    PointCell pc;
+    point_level(a, *level_tables(L), __uint_as_float(~s.key), pc);
+    lev[k] = pc.j0;
+    atomicAdd(&gcnt[pc.j0], 1);
+    atomicAdd(&gsum[pc.j0], int(mine[k]));
+    atomicMin(&gx0[pc.j0], rx);
+    atomicMin(&gy0[pc.j0], ry);
+    atomicMax(&gx1[pc.j0], rx + bx);
+    atomicMax(&gy1[pc.j0], ry + by);
+  }
+  __syncthreads();
+  // joint groups, a thread per first level; then the planes of the other levels, each on its own
+  const int t = threadIdx.x;
+  int cnt = t < SWENSE_MAX_LEVELS ? gcnt[t] : 0;
+  const int gbx = cnt ? gx1[t] - gx0[t] : 0, gby = cnt ? gy1[t] - gy0[t] : 0;
+  long long gu = ((long long)gbx * gby + PLANE_UNIT - 1) / PLANE_UNIT;
+  if (cnt && gu > gsum[t]) {
+    cnt = 0;
+    gu = 0;
+    gpos[t] = -1;                                  // not joint
+  }
+  const int first = int(block_scan(cnt, ws, sum)), joint = int(sum);
+  const int id = int(block_scan(cnt ? 1 : 0, ws, sum));
+  int groups = int(sum);
+  const int u0 = int(block_scan(gu, ws, sum));
+  int gunits = int(sum);
+  if (cnt) {
+    g.groups[id] = PlaneGroup{u0, first, cnt, 0, gx0[t], gy0[t], gbx, gby};
+    gpos[t] = first;
+  }
+  __syncthreads();
+  int alone = 0;
+  long long aunits = 0;
+  for (int k = 0; k < PER; ++k) {
+    if (!mine[k]) continue;
+    if (gpos[lev[k]] >= 0) {
+      g.members[atomicAdd(&gpos[lev[k]], 1)] = t * PER + k;
+    } else {
+      ++alone;
+      aunits += mine[k];
+    }
+  }
+  int ai = int(block_scan(alone, ws, sum));
+  const int n_alone = int(sum);
+  int au = gunits + int(block_scan(aunits, ws, sum));
+  gunits += int(sum);
+  for (int k = 0; k < PER; ++k) {
+    if (!mine[k] || gpos[lev[k]] >= 0) continue;
+    const int i = t * PER + k;
+    const PlaneSlot s = g.slots[i];
+    int rx, ry, bx, by;
+    plane_box(a, s, rx, ry, bx, by);
+    g.members[joint + ai] = i;
+    g.groups[groups + ai] = PlaneGroup{au, joint + ai, 1, 0, rx, ry, bx, by};
+    au += int(mine[k]);
+    ++ai;
+  }
+  groups += n_alone;
+  __threadfence_block();
+  __syncthreads();
+  int np = 0, nt = 0, ng = 0;
+  for (int c0 = 0; c0 < chunks; c0 += 1024) {
+    const int c = c0 + t;
+    int kind = -1;
+    if (c < chunks) {
+      const int2 sl = g.chunk_slot[c];
+      kind = sl.x >= 0 && sl.y >= 0 && g.slots[sl.x].off >= 0 && g.slots[sl.y].off >= 0 ? 0
+             : !plan_is_global(plan[c], a.nz)                                           ? 1
+                                                                                        : 2;
+      if (kind != 0) g.chunk_slot[c] = make_int2(-1, -1);
+    }
+    const long long pre = block_scan(kind < 0 ? 0 : 1ll << (20 * kind), ws, sum);
+    if (kind == 0) g.l_plane[np + int(pre & 0xfffff)] = c;
+    if (kind == 1) g.l_tile[nt + int(pre >> 20 & 0xfffff)] = c;
+    np += int(sum & 0xfffff);
+    nt += int(sum >> 20 & 0xfffff);
+    ng += int(sum >> 40);
+  }
+  if (t == 0) {
+    g.n->groups = groups;
+    g.n->units = gunits;
+    g.n->n_plane = np;
+    g.n->n_tile = nt;
+    g.n->n_global = ng;
+  }
+}
+
+// The planes: a thread per column of a group's box, its four levels blended in time once, then a
+// weighted sum and a store for each of the group's planes that holds the column.
+template <bool P2>
+__global__ void __launch_bounds__(BOX_THREADS, 4) k_plane_collapse(const __grid_constant__ InterpArgs a,
+                                                                    const __grid_constant__ Levels L,
+                                                                    const int4* __restrict__ plan, GatherLists g) {
+  const int groups = g.n->groups, units = groups ? g.n->units : 0;
+  if (units == 0) return;
+  const int4 ref = plan[0];
+  const size_t plane = size_t(a.Nyr) * a.Nxr, tl_stride = size_t(a.nz) * plane;
+  const LevelTables& T = *level_tables(L);
+  constexpr int BATCH = 64;                        // planes whose weights and boxes are in shared memory
+  __shared__ float4 swz[BATCH];
+  __shared__ int4 sbx[BATCH];                      // rx, ry, bx, by
+  __shared__ int soff[BATCH];
+  for (int u = blockIdx.x; u < units; u += gridDim.x) {
+    int lo = 0, hi = groups - 1;                   // last group whose first unit <= u
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (g.groups[mid].unit0 <= u) lo = mid;
+      else hi = mid - 1;
+    }
+    const PlaneGroup e = g.groups[lo];
+    // threads past the box's end repeat its last column and store nothing
+    const int ci = (u - e.unit0) * PLANE_UNIT + int(threadIdx.x), c = min(ci, e.bx * e.by - 1);
+    const int cy = e.ry + c / e.bx, cx = e.rx + c % e.bx;     // relative to chunk 0's box
+    const size_t col = size_t(a.Nyr > 1 ? wrapi<P2>(ref.y + cy, a.Nyr) : 0) * a.Nxr + wrapi<P2>(ref.x + cx, a.Nxr);
+    PointCell pc;
+    point_level(a, T, __uint_as_float(~g.slots[g.members[e.first]].key), pc);
+    const float4* src = a.nodes + size_t(pc.j0) * plane + col;
+    float4 v[4];
+    float et = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int tl = 0; tl < a.n_tl; ++tl) {
+      const float w = a.wt[tl];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 n = __ldg(&src[size_t(tl) * tl_stride + size_t(q) * plane]);
+        v[q].x = fmaf(w, n.x, v[q].x);
+        v[q].y = fmaf(w, n.y, v[q].y);
+        v[q].z = fmaf(w, n.z, v[q].z);
+        v[q].w = fmaf(w, n.w, v[q].w);
+      }
+      et = fmaf(w, __ldg(&a.eta[size_t(tl) * plane + col]), et);
+    }
+    for (int k0 = 0; k0 < e.n; k0 += BATCH) {
+      const int nk = min(BATCH, e.n - k0);
+      __syncthreads();                             // the previous batch has been read
+      if (threadIdx.x < nk) {
+        const PlaneSlot& s = g.slots[g.members[e.first + k0 + threadIdx.x]];
+        int rx, ry, bx, by;
+        plane_box(a, s, rx, ry, bx, by);
+        point_level(a, T, __uint_as_float(~s.key), pc);
+        swz[threadIdx.x] = make_float4(pc.wz[0], pc.wz[1], pc.wz[2], pc.wz[3]);
+        sbx[threadIdx.x] = make_int4(rx, ry, bx, by);
+        soff[threadIdx.x] = s.off;
+      }
+      __syncthreads();
+      for (int k = 0; k < nk; ++k) {
+        const int4 b = sbx[k];
+        const int lx = cx - b.x, ly = cy - b.y;
+        if (ci != c || lx < 0 || lx >= b.z || ly < 0 || ly >= b.w) continue;
+        const float4 w = swz[k];
+        float4 o = make_float4(w.x * v[0].x, w.x * v[0].y, w.x * v[0].z, w.x * v[0].w);
+        const float wq[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int q = 1; q < 4; ++q) {
+          o.x = fmaf(wq[q], v[q].x, o.x);
+          o.y = fmaf(wq[q], v[q].y, o.y);
+          o.z = fmaf(wq[q], v[q].z, o.z);
+          o.w = fmaf(wq[q], v[q].w, o.w);
+        }
+        const int i = soff[k] + ly * b.z + lx;
+        g.cols[i] = o;
+        g.etas[i] = et;
+      }
+    }
+  }
+}
+
+// WPTS points from their planes by one warp, four lanes a point (as gather_warp).
+template <bool P2, int WPTS>
+__device__ __forceinline__ void plane_warp(const InterpArgs& a, const Levels& L, const GatherLists& g, int4 ref, int2 sl,
+                                           int64_t p0, GatherRec* rec) {
+  const int lane = threadIdx.x & 31, k = lane & 3;
+  const bool two_d = a.Nyr == 1;
+  const int64_t i = p0 + lane;
+  float z = 0.f;
+  if (WPTS == 32 || lane < WPTS) {
+    const int64_t ic = i < a.np ? i : a.np - 1;    // lanes past the end repeat the last point
+    z = __ldg(&a.pts[3 * ic + 2]);
+    PointCell c;
+    point_xy<P2>(a, __ldg(&a.pts[3 * ic]), __ldg(&a.pts[3 * ic + 1]), c);
+    const PlaneSlot& s = g.slots[~__float_as_uint(z) == g.slots[sl.x].key ? sl.x : sl.y];
+    int rx, ry, bx, by;
+    plane_box(a, s, rx, ry, bx, by);
+    const int lx = min(max(wrapi<P2>(c.ix - 1 - (ref.x + rx), a.Nxr), 0), bx - 4);
+    const int ly = two_d ? 0 : min(max(wrapi<P2>(c.iy - 1 - (ref.y + ry), a.Nyr), 0), by - 4);
+    GatherRec& r = rec[lane];
+    r.cell = make_int4(s.off + ly * bx + lx, bx, 0, 0);
+    r.wy = make_float4(c.wy[0], c.wy[1], c.wy[2], c.wy[3]);
+    *reinterpret_cast<float4*>(r.wx) = make_float4(c.wx[0], c.wx[1], c.wx[2], c.wx[3]);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int s = 0; s < WPTS / 8; ++s) {
+    GatherRec& r = rec[8 * s + (lane >> 2)];
+    const int4 c = r.cell;
+    const float4 wy = r.wy;
+    const float wxk = r.wx[k];
+    const float wyb[4] = {wy.x, wy.y, wy.z, wy.w};
+    unsigned long long uv = 0ull, wt = 0ull;
+    float e = 0.f;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      if (b > 0 && two_d) break;
+      const int o = c.x + b * c.y + k;
+      const float4 v = __ldg(&g.cols[o]);
+      const unsigned long long w2 = pack2(wyb[b], wyb[b]);
+      fma2(uv, w2, pack2(v.x, v.y));
+      fma2(wt, w2, pack2(v.z, v.w));
+      e = fmaf(wyb[b], __ldg(&g.etas[o]), e);
+    }
+    quad_sum(uv, wt, e, wxk, k, r);
+  }
+  __syncwarp();
+  if ((WPTS == 32 || lane < WPTS) && i < a.np) {
+    const float4 f = *reinterpret_cast<const float4*>(rec[lane].wx);
+    store_point(a, i, f, rec[lane].eta, z, z >= L.z[0] && z <= L.z[a.nz - 1]);
+  }
+}
+
+// The chunks that read planes, from their list.
+template <bool P2>
+__global__ void __launch_bounds__(BOX_THREADS, 5) k_interp_planes(const __grid_constant__ InterpArgs a,
+                                                                   const __grid_constant__ Levels L,
+                                                                   const int4* __restrict__ plan,
+                                                                   const __grid_constant__ GatherLists g) {
+  __shared__ GatherRec rec[BOX_THREADS];
+  const int n = g.n->n_plane;
+  for (int li = blockIdx.x; li < n; li += gridDim.x) {
+    const int chunk = g.l_plane[li];
+    const int2 sl = g.chunk_slot[chunk];
+#pragma unroll 1
+    for (int k = 0; k < BOX_PPT; ++k) {
+      const int64_t p0 = int64_t(chunk) * BOX_PTS + k * BOX_THREADS + (threadIdx.x & ~31);
+      if (p0 >= a.np) break;                       // uniform over the warp
+      plane_warp<P2, 32>(a, L, g, plan[0], sl, p0, rec + (threadIdx.x & ~31));
+      __syncwarp();                                // the records are rewritten by the next turn
+    }
+  }
+}
+
+// The chunks with a staged tile, taken from their list.
+template <bool P2>
+__global__ void __launch_bounds__(BOX_THREADS, 3) k_interp_tiles(const __grid_constant__ InterpArgs a,
+                                                                  const __grid_constant__ Levels L,
+                                                                  const int4* __restrict__ plan, GatherLists g) {
+  extern __shared__ float4 sbox[];
+  float* seta = reinterpret_cast<float*>(sbox + BOX_NODES);
+  __shared__ LevelTables zs;
+  const int n = g.n->n_tile;
+  if (int(blockIdx.x) >= n) return;
+  fill_level_tables(zs, L);
+  for (int li = blockIdx.x; li < n; li += gridDim.x) {
+    __syncthreads();                               // shared memory free for the next chunk
+    const int chunk = g.l_tile[li];
+    box_chunk<P2, false>(a, zs, chunk, plan[chunk], sbox, seta);
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1413,6 +1840,56 @@ extern "C" int swense_interp_learned(const swense_grid* g, double t, const float
 namespace swense {
 namespace {
 
+size_t up256(size_t b) { return (b + 255) & ~size_t(255); }
+
+// Scratch of the gather by kinds of chunks, after the counters and the plan: 2 columns per point, at
+// most 2^26, which holds a mesh's planes with room to spare.
+int plane_units(int64_t np) { return int(std::min<int64_t>(2 * np, int64_t(1) << 26) / PLANE_UNIT); }
+size_t lists_bytes(int64_t np, int64_t chunks) {
+  const size_t cols = size_t(plane_units(np)) * PLANE_UNIT;
+  return up256(PLANE_SLOTS * sizeof(PlaneSlot)) + up256(PLANE_SLOTS * sizeof(PlaneGroup)) +
+         up256(PLANE_SLOTS * sizeof(int)) + up256(chunks * sizeof(int2)) + 2 * up256(chunks * sizeof(int)) + up256(cols * sizeof(float4)) + up256(cols * sizeof(float));
+}
+GatherLists lists_in(char* c, int64_t np, int64_t chunks, void* counts) {
+  const size_t cols = size_t(plane_units(np)) * PLANE_UNIT;
+  GatherLists g;
+  auto take = [&](size_t b) { char* q = c; c += up256(b); return q; };
+  g.n = static_cast<GatherCounts*>(counts);
+  g.slots = reinterpret_cast<PlaneSlot*>(take(PLANE_SLOTS * sizeof(PlaneSlot)));
+  g.groups = reinterpret_cast<PlaneGroup*>(take(PLANE_SLOTS * sizeof(PlaneGroup)));
+  g.members = reinterpret_cast<int*>(take(PLANE_SLOTS * sizeof(int)));
+  g.chunk_slot = reinterpret_cast<int2*>(take(chunks * sizeof(int2)));
+  g.l_plane = reinterpret_cast<int*>(take(chunks * sizeof(int)));
+  g.l_tile = reinterpret_cast<int*>(take(chunks * sizeof(int)));
+  g.cols = reinterpret_cast<float4*>(take(cols * sizeof(float4)));
+  g.etas = reinterpret_cast<float*>(take(cols * sizeof(float)));
+  g.max_units = plane_units(np);
+  return g;
+}
+
+template <bool P2>
+int interp_by_kind(const InterpArgs& a, const Levels& lev, const int4* plan, int chunks, int sms, const GatherLists& g,
+                   cudaStream_t stream) {
+  SWENSE_CUDA_TRY(cudaMemsetAsync(g.slots, 0, PLANE_SLOTS * sizeof(PlaneSlot), stream));
+  k_gather_register<P2><<<unsigned((chunks + 255) / 256), 256, 0, stream>>>(a, plan, chunks, g);
+  SWENSE_CUDA_TRY(cudaGetLastError());
+  k_gather_lists<<<1, 1024, 0, stream>>>(a, lev, plan, chunks, g);
+  SWENSE_CUDA_TRY(cudaGetLastError());
+  k_plane_collapse<P2><<<unsigned(sms * 4), BOX_THREADS, 0, stream>>>(a, lev, plan, g);
+  SWENSE_CUDA_TRY(cudaGetLastError());
+  SWENSE_CUDA_TRY(cudaFuncSetAttribute((const void*)k_interp_tiles<P2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       int(BOX_SMEM)));
+  k_interp_tiles<P2><<<unsigned(sms * 3), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan, g);
+  SWENSE_CUDA_TRY(cudaGetLastError());
+  k_interp_planes<P2><<<unsigned(sms * 5), BOX_THREADS, 0, stream>>>(a, lev, plan, g);
+  SWENSE_CUDA_TRY(cudaGetLastError());
+  k_interp_global<P2><<<unsigned((a.np + GLOBAL_PTS - 1) / GLOBAL_PTS), BOX_THREADS, 0, stream>>>(
+      a, lev, plan, &g.n->n_global, g.chunk_slot);
+  SWENSE_CUDA_TRY(cudaGetLastError());
+  count_launches(6);
+  return SWENSE_OK;
+}
+
 // plan_in: a plan made earlier by swense_interp_plan for these points and this grid geometry
 // (NULL: make one in the workspace first).
 int interp_impl(const swense_grid* g, double t, const float* pts, const int32_t* perm, int64_t np,
@@ -1423,9 +1900,20 @@ int interp_impl(const swense_grid* g, double t, const float* pts, const int32_t*
   Levels lev;
   int st = prepare_interp(g, t, pts, np, p_mode, rho, grav, &a, &lev);
   if (st) return st;
-  // workspace: [0, 256) out-of-range counter, then one int4 box plan per 1024-point chunk
+  // workspace: [0, 256) counters, one int4 box plan per 1024-point chunk (unless given), and for many
+  // points the lists and planes of the gather by kinds, which is passed over where they cannot be had
+  const int64_t blocks = (np + BOX_PTS - 1) / BOX_PTS;
+  const size_t b_plan = 256 + (plan_in ? 0 : up256(size_t(blocks) * sizeof(int4)));
+  // sparse point sets (fewer points than a quarter of a time level's nodes): a chunk's stencils rarely
+  // fit a tile
+  const bool sparse = double(np) < 0.25 * double(a.Nxr) * double(a.Nyr) * double(a.nz);
+  bool kinds = sparse && np >= LAYER_POINTS && blocks < (int64_t(1) << 31) / (BOX_PTS / GLOBAL_PTS);
   void* ws = nullptr;
-  st = workspace(256 + (plan_in ? 0 : size_t((np + BOX_PTS - 1) / BOX_PTS) * sizeof(int4)), stream, &ws);
+  st = kinds ? workspace(b_plan + lists_bytes(np, blocks), stream, &ws) : SWENSE_OK;
+  if (st || !kinds) {
+    kinds = false;
+    st = workspace(b_plan, stream, &ws);
+  }
   if (st) return st;
   unsigned long long* d_count = nullptr;
   if (n_out_of_range) {
@@ -1440,7 +1928,6 @@ int interp_impl(const swense_grid* g, double t, const float* pts, const int32_t*
     a.o_p = p;
     a.n_oor = d_count;
     a.perm = perm;
-    const int64_t blocks = (np + BOX_PTS - 1) / BOX_PTS;
     if (blocks >= (int64_t(1) << 31)) return fail(SWENSE_ERR_SIZE, "too many points for one call");
     // Fewer chunks than SMs: planning and staging would be two launches of a few blocks each, bound by
     // latency (18 + 25 us for 50,000 points of a 2-D wave); the gather without tiles fills the GPU from
@@ -1458,30 +1945,37 @@ int interp_impl(const swense_grid* g, double t, const float* pts, const int32_t*
       count_launches(1);
       plan = pw;
     }
-    // Sparse point sets (fewer points than a quarter of a time level's nodes: a chunk's
-    // stencils then rarely fit a tile) send the chunks without a tile to k_interp_global, where
-    // L1 is not reduced by the tile; dense ones (meshes at their grid's resolution) gather the
-    // rare such chunks inside k_interp_box and skip the second launch.
-    const bool split = small || double(np) < 0.25 * double(a.Nxr) * double(a.Nyr) * double(a.nz);
-    const void* kbox = a.p2 ? (split ? (const void*)k_interp_box<true, true> : (const void*)k_interp_box<true, false>)
-                            : (split ? (const void*)k_interp_box<false, true> : (const void*)k_interp_box<false, false>);
-    SWENSE_CUDA_TRY(cudaFuncSetAttribute(kbox, cudaFuncAttributeMaxDynamicSharedMemorySize, int(BOX_SMEM)));
-    if (split) {
-      if (!small) {
-        if (a.p2) k_interp_box<true, true><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
-        else k_interp_box<false, true><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
+    if (kinds) {
+      const GatherLists g = lists_in(static_cast<char*>(ws) + b_plan, np, blocks, ws);
+      st = a.p2 ? interp_by_kind<true>(a, lev, plan, int(blocks), sms, g, stream)
+                : interp_by_kind<false>(a, lev, plan, int(blocks), sms, g, stream);
+      if (st) return st;
+    }
+    // Sparse sets send the chunks without a tile to k_interp_global, where L1 is not reduced by the
+    // tile; dense ones (meshes at their grid's resolution) gather the rare such chunks inside
+    // k_interp_box and skip the second launch.
+    const bool split = small || sparse;
+    if (!kinds) {
+      const void* kbox = a.p2 ? (split ? (const void*)k_interp_box<true, true> : (const void*)k_interp_box<true, false>)
+                              : (split ? (const void*)k_interp_box<false, true> : (const void*)k_interp_box<false, false>);
+      SWENSE_CUDA_TRY(cudaFuncSetAttribute(kbox, cudaFuncAttributeMaxDynamicSharedMemorySize, int(BOX_SMEM)));
+      if (split) {
+        if (!small) {
+          if (a.p2) k_interp_box<true, true><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
+          else k_interp_box<false, true><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
+          count_launches(1);
+        }
+        const unsigned gctas = unsigned((np + GLOBAL_PTS - 1) / GLOBAL_PTS);
+        if (a.p2) k_interp_global<true><<<gctas, BOX_THREADS, 0, stream>>>(a, lev, plan, nullptr, nullptr);
+        else k_interp_global<false><<<gctas, BOX_THREADS, 0, stream>>>(a, lev, plan, nullptr, nullptr);
+        count_launches(1);
+      } else {
+        if (a.p2) k_interp_box<true, false><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
+        else k_interp_box<false, false><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
         count_launches(1);
       }
-      const unsigned gctas = unsigned((np + GLOBAL_PTS - 1) / GLOBAL_PTS);
-      if (a.p2) k_interp_global<true><<<gctas, BOX_THREADS, 0, stream>>>(a, lev, plan);
-      else k_interp_global<false><<<gctas, BOX_THREADS, 0, stream>>>(a, lev, plan);
-      count_launches(1);
-    } else {
-      if (a.p2) k_interp_box<true, false><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
-      else k_interp_box<false, false><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
-      count_launches(1);
+      SWENSE_CUDA_TRY(cudaGetLastError());
     }
-    SWENSE_CUDA_TRY(cudaGetLastError());
   }
   if (n_out_of_range) {
     unsigned long long h = 0;
