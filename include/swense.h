@@ -180,9 +180,9 @@ int swense_fields_on_grid_noalloc(const swense_modes* modes, int32_t n_tl, const
  * and used by later calls. No counterpart in the paper. Writes the grid (same outputs as
  * swense_fields_on_grid), synchronises the stream, must not be captured. 2-D grids have a
  * single path (nothing to tune; *lpc_out = -1).
- * lpc_out (0 = shared-memory path), chunk_bytes_out, row_variant_out (0 = the row pass reads the
- * intermediate straight from memory; 4 = each warp's rows staged in shared memory by bulk
- * asynchronous copies, 256- to 1024-point rows; 5 = as 0 with chunk c's row pass on a
+ * lpc_out (0 = shared-memory path), chunk_bytes_out, row_variant_out (0 = the row pass takes
+ * its rows from shared memory, where bulk asynchronous copies put them, a block at a time; 4 = the
+ * same by the warp with radix-8 transforms, 256- to 1024-point rows; 5 = as 0 with chunk c's row pass on a
  * library-internal second stream while chunk c+1's column pass runs on `stream`, two intermediate
  * buffers, joined back before the call's work ends; 1, 2 and 3, and 16 more than any of them, name
  * earlier variants and run as 0):

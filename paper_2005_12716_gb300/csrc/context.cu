@@ -173,8 +173,8 @@ int swense_async_status(int32_t reset, void* stream) {
   if (!st) st = swense::direct_async_flag(reset != 0, &direct);
   if (st) return st;
   if (grid)
-    return swense::fail(SWENSE_ERR_TIMEOUT, "a bounded wait of the staged row pass (k_row_tma) gave "
-                                            "up; the grid rows of that warp were not written");
+    return swense::fail(SWENSE_ERR_TIMEOUT, "a bounded wait of a staged row pass (k_row_w, k_row_tma) gave "
+                                            "up; the grid rows of that block or warp were not written");
   if (direct)
     return swense::fail(SWENSE_ERR_TIMEOUT, "a bounded wait of the tensor-core direct sum "
                                             "(k_direct_tc) gave up; the outputs of that tile were "

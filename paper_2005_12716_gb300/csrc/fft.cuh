@@ -412,7 +412,9 @@ namespace swense {
 // ------------------------------------------------------------------------------------------------
 // Wide-radix inverse DFTs in two or three Stockham passes: N = R0 R1 (R2), with R0 elements a thread.
 // A 16- or 32-point DFT in registers replaces two or three radix-8/-4 passes and their exchanges, so a
-// transform of up to 1024 points goes through shared memory once and one of 2048 points twice.
+// transform of up to 1024 points goes through shared memory once and one of 2048 points twice. (Columns
+// of 512 and 1024 points as 16 x 16 x N/256, with 24 warps per SM instead of 16 but a second exchange,
+// were slower: eight levels of 1024 x 1024 columns 155 against 145 us, 64 of 512 x 512 130 against 101.)
 // Pass p with stride NS and radix R: butterfly j reads x[j + r N/R], multiplies by
 // e^{2 pi i (j mod NS) r / (NS R)} and writes y[(j / NS) NS R + (j mod NS) + r NS].
 
@@ -502,8 +504,8 @@ __host__ __device__ constexpr int wide_exponent(int i) {          // of twiddle 
 }
 
 // Two row transforms side by side by T = N / R0 threads (t = 0 .. T-1): element e of thread t holds
-// position t + T e on entry, and element wide_row_elem(b, r) position wide_row_pos(t, b, r) on exit.
-// Both buffers are padded by one element in R0, which makes every exchange conflict-free.
+// position t + T e on entry, and element elem(b, r) position pos(t, b, r) on exit. The buffer is padded
+// by one element in R0, which makes every exchange conflict-free.
 template <int N>
 struct WideRow {
   static constexpr int R0 = N >= 128 ? 16 : 8, R1 = N >= 256 ? 16 : N / R0, R2 = N / (R0 * R1);
@@ -516,26 +518,43 @@ struct WideRow {
     if constexpr (T <= 32) __syncwarp();
     else __syncthreads();
   }
+  // TWO: a buffer for each transform (b1, b2) and their exchanges side by side; otherwise they take the
+  // one buffer b1 in turn: half the shared memory, for two more barriers an exchange.
+  template <bool TWO, class Put, class Get>
+  __device__ static __forceinline__ void exchange(float2 (&z1)[E], float2 (&z2)[E], float2* b1, float2* b2, Put put,
+                                                  Get get) {
+    put(z1, b1);
+    if constexpr (TWO) put(z2, b2);
+    sync();
+    get(z1, b1);
+    if constexpr (TWO) get(z2, b2);
+    sync();
+    if constexpr (!TWO) {
+      put(z2, b1);
+      sync();
+      get(z2, b1);
+      sync();
+    }
+  }
+  template <bool TWO>
   __device__ static __forceinline__ void fft2(float2 (&z1)[E], float2 (&z2)[E], const float2* __restrict__ tw,
                                               float2* b1, float2* b2, int t) {
+    constexpr int B1 = E / R1, S1 = N / R1;        // S1 is a multiple of R0: the pad index splits
+    auto put0 = [&](float2 (&z)[E], float2* buf) {
+#pragma unroll
+      for (int r = 0; r < R0; ++r) buf[t * (R0 + 1) + r] = z[dft_slot<R0>(r)];
+    };
+    auto get0 = [&](float2 (&z)[E], float2* buf) {
+#pragma unroll
+      for (int b = 0; b < B1; ++b) {
+        const int jj = t + T * b, base = jj + jj / R0;
+#pragma unroll
+        for (int r = 0; r < R1; ++r) z[b * R1 + r] = buf[base + r * (S1 + S1 / R0)];
+      }
+    };
     wide_dft<R0>(z1);
     wide_dft<R0>(z2);
-#pragma unroll
-    for (int r = 0; r < R0; ++r) {
-      b1[t * (R0 + 1) + r] = z1[dft_slot<R0>(r)];
-      b2[t * (R0 + 1) + r] = z2[dft_slot<R0>(r)];
-    }
-    sync();
-    constexpr int B1 = E / R1, S1 = N / R1;        // S1 is a multiple of R0: the pad index splits
-#pragma unroll
-    for (int b = 0; b < B1; ++b) {
-      const int jj = t + T * b, base = jj + jj / R0;
-#pragma unroll
-      for (int r = 0; r < R1; ++r) {
-        z1[b * R1 + r] = b1[base + r * (S1 + S1 / R0)];
-        z2[b * R1 + r] = b2[base + r * (S1 + S1 / R0)];
-      }
-    }
+    exchange<TWO>(z1, z2, b1, b2, put0, get0);
 #pragma unroll
     for (int b = 0; b < B1; ++b) {
       const int jm = (t + T * b) % R0;
@@ -550,22 +569,23 @@ struct WideRow {
     }
     if constexpr (R2 > 1) {
       static_assert(R2 == 1 || (R0 == 16 && R1 == 16), "three passes start with 16 x 16");
-      sync();                                      // every thread has read the first exchange
       const int wb = (t / 16) * 272 + t % 16;
+      auto put1 = [&](float2 (&z)[E], float2* buf) {
 #pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        b1[wb + 17 * r] = z1[dft_slot<16>(r)];
-        b2[wb + 17 * r] = z2[dft_slot<16>(r)];
-      }
-      sync();
+        for (int r = 0; r < 16; ++r) buf[wb + 17 * r] = z[dft_slot<16>(r)];
+      };
+      auto get1 = [&](float2 (&z)[E], float2* buf) {
+#pragma unroll
+        for (int b = 0; b < BL; ++b) {
+          const int jj = t + T * b, base = jj + jj / 16;
+#pragma unroll
+          for (int r = 0; r < R2; ++r) z[b * R2 + r] = buf[base + 272 * r];
+        }
+      };
+      exchange<TWO>(z1, z2, b1, b2, put1, get1);
 #pragma unroll
       for (int b = 0; b < BL; ++b) {
-        const int jj = t + T * b, base = jj + jj / 16;
-#pragma unroll
-        for (int r = 0; r < R2; ++r) {
-          z1[b * R2 + r] = b1[base + 272 * r];
-          z2[b * R2 + r] = b2[base + 272 * r];
-        }
+        const int jj = t + T * b;
 #pragma unroll
         for (int r = 1; r < R2; ++r) {
           const float2 w = __ldg(&tw[kWideTw3 + N + 256 * r + jj]);

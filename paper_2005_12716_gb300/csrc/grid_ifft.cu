@@ -481,69 +481,109 @@ __global__ void __launch_bounds__(ColCfg<N>::kThr, ColCfg<N>::kMin) k_col_w(ColA
   }
 }
 
+// Set when a bounded wait of a staged row pass gives up; the host reads and clears it with
+// swense_async_status.
+__device__ int g_async_timeout;
+
 // Row pass over the transposed intermediate for rows of 32 to 2048 points: T = N / R0 threads per grid
-// row, its four modal fields loaded straight from G (neighbouring threads read neighbouring m),
-// packed as Z1 = U + iV and Z2 = W + iT over the full x spectrum, both transformed side by side
-// (WideRow), stored as float4. Loads are cached in L1: at padding 1 a row reads each value twice, as
-// mode m and mirrored as N - m. Eight levels of 1024 x 2048 nodes at padding 4: 108 -> 72 us; at
-// padding 1 the loads of the intermediate bound it, 149 us (124 with radix-8 passes, whose six blocks
-// per SM hid more of them; the columns' gain outweighs it). Variants at 5 blocks per SM spill.
-template <int N>
-__global__ void __launch_bounds__(WideRow<N>::T * WideRow<N>::kRows, WideRow<N>::E == 16 ? 4 : 8) k_row_w(RowArgs a) {
+// row; its four modal fields packed as Z1 = U + iV and Z2 = W + iT over the full x spectrum, both
+// transformed (WideRow), stored as float4. Persistent blocks take kRows rows of a slot at a time, whose
+// fields (contiguous in G) arrive in shared memory by bulk copies on the block's mbarrier, the next
+// rows' while the current ones are transformed: at padding 1 a row is 32 KB read twice (as mode m and
+// mirrored as N - m), which straight loads could only fetch a third at a time for want of registers.
+// A wait that does not complete within its bound sets the error flag and ends the block, as one.
+// Eight levels of 1024 x 2048 nodes: at padding 1 149 -> 97 us (5.5 TB/s with the
+// intermediate from memory), at padding 4 (a quarter of the input) 76 us; radix-8 passes with
+// straight loads took 124 and 108.
+// TWO: an exchange buffer for each of the two transforms, where the staged rows leave the room.
+template <int N, bool TWO>
+__global__ void __launch_bounds__(WideRow<N>::T * WideRow<N>::kRows, WideRow<N>::E == 16 ? 4 : 8) k_row_w(RowArgs a, int items) {
   using W = WideRow<N>;
-  extern __shared__ float2 sm[];                 // two exchange buffers per row
+  extern __shared__ __align__(16) unsigned char smraw[];
   const int t = threadIdx.x % W::T, rr = threadIdx.x / W::T;
-  const int y = blockIdx.x * W::kRows + rr;      // the row count is a multiple of kRows
-  const int level = blockIdx.y;
   const size_t fs = size_t(a.Nyr) * a.ldG;
-  const float2* row = a.G + size_t(level) * 4 * fs + size_t(y) * a.ldG;
-  const bool is_eta = a.lev0 + level >= a.n_lev;   // one field: Z1 = eta, the others zero
-  float2 z1[W::E], z2[W::E];
+  const unsigned span = unsigned(W::kRows * a.ldG) * unsigned(sizeof(float2));   // bytes per field
+  float2* stg = reinterpret_cast<float2*>(smraw);
+  float2* buf = reinterpret_cast<float2*>(smraw + 4 * size_t(span)) + rr * (TWO ? 2 : 1) * W::kBuf;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smraw + 4 * size_t(span) + size_t(W::kRows) * (TWO ? 2 : 1) * W::kBuf * sizeof(float2));
+  const int yblocks = a.Nyr / W::kRows;            // the row count is a multiple of kRows
+  auto issue = [&](int item) {                     // by one thread
+    const int level = item / yblocks, y0 = (item - level * yblocks) * W::kRows;
+    const int nf = a.lev0 + level >= a.n_lev ? 1 : 4;   // eta: one field
+    const float2* src = a.G + size_t(level) * 4 * fs + size_t(y0) * a.ldG;
+    fence_proxy_async();                           // earlier reads of the buffer come first
+    mbar_arrive_expect_tx(bar, nf * span);
+    for (int f = 0; f < nf; ++f) bulk_g2s(stg + size_t(f) * W::kRows * a.ldG, src + f * fs, span, bar);
+  };
+  int item = blockIdx.x;
+  if (item >= items) return;
+  if (threadIdx.x == 0) {
+    mbar_init(bar, 1);
+    fence_mbar_init();
+    fence_proxy_async();
+    issue(item);
+  }
+  __syncthreads();
+  for (unsigned ph = 0; item < items; ph ^= 1u) {
+    const bool done = mbar_wait(bar, ph, a.polls);
+    if (__syncthreads_or(!done)) {                 // one thread gave up: the whole block leaves
+      if (threadIdx.x == 0) atomicExch(&g_async_timeout, 1);
+      mbar_wait(bar, ph, a.polls);                 // the copy waited on is the only one in flight
+      __syncthreads();
+      return;
+    }
+    const int level = item / yblocks, y = (item - level * yblocks) * W::kRows + rr;
+    const bool is_eta = a.lev0 + level >= a.n_lev;   // one field: Z1 = eta, the others zero
+    const float2* S = stg + size_t(rr) * a.ldG;
+    const size_t ss = size_t(W::kRows) * a.ldG;
+    float2 z1[W::E], z2[W::E];
 #pragma unroll
-  for (int e = 0; e < W::E; ++e) {
-    // positions of the upper half hold the mirrored (conjugate) modes N - p
-    const int p = t + W::T * e, mm = e < W::E / 2 ? p : N - p;
-    float2 U = make_float2(0.f, 0.f), V = U, X = U, Y = U;
-    if (mm < a.Mh) {
-      U = row[mm];
-      if (!is_eta) {
-        V = row[fs + mm];
-        X = row[2 * fs + mm];
-        Y = row[3 * fs + mm];
+    for (int e = 0; e < W::E; ++e) {
+      // positions of the upper half hold the mirrored (conjugate) modes N - p
+      const int p = t + W::T * e, mm = e < W::E / 2 ? p : N - p;
+      float2 U = make_float2(0.f, 0.f), V = U, X = U, Y = U;
+      if (mm < a.Mh) {
+        U = S[mm];
+        if (!is_eta) {
+          V = S[ss + mm];
+          X = S[2 * ss + mm];
+          Y = S[3 * ss + mm];
+        }
+      }
+      if (e >= W::E / 2) {
+        z1[e] = make_float2(U.x + V.y, V.x - U.y);
+        z2[e] = make_float2(X.x + Y.y, Y.x - X.y);
+      } else if (e == 0 && t == 0) {               // m = 0: the real parts only
+        z1[e] = make_float2(U.x, V.x);
+        z2[e] = make_float2(X.x, Y.x);
+      } else {
+        z1[e] = make_float2(U.x - V.y, U.y + V.x);
+        z2[e] = make_float2(X.x - Y.y, X.y + Y.x);
       }
     }
-    if (e >= W::E / 2) {
-      z1[e] = make_float2(U.x + V.y, V.x - U.y);
-      z2[e] = make_float2(X.x + Y.y, Y.x - X.y);
-    } else if (e == 0 && t == 0) {               // m = 0: the real parts only
-      z1[e] = make_float2(U.x, V.x);
-      z2[e] = make_float2(X.x, Y.x);
+    __syncthreads();                               // the staged rows have been read
+    const int next = item + int(gridDim.x);
+    if (threadIdx.x == 0 && next < items) issue(next);
+    W::template fft2<TWO>(z1, z2, a.tw, buf, TWO ? buf + W::kBuf : buf, t);
+    if (is_eta) {
+      float* out = a.eta + (size_t(a.lev0 + level - a.n_lev) * a.Nyr + y) * N;
+#pragma unroll
+      for (int b = 0; b < W::BL; ++b)
+#pragma unroll
+        for (int r = 0; r < W::RL; ++r) __stcs(&out[W::pos(t, b, r)], z1[W::elem(b, r)].x);
     } else {
-      z1[e] = make_float2(U.x - V.y, U.y + V.x);
-      z2[e] = make_float2(X.x - Y.y, X.y + Y.x);
+      float4* out = a.nodes + (size_t(a.lev0 + level) * a.Nyr + y) * N;
+#pragma unroll
+      for (int b = 0; b < W::BL; ++b)
+#pragma unroll
+        for (int r = 0; r < W::RL; ++r) {
+          const int e = W::elem(b, r);
+          __stcs(&out[W::pos(t, b, r)], make_float4(z1[e].x, z1[e].y, z2[e].x, z2[e].y));
+        }
     }
+    discard_rows(a.G + size_t(level) * 4 * fs + size_t(y) * a.ldG, fs, is_eta ? 1 : 4, a.ldG, t, W::T);
+    item = next;
   }
-  float2* b1 = sm + size_t(rr) * 2 * W::kBuf;
-  W::fft2(z1, z2, a.tw, b1, b1 + W::kBuf, t);
-  if (is_eta) {
-    float* out = a.eta + (size_t(a.lev0 + level - a.n_lev) * a.Nyr + y) * N;
-#pragma unroll
-    for (int b = 0; b < W::BL; ++b)
-#pragma unroll
-      for (int r = 0; r < W::RL; ++r) __stcs(&out[W::pos(t, b, r)], z1[W::elem(b, r)].x);
-    discard_rows(row, fs, 1, a.ldG, t, W::T);
-    return;
-  }
-  float4* out = a.nodes + (size_t(a.lev0 + level) * a.Nyr + y) * N;
-#pragma unroll
-  for (int b = 0; b < W::BL; ++b)
-#pragma unroll
-    for (int r = 0; r < W::RL; ++r) {
-      const int e = W::elem(b, r);
-      __stcs(&out[W::pos(t, b, r)], make_float4(z1[e].x, z1[e].y, z2[e].x, z2[e].y));
-    }
-  // every thread's reads of the row came before the last exchange's barrier
-  discard_rows(row, fs, 4, a.ldG, t, W::T);
 }
 
 // Row pass for 4096- and 8192-point rows: one block of kThreads per grid row of one level, inputs
@@ -611,8 +651,6 @@ __global__ void __launch_bounds__(256, N >= 8192 ? 1 : 2) k_row_tb(RowArgs a) {
 // the warp decides together (every lane must have seen its copy complete), waits, also bounded,
 // for the copy it still has in flight, and leaves as one. The host reads and clears the flag
 // with swense_async_status.
-__device__ int g_async_timeout;
-
 template <int N>
 __global__ void __launch_bounds__(256, N >= 1024 ? 1 : 2) k_row_tma(RowArgs a, int rpw) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -744,10 +782,21 @@ int launch_col_w(const ColArgs& c, const Levels& L, int nl, cudaStream_t stream)
 template <int N>
 int launch_row_w(const RowArgs& r, int nl, cudaStream_t stream) {
   using W = WideRow<N>;
-  const size_t smem = size_t(W::kRows) * 2 * W::kBuf * sizeof(float2);
-  int st = set_smem((const void*)k_row_w<N>, smem);
+  const int per_sm = W::E == 16 ? 4 : 8;
+  const size_t stage = size_t(4) * W::kRows * r.ldG * sizeof(float2), buf = size_t(W::kRows) * W::kBuf * sizeof(float2);
+  // 227 KB of shared memory per SM, 1 KB of it reserved per block
+  const bool two = (stage + 2 * buf + 1152) * per_sm <= size_t(227) * 1024;
+  const size_t smem = stage + (two ? 2 : 1) * buf + sizeof(uint64_t);
+  const void* fn = two ? (const void*)k_row_w<N, true> : (const void*)k_row_w<N, false>;
+  int st = set_smem(fn, smem);
   if (st) return st;
-  k_row_w<N><<<dim3(unsigned(r.Nyr / W::kRows), unsigned(nl)), W::T * W::kRows, smem, stream>>>(r);
+  int dev = 0, sms = 0;
+  SWENSE_CUDA_TRY(cudaGetDevice(&dev));
+  SWENSE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int items = nl * (r.Nyr / W::kRows);
+  const unsigned grid = unsigned(std::min(items, sms * per_sm));
+  if (two) k_row_w<N, true><<<grid, W::T * W::kRows, smem, stream>>>(r, items);
+  else k_row_w<N, false><<<grid, W::T * W::kRows, smem, stream>>>(r, items);
   SWENSE_CUDA_TRY(cudaGetLastError());
   count_launches(1);
   return SWENSE_OK;
