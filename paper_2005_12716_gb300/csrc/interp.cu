@@ -231,6 +231,11 @@ constexpr int BOX_PTS = BOX_THREADS * BOX_PPT;
 constexpr int BOX_NODES = 4096;                    // float4 nodes (64 KB; 99 % of the 1024-point mesh chunks fit)
 constexpr int BOX_COLS = BOX_NODES / 4;             // eta columns (a box has at least 4 levels)
 constexpr size_t BOX_SMEM = size_t(BOX_NODES) * sizeof(float4) + size_t(BOX_COLS) * sizeof(float);
+// Tile of the batched gather: points binned in rows of tiles put 1024 of them in a box of
+// (256 / d + 3) x 7 x 4 nodes at d points per node, or of whole rows of a narrow grid; 6400 nodes
+// (two CTAs per SM) hold that from d = 1.1 on, 4096 only from 1.8 on.
+constexpr int BATCH_NODES = 6400, BATCH_COLS = BATCH_NODES / 4;
+constexpr size_t BATCH_SMEM = size_t(BATCH_NODES) * sizeof(float4) + size_t(BATCH_COLS) * sizeof(float);
 // Level-flat chunks (every point at the same z, as the cell and face centres of one layer of an
 // extruded mesh) stage one z-collapsed plane instead of the box: float4 columns and eta.
 constexpr int FLAT_COLS = 3456;
@@ -524,8 +529,8 @@ __host__ __device__ __forceinline__ int64_t plan_blocks(int64_t np) {
   return ((np + BOX_PTS - 1) / BOX_PTS + PLAN_WARPS - 1) / PLAN_WARPS;
 }
 
-// Plan of chunk `chunk` of the points of `a`, by one warp (no block barrier).
-template <bool P2>
+// Plan of chunk `chunk` of the points of `a`, by one warp (no block barrier), for tiles of NODES nodes.
+template <bool P2, int NODES = BOX_NODES>
 __device__ __forceinline__ void plan_chunk(const InterpArgs& a, const LevelTables& zs, int64_t chunk,
                                            int4* __restrict__ plan, int lane) {
   const int64_t p0 = chunk * BOX_PTS;
@@ -592,22 +597,22 @@ __device__ __forceinline__ void plan_chunk(const InterpArgs& a, const LevelTable
   const bool flat = __all_sync(0xffffffffu, same_z);
   const bool flat2 = !flat && __all_sync(0xffffffffu, two_z);
   if (lane != 0) return;
-  // box: x nodes rel (mn0-1) .. (mx0+2), y likewise (one row in 2-D), levels mn2 .. mx2+3
-  const int bx = mx[0] - mn[0] + 4;
+  // box: x nodes rel (mn0-1) .. (mx0+2), y likewise (one row in 2-D), levels mn2 .. mx2+3; one that laps
+  // the periodic grid is the whole period and three nodes more, so that every stencil is contiguous
+  const int bx = min(mx[0] - mn[0] + 4, a.Nxr + 3);
   const int sbx = bx + ((4 - bx) & 7);
-  const int by = a.Nyr > 1 ? mx[1] - mn[1] + 4 : 1;
+  const int by = a.Nyr > 1 ? min(mx[1] - mn[1] + 4, a.Nyr + 3) : 1;
   const int bz = mx[2] - mn[2] + 4;
   const int zst = box_zstride(sbx, by);
-  const bool inside_grid = bx <= a.Nxr && by <= a.Nyr;
-  const bool fits = int64_t(zst) * bz <= BOX_NODES && int64_t(sbx) * by <= BOX_COLS && inside_grid;
-  const bool fits_flat = flat && int64_t(sbx) * by <= FLAT_COLS && inside_grid;
-  const bool fits_two = flat2 && int64_t(sbx) * by <= FLAT2_COLS && inside_grid;
+  const bool fits = int64_t(zst) * bz <= NODES && int64_t(sbx) * by <= NODES / 4 && bx < 2048 && by < 2048;
+  const bool fits_flat = flat && int64_t(sbx) * by <= FLAT_COLS;
+  const bool fits_two = flat2 && int64_t(sbx) * by <= FLAT2_COLS;
   const int x0 = wrapi<P2>(refx + mn[0] - 1, a.Nxr);
   const int y0 = a.Nyr > 1 ? wrapi<P2>(refy + mn[1] - 1, a.Nyr) : 0;
   plan[chunk] = fits_flat  ? make_int4(x0, y0, mn[2] | FLAT_BIT, bx | (by << 12))
               : fits_two   ? make_int4(x0, y0, FLAT_BIT | FLAT2_BIT, bx | (by << 12))
               : fits       ? make_int4(x0, y0, mn[2], bx | (by << 11) | (bz << 22))
-              : (flat || flat2) && inside_grid
+              : flat || flat2
                   ? make_int4(x0, y0, flat ? FLAT_BIT : FLAT_BIT | FLAT2_BIT, int(0x80000000u | unsigned(bx) | unsigned(by) << 14))
                   : make_int4(x0, y0, mn[2], -1);
 }
@@ -1278,22 +1283,27 @@ __global__ void __launch_bounds__(BOX_THREADS) k_interp_plan_batch(const BatchIn
   copy_words(sa, &inst[i].a, int(sizeof(InterpArgs)), lane, 32);
   copy_words(zs, &inst[i].L, int(sizeof(LevelTables)), lane, 32);
   __syncwarp();
-  plan_chunk<true>(*sa, *zs, c - chunk0[i], plan + chunk0[i], lane);
+  plan_chunk<true, BATCH_NODES>(*sa, *zs, c - chunk0[i], plan + chunk0[i], lane);
 }
 
-__global__ void __launch_bounds__(BOX_THREADS, 3) k_interp_box_batch(const BatchInst* __restrict__ inst,
+// The chunks with a staged tile, by persistent blocks.
+__global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_box_batch(const BatchInst* __restrict__ inst,
                                                                       const int64_t* __restrict__ chunk0, int n,
                                                                       const int4* __restrict__ plan,
                                                                       unsigned* __restrict__ counter) {
   extern __shared__ float4 sbox[];
-  float* seta = reinterpret_cast<float*>(sbox + BOX_NODES);
+  float* seta = reinterpret_cast<float*>(sbox + BATCH_NODES);
   __shared__ LevelTables zs;
   __shared__ InterpArgs sa;
   __shared__ int64_t s_item;
   const int64_t total = chunk0[n];
   int cur = -1;
   for (;;) {
-    if (threadIdx.x == 0) s_item = int64_t(atomicAdd(counter, 1u));
+    if (threadIdx.x == 0) {                         // the next chunk with a tile
+      int64_t c = int64_t(atomicAdd(counter, 1u));
+      while (c < total && plan_is_global(plan[c], inst[batch_instance(chunk0, n, c)].a.nz)) c = int64_t(atomicAdd(counter, 1u));
+      s_item = c;
+    }
     __syncthreads();
     const int64_t c = s_item;
     if (c >= total) break;                          // uniform over the CTA
@@ -1304,9 +1314,29 @@ __global__ void __launch_bounds__(BOX_THREADS, 3) k_interp_box_batch(const Batch
       cur = i;
     }
     __syncthreads();                                // arguments and tables in place
-    box_chunk<true>(sa, zs, c - chunk0[i], plan[c], sbox, seta);
+    box_chunk<true, false>(sa, zs, c - chunk0[i], plan[c], sbox, seta);
     __syncthreads();                                // shared memory free for the next chunk
   }
+}
+
+// The others, straight from the grid in point order (as k_interp_global): without a tile's shared
+// memory L1 holds the rows that neighbouring points share. Eight uneven instances, 4.2 M points at
+// four time levels: 1.84 -> 1.06 ms, 0.35 of it the tiles of the dense instance (3.1 M points).
+__global__ void __launch_bounds__(BOX_THREADS, 5) k_interp_global_batch(const BatchInst* __restrict__ inst,
+                                                                         const int64_t* __restrict__ chunk0, int n,
+                                                                         const int4* __restrict__ plan) {
+  __shared__ GatherRec rec[GLOBAL_PTS];
+  __shared__ InterpArgs sa;
+  constexpr int SUB = BOX_PTS / GLOBAL_PTS;
+  const int64_t c = blockIdx.x / SUB;
+  const int i = batch_instance(chunk0, n, c);
+  if (!plan_is_global(plan[c], inst[i].a.nz)) return;   // uniform over the block
+  copy_words(&sa, &inst[i].a, int(sizeof(InterpArgs)), threadIdx.x, blockDim.x);
+  __syncthreads();
+  const int warp = threadIdx.x >> 5;
+  const int64_t p0 = (c - chunk0[i]) * BOX_PTS + (blockIdx.x % SUB) * GLOBAL_PTS + warp * GLOBAL_WPTS;
+  if (p0 >= sa.np) return;                          // uniform over the warp
+  gather_warp<true, GLOBAL_WPTS>(sa, *level_tables(inst[i].L), p0, rec + warp * GLOBAL_WPTS);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2153,7 +2183,7 @@ int interp_batch(const GatherItem* items, int n, int32_t p_mode, double rho, dou
   int st = batch_tables(items, n, p_mode, rho, grav, stream, &d_inst, &d_chunk0, &nchunks);
   if (st) return st;
   if (nchunks == 0) return SWENSE_OK;
-  if (nchunks >= (int64_t(1) << 31)) return fail(SWENSE_ERR_SIZE, "too many point chunks in one batch");
+  if (nchunks >= (int64_t(1) << 31) / (BOX_PTS / GLOBAL_PTS)) return fail(SWENSE_ERR_SIZE, "too many point chunks in one batch");
   unsigned* counter = static_cast<unsigned*>(ws);
   int4* plan = reinterpret_cast<int4*>(static_cast<char*>(ws) + 256);
   const size_t plan_smem = size_t(PLAN_WARPS) * (sizeof(InterpArgs) + sizeof(LevelTables));
@@ -2164,16 +2194,18 @@ int interp_batch(const GatherItem* items, int n, int32_t p_mode, double rho, dou
   SWENSE_CUDA_TRY(cudaGetLastError());
   SWENSE_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned), stream));
   SWENSE_CUDA_TRY(cudaFuncSetAttribute((const void*)k_interp_box_batch,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, int(BOX_SMEM)));
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, int(BATCH_SMEM)));
   int dev = 0, sms = 0, per_sm = 0;
   SWENSE_CUDA_TRY(cudaGetDevice(&dev));
   SWENSE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   SWENSE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_interp_box_batch, BOX_THREADS,
-                                                                BOX_SMEM));
+                                                                BATCH_SMEM));
   const int64_t ctas = std::min<int64_t>(nchunks, int64_t(std::max(1, sms * std::max(1, per_sm))));
-  k_interp_box_batch<<<unsigned(ctas), BOX_THREADS, BOX_SMEM, stream>>>(d_inst, d_chunk0, n, plan, counter);
+  k_interp_box_batch<<<unsigned(ctas), BOX_THREADS, BATCH_SMEM, stream>>>(d_inst, d_chunk0, n, plan, counter);
   SWENSE_CUDA_TRY(cudaGetLastError());
-  count_launches(2);
+  k_interp_global_batch<<<unsigned(nchunks * (BOX_PTS / GLOBAL_PTS)), BOX_THREADS, 0, stream>>>(d_inst, d_chunk0, n, plan);
+  SWENSE_CUDA_TRY(cudaGetLastError());
+  count_launches(3);
   return SWENSE_OK;
 }
 
