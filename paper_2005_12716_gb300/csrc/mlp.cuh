@@ -48,9 +48,10 @@ __device__ __forceinline__ unsigned ld_u32(const __nv_bfloat16* p) {
   return *reinterpret_cast<const unsigned*>(p);
 }
 
-// GELU, tanh form: 0.5 x (1 + tanh(u)), u = sqrt(2/pi) (x + 0.044715 x^3), with
+// GELU, tanh form: 0.5 x (1 + tanh(u)), u = sqrt(2/pi) (x + 0.044715 x^3). Training's form, with
 // tanh(u) = 1 - 2 / (1 + e^{2u}) (saturates correctly at both ends; absolute error ~1e-7 near
-// u = 0, far below the BF16 operands it feeds).
+// u = 0, far below the BF16 operands it feeds): its activations are rounded to BF16, where another
+// form's last bit can flip a rounding, and a run goes on from an older checkpoint bit for bit.
 __device__ __forceinline__ float gelu_tanh_u(float x) {
   const float c = 0.7978845608028654f;
   const float u = c * fmaf(0.044715f * x, x * x, x);
@@ -62,32 +63,64 @@ __device__ __forceinline__ float gelu_grad(float x) {
   const float t = gelu_tanh_u(x);
   return 0.5f * (1.f + t) + 0.5f * x * (1.f - t * t) * c * fmaf(3.f * 0.044715f, x * x, 1.f);
 }
+// Inference's form, x / (1 + e^{-2u}): the same function in seven instructions instead of twelve and
+// without the cancellation; the exponential is one of two (2 log2(e) sqrt(2/pi) folded into the
+// polynomial), and an overflowing one gives 0, as it should.
+__device__ __forceinline__ float gelu_fast(float x) {
+  const float k1 = -2.f * 1.4426950408889634f * 0.7978845608028654f, k3 = k1 * 0.044715f;
+  float e;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x * fmaf(k3, x * x, k1)));
+  return __fdividef(x, 1.f + e);
+}
 
 // ------------------------------------------------------------------------------ forward
-// Layer with K = 16 * KS inputs held as A fragments (hi and optional lo), N = 8 * NT outputs.
+// B fragments of 8 outputs (rows n of W) and 32 (or 16) inputs from k on: the 8 x 8 blocks that the lanes
+// of each quarter (half) warp point at, row by row.
+__device__ __forceinline__ void load_b32(const __nv_bfloat16* W, int ldw, int lane, unsigned (&b)[4]) {
+  const unsigned a = unsigned(__cvta_generic_to_shared(W + (lane & 7) * ldw + 8 * (lane >> 3)));
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]) : "r"(a));
+}
+__device__ __forceinline__ void load_b16(const __nv_bfloat16* W, int ldw, int lane, unsigned (&b)[2]) {
+  const unsigned a = unsigned(__cvta_generic_to_shared(W + (lane & 7) * ldw + 8 * ((lane >> 3) & 1)));
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(b[0]), "=r"(b[1]) : "r"(a));
+}
+
+// Layer with K = 16 * KS inputs held as A fragments (hi and optional lo), N = 8 * NT outputs; W in
+// shared memory, rows 16-byte aligned.
 template <int KS, int NT, bool SPLIT>
 __device__ __forceinline__ void layer(float (&z)[NT][4], const unsigned (&ahi)[KS][4],
                                       const unsigned (&alo)[KS][4], const __nv_bfloat16* W, int ldw,
                                       const float* bias, int lane) {
-  const int g = lane >> 2, t = lane & 3;
+  const int t = lane & 3;
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) {
-    const float bb0 = bias[8 * nt + 2 * t], bb1 = bias[8 * nt + 2 * t + 1];
-    z[nt][0] = bb0;
-    z[nt][1] = bb1;
-    z[nt][2] = bb0;
-    z[nt][3] = bb1;
+    const float2 bb = *reinterpret_cast<const float2*>(&bias[8 * nt + 2 * t]);
+    z[nt][0] = bb.x;
+    z[nt][1] = bb.y;
+    z[nt][2] = bb.x;
+    z[nt][3] = bb.y;
+    const __nv_bfloat16* wr = W + 8 * nt * ldw;
 #pragma unroll
-    for (int kk = 0; kk < KS; ++kk) {
-      const __nv_bfloat16* wr = W + (8 * nt + g) * ldw + 16 * kk + 2 * t;
-      const unsigned b0 = ld_u32(wr), b1 = ld_u32(wr + 8);
-      mma16816(z[nt], ahi[kk], b0, b1);
-      if (SPLIT) mma16816(z[nt], alo[kk], b0, b1);
+    for (int kk = 0; kk + 1 < KS; kk += 2) {
+      unsigned b[4];
+      load_b32(wr + 16 * kk, ldw, lane, b);
+      mma16816(z[nt], ahi[kk], b[0], b[1]);
+      if (SPLIT) mma16816(z[nt], alo[kk], b[0], b[1]);
+      mma16816(z[nt], ahi[kk + 1], b[2], b[3]);
+      if (SPLIT) mma16816(z[nt], alo[kk + 1], b[2], b[3]);
+    }
+    if constexpr (KS & 1) {
+      unsigned b[2];
+      load_b16(wr + 16 * (KS - 1), ldw, lane, b);
+      mma16816(z[nt], ahi[KS - 1], b[0], b[1]);
+      if (SPLIT) mma16816(z[nt], alo[KS - 1], b[0], b[1]);
     }
   }
 }
 
-// Accumulator fragments (16 x 8*NT, FP32) -> A fragments (16 x 16*NT/2) after GELU.
+// Accumulator fragments (16 x 8*NT, FP32) -> A fragments (16 x 16*NT/2) after GELU: hi and lo halves for
+// inference, BF16 for training.
 template <int NT, bool SPLIT>
 __device__ __forceinline__ void to_a(const float (&z)[NT][4], unsigned (&ahi)[NT / 2][4],
                                      unsigned (&alo)[NT / 2][4]) {
@@ -96,7 +129,8 @@ __device__ __forceinline__ void to_a(const float (&z)[NT][4], unsigned (&ahi)[NT
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const float* c = z[2 * kk + h];
-      const float g0 = gelu(c[0]), g1 = gelu(c[1]), g2 = gelu(c[2]), g3 = gelu(c[3]);
+      auto act = [](float x) { return SPLIT ? gelu_fast(x) : gelu(x); };
+      const float g0 = act(c[0]), g1 = act(c[1]), g2 = act(c[2]), g3 = act(c[3]);
       if (SPLIT) {
         bf2_split(g0, g1, ahi[kk][2 * h], alo[kk][2 * h]);
         bf2_split(g2, g3, ahi[kk][2 * h + 1], alo[kk][2 * h + 1]);
