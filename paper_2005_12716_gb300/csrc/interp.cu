@@ -1350,8 +1350,9 @@ __global__ void __launch_bounds__(BOX_THREADS, 5) k_interp_global_batch(const Ba
 //     max |value|, the normalised values (hi + lo BF16) feed layers 1-3, and the lane holding
 //     column f of row (point, f) writes lagrange + s_f * out_scale * y[f];
 //   C (one thread per point): Bernoulli, NaN outside the levels, stores.
-// Bound by instruction issue; with weight fragments loaded four at a time (ldmatrix) and GELU in seven
-// instructions, 8.2 M mesh points take 4.75 ms (5.79 before).
+// Bound by instruction issue (50 % of cycles) and the warp MMAs (45 %), which hardly overlap; with weight
+// fragments loaded four at a time (ldmatrix), GELU of two values in nine instructions and the offsets in
+// half a step, 8.2 M mesh points take 4.45 ms (5.79 before).
 struct LPoint {
   int base;                 // staged node index of stencil node (x 0, y 0, level 0)
   float w[12];              // wx[4], wy[4], wz[4]; the corrected fields overwrite w[0..3]
@@ -1393,7 +1394,7 @@ __device__ __forceinline__ void learned_tiles(const float4* nodes, int SY, int S
     const int j0 = 4 * t + (g >> 2), j1 = j0 + 2;      // points of rows g and g + 8
     if (4 * t >= npts) break;                          // uniform over the warp
     float lag[2], sc[2];
-    unsigned xh[5][4], xl[5][4];
+    unsigned xh[4][4], xl[4][4], xo[2];
     float v[2][4][4];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -1423,34 +1424,23 @@ __device__ __forceinline__ void learned_tiles(const float4* nodes, int SY, int S
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const float inv = 1.f / sc[h];
-        bf2_split(v[h][kk][0] * inv, v[h][kk][1] * inv, xh[kk][h], xl[kk][h]);
-        bf2_split(v[h][kk][2] * inv, v[h][kk][3] * inv, xh[kk][2 + h], xl[kk][2 + h]);
+        const float2 iv = make_float2(inv, inv);
+        bf2_split(pmul(make_float2(v[h][kk][0], v[h][kk][1]), iv), xh[kk][h], xl[kk][h]);
+        bf2_split(pmul(make_float2(v[h][kk][2], v[h][kk][3]), iv), xh[kk][2 + h], xl[kk][2 + h]);
       }
     }
-    // inputs 64..79: dx, dy, dz, then zeros (columns 2q, 2q+1 of the fifth k-tile)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const LPoint& P = rec[min(h ? j1 : j0, npts - 1)];
-      const float o0 = q == 0 ? P.off[0] : (q == 1 ? P.off[2] : 0.f);
-      const float o1 = q == 0 ? P.off[1] : 0.f;
-      bf2_split(o0, o1, xh[4][h], xl[4][h]);
-      xh[4][2 + h] = xl[4][2 + h] = 0u;
+      xo[h] = offsets_a(P.off[0], P.off[1], P.off[2], q);
     }
-    float z1[8][4];
-    layer<5, 8, true>(z1, xh, xl, &W.w1[0][0], W1LD, W.b1, lane);
-    unsigned h1h[4][4], h1l[4][4];
-    to_a<8, true>(z1, h1h, h1l);
-    float z2[8][4];
-    layer<4, 8, true>(z2, h1h, h1l, &W.w2[0][0], W2LD, W.b2, lane);
-    unsigned h2h[4][4], h2l[4][4];
-    to_a<8, true>(z2, h2h, h2l);
-    float o[1][4];
-    layer<4, 1, true>(o, h2h, h2l, &W.w3[0][0], W2LD, W.b3, lane);
+    float o[4];
+    infer(o, xh, xl, xo, W, W1LD, W2LD, lane);
     __syncwarp();                                      // every lane has read its records
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int jh = h ? j1 : j0;
-      const float yv = (f & 1) ? o[0][2 * h + 1] : o[0][2 * h];   // a select, not a local array
+      const float yv = (f & 1) ? o[2 * h + 1] : o[2 * h];   // a select, not a local array
       if ((f >> 1) == q && jh < npts) rec[jh].w[f] = fmaf(sc[h] * W.out_scale, yv, lag[h]);
     }
     __syncwarp();
@@ -1472,8 +1462,10 @@ __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_
     const uint4* g1 = reinterpret_cast<const uint4*>(&Wg->w1[0][0]);
     const uint4* g2 = reinterpret_cast<const uint4*>(&Wg->w2[0][0]);
     const uint4* g3 = reinterpret_cast<const uint4*>(&Wg->w3[0][0]);
-    for (int i = threadIdx.x; i < NH * KIN / 8; i += blockDim.x)
-      *reinterpret_cast<uint4*>(&W.w1[i / (KIN / 8)][8 * (i % (KIN / 8))]) = __ldg(&g1[i]);
+    for (int i = threadIdx.x; i < NH * KIN / 8; i += blockDim.x) {
+      const uint4 w = __ldg(&g1[i]);
+      *reinterpret_cast<uint4*>(&W.w1[i / (KIN / 8)][8 * (i % (KIN / 8))]) = i % (KIN / 8) == 8 ? repeat_offsets(w) : w;
+    }
     for (int i = threadIdx.x; i < NH * NH / 8; i += blockDim.x)
       *reinterpret_cast<uint4*>(&W.w2[i / (NH / 8)][8 * (i % (NH / 8))]) = __ldg(&g2[i]);
     for (int i = threadIdx.x; i < NO * NH / 8; i += blockDim.x)

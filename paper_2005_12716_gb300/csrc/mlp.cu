@@ -56,27 +56,23 @@ __global__ void k_mlp_pack(const float* __restrict__ P, Packed* __restrict__ out
   if (i < NO) out->b3[i] = i < NOUT ? P[OFF_B3 + i] : 0.f;
 }
 
-// A fragments of 16 rows of x (FP32, leading dimension XLD, columns >= NIN read as 0).
-__device__ __forceinline__ void load_x(const float* __restrict__ x, int64_t row0, int64_t rows,
-                                       unsigned (&ahi)[5][4], unsigned (&alo)[5][4], int lane) {
+// A fragments of 16 rows of x (FP32, leading dimension XLD; rows past the end read as 0).
+__device__ __forceinline__ void load_x(const float* __restrict__ x, int64_t row0, int64_t rows, unsigned (&ahi)[4][4],
+                                       unsigned (&alo)[4][4], unsigned (&off)[2], int lane) {
   const int g = lane >> 2, t = lane & 3;
-  const int64_t r[2] = {row0 + g, row0 + g + 8};
-  const float* xr[2];
 #pragma unroll
-  for (int h = 0; h < 2; ++h) xr[h] = r[h] < rows ? x + r[h] * XLD : nullptr;
+  for (int h = 0; h < 2; ++h) {                    // a0, a2: row g; a1, a3: row g + 8
+    const int64_t r = row0 + g + 8 * h;
+    const float* xr = r < rows ? x + r * XLD : nullptr;
+    auto at = [&](int col) { return xr ? __ldg(&xr[col]) : 0.f; };
 #pragma unroll
-  for (int kk = 0; kk < 5; ++kk) {
+    for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int h = q & 1;                         // a0, a2: row g; a1, a3: row g + 8
-      const int col = 16 * kk + 2 * t + (q >= 2 ? 8 : 0);
-      float v0 = 0.f, v1 = 0.f;
-      if (xr[h]) {
-        if (col < NIN) v0 = __ldg(&xr[h][col]);
-        if (col + 1 < NIN) v1 = __ldg(&xr[h][col + 1]);
+      for (int q = 0; q < 2; ++q) {
+        const int col = 16 * kk + 2 * t + 8 * q;
+        bf2_split(at(col), at(col + 1), ahi[kk][h + 2 * q], alo[kk][h + 2 * q]);
       }
-      bf2_split(v0, v1, ahi[kk][q], alo[kk][q]);
-    }
+    off[h] = offsets_a(at(64), at(65), at(66), t);
   }
 }
 
@@ -85,33 +81,26 @@ __global__ void __launch_bounds__(128) k_mlp_forward(const Packed* __restrict__ 
                                                      int64_t rows, float* __restrict__ y) {
   __shared__ Packed s;
   {
-    const int4* src = reinterpret_cast<const int4*>(P);
-    int4* dst = reinterpret_cast<int4*>(&s);
-    for (int i = threadIdx.x; i < int(sizeof(Packed) / 16); i += blockDim.x) dst[i] = src[i];
+    const uint4* src = reinterpret_cast<const uint4*>(P);
+    uint4* dst = reinterpret_cast<uint4*>(&s);
+    for (int i = threadIdx.x; i < int(sizeof(Packed) / 16); i += blockDim.x)
+      dst[i] = i < NH * KIN / 8 && i % (KIN / 8) == 8 ? repeat_offsets(src[i]) : src[i];
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
   for (int64_t row0 = (int64_t(blockIdx.x) * 4 + warp) * 16; row0 < rows;
        row0 += int64_t(gridDim.x) * 64) {
-    unsigned xh[5][4], xl[5][4];
-    load_x(x, row0, rows, xh, xl, lane);
-    float z1[8][4];
-    layer<5, 8, true>(z1, xh, xl, &s.w1[0][0], KIN, s.b1, lane);
-    unsigned h1h[4][4], h1l[4][4];
-    to_a<8, true>(z1, h1h, h1l);
-    float z2[8][4];
-    layer<4, 8, true>(z2, h1h, h1l, &s.w2[0][0], NH, s.b2, lane);
-    unsigned h2h[4][4], h2l[4][4];
-    to_a<8, true>(z2, h2h, h2l);
-    float o[1][4];
-    layer<4, 1, true>(o, h2h, h2l, &s.w3[0][0], NH, s.b3, lane);
+    unsigned xh[4][4], xl[4][4], xo[2];
+    load_x(x, row0, rows, xh, xl, xo, lane);
+    float o[4];
+    infer(o, xh, xl, xo, s, KIN, NH, lane);
     // row r uses output column r % 4: c0/c1 hold columns 2t, 2t+1 of row g, c2/c3 of row g+8
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int64_t r = row0 + g + 8 * h;
       const int f = (g + 8 * h) & 3;               // row0 is a multiple of 16
-      const float yv = (f & 1) ? o[0][2 * h + 1] : o[0][2 * h];   // a select, not a local array
+      const float yv = (f & 1) ? o[2 * h + 1] : o[2 * h];   // a select, not a local array
       if (r < rows && (f >> 1) == t) y[r] = yv * s.out_scale;
     }
   }
@@ -167,7 +156,7 @@ __global__ void __launch_bounds__(TTHR, 1) k_mlp_train(TrainArgs a) {
     for (int r0 = blockIdx.x * TROWS; r0 < a.B; r0 += step) {
       sync();                                      // the tile's x rows are in place
       const int w0 = 16 * warp;
-      unsigned xh[5][4], unused0[5][4];
+      unsigned xh[5][4];
 #pragma unroll
       for (int kk = 0; kk < 5; ++kk)
 #pragma unroll
@@ -176,15 +165,15 @@ __global__ void __launch_bounds__(TTHR, 1) k_mlp_train(TrainArgs a) {
           xh[kk][q] = col < XS ? bf2(s.x[r][col], s.x[r][col + 1]) : 0u;
         }
       float z1[8][4];
-      layer<5, 8, false>(z1, xh, unused0, &s.p.w1[0][0], KIN, s.p.b1, lane);
-      unsigned h1[4][4], unused1[4][4];
-      to_a<8, false>(z1, h1, unused1);
+      layer<5, 8>(z1, xh, &s.p.w1[0][0], KIN, s.p.b1, lane);
+      unsigned h1[4][4];
+      to_a<8>(z1, h1);
       float z2[8][4];
-      layer<4, 8, false>(z2, h1, unused1, &s.p.w2[0][0], NH, s.p.b2, lane);
-      unsigned h2[4][4], unused2[4][4];
-      to_a<8, false>(z2, h2, unused2);
+      layer<4, 8>(z2, h1, &s.p.w2[0][0], NH, s.p.b2, lane);
+      unsigned h2[4][4];
+      to_a<8>(z2, h2);
       float o[1][4];
-      layer<4, 1, false>(o, h2, unused2, &s.p.w3[0][0], NH, s.p.b3, lane);
+      layer<4, 1>(o, h2, &s.p.w3[0][0], NH, s.p.b3, lane);
       // dY: only the row's own output column carries 2 (y - target) / B
       float dyf[4];
 #pragma unroll

@@ -25,6 +25,11 @@ __device__ __forceinline__ void bf2_split(float a, float b, unsigned& hi, unsign
   const float ha = __uint_as_float(hi << 16), hb = __uint_as_float(hi & 0xffff0000u);
   lo = bf2(a - ha, b - hb);
 }
+__device__ __forceinline__ void bf2_split(float2 v, unsigned& hi, unsigned& lo) {
+  hi = bf2(v.x, v.y);
+  const float2 r = csub(v, make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)));
+  lo = bf2(r.x, r.y);
+}
 
 __device__ __forceinline__ void mma16816(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
   asm volatile(
@@ -32,6 +37,14 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const unsigned (&a)[4], 
       "{%0,%1,%2,%3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// Eight inputs: A a0 (g, 2q..2q+1), a1 (g+8, 2q..2q+1); B b0 rows 2q..2q+1 of column g.
+__device__ __forceinline__ void mma1688(float (&d)[4], const unsigned (&a)[2], unsigned b0) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(b0));
 }
 
 // 16-byte global -> shared asynchronous copy (src_bytes < 16 zero-fills the rest).
