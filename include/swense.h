@@ -611,13 +611,14 @@ int swense_relax_cells(const float* cell_xyz, const float* cell_zext, const floa
 
 /*
  * swense_async_status — errors of bounded device-side waits (no passage of the paper: library
- * housekeeping). Kernels that wait on asynchronous copies (the staged row pass of
- * swense_fields_on_grid, row variant 4) give every wait an iteration limit; a wait that runs
- * out sets a per-device flag and its warp returns without writing its grid rows, so the call
- * that launched it has already returned SWENSE_OK. This call synchronises `stream`, reads the
- * flag of the current device and, when reset != 0, clears it.
- * Returns SWENSE_ERR_TIMEOUT if a wait gave up since the flag was last cleared (the grid of that
- * call is incomplete), else SWENSE_OK; CUDA on a failed copy.
+ * housekeeping). Kernels that wait on asynchronous copies or on the tensor cores (the staged row
+ * passes of swense_fields_on_grid, the tensor-core sum of swense_direct, swense_interp_learned)
+ * give every wait an iteration limit; a wait that runs out sets a per-device flag and leaves its
+ * outputs unwritten (the learned gather: NaN), so the call that launched it has already returned
+ * SWENSE_OK. This call synchronises `stream`, reads the flags of the current device and, when
+ * reset != 0, clears them.
+ * Returns SWENSE_ERR_TIMEOUT if a wait gave up since the flags were last cleared (the outputs of
+ * that call are incomplete), else SWENSE_OK; CUDA on a failed copy.
  */
 int swense_async_status(int32_t reset, void* stream);
 

@@ -168,9 +168,10 @@ const char* swense_strerror(int status) {
 
 int swense_async_status(int32_t reset, void* stream) {
   SWENSE_CUDA_TRY(cudaStreamSynchronize(static_cast<cudaStream_t>(stream)));
-  int grid = 0, direct = 0;
+  int grid = 0, direct = 0, learned = 0;
   int st = swense::grid_async_flag(reset != 0, &grid);
   if (!st) st = swense::direct_async_flag(reset != 0, &direct);
+  if (!st) st = swense::learned_async_flag(reset != 0, &learned);
   if (st) return st;
   if (grid)
     return swense::fail(SWENSE_ERR_TIMEOUT, "a bounded wait of a staged row pass (k_row_w, k_row_tma) gave "
@@ -179,6 +180,9 @@ int swense_async_status(int32_t reset, void* stream) {
     return swense::fail(SWENSE_ERR_TIMEOUT, "a bounded wait of the tensor-core direct sum "
                                             "(k_direct_tc) gave up; the outputs of that tile were "
                                             "not written");
+  if (learned)
+    return swense::fail(SWENSE_ERR_TIMEOUT, "a bounded wait of the learned gather (k_interp_learned) gave "
+                                            "up; u, v, w, p of those points are NaN");
   return SWENSE_OK;
 }
 

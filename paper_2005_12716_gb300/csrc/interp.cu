@@ -17,6 +17,8 @@
 
 #include "internal.cuh"
 #include "mlp.cuh"
+#include "tcgen05.cuh"
+#include "tma.cuh"
 
 namespace swense {
 namespace {
@@ -1342,140 +1344,140 @@ __global__ void __launch_bounds__(BOX_THREADS, 5) k_interp_global_batch(const Ba
 // ---------------------------------------------------------------------------------------------
 // Fused learned gather: the plain Lagrange gather, the network's inputs and its three layers in
 // one kernel, per 1024-point chunk. The chunk's stencils come from the staged box (as in
-// k_interp_box) when it fits, else from per-point stencil arrays gathered from global memory
-// (64 points at a time) in the same shared memory. Per sub-batch of points:
+// k_interp_box) when it fits, else from per-point stencil arrays gathered from global memory in the
+// same shared memory. Each of the block's two warpgroups takes half of the chunk, some points at a time:
 //   A (one thread per point): cell, Lagrange weights, offsets, eta, stencil base -> LPoint;
-//   B (warps, m16n8k16): rows (point, field), 16 rows = 4 points x 4 fields per tile; each lane
-//     reads its fragment's stencil values, the quad reduces the row's Lagrange value and
-//     max |value|, the normalised values (hi + lo BF16) feed layers 1-3, and the lane holding
-//     column f of row (point, f) writes lagrange + s_f * out_scale * y[f];
+//   B (one thread per row = point and field, 32 points at a time): stencil values, Lagrange value and
+//     max |value|; the normalised values (hi + lo BF16) go to tensor memory as the A operand of layer 1,
+//     its accumulators come back through GELU as the A operand of layer 2, and layer 3's one output of
+//     the row is an FP32 dot product; lagrange + s_f * out_scale * y[f] is the result;
 //   C (one thread per point): Bernoulli, NaN outside the levels, stores.
-// Bound by instruction issue (50 % of cycles) and the warp MMAs (45 %), which hardly overlap; with weight
-// fragments loaded four at a time (ldmatrix), GELU of two values in nine instructions and the offsets in
-// half a step, 8.2 M mesh points take 4.45 ms (5.79 before).
-struct LPoint {
-  int base;                 // staged node index of stencil node (x 0, y 0, level 0)
+// Bound by instruction issue (51 % of cycles, 17 % of the tensor cores'): 55 % of it GELU and the splits.
+// A row per thread and the fifth-generation tensor cores leave about 850 issue slots per 16 rows where
+// fragments of warp MMAs took 1260 and another 1140 cycles of the MMA pipe that did not overlap with them:
+// 8.2 M mesh points 4.45 -> 3.00 ms. Two warpgroups a block and two blocks an SM fill one another's waits.
+// Offsets and biases are a k-step of their own: a row's inputs 64..79 are the hi halves of dx, dy, dz,
+// their lo halves and three ones, against the offsets' weights twice and the bias in three BF16 parts
+// (its 24 bits); layer 2 repeats it with weights of zero.
+struct alignas(16) LPoint {
   float w[12];              // wx[4], wy[4], wz[4]; the corrected fields overwrite w[0..3]
   float off[3];             // dx, dy in the cell; dz in the stencil's middle level interval
+  int base;                 // staged node index of stencil node (x 0, y 0, level 0)
   float eta, z;
   int inside, pad_;
 };
-static_assert(sizeof(LPoint) == 80, "LPoint layout");
+static_assert(sizeof(LPoint) == 80, "eight neighbouring records start in eight different groups of banks");
 
 using mlpnet::PackedFwd;
 
-// Shared-memory copy of the forward weights with padded rows: the B-fragment loads of a warp
-// (row 8 nt + g, word 8 kk + q) then fall into 32 different banks (an unpadded 64-wide row
-// maps all eight g to one bank).
-constexpr int W1LD = mlpnet::KIN + 8, W2LD = mlpnet::NH + 8;
-struct WeightsSmem {
-  __nv_bfloat16 w1[mlpnet::NH][W1LD];
-  __nv_bfloat16 w2[mlpnet::NH][W2LD];
-  __nv_bfloat16 w3[mlpnet::NO][W2LD];
-  float b1[mlpnet::NH], b2[mlpnet::NH], b3[mlpnet::NO];
-  float out_scale, pad_[3];
+constexpr int LRN_WG = BOX_THREADS / 128;              // warpgroups
+constexpr int LRN_SB = 64, LRN_SB_PP = 32;             // points per step of a warpgroup: staged box, per-point stencils
+constexpr int LRN_K = 16 * 5, LRN_LBO = mlpnet::NH / 8 * 128;   // bytes between neighbouring core matrices along K
+constexpr uint32_t LRN_COLS = 128;                     // tensor-memory columns a warpgroup: A hi 0, A lo 32, D 64
+constexpr uint32_t LRN_IDESC = tc::idesc_bf16_f32(128, mlpnet::NH);
+static_assert(LRN_WG * LRN_SB_PP * 64 <= BOX_NODES, "per-point stencils fit the box area");
+static_assert(mlpnet::KIN == LRN_K && mlpnet::NIN == 67 && mlpnet::NH == 64 && mlpnet::NOUT == 4, "the layout above");
+
+struct LearnedSmem {
+  unsigned char w1[LRN_K / 8 * LRN_LBO], w2[LRN_K / 8 * LRN_LBO];   // K-major core matrices
+  unsigned char xo[LRN_WG + 1][128 * 16];              // inputs 64..71 of a warpgroup's rows; last: 72..79 of any
+  float4 w3[mlpnet::NH / 4][mlpnet::NOUT];
+  float b3[mlpnet::NOUT];
+  float out_scale;
+  uint32_t tmem;
+  alignas(8) uint64_t bar[LRN_WG];
 };
-
-constexpr int LRN_SB = 128;                            // points per sub-batch (box mode)
-constexpr int LRN_SB_PP = 64;                          // points per sub-batch (per-point stencils)
-static_assert(LRN_SB_PP * 64 <= BOX_NODES, "per-point stencils fit the box area");
 constexpr size_t LRN_SMEM = size_t(BOX_NODES) * sizeof(float4) + size_t(BOX_COLS) * sizeof(float) +
-                            size_t(LRN_SB) * sizeof(LPoint) + sizeof(WeightsSmem);
+                            size_t(LRN_WG) * LRN_SB * sizeof(LPoint) + sizeof(LearnedSmem);
+static_assert(2 * (LRN_SMEM + 1024) <= 228 * 1024, "two blocks an SM");
 
-// Phase B for `ntile` 16-row tiles of this warp. Node (x k, y b, level q) of point j is
-// nodes[rec[j].base + q * SZ + b * SY + k].
-__device__ __forceinline__ void learned_tiles(const float4* nodes, int SY, int SZ, LPoint* rec,
-                                              const WeightsSmem& W, int tile0, int ntile, int npts) {
-  using namespace mlpnet;
-  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
-  const int f = g & 3;                                 // field of rows g and g + 8
-  const float* nf = reinterpret_cast<const float*>(nodes) + f;
-  for (int t = tile0; t < tile0 + ntile; ++t) {
-    const int j0 = 4 * t + (g >> 2), j1 = j0 + 2;      // points of rows g and g + 8
-    if (4 * t >= npts) break;                          // uniform over the warp
-    float lag[2], sc[2];
-    unsigned xh[4][4], xl[4][4], xo[2];
-    float v[2][4][4];
+// Set when a wait for the tensor cores gives up; the host reads and clears it with swense_async_status.
+__device__ int g_learned_timeout;
+
+__device__ __forceinline__ void wg_sync(int wg) { asm volatile("bar.sync %0, 128;" ::"r"(1 + wg) : "memory"); }
+
+// Eight inputs (k-chunk kc) of output n of a layer with K plain inputs and 16 more for offsets and bias.
+__device__ __forceinline__ uint4 learned_weights(const __nv_bfloat16* w, const float* bias, bool offsets, int ldw, int n, int kc) {
+  if (kc < 8) return __ldg(reinterpret_cast<const uint4*>(w + n * ldw) + kc);
+  const float b = __ldg(&bias[n]);
+  unsigned h, l, l2, unused;
+  bf2_split(b, 0.f, h, l);
+  bf2_split(b - __uint_as_float(h << 16) - __uint_as_float(l << 16), 0.f, l2, unused);
+  if (kc == 9) return make_uint4(l2 & 0xffffu, 0u, 0u, 0u);
+  uint4 v = make_uint4(0u, 0u, 0u, 0u);
+  if (offsets) v = mlpnet::repeat_offsets(__ldg(reinterpret_cast<const uint4*>(w + n * ldw) + kc));
+  v.w = (h & 0xffffu) | (l << 16);
+  return v;
+}
+
+// One layer of a warpgroup's 128 rows, by one thread: D = [A hi + A lo | offsets] x W.
+__device__ __forceinline__ void learned_mma(uint32_t ta, const unsigned char* w, const unsigned char* xo, uint32_t xo_lbo,
+                                            uint64_t* bar) {
+  tc::fence_after();
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const LPoint& P = rec[min(h ? j1 : j0, npts - 1)];
-      const int base = P.base;
-      float lg = 0.f, mx = 0.f;
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int b = (q >> 1) + 2 * (e >> 1), k = 2 * (q & 1) + (e & 1);
-          const float val = nf[4 * (base + kk * SZ + b * SY + k)];
-          v[h][kk][e] = val;
-          lg = fmaf(P.w[8 + kk] * P.w[4 + b] * P.w[k], val, lg);
-          mx = fmaxf(mx, fabsf(val));
-        }
-      }
-      lg += __shfl_xor_sync(0xffffffffu, lg, 1);
-      lg += __shfl_xor_sync(0xffffffffu, lg, 2);
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-      lag[h] = lg;
-      sc[h] = mx + 1e-30f;
-    }
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float inv = 1.f / sc[h];
-        const float2 iv = make_float2(inv, inv);
-        bf2_split(pmul(make_float2(v[h][kk][0], v[h][kk][1]), iv), xh[kk][h], xl[kk][h]);
-        bf2_split(pmul(make_float2(v[h][kk][2], v[h][kk][3]), iv), xh[kk][2 + h], xl[kk][2 + h]);
-      }
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const LPoint& P = rec[min(h ? j1 : j0, npts - 1)];
-      xo[h] = offsets_a(P.off[0], P.off[1], P.off[2], q);
-    }
-    float o[4];
-    infer(o, xh, xl, xo, W, W1LD, W2LD, lane);
-    __syncwarp();                                      // every lane has read its records
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int jh = h ? j1 : j0;
-      const float yv = (f & 1) ? o[2 * h + 1] : o[2 * h];   // a select, not a local array
-      if ((f >> 1) == q && jh < npts) rec[jh].w[f] = fmaf(sc[h] * W.out_scale, yv, lag[h]);
-    }
-    __syncwarp();
+  for (int ks = 0; ks < 4; ++ks) {
+    const uint64_t wd = tc::smem_desc(w + 2 * ks * LRN_LBO, LRN_LBO, 128u);
+    tc::mma_ts(ta + 64u, ta + 8u * ks, wd, LRN_IDESC, ks > 0 ? 1u : 0u);
+    tc::mma_ts(ta + 64u, ta + 32u + 8u * ks, wd, LRN_IDESC, 1u);
   }
+  tc::mma_ss(ta + 64u, tc::smem_desc(xo, xo_lbo, 128u), tc::smem_desc(w + 8 * LRN_LBO, LRN_LBO, 128u), LRN_IDESC, 1u);
+  tc::commit(bar);
+}
+
+// Accumulators 32 hf .. 32 hf + 31 of this thread's row after GELU, in pairs.
+__device__ __forceinline__ void learned_activations(uint32_t lanes, int hf, float2 (&g)[16]) {
+  uint32_t r0[16], r1[16];
+  tc::ld_x16(lanes + 64u + 32u * hf, r0);
+  tc::ld_x16(lanes + 64u + 32u * hf + 16u, r1);
+  tc::wait_ld();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    g[i] = mlpnet::gelu_fast2(make_float2(__uint_as_float(r0[2 * i]), __uint_as_float(r0[2 * i + 1])));
+    g[8 + i] = mlpnet::gelu_fast2(make_float2(__uint_as_float(r1[2 * i]), __uint_as_float(r1[2 * i + 1])));
+  }
+}
+
+// 32 values of a row (pairs) as hi and lo BF16 halves into the A operand's words 16 hf .. 16 hf + 15.
+__device__ __forceinline__ void learned_store_a(uint32_t lanes, int hf, const float2 (&g)[16]) {
+  uint32_t hi[16], lo[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) bf2_split(g[i], hi[i], lo[i]);
+  tc::st_x16(lanes + 16u * hf, hi);
+  tc::st_x16(lanes + 32u + 16u * hf, lo);
 }
 
 __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_constant__ InterpArgs a, const __grid_constant__ Levels L,
                                                                     const int4* __restrict__ plan,
                                                                     const PackedFwd* __restrict__ Wg) {
+  using namespace mlpnet;
   extern __shared__ float4 sbox[];
   float* seta = reinterpret_cast<float*>(sbox + BOX_NODES);
-  LPoint* rec = reinterpret_cast<LPoint*>(seta + BOX_COLS);
-  WeightsSmem& W = *reinterpret_cast<WeightsSmem*>(rec + LRN_SB);
-  __shared__ LevelTables zs;
-  fill_level_tables(zs, L);
-  {
-    // rows re-strided into the padded layout, 16 bytes (8 bf16) at a time
-    using namespace mlpnet;
-    const uint4* g1 = reinterpret_cast<const uint4*>(&Wg->w1[0][0]);
-    const uint4* g2 = reinterpret_cast<const uint4*>(&Wg->w2[0][0]);
-    const uint4* g3 = reinterpret_cast<const uint4*>(&Wg->w3[0][0]);
-    for (int i = threadIdx.x; i < NH * KIN / 8; i += blockDim.x) {
-      const uint4 w = __ldg(&g1[i]);
-      *reinterpret_cast<uint4*>(&W.w1[i / (KIN / 8)][8 * (i % (KIN / 8))]) = i % (KIN / 8) == 8 ? repeat_offsets(w) : w;
-    }
-    for (int i = threadIdx.x; i < NH * NH / 8; i += blockDim.x)
-      *reinterpret_cast<uint4*>(&W.w2[i / (NH / 8)][8 * (i % (NH / 8))]) = __ldg(&g2[i]);
-    for (int i = threadIdx.x; i < NO * NH / 8; i += blockDim.x)
-      *reinterpret_cast<uint4*>(&W.w3[i / (NH / 8)][8 * (i % (NH / 8))]) = __ldg(&g3[i]);
-    for (int i = threadIdx.x; i < NH; i += blockDim.x) {
-      W.b1[i] = __ldg(&Wg->b1[i]);
-      W.b2[i] = __ldg(&Wg->b2[i]);
-    }
-    if (threadIdx.x < NO) W.b3[threadIdx.x] = __ldg(&Wg->b3[threadIdx.x]);
-    if (threadIdx.x == 0) W.out_scale = __ldg(&Wg->out_scale);
+  LPoint* recs = reinterpret_cast<LPoint*>(seta + BOX_COLS);
+  LearnedSmem& W = *reinterpret_cast<LearnedSmem*>(recs + LRN_WG * LRN_SB);
+  const LevelTables& zs = *level_tables(L);
+  for (int i = threadIdx.x; i < NH * (LRN_K / 8); i += blockDim.x) {
+    const int n = i / (LRN_K / 8), kc = i % (LRN_K / 8), o = kc * LRN_LBO + (n / 8) * 128 + (n % 8) * 16;
+    *reinterpret_cast<uint4*>(W.w1 + o) = learned_weights(&Wg->w1[0][0], Wg->b1, true, KIN, n, kc);
+    *reinterpret_cast<uint4*>(W.w2 + o) = learned_weights(&Wg->w2[0][0], Wg->b2, false, NH, n, kc);
+  }
+  if (threadIdx.x < 128)                               // input 72 is 1, 73..79 are 0
+    *reinterpret_cast<uint4*>(W.xo[LRN_WG] + 16 * threadIdx.x) = make_uint4(0x3f80u, 0u, 0u, 0u);
+  if (threadIdx.x < NH) {
+    const int k4 = threadIdx.x / NOUT, f = threadIdx.x % NOUT;
+    const uint2 w = __ldg(reinterpret_cast<const uint2*>(&Wg->w3[f][4 * k4]));
+    W.w3[k4][f] = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                              __uint_as_float(w.y & 0xffff0000u));
+  }
+  if (threadIdx.x < NOUT) W.b3[threadIdx.x] = __ldg(&Wg->b3[threadIdx.x]);
+  if (threadIdx.x == 0) {
+    W.out_scale = __ldg(&Wg->out_scale);
+    for (int i = 0; i < LRN_WG; ++i) mbar_init(&W.bar[i], 1);
+    fence_mbar_init();
+  }
+  __syncwarp();
+  if (threadIdx.x < 32) {
+    tc::alloc(&W.tmem, LRN_WG * LRN_COLS);
+    tc::relinquish();
   }
   const int64_t p0 = int64_t(blockIdx.x) * BOX_PTS;
   const int4 pl = plan[blockIdx.x];
@@ -1486,9 +1488,7 @@ __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_
   int l0 = bp.l0, bz = bp.bz;
   bool box3d = bp.box3d;
   if (bp.two) {
-    // a chunk across two layers: the box spans the level windows of its first and last
-    // point's z (the level tables are complete after this barrier)
-    __syncthreads();
+    // a chunk across two layers: the box spans the level windows of its first and last point's z
     PointCell ca, cb;
     point_level(a, zs, __ldg(&a.pts[3 * p0 + 2]), ca);
     point_level(a, zs, __ldg(&a.pts[3 * ((p0 + BOX_PTS < a.np ? p0 + BOX_PTS : a.np) - 1) + 2]), cb);
@@ -1500,52 +1500,80 @@ __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_
   const int x0 = bp.x0, y0 = bp.y0;
   const size_t plane = size_t(a.Nyr) * a.Nxr;
   if (boxed) stage_box(a, x0, y0, l0, bx, by, bz, sbx, zst, sbox, seta);
+  fence_proxy_async();                                 // the weights, read by the tensor cores
+  tc::fence_before();
   __syncthreads();
+  tc::fence_after();
+  const int wg = threadIdx.x >> 7, t = threadIdx.x & 127, f = t & 3;
+  const uint32_t ta = W.tmem + uint32_t(wg) * LRN_COLS, lanes = ta + (uint32_t(t & 96) << 16);
+  unsigned char* xo = W.xo[wg];
+  const uint32_t xo_lbo = uint32_t(LRN_WG - wg) * uint32_t(sizeof(W.xo[0]));
+  uint64_t* bar = &W.bar[wg];
+  LPoint* rec = recs + wg * LRN_SB;
+  float4* own = sbox + wg * (LRN_SB_PP * 64);          // the warpgroup's per-point stencils
+  const float* nf = reinterpret_cast<const float*>(boxed ? sbox : own) + f;
+  const int SY = boxed ? sbx : 4, SZ = boxed ? zst : 16;
   const int SB = boxed ? LRN_SB : LRN_SB_PP;
-  const int warp = threadIdx.x >> 5;
-  for (int s0 = 0; s0 < BOX_PTS; s0 += SB) {
-    const int npts = int(a.np - (p0 + s0) < int64_t(SB) ? a.np - (p0 + s0) : int64_t(SB));
-    if (npts <= 0) break;                              // uniform over the block
+  const int64_t q0 = p0 + int64_t(wg) * (BOX_PTS / LRN_WG);
+  unsigned ph = 0;
+  bool bad = false;
+  // every thread of the warpgroup has its share of the operands in place -> the accumulators are ready
+  auto run_layer = [&](const unsigned char* w) {
+    tc::wait_st();
+    fence_proxy_async();
+    tc::fence_before();
+    wg_sync(wg);
+    if (t == 0 && !bad) learned_mma(ta, w, xo, xo_lbo, bar);
+    __syncwarp();
+    if (!bad) bad = !mbar_wait(bar, ph);
+    ph ^= 1u;
+    __syncwarp();
+    tc::fence_after();
+  };
+  for (int s0 = 0; s0 < BOX_PTS / LRN_WG; s0 += SB) {
+    const int npts = int(a.np - (q0 + s0) < int64_t(SB) ? a.np - (q0 + s0) : int64_t(SB));
+    if (npts <= 0) break;                              // uniform over the warpgroup
     // ---- A
+    auto record = [&](LPoint& P, const PointCell& c, float px, float py, float pz, int base, float e) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        P.w[k] = c.wx[k];
+        P.w[4 + k] = c.wy[k];
+        P.w[8 + k] = c.wz[k];
+      }
+      float fx, fy;
+      int ixx, iyy;
+      locate(px, a.sx_hi, a.sx_lo, a.Nxr, ixx, fx);
+      locate(py, a.sy_hi, a.sy_lo, a.Nyr, iyy, fy);
+      const float z1 = zs.z[c.j0 + 1], z2 = zs.z[c.j0 + 2];
+      P.off[0] = fx;
+      P.off[1] = fy;
+      P.off[2] = (pz - z1) / (z2 - z1);
+      P.base = base;
+      P.eta = e;
+      P.z = pz;
+      P.inside = c.inside;
+    };
     if (boxed) {
-      const int t = threadIdx.x;
       if (t < npts) {
-        const int64_t i = p0 + s0 + t;
+        const int64_t i = q0 + s0 + t;
         const float px = __ldg(&a.pts[3 * i]), py = __ldg(&a.pts[3 * i + 1]), pz = __ldg(&a.pts[3 * i + 2]);
         const PointCell c = point_cell(a, zs, px, py, pz);
         const int lx = min(max((c.ix - 1 - x0) & (a.Nxr - 1), 0), bx - 4);
         const int ly = min(max((c.iy - 1 - y0) & (a.Nyr - 1), 0), by - 4);
         const int lz = min(max(c.j0 - l0, 0), bz - 4);
-        LPoint& P = rec[t];
-        P.base = lz * zst + ly * sbx + lx;
         float e = 0.f;
 #pragma unroll
         for (int b = 0; b < 4; ++b)
 #pragma unroll
           for (int k = 0; k < 4; ++k) e = fmaf(c.wy[b] * c.wx[k], seta[(ly + b) * sbx + lx + k], e);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          P.w[k] = c.wx[k];
-          P.w[4 + k] = c.wy[k];
-          P.w[8 + k] = c.wz[k];
-        }
-        float fx, fy;
-        int ixx, iyy;
-        locate(px, a.sx_hi, a.sx_lo, a.Nxr, ixx, fx);
-        locate(py, a.sy_hi, a.sy_lo, a.Nyr, iyy, fy);
-        const float z1 = zs.z[c.j0 + 1], z2 = zs.z[c.j0 + 2];
-        P.off[0] = fx;
-        P.off[1] = fy;
-        P.off[2] = (pz - z1) / (z2 - z1);
-        P.eta = e;
-        P.z = pz;
-        P.inside = c.inside;
+        record(rec[t], c, px, py, pz, lz * zst + ly * sbx + lx, e);
       }
     } else {
       // per-point stencils: four threads per point, each blends 16 of its 64 nodes
-      const int j = threadIdx.x >> 2, qq = threadIdx.x & 3;
+      const int j = t >> 2, qq = t & 3;
       if (j < npts) {
-        const int64_t i = p0 + s0 + j;
+        const int64_t i = q0 + s0 + j;
         const float px = __ldg(&a.pts[3 * i]), py = __ldg(&a.pts[3 * i + 1]), pz = __ldg(&a.pts[3 * i + 2]);
         const PointCell c = point_cell(a, zs, px, py, pz);
         const size_t tl_stride = size_t(a.nz) * plane;
@@ -1563,11 +1591,9 @@ __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_
             v.z = fmaf(w, gv.z, v.z);
             v.w = fmaf(w, gv.w, v.w);
           }
-          sbox[64 * j + node] = v;
+          own[64 * j + node] = v;
         }
         if (qq == 0) {
-          LPoint& P = rec[j];
-          P.base = 64 * j;
           float e = 0.f;
           for (int tl = 0; tl < a.n_tl; ++tl)
 #pragma unroll
@@ -1577,40 +1603,95 @@ __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_
                 e = fmaf(a.wt[tl] * c.wy[b] * c.wx[k],
                          __ldg(&a.eta[size_t(tl) * plane + size_t((c.iy - 1 + b) & (a.Nyr - 1)) * a.Nxr +
                                       ((c.ix - 1 + k) & (a.Nxr - 1))]), e);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            P.w[k] = c.wx[k];
-            P.w[4 + k] = c.wy[k];
-            P.w[8 + k] = c.wz[k];
-          }
-          float fx, fy;
-          int ixx, iyy;
-          locate(px, a.sx_hi, a.sx_lo, a.Nxr, ixx, fx);
-          locate(py, a.sy_hi, a.sy_lo, a.Nyr, iyy, fy);
-          const float z1 = zs.z[c.j0 + 1], z2 = zs.z[c.j0 + 2];
-          P.off[0] = fx;
-          P.off[1] = fy;
-          P.off[2] = (pz - z1) / (z2 - z1);
-          P.eta = e;
-          P.z = pz;
-          P.inside = c.inside;
+          record(rec[j], c, px, py, pz, 64 * j, e);
         }
       }
     }
-    __syncthreads();
-    // ---- B: SB points = SB / 4 tiles, spread over the warps
-    const int ntiles = (npts + 3) / 4, per = (SB / 4 + (blockDim.x >> 5) - 1) / (blockDim.x >> 5);
-    if (boxed) learned_tiles(sbox, sbx, zst, rec, W, warp * per, min(per, max(ntiles - warp * per, 0)), npts);
-    else learned_tiles(sbox, 4, 16, rec, W, warp * per, min(per, max(ntiles - warp * per, 0)), npts);
-    __syncthreads();
-    // ---- C
-    if (threadIdx.x < npts) {
-      const LPoint& P = rec[threadIdx.x];
-      store_point(a, p0 + s0 + threadIdx.x, make_float4(P.w[0], P.w[1], P.w[2], P.w[3]), P.eta, P.z,
-                  P.inside != 0);
+    wg_sync(wg);
+    // ---- B (rows past the last point repeat it and are not kept)
+    for (int g0 = 0; g0 < npts; g0 += 32) {
+      const int j = g0 + (t >> 2);
+      float lag = 0.f, mx = 0.f;
+      {
+        const LPoint& P = rec[min(j, npts - 1)];
+        const float4 w4x = *reinterpret_cast<const float4*>(&P.w[0]), w4y = *reinterpret_cast<const float4*>(&P.w[4]),
+                     w4z = *reinterpret_cast<const float4*>(&P.w[8]), o4 = *reinterpret_cast<const float4*>(&P.off[0]);
+        const float wx[4] = {w4x.x, w4x.y, w4x.z, w4x.w}, wy[4] = {w4y.x, w4y.y, w4y.z, w4y.w},
+                    wz[4] = {w4z.x, w4z.y, w4z.z, w4z.w};
+        const float* src = nf + 4 * __float_as_int(o4.w);
+        float2 v[2][16];
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+          float sy = 0.f;
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            float x[4], sx = 0.f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              x[k] = src[4 * (kk * SZ + b * SY + k)];
+              sx = fmaf(wx[k], x[k], sx);
+              mx = fmaxf(mx, fabsf(x[k]));
+            }
+            sy = fmaf(wy[b], sx, sy);
+            v[kk >> 1][8 * (kk & 1) + 2 * b] = make_float2(x[0], x[1]);
+            v[kk >> 1][8 * (kk & 1) + 2 * b + 1] = make_float2(x[2], x[3]);
+          }
+          lag = fmaf(wz[kk], sy, lag);
+        }
+        mx += 1e-30f;
+        const float inv = 1.f / mx;
+        __syncwarp();
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[hf][i] = pmul(v[hf][i], make_float2(inv, inv));
+          learned_store_a(lanes, hf, v[hf]);
+        }
+        unsigned h, l, hz, lz;
+        bf2_split(o4.x, o4.y, h, l);
+        bf2_split(o4.z, 0.f, hz, lz);
+        *reinterpret_cast<uint4*>(xo + 16 * t) =
+            make_uint4(h, (hz & 0xffffu) | (l << 16), (l >> 16) | (lz << 16), 0x3f803f80u);
+      }
+      run_layer(W.w1);
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        float2 g[16];
+        learned_activations(lanes, hf, g);
+        learned_store_a(lanes, hf, g);
+      }
+      run_layer(W.w2);
+      float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        float2 g[16];
+        learned_activations(lanes, hf, g);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float4 w = W.w3[8 * hf + i][f];
+          acc = pfma(g[2 * i], make_float2(w.x, w.y), acc);
+          acc = pfma(g[2 * i + 1], make_float2(w.z, w.w), acc);
+        }
+      }
+      const float y = acc.x + acc.y + W.b3[f];
+      if (j < npts) rec[j].w[f] = bad ? __int_as_float(0x7fc00000) : fmaf(mx * W.out_scale, y, lag);
     }
-    __syncthreads();
+    wg_sync(wg);
+    // ---- C
+    if (t < npts) {
+      const LPoint& P = rec[t];
+      store_point(a, q0 + s0 + t, make_float4(P.w[0], P.w[1], P.w[2], P.w[3]), P.eta, P.z, P.inside != 0);
+    }
+    wg_sync(wg);
   }
+  if (bad) {
+    atomicExch(&g_learned_timeout, 1);
+    mbar_wait(bar, ph ^ 1u);                           // the MMAs may still be in flight
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  if (threadIdx.x < 32) tc::dealloc(W.tmem, LRN_WG * LRN_COLS);
 }
 
 void split(double v, float& hi, float& lo) {
@@ -1812,6 +1893,21 @@ extern "C" int swense_mlp_features(const swense_grid* g, double t, const float* 
   count_launches(1);
   return SWENSE_OK;
 }
+
+namespace swense {
+
+int learned_async_flag(bool reset, int* was_set) {
+  int v = 0;
+  SWENSE_CUDA_TRY(cudaMemcpyFromSymbol(&v, g_learned_timeout, sizeof(int)));
+  if (reset && v) {
+    const int zero = 0;
+    SWENSE_CUDA_TRY(cudaMemcpyToSymbol(g_learned_timeout, &zero, sizeof(int)));
+  }
+  *was_set = v;
+  return SWENSE_OK;
+}
+
+}  // namespace swense
 
 extern "C" int swense_interp_learned(const swense_grid* g, double t, const float* pts, int64_t np,
                                      float* eta, float* u, float* v, float* w, float* p,

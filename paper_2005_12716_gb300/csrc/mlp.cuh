@@ -190,8 +190,7 @@ __device__ __forceinline__ void activate(const float (&z)[2][4], unsigned (&hi)[
 }
 
 // The three layers of 16 rows (xo: offsets_a of rows g and g + 8). The MMAs of the next 16 outputs stand
-// between a block's own and its activation, which hides part of either (layer by layer, with two padded
-// steps for the offsets and one GELU at a time, the learned gather of 8.2 M points took 4.75 ms, so 4.45).
+// between a block's own and its activation, which hides part of either.
 template <class Weights>
 __device__ __forceinline__ void infer(float (&o)[4], const unsigned (&xh)[4][4], const unsigned (&xl)[4][4],
                                       const unsigned (&xo)[2], const Weights& W, int ld1, int ld2, int lane) {
