@@ -172,7 +172,8 @@ int swense_fields_on_grid_noalloc(const swense_modes* modes, int32_t n_tl, const
 /*
  * swense_autotune_grid — choose the launch shape of swense_fields_on_grid for this grid shape
  * (the transform path: the wide-radix transform pair with 1, 2 or 4 levels per column-transform
- * block, or the shared-memory kernels; the level-chunk size among 16, 32, 64, 96, 128, 256 MB; and
+ * block, or the shared-memory kernels; the level-chunk size among 16, 32, 64, 96, 128 and 256 MB, the
+ * last of which stands for the default's chunks of up to 512 MB; and
  * the row pass's form) by
  * timing each candidate five times on `stream` (best of five, each from a cold L2: the
  * workspace, grown to at least 256 MB, is overwritten before each repetition); the choice is
@@ -198,7 +199,7 @@ int swense_autotune_grid(const swense_modes* modes, int32_t n_tl, const double* 
  * (nx, ny, pad_n, nz), e.g. a choice that swense_autotune_grid returned in an earlier process.
  * lpc: -1 (forget any choice: untuned defaults again), 0 (shared-memory path), 1, 2 or 4 levels
  * per column block;
- * chunk_bytes in [1 MiB, 1 GiB] (level chunk); row_variant 0..5, or 16 more (see
+ * chunk_bytes in [1 MiB, 1 GiB] (level chunk; 256 MiB: the default's, up to 512 MiB); row_variant 0..5, or 16 more (see
  * swense_autotune_grid). Results do not depend on the choice beyond FP32 rounding. No
  * counterpart in the paper. Errors: SWENSE_ERR_ARG for values outside those sets.
  */
@@ -308,8 +309,9 @@ typedef struct swense_instance {
  * and then every instance's gather (as swense_interp, or swense_interp_permuted when perm is
  * set). The reconstructions run concurrently on four library streams forked from `stream`
  * (largest instance first, round robin, each stream in its own part of the workspace); after
- * they are joined back, one launch plans the point chunks of all instances and one persistent
- * launch gathers them, its CTAs taking chunks from a device queue. Fork and join are events,
+ * they are joined back, one launch plans the point chunks of all instances, one persistent launch
+ * gathers those whose stencils fit a staged tile, its CTAs taking chunks from a device queue, and
+ * one launch gathers the others. Fork and join are events,
  * so one call can be captured as a single CUDA graph and replayed as one launch. The first call
  * with a given set of instances must be made outside any capture: it sizes the workspace and
  * uploads the gather tables (arguments and level tables of every instance; a captured call

@@ -324,9 +324,11 @@ __global__ void __launch_bounds__(256) k_form_modes(FormArgs a, PropTimes T) {
 
 constexpr int kThreads = 256;
 constexpr size_t kSmemBudget = 64 * 1024;
-// Level chunks of 256 MB: a pass then has whole waves of blocks (2048 x 1024 modes: 9.5 ms for 256
-// levels, against 10.3 at 64 MB and 11.8 at 32 MB), which outweighs an intermediate that stays in L2.
-constexpr size_t kChunkBytes = size_t(256) << 20;
+// Level chunks of at most 512 MB, of equal size: each pass pays its first and last wave of blocks (about
+// 20 us) once a chunk, which outweighs an intermediate that stays in L2 (2048 x 1024 modes, 256 levels:
+// 7.44 ms, 7.89 at 256 MB, 9.07 at 64 MB; 512 x 256 modes, 128 levels in one chunk instead of one and a
+// rest of two slots: 13 us less). The largest size a tuned choice names, 256 MB, stands for it too.
+constexpr size_t kChunkBytes = size_t(512) << 20, kChunkNominal = size_t(256) << 20;
 constexpr int kColLevels = 1;   // levels per column-transform CTA
 
 int set_smem(const void* fn, size_t bytes) {
@@ -943,14 +945,20 @@ int grid_slots(const GridPlan& p, const Shape& s) {
 }
 
 int chunk_slots(const GridPlan& p, const Shape& s, size_t bytes) {
+  if (bytes == kChunkNominal) bytes = kChunkBytes;
   return int(std::max<size_t>(1, std::min<size_t>(size_t(grid_slots(p, s)), bytes / p.per_level)));
+}
+// The same number of chunks, of equal size: no short one at the end.
+int even_chunk(const GridPlan& p, const Shape& s, int chunk) {
+  const int n = grid_slots(p, s), k = (n + chunk - 1) / chunk;
+  return (n + k - 1) / k;
 }
 Shape grid_shape(const GridPlan& p) {
   const Tune tn = tuned(p.nx, p.ny, p.pad, p.nz);
   Shape s;
   s.lpc = tn.lpc >= 0 ? tn.lpc : (pair_path(p.ny, p.Nxr, p.Nyr) ? kColLevels : 0);
   s.rowv = tn.lpc >= 0 ? tn.rowv : 0;
-  s.chunk = p.ny > 1 ? chunk_slots(p, s, tn.chunk_bytes) : 0;
+  s.chunk = p.ny > 1 ? even_chunk(p, s, chunk_slots(p, s, tn.chunk_bytes)) : 0;
   return s;
 }
 
@@ -965,6 +973,17 @@ size_t modes_bytes(const GridPlan& p, bool pair) {
 size_t scratch_bytes(const GridPlan& p, int chunk, int nbuf, bool pair) {
   const size_t g_bytes = p.ny > 1 ? size_t(chunk) * p.per_level : 0;
   return align256(modes_bytes(p, pair)) + align256(p.geta_bytes) + size_t(nbuf) * align256(g_bytes);
+}
+
+// Workspace of a request (`extra` bytes more); where that much cannot be had, of smaller chunks.
+int shape_workspace(const GridPlan& p, Shape* s, int nbuf, size_t extra, cudaStream_t stream, void** ws) {
+  for (;;) {
+    const size_t bytes = scratch_bytes(p, s->chunk, nbuf, runs_pair(p, s->lpc)) + extra;
+    if (!bytes) return SWENSE_OK;
+    const int st = workspace(bytes, stream, ws);
+    if (st != SWENSE_ERR_OOM || s->chunk <= 1) return st;
+    s->chunk = (s->chunk + 1) / 2;
+  }
 }
 
 // Library-internal second stream and events (per device) for the two-stream transform
@@ -1329,8 +1348,7 @@ int fields_on_grid_shifted(const GridPlan& p, const swense_modes* md, const doub
   sp.Nyr = p.ny > 1 ? int64_t(p2) * p.ny : 1;
   sp.per_level = size_t(4) * sp.Nyr * trans_ld(sp.Mh) * sizeof(float2);
   sp.geta_bytes = p.ny > 1 ? size_t(sp.Nyr) * sp.Mh * sizeof(float2) : 0;
-  const Shape shape = grid_shape(sp);                         // one stream for the sub-grids
-  const size_t scratch = align256(scratch_bytes(sp, shape.chunk, 1, runs_pair(sp, shape.lpc)));
+  Shape shape = grid_shape(sp);                               // one stream for the sub-grids
   const int64_t sub_nodes = int64_t(p.n_tl) * p.nz * sp.Nyr * sp.Nxr;
   const int64_t sub_eta = int64_t(p.n_tl) * sp.Nyr * sp.Nxr;
   const int64_t nmodes = int64_t(md->n_snap) * p.ny * p.nxh1;
@@ -1338,8 +1356,9 @@ int fields_on_grid_shifted(const GridPlan& p, const swense_modes* md, const doub
   const size_t b_eta = align256(size_t(sub_eta) * sizeof(float));
   const size_t b_modes = align256(size_t(nmodes) * sizeof(float2));
   void* ws = nullptr;
-  int st = workspace(scratch + b_nodes + b_eta + 3 * b_modes, stream, &ws);
+  int st = shape_workspace(sp, &shape, 1, b_nodes + b_eta + 3 * b_modes, stream, &ws);
   if (st) return st;
+  const size_t scratch = align256(scratch_bytes(sp, shape.chunk, 1, runs_pair(sp, shape.lpc)));
   char* base = static_cast<char*>(ws);
   float4* snodes = reinterpret_cast<float4*>(base + scratch);
   float* seta = reinterpret_cast<float*>(base + scratch + b_nodes);
@@ -1385,13 +1404,10 @@ extern "C" int swense_fields_on_grid(const swense_modes* md, int32_t n_tl, const
   int st = plan_grid(md, n_tl, t, desc, nodes, eta, &p);
   if (st) return st;
   if (!is_pow2(p.pad)) return fields_on_grid_shifted(p, md, t, nodes, eta, stream);
-  const Shape shape = grid_shape(p);
+  Shape shape = grid_shape(p);
   void* ws = nullptr;
-  const size_t ws_bytes = scratch_bytes(p, shape.chunk, shape.rowv == 5 ? 2 : 1, runs_pair(p, shape.lpc));
-  if (ws_bytes) {
-    st = workspace(ws_bytes, stream, &ws);
-    if (st) return st;
-  }
+  st = shape_workspace(p, &shape, shape.rowv == 5 ? 2 : 1, 0, stream, &ws);
+  if (st) return st;
   return launch_grid(p, md, t, nodes, eta, ws, shape, stream, shape.rowv == 5, true);
 }
 
@@ -1443,7 +1459,7 @@ extern "C" int swense_autotune_grid(const swense_modes* md, int32_t n_tl, const 
     // evicts the grid): the workspace, sized for the largest candidate and at least twice the
     // L2, is overwritten before each repetition (its contents are scratch).
     constexpr size_t kFlushBytes = size_t(256) << 20;
-    const int max_chunk = chunk_slots(p, Shape{0, 1, 0}, size_t(256) << 20);
+    const int max_chunk = chunk_slots(p, Shape{0, 1, 0}, kChunkBytes);
     const size_t ws_all = std::max(scratch_bytes(p, max_chunk, 2, pair_path(p.ny, p.Nxr, p.Nyr)), kFlushBytes);
     {
       void* ws = nullptr;
@@ -1459,7 +1475,7 @@ extern "C" int swense_autotune_grid(const swense_modes* md, int32_t n_tl, const 
       for (size_t mb : {16, 32, 64, 96, 128, 256}) {
         const size_t cb = mb << 20;
         Shape shape{0, lpc, rowv};
-        shape.chunk = chunk_slots(p, shape, cb);
+        shape.chunk = even_chunk(p, shape, chunk_slots(p, shape, cb));
         void* ws = nullptr;
         st = workspace(ws_all, stream, &ws);
         if (!st) st = launch_grid(p, md, t, nodes, eta, ws, shape, stream, rowv == 5, true);   // warm
