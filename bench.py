@@ -301,7 +301,7 @@ def job_throughput(units_per_rank, world, ms_per_step):
 
 GATHER_SOURCES = ("csrc/interp.cu", "csrc/internal.cuh")
 GRID_SOURCES = ("csrc/grid_ifft.cu", "csrc/fft.cuh", "csrc/internal.cuh")
-GRID_STAGE = "grid_ifft (stage 1: k_propagate, eta k_pass_a/k_pass_b, k_col_t, k_row_t)"
+GRID_STAGE = "grid_ifft (stage 1: k_form_modes, k_col_w, k_row_w)"
 
 
 def kernel_source_hash(files=GATHER_SOURCES):
@@ -321,13 +321,13 @@ def kernel_source_hash(files=GATHER_SOURCES):
 # the hash of the kernel's sources and the workload they were taken on; a changed kernel or
 # workload invalidates them (traffic is then reported as null).
 NCU_TRAFFIC = {
-    "k_interp_box": {"bytes": 114632192 + 113704704, "hash": "709995ea123f7df2",
+    "k_interp_box": {"bytes": 105900000 + 127300000, "hash": "92ee0328a2d6767e",
                      "workload": "jonswap3d: 512x256 modes, 64 levels, pad 1, 2 time levels, "
                                  "2048000 cell + 6177280 face centres (cylinder O-grid)"},
-    # all 13 launches of one step, caches kept between them (--cache-control none), launch shape
-    # lpc 4, 64 MB level chunks, row variant 2
-    GRID_STAGE: {"bytes": 284673536, "hash": "a8dc3ee11c502d0a",
-                 "taken_with": {"lpc": 4, "chunk_bytes": 64 << 20, "row_variant": 2},
+    # the three launches of one step, caches kept between them (--cache-control none), untuned launch
+    # shape: one chunk of 130 slots, whose intermediate goes through memory
+    GRID_STAGE: {"bytes": 6300000 + 266600000 + 527600000, "hash": "1e958107ea5274bd",
+                 "taken_with": {"lpc": 1, "chunk_bytes": 512 << 20, "row_variant": 0},
                  "workload": "jonswap3d: 512x256 modes, 64 levels, pad 1, 2 time levels, "
                              "2048000 cell + 6177280 face centres (cylinder O-grid)"},
 }

@@ -1,9 +1,9 @@
 // Many independent sea states in one call (workload of uneven instances). The reconstructions
 // run concurrently on library streams forked from the caller's stream (largest instance first,
 // round robin, each stream with its own part of the workspace, so small grids that cannot fill
-// the GPU alone run side by side); after the join, every instance's gather goes through one
-// planning launch and one persistent gather launch over a device queue of all the instances'
-// point chunks (interp_batch). The fork and join are events, so a whole call can be captured as
+// the GPU alone run side by side); after the join, the gathers of all instances go through one
+// planning launch, one persistent launch over a device queue of the point chunks that fit a tile and one
+// launch for the other chunks (interp_batch). The fork and join are events, so a whole call can be captured as
 // one CUDA graph and replayed as one launch. The first call (outside any capture) sizes the
 // workspace and uploads the gather tables.
 #include <algorithm>

@@ -6,6 +6,7 @@
 
 #include "fft.cuh"
 #include "internal.cuh"
+#include "mlp.cuh"
 
 namespace swense {
 

@@ -37,7 +37,6 @@ void count_launches(int n);
 // (and cleared when reset) on the current device; *was_set != 0 when a wait gave up.
 int grid_async_flag(bool reset, int* was_set);
 int direct_async_flag(bool reset, int* was_set);
-int learned_async_flag(bool reset, int* was_set);
 
 // Near-body direct sums (direct.cu, direct_tc.cu). direct_tc: the tensor-core split-BF16 path;
 // direct_split_sorted: the per-pair split-BF16 kernel over points sorted by the tensor-core path

@@ -6,8 +6,8 @@
 //   layers 67 -> 64 -> 64 -> 4, GELU (tanh form) on the hidden layers, output y[f] used,
 //   correction  f = lagrange_f + s_f y[f], pressure from the corrected fields (Bernoulli).
 //
-// Tensor cores: BF16 mma.sync (m16n8k16) with FP32 accumulation; one warp owns 16 rows, and a
-// layer's accumulator fragments become the next layer's A fragments in registers. Inference
+// Tensor cores: BF16 mma.sync (m16n8k16) with FP32 accumulation (the fused gather in interp.cu runs the
+// same network on tcgen05); one warp owns 16 rows, and a layer's accumulator fragments become the next layer's A fragments in registers. Inference
 // splits inputs and activations into BF16 hi + lo (two MMAs per step) so the result tracks an
 // FP64 evaluation of the same BF16 weights to ~1e-5; training uses plain BF16 operands.
 // Weight gradients (sums over the batch) are formed on the CUDA cores in FP32 by the block that made

@@ -1,6 +1,6 @@
 // The learned-correction network shared by the training kernels and the fused gather: sizes,
-// parameter offsets, the BF16 packed weight layout, GELU, and the per-warp layer step on
-// m16n8k16 fragments (see mlp.cu for the network's definition).
+// parameter offsets, the BF16 packed weight layout, GELU, and the per-warp layers of training and
+// plain inference on m16n8k16 fragments (see mlp.cu for the network's definition).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -11,6 +11,10 @@
 #include "mma.cuh"
 
 namespace swense {
+
+// The error flag of the learned gather's bounded waits (as grid_async_flag).
+int learned_async_flag(bool reset, int* was_set);
+
 namespace mlpnet {
 
 constexpr int NIN = 67, KIN = 80, NH = 64, NOUT = 4, NO = 8, XLD = 68;
