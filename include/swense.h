@@ -645,6 +645,15 @@ int swense_selftest_wait_timeout(void* stream);
 int swense_selftest_direct_wait_timeout(int32_t on);
 
 /*
+ * swense_selftest_learned_wait_timeout — self-test switch of the learned gather's bounded waits (no
+ * passage of the paper: library housekeeping). While on (on != 0) for the current device, every
+ * swense_interp_learned call issues no MMA and limits each wait to a few polls: every wait runs out,
+ * u, v, w and p of all points are NaN (eta does not depend on the waits), and swense_async_status then
+ * returns SWENSE_ERR_TIMEOUT. Switch it off (on = 0) before any real call. Errors: UNSUPPORTED, CUDA.
+ */
+int swense_selftest_learned_wait_timeout(int32_t on);
+
+/*
  * swense_direct_stats — tiles of the last SWENSE_DIRECT_SPLIT_BF16 call on the current device
  * (no passage of the paper): *tiles = tiles of 128 z-sorted points, *fallback_tiles = those whose
  * z range was too wide for the tensor-core expansion and went to the per-pair kernel (0 and 0

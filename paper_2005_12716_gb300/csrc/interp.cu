@@ -1397,6 +1397,11 @@ static_assert(2 * (LRN_SMEM + 1024) <= 228 * 1024, "two blocks an SM");
 // Set when a wait for the tensor cores gives up; the host reads and clears it with swense_async_status.
 __device__ int g_learned_timeout;
 
+// Limit of those waits; withhold: no MMA is issued, so that every wait runs out (self-test).
+struct LearnedWaits {
+  int polls, withhold;
+};
+
 __device__ __forceinline__ void wg_sync(int wg) { asm volatile("bar.sync %0, 128;" ::"r"(1 + wg) : "memory"); }
 
 // Eight inputs (k-chunk kc) of output n of a layer with K plain inputs and 16 more for offsets and bias.
@@ -1451,7 +1456,7 @@ __device__ __forceinline__ void learned_store_a(uint32_t lanes, int hf, const fl
 
 __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_constant__ InterpArgs a, const __grid_constant__ Levels L,
                                                                     const int4* __restrict__ plan,
-                                                                    const PackedFwd* __restrict__ Wg) {
+                                                                    const PackedFwd* __restrict__ Wg, LearnedWaits waits) {
   using namespace mlpnet;
   extern __shared__ float4 sbox[];
   float* seta = reinterpret_cast<float*>(sbox + BOX_NODES);
@@ -1526,10 +1531,10 @@ __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_
     fence_proxy_async();
     tc::fence_before();
     wg_sync(wg);
-    if (t == 0 && !bad) learned_mma(ta, w, xo, xo_lbo, bar);
+    if (t == 0 && !bad && !waits.withhold) learned_mma(ta, w, xo, xo_lbo, bar);
     __syncwarp();
-    if (!bad) bad = !mbar_wait(bar, ph);
-    ph ^= 1u;
+    if (!bad) bad = !mbar_wait(bar, ph, waits.polls);
+    if (!bad) ph ^= 1u;                                // a thread that gave up stays at the phase it gave up on
     __syncwarp();
     tc::fence_after();
   };
@@ -1689,7 +1694,9 @@ __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_
   }
   if (bad) {
     atomicExch(&g_learned_timeout, 1);
-    mbar_wait(bar, ph ^ 1u);                           // the MMAs may still be in flight
+    // thread 0 issues a layer only after it has seen the one before complete, so the MMAs that may still be
+    // in flight are those of the phase it gave up on
+    if (t == 0) mbar_wait(bar, ph, waits.polls);
   }
   tc::fence_before();
   __syncthreads();
@@ -1898,6 +1905,21 @@ extern "C" int swense_mlp_features(const swense_grid* g, double t, const float* 
 }
 
 namespace swense {
+namespace {
+
+std::mutex g_learned_selftest_mutex;
+bool g_learned_selftest[64];      // per device (swense_selftest_learned_wait_timeout)
+
+int learned_waits(LearnedWaits* w) {
+  int dev = 0;
+  SWENSE_CUDA_TRY(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lock(g_learned_selftest_mutex);
+  const bool on = dev >= 0 && dev < 64 && g_learned_selftest[dev];
+  *w = on ? LearnedWaits{8, 1} : LearnedWaits{kMbarPolls, 0};
+  return SWENSE_OK;
+}
+
+}  // namespace
 
 int learned_async_flag(bool reset, int* was_set) {
   int v = 0;
@@ -1911,6 +1933,15 @@ int learned_async_flag(bool reset, int* was_set) {
 }
 
 }  // namespace swense
+
+extern "C" int swense_selftest_learned_wait_timeout(int32_t on) {
+  int dev = 0;
+  SWENSE_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return fail(SWENSE_ERR_UNSUPPORTED, "device index too large");
+  std::lock_guard<std::mutex> lock(g_learned_selftest_mutex);
+  g_learned_selftest[dev] = on != 0;
+  return SWENSE_OK;
+}
 
 extern "C" int swense_interp_learned(const swense_grid* g, double t, const float* pts, int64_t np,
                                      float* eta, float* u, float* v, float* w, float* p,
@@ -1946,8 +1977,11 @@ extern "C" int swense_interp_learned(const swense_grid* g, double t, const float
     SWENSE_CUDA_TRY(cudaGetLastError());
     SWENSE_CUDA_TRY(cudaFuncSetAttribute((const void*)k_interp_learned,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, int(LRN_SMEM)));
+    LearnedWaits waits;
+    st = learned_waits(&waits);
+    if (st) return st;
     k_interp_learned<<<unsigned(blocks), BOX_THREADS, LRN_SMEM, stream>>>(
-        a, lev, plan, static_cast<const PackedFwd*>(packed));
+        a, lev, plan, static_cast<const PackedFwd*>(packed), waits);
     SWENSE_CUDA_TRY(cudaGetLastError());
     count_launches(2);
   }
