@@ -645,6 +645,16 @@ int swense_selftest_wait_timeout(void* stream);
 int swense_selftest_direct_wait_timeout(int32_t on);
 
 /*
+ * swense_selftest_grid_wait_timeout — self-test switch of the staged row passes' bounded waits (no
+ * passage of the paper: library housekeeping). While on (on != 0) for the current device, the rows of
+ * every grid whose row pass stages them by bulk copies (3-D grids with columns of 32 to 1024 nodes and
+ * rows of 32 to 2048) are not copied and each wait is limited to a few polls: every wait runs out, the
+ * grid's rows are not written, and swense_async_status then returns SWENSE_ERR_TIMEOUT. Switch it off
+ * (on = 0) before any real call. Errors: UNSUPPORTED, CUDA.
+ */
+int swense_selftest_grid_wait_timeout(int32_t on);
+
+/*
  * swense_selftest_learned_wait_timeout — self-test switch of the learned gather's bounded waits (no
  * passage of the paper: library housekeeping). While on (on != 0) for the current device, every
  * swense_interp_learned call issues no MMA and limits each wait to a few polls: every wait runs out,

@@ -124,6 +124,7 @@ _SIGS = {
     "swense_async_status": (ctypes.c_int, [ctypes.c_int32, ctypes.c_void_p]),
     "swense_selftest_wait_timeout": (ctypes.c_int, [ctypes.c_void_p]),
     "swense_selftest_direct_wait_timeout": (ctypes.c_int, [ctypes.c_int32]),
+    "swense_selftest_grid_wait_timeout": (ctypes.c_int, [ctypes.c_int32]),
     "swense_selftest_learned_wait_timeout": (ctypes.c_int, [ctypes.c_int32]),
     "swense_direct_stats": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]),
     "swense_selftest_tc_gemm": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
@@ -366,6 +367,10 @@ def swense_selftest_wait_timeout(stream=None):
 
 def swense_selftest_direct_wait_timeout(on):
     _check(load().swense_selftest_direct_wait_timeout(1 if on else 0))
+
+
+def swense_selftest_grid_wait_timeout(on):
+    _check(load().swense_selftest_grid_wait_timeout(1 if on else 0))
 
 
 def swense_selftest_learned_wait_timeout(on):

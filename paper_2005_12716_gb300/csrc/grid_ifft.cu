@@ -356,8 +356,8 @@ struct RowArgs {
   const float2* tw;
   int Mh, Nxr, Nyr, lev0, n_lev;
   int ldG;               // m stride of the transposed intermediate
-  int polls;             // k_row_tma: polls of a bounded wait before it gives up
-  int selftest;          // k_row_tma: 1 = issue no copy, so every wait runs out (self-test)
+  int polls;             // staged rows: polls of a bounded wait before it gives up
+  int selftest;          // staged rows: 1 = issue no copy, so every wait runs out (self-test)
 };
 
 // m stride of the transposed intermediate: a whole number of 128-byte lines per field row, so
@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(WideRow<N>::T * WideRow<N>::kRows, WideRow<N>:
     const float2* src = a.G + size_t(level) * 4 * fs + size_t(y0) * a.ldG;
     fence_proxy_async();                           // earlier reads of the buffer come first
     mbar_arrive_expect_tx(bar, nf * span);
-    for (int f = 0; f < nf; ++f) bulk_g2s(stg + size_t(f) * W::kRows * a.ldG, src + f * fs, span, bar);
+    for (int f = 0; f < nf && !a.selftest; ++f) bulk_g2s(stg + size_t(f) * W::kRows * a.ldG, src + f * fs, span, bar);
   };
   int item = blockIdx.x;
   if (item >= items) return;
@@ -986,6 +986,16 @@ int shape_workspace(const GridPlan& p, Shape* s, int nbuf, size_t extra, cudaStr
   }
 }
 
+// Self-test of the staged rows' waits, per device (swense_selftest_grid_wait_timeout).
+std::mutex g_selftest_mutex;
+bool g_selftest[64];
+bool g_row_selftest() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  std::lock_guard<std::mutex> lock(g_selftest_mutex);
+  return g_selftest[dev];
+}
+
 // Library-internal second stream and events (per device) for the two-stream transform
 // pipeline: chunk c's row pass runs on the second stream while chunk c+1's column pass runs on
 // the caller's stream, with two intermediate buffers. Created on first use; recording, waiting
@@ -1240,8 +1250,9 @@ int launch_grid(const GridPlan& p, const swense_modes* md, const double* t, floa
   ra.Nxr = int(Nxr);
   ra.Nyr = int(Nyr);
   ra.n_lev = ca.n_lev;
-  ra.polls = kMbarPolls;
-  ra.selftest = 0;
+  const bool selftest = g_row_selftest();
+  ra.polls = selftest ? 8 : kMbarPolls;
+  ra.selftest = selftest;
   ca.ldG = ra.ldG = ld;
   const int slots = grid_slots(p, shape);
   for (int l0 = 0; l0 < slots; l0 += chunk) {
@@ -1533,7 +1544,7 @@ extern "C" int swense_set_grid_tune(int32_t nx, int32_t ny, int32_t pad_n, int32
 }
 
 // ---------------------------------------------------------------------------------------------
-// Bounded device-side waits report here: the flag of this translation unit (k_row_tma).
+// Bounded device-side waits report here: the flag of this translation unit (k_row_w, k_row_tma).
 namespace swense {
 
 int grid_async_flag(bool reset, int* was_set) {
@@ -1548,6 +1559,15 @@ int grid_async_flag(bool reset, int* was_set) {
 }
 
 }  // namespace swense
+
+extern "C" int swense_selftest_grid_wait_timeout(int32_t on) {
+  int dev = 0;
+  SWENSE_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return fail(SWENSE_ERR_UNSUPPORTED, "device index too large");
+  std::lock_guard<std::mutex> lock(g_selftest_mutex);
+  g_selftest[dev] = on != 0;
+  return SWENSE_OK;
+}
 
 extern "C" int swense_selftest_wait_timeout(void* stream_) {
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);

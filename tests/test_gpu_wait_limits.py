@@ -49,3 +49,34 @@ def test_learned_gather_wait_that_runs_out(env, n, flat):
     assert S.swense_async_status(reset=True) == 0
     for k, v in want.items():
         assert torch.equal(again[k], v), k
+
+
+# rows of one thread's exchange up to a block a row; one and two exchange buffers; one chunk and several
+@pytest.mark.parametrize("nx,ny,pad,rowv,chunk", [(32, 32, 1, 0, 512), (64, 32, 4, 0, 1), (256, 64, 1, 0, 1), (256, 64, 2, 5, 1),
+                                                  (2048, 32, 1, 0, 4), (512, 32, 4, 0, 512), (512, 64, 1, 4, 1)])
+def test_row_pass_wait_that_runs_out(env, nx, ny, pad, rowv, chunk):
+    torch, S, api = env
+    from wavegen import seas
+    rng = np.random.default_rng(nx)
+    sea = seas.linear_sea(nx, ny, nx / 16, ny / 16, seas.random_linear_components(nx, ny, nx / 16, ny / 16, 6, 0.01, rng))
+    z, tl = np.linspace(-1.0, 0.05, 7).astype(np.float32), [0.0, 0.1]
+    modes = api.upload_modes(sea)
+    S.swense_set_grid_tune(nx, ny, pad, len(z), 1, chunk << 20, rowv)
+    try:
+        want = api.fields_on_grid(modes, z, pad, tl)
+        g = api.alloc_grid(modes, z, pad, tl)
+        g.nodes.fill_(7.0)
+        assert S.swense_async_status(reset=True) == 0
+        S.swense_selftest_grid_wait_timeout(True)
+        try:
+            api.fields_on_grid(modes, z, pad, tl, out=g)
+            st = S.swense_async_status(reset=True, raise_on_error=False)
+        finally:
+            S.swense_selftest_grid_wait_timeout(False)
+        assert st == -6 and S.swense_strerror(st) == "SWENSE_ERR_TIMEOUT"
+        assert bool((g.nodes == 7.0).all())                    # no row was written
+        api.fields_on_grid(modes, z, pad, tl, out=g)
+        assert S.swense_async_status(reset=True) == 0
+        assert torch.equal(g.nodes, want.nodes) and torch.equal(g.eta, want.eta)
+    finally:
+        S.swense_set_grid_tune(nx, ny, pad, len(z), -1)
