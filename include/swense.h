@@ -18,7 +18,8 @@
  *   "host" pointers are read before the call returns. The caller owns every buffer it passes.
  *   The library keeps a per-device scratch workspace (allocated with cudaMalloc on first use,
  *   grown on demand, freed by swense_release); entry points that may grow it must not be
- *   called for the first time inside a CUDA stream capture.
+ *   called for the first time inside a CUDA stream capture. Where memory is short, calls that take
+ *   more scratch only to be faster do with what is held, in a capture as outside one.
  * - `stream` is a cudaStream_t passed as void* (NULL = legacy default stream). All device work
  *   is enqueued on it; calls return before it runs unless documented otherwise.
  * - Calls that overlap on the GPU (different streams, no ordering) race on the library's scratch
@@ -681,6 +682,13 @@ int swense_direct_stats(int64_t* tiles, int64_t* fallback_tiles, void* stream);
  */
 int swense_selftest_tc_gemm(const float* A, const float* B, float* D, int32_t N, int32_t K,
                             int32_t variant, void* stream);
+
+/*
+ * swense_selftest_workspace_limit — self-test of the library on a device short of memory (no passage of
+ * the paper: library housekeeping): while bytes > 0, growing the current device's scratch workspace
+ * beyond that many bytes fails as if the device had no more. 0: no limit. Errors: UNSUPPORTED, CUDA.
+ */
+int swense_selftest_workspace_limit(int64_t bytes);
 
 /* Bytes of scratch workspace currently held on the current device. */
 int64_t swense_workspace_bytes(void);

@@ -125,6 +125,7 @@ _SIGS = {
     "swense_selftest_wait_timeout": (ctypes.c_int, [ctypes.c_void_p]),
     "swense_selftest_direct_wait_timeout": (ctypes.c_int, [ctypes.c_int32]),
     "swense_selftest_grid_wait_timeout": (ctypes.c_int, [ctypes.c_int32]),
+    "swense_selftest_workspace_limit": (ctypes.c_int, [ctypes.c_int64]),
     "swense_selftest_learned_wait_timeout": (ctypes.c_int, [ctypes.c_int32]),
     "swense_direct_stats": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]),
     "swense_selftest_tc_gemm": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
@@ -371,6 +372,10 @@ def swense_selftest_direct_wait_timeout(on):
 
 def swense_selftest_grid_wait_timeout(on):
     _check(load().swense_selftest_grid_wait_timeout(1 if on else 0))
+
+
+def swense_selftest_workspace_limit(nbytes):
+    _check(load().swense_selftest_workspace_limit(int(nbytes)))
 
 
 def swense_selftest_learned_wait_timeout(on):

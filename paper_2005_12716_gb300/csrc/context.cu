@@ -1,6 +1,8 @@
 // Per-device scratch workspace, twiddle table and error reporting.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <cstdint>
 #include <mutex>
 #include <string>
 
@@ -35,7 +37,14 @@ struct DeviceState {
   void* ws = nullptr;
   size_t ws_bytes = 0;
   bool tw_ready = false;
+  // Smallest optional request that could not be had, and how many more of at least its size are answered
+  // so without another try: a failing allocation on every call would cost more than the larger scratch
+  // gives, and memory may come free later.
+  size_t refused = SIZE_MAX;
+  int refusals_left = 0;
+  size_t limit = SIZE_MAX;      // self-test: larger allocations fail (swense_selftest_workspace_limit)
 };
+constexpr int kRefusals = 256;
 
 std::mutex g_mutex;
 DeviceState g_dev[kMaxDevices];
@@ -63,7 +72,27 @@ int current_device(int* dev) {
 
 }  // namespace
 
-int workspace(size_t bytes, cudaStream_t stream, void** out) {
+namespace {
+
+// A new workspace in place of the device's own, which is freed once the new one is there.
+cudaError_t replace_workspace(DeviceState& d, size_t want) {
+  void* p = nullptr;
+  const cudaError_t e = want > d.limit ? cudaErrorMemoryAllocation : cudaMalloc(&p, want);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return e;
+  }
+  if (d.ws) {
+    cudaDeviceSynchronize();                     // work in flight may still use the old one
+    cudaFree(d.ws);
+  }
+  d.ws = p;
+  d.ws_bytes = want;
+  if (want >= d.refused) d.refused = SIZE_MAX;
+  return cudaSuccess;
+}
+
+int grow(size_t bytes, cudaStream_t stream, void** out, bool optional) {
   int dev;
   int st = current_device(&dev);
   if (st) return st;
@@ -76,27 +105,36 @@ int workspace(size_t bytes, cudaStream_t stream, void** out) {
   }
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   SWENSE_CUDA_TRY(cudaStreamIsCapturing(stream, &cap));
-  if (cap != cudaStreamCaptureStatusNone)
+  const bool capturing = cap != cudaStreamCaptureStatusNone;
+  if (optional && (capturing || (bytes >= d.refused && d.refusals_left-- > 0))) return SWENSE_ERR_OOM;
+  if (capturing)
     return fail(SWENSE_ERR_ARG, "scratch workspace must grow, which is not allowed during stream "
                                 "capture; make one call with the same sizes before capturing");
-  if (d.ws) {
+  const size_t want = bytes + bytes / 4;         // headroom so small growth does not reallocate
+  cudaError_t e = replace_workspace(d, want);
+  if (e != cudaSuccess && optional) {
+    d.refused = std::min(d.refused, bytes);
+    d.refusals_left = kRefusals;
+    return SWENSE_ERR_OOM;
+  }
+  if (e != cudaSuccess && d.ws) {                // no room for both: give up the old one first
     SWENSE_CUDA_TRY(cudaDeviceSynchronize());
     SWENSE_CUDA_TRY(cudaFree(d.ws));
     d.ws = nullptr;
     d.ws_bytes = 0;
+    e = replace_workspace(d, want);
   }
-  size_t want = bytes + bytes / 4;  // headroom so small growth does not reallocate
-  cudaError_t e = cudaMalloc(&d.ws, want);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    d.ws = nullptr;
+  if (e != cudaSuccess)
     return fail(SWENSE_ERR_OOM, "cudaMalloc of the scratch workspace (" + std::to_string(want) +
                                     " bytes) failed: " + cudaGetErrorString(e));
-  }
-  d.ws_bytes = want;
   *out = d.ws;
   return SWENSE_OK;
 }
+
+}  // namespace
+
+int workspace(size_t bytes, cudaStream_t stream, void** out) { return grow(bytes, stream, out, false); }
+int workspace_optional(size_t bytes, cudaStream_t stream, void** out) { return grow(bytes, stream, out, true); }
 
 int twiddles(cudaStream_t stream, const float2** out) {
   int dev;
@@ -147,6 +185,17 @@ int swense_release(void) {
   }
   d.ws = nullptr;
   d.ws_bytes = 0;
+  d.refused = SIZE_MAX;
+  d.refusals_left = 0;
+  return SWENSE_OK;
+}
+
+int swense_selftest_workspace_limit(int64_t bytes) {
+  int dev = 0;
+  int st = swense::current_device(&dev);
+  if (st) return st;
+  std::lock_guard<std::mutex> lock(swense::g_mutex);
+  swense::g_dev[dev].limit = bytes > 0 ? size_t(bytes) : SIZE_MAX;
   return SWENSE_OK;
 }
 

@@ -975,15 +975,31 @@ size_t scratch_bytes(const GridPlan& p, int chunk, int nbuf, bool pair) {
   return align256(modes_bytes(p, pair)) + align256(p.geta_bytes) + size_t(nbuf) * align256(g_bytes);
 }
 
-// Workspace of a request (`extra` bytes more); where that much cannot be had, of smaller chunks.
+// Workspace of a request (`extra` bytes more); where that much cannot be had, or would have to be got
+// during a capture, of smaller chunks, down to one slot, and at last of the shared-memory path, whose
+// modes take less. First without giving up the present workspace (a smaller chunk is better than a free
+// and an allocation on every call), then, should it not even hold one slot, whatever it takes.
+constexpr size_t kChunkNeeded = size_t(64) << 20;
 int shape_workspace(const GridPlan& p, Shape* s, int nbuf, size_t extra, cudaStream_t stream, void** ws) {
-  for (;;) {
-    const size_t bytes = scratch_bytes(p, s->chunk, nbuf, runs_pair(p, s->lpc)) + extra;
-    if (!bytes) return SWENSE_OK;
-    const int st = workspace(bytes, stream, ws);
-    if (st != SWENSE_ERR_OOM || s->chunk <= 1) return st;
-    s->chunk = (s->chunk + 1) / 2;
+  const Shape first = *s;
+  Shape shared = first;
+  shared.lpc = 0;
+  shared.chunk = chunk_slots(p, shared, kChunkNeeded);
+  int st = SWENSE_OK;
+  for (int pass = 0; pass < 2; ++pass) {
+    for (Shape t : {first, shared}) {
+      if (pass == 1) t.chunk = std::min(t.chunk, chunk_slots(p, t, kChunkNeeded));
+      for (;; t.chunk = (t.chunk + 1) / 2) {
+        const size_t bytes = scratch_bytes(p, t.chunk, nbuf, runs_pair(p, t.lpc)) + extra;
+        st = !bytes ? SWENSE_OK : pass == 0 ? workspace_optional(bytes, stream, ws) : workspace(bytes, stream, ws);
+        *s = t;
+        if (st != SWENSE_ERR_OOM && st != SWENSE_ERR_ARG) return st;   // ARG: growth during a capture
+        if (t.chunk <= 1) break;
+      }
+      if (!runs_pair(p, first.lpc)) break;
+    }
   }
+  return st;
 }
 
 // Self-test of the staged rows' waits, per device (swense_selftest_grid_wait_timeout).

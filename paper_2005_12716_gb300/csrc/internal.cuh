@@ -22,8 +22,12 @@ int cuda_fail(cudaError_t e, const char* what);
 
 // ---------------------------------------------------------------- per-device scratch
 // Returns a device pointer to at least `bytes` bytes of scratch (256-byte aligned), growing the
-// device's workspace if needed. Growing synchronises the device and is refused during capture.
+// device's workspace if needed. Growing synchronises the device and is refused during capture. The
+// old workspace is freed after the new one is had, or before it where there is no room for both.
 int workspace(size_t bytes, cudaStream_t stream, void** out);
+// The same for scratch a call can do without: where it cannot be had beside the present workspace, or
+// during a capture that would have to grow it, SWENSE_ERR_OOM and the workspace as it was.
+int workspace_optional(size_t bytes, cudaStream_t stream, void** out);
 
 // Twiddle array: the plain table e^{+2 pi i j / SWENSE_MAX_FFT}, j < SWENSE_MAX_FFT, followed by
 // the Stockham passes' pass-major tables (fft.cuh, stk_twp). The first call on a device fills it

@@ -2066,7 +2066,7 @@ int interp_impl(const swense_grid* g, double t, const float* pts, const int32_t*
   const bool sparse = double(np) < 0.25 * double(a.Nxr) * double(a.Nyr) * double(a.nz);
   bool kinds = sparse && np >= LAYER_POINTS && blocks < (int64_t(1) << 31) / (BOX_PTS / GLOBAL_PTS);
   void* ws = nullptr;
-  st = kinds ? workspace(b_plan + lists_bytes(np, blocks), stream, &ws) : SWENSE_OK;
+  st = kinds ? workspace_optional(b_plan + lists_bytes(np, blocks), stream, &ws) : SWENSE_OK;
   if (st || !kinds) {
     kinds = false;
     st = workspace(b_plan, stream, &ws);
