@@ -7,6 +7,7 @@
 // one CUDA graph and replayed as one launch. The first call (outside any capture) sizes the
 // workspace and uploads the gather tables.
 #include <algorithm>
+#include <cstdint>
 #include <mutex>
 #include <numeric>
 #include <vector>
@@ -55,16 +56,25 @@ extern "C" int swense_batch_run(const swense_instance* inst, int32_t n, int32_t 
   if (n < 0) return fail(SWENSE_ERR_ARG, "negative instance count");
   if (n == 0) return SWENSE_OK;
   if (!inst) return fail(SWENSE_ERR_ARG, "NULL instance array");
-  // scratch of each reconstruction (its tuned launch shape) and the gather items
+  // launch shape of each reconstruction (the tuned one, with chunks within `limit`) and the largest scratch
+  std::vector<GridShape> shapes(static_cast<size_t>(n));
   size_t slice = 0;
+  auto size_slice = [&](size_t limit) {
+    slice = 0;
+    for (int32_t i = 0; i < n; ++i) {
+      const swense_instance& c = inst[i];
+      size_t b = 0;
+      const int e = grid_scratch(&c.modes, c.n_tl, c.t_levels, &c.desc, c.nodes, c.eta, limit, &shapes[size_t(i)], &b);
+      if (e) return e;
+      slice = std::max(slice, align256(b));
+    }
+    return int(SWENSE_OK);
+  };
+  // the gather items
   std::vector<GatherItem> items(static_cast<size_t>(n));
   std::vector<double> weight(static_cast<size_t>(n));
   for (int32_t i = 0; i < n; ++i) {
     const swense_instance& c = inst[i];
-    size_t b = 0;
-    int st = grid_scratch(&c.modes, c.n_tl, c.t_levels, &c.desc, c.nodes, c.eta, &b);
-    if (st) return st;
-    slice = std::max(slice, align256(b));
     GatherItem& it = items[size_t(i)];
     it.grid = swense_grid{};
     it.grid.nodes = c.nodes;
@@ -92,8 +102,22 @@ extern "C" int swense_batch_run(const swense_instance* inst, int32_t n, int32_t 
   size_t gbytes = 0;
   int st = interp_batch_bytes(items.data(), n, &gbytes);
   if (st) return st;
+  // The streams' parts at full size; where that cannot be had (or would have to be got during a capture),
+  // of smaller chunks, first without giving up the present workspace, as for a single grid.
   void* ws = nullptr;
-  st = workspace(size_t(kBatchStreams) * slice + gbytes, stream, &ws);
+  constexpr size_t kMB = size_t(1) << 20;
+  constexpr size_t kLimits[] = {SIZE_MAX, 256 * kMB, 128 * kMB, 64 * kMB, 16 * kMB, 4 * kMB, kMB, 0};
+  for (int pass = 0; pass < 2 && !ws; ++pass)
+    for (size_t limit : kLimits) {
+      if (pass == 1 && limit > 64 * kMB) continue;
+      st = size_slice(limit);
+      if (st) return st;
+      const size_t bytes = size_t(kBatchStreams) * slice + gbytes;
+      st = pass == 0 ? workspace_optional(bytes, stream, &ws) : workspace(bytes, stream, &ws);
+      if (!st) break;
+      ws = nullptr;
+      if (st != SWENSE_ERR_OOM && st != SWENSE_ERR_ARG) return st;
+    }
   if (st) return st;
   BatchStreams* bs = nullptr;
   st = batch_streams(&bs);
@@ -109,7 +133,7 @@ extern "C" int swense_batch_run(const swense_instance* inst, int32_t n, int32_t 
   for (int j = 0; j < n && !first_err; ++j) {
     const int i = order[size_t(j)], k = j % kBatchStreams;
     const swense_instance& c = inst[i];
-    first_err = grid_with_scratch(&c.modes, c.n_tl, c.t_levels, &c.desc, c.nodes, c.eta,
+    first_err = grid_with_scratch(&c.modes, c.n_tl, c.t_levels, &c.desc, c.nodes, c.eta, shapes[size_t(i)],
                                   static_cast<char*>(ws) + size_t(k) * slice, bs->s[k]);
   }
   // join (also after an error, so that no stream is left forked from a capture)

@@ -931,9 +931,7 @@ int plan_grid(const swense_modes* md, int32_t n_tl, const double* t, const swens
 
 // The launch shape of a request: the tuned one of its grid shape, else the transposed pair where it
 // applies and the shared-memory path elsewhere.
-struct Shape {
-  int chunk, lpc, rowv;   // chunk: levels (the pair: slots, of all time levels and eta) per chunk
-};
+using Shape = GridShape;
 
 // Whether a launch shape runs the transposed pair, and with eta's transforms among its slots (the
 // row passes of 4096 points and more and the staged one take levels only).
@@ -1440,28 +1438,30 @@ extern "C" int swense_fields_on_grid(const swense_modes* md, int32_t n_tl, const
 
 namespace swense {
 
-// Scratch one swense_fields_on_grid call needs with its current launch shape, and the same call
+// Launch shape and scratch of one swense_fields_on_grid call, and the same call
 // with that scratch supplied (no library stream: the eta transform and, for variant 5, the row
 // passes stay on `stream`), for callers that run several reconstructions concurrently, each in
 // its own part of the workspace (swense_batch_run).
 int grid_scratch(const swense_modes* md, int32_t n_tl, const double* t, const swense_grid_desc* desc,
-                 float* nodes, float* eta, size_t* bytes) {
+                 float* nodes, float* eta, size_t chunk_limit, GridShape* shape, size_t* bytes) {
   GridPlan p;
   int st = plan_grid(md, n_tl, t, desc, nodes, eta, &p);
   if (st) return st;
   if (!is_pow2(p.pad)) return fail(SWENSE_ERR_UNSUPPORTED, "batched grids take power-of-two padding factors");
-  const Shape shape = grid_shape(p);
-  *bytes = scratch_bytes(p, shape.chunk, 1, runs_pair(p, shape.lpc));
+  *shape = grid_shape(p);
+  if (chunk_limit == 0) shape->lpc = 0;
+  if (p.ny > 1) shape->chunk = std::min(shape->chunk, chunk_slots(p, *shape, chunk_limit));
+  *bytes = scratch_bytes(p, shape->chunk, 1, runs_pair(p, shape->lpc));
   return SWENSE_OK;
 }
 
 int grid_with_scratch(const swense_modes* md, int32_t n_tl, const double* t, const swense_grid_desc* desc,
-                      float* nodes, float* eta, void* ws, cudaStream_t stream) {
+                      float* nodes, float* eta, const GridShape& shape, void* ws, cudaStream_t stream) {
   GridPlan p;
   int st = plan_grid(md, n_tl, t, desc, nodes, eta, &p);
   if (st) return st;
   if (!is_pow2(p.pad)) return fail(SWENSE_ERR_UNSUPPORTED, "batched grids take power-of-two padding factors");
-  return launch_grid(p, md, t, nodes, eta, ws, grid_shape(p), stream, false, false);
+  return launch_grid(p, md, t, nodes, eta, ws, shape, stream, false, false);
 }
 
 }  // namespace swense
@@ -1487,13 +1487,21 @@ extern "C" int swense_autotune_grid(const swense_modes* md, int32_t n_tl, const 
     // L2, is overwritten before each repetition (its contents are scratch).
     constexpr size_t kFlushBytes = size_t(256) << 20;
     const int max_chunk = chunk_slots(p, Shape{0, 1, 0}, kChunkBytes);
-    const size_t ws_all = std::max(scratch_bytes(p, max_chunk, 2, pair_path(p.ny, p.Nxr, p.Nyr)), kFlushBytes);
-    {
+    bool pp = pair_path(p.ny, p.Nxr, p.Nyr);
+    size_t ws_all = 0;
+    for (;; pp = false) {                        // the pair's candidates only where its scratch can be had
+      const size_t chunks = pp ? scratch_bytes(p, max_chunk, 2, true)
+                               : scratch_bytes(p, chunk_slots(p, Shape{0, 0, 0}, kFlushBytes), 1, false);
+      ws_all = std::max(chunks, kFlushBytes);
       void* ws = nullptr;
       st = workspace(ws_all, stream, &ws);
-      if (st) return st;
+      if (st && !(st == SWENSE_ERR_OOM && pp)) {
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        return st;
+      }
+      if (!st) break;
     }
-    const bool pp = pair_path(p.ny, p.Nxr, p.Nyr);
     for (int lpc : {0, 1, 2, 4})
     for (int rowv : {0, 4, 5}) {
       if (lpc > 0 && !pp) continue;

@@ -49,10 +49,15 @@ int direct_async_flag(bool reset, int* was_set);
 int direct_tc(const swense_modes* md, double t, const float* pts, int64_t np, float* eta, float* u,
               float* v, float* w, float* p, int32_t p_mode, double rho, double grav, cudaStream_t stream);
 // Grid reconstruction with caller-supplied scratch (grid_ifft.cu), for concurrent batches.
+// grid_scratch: the launch shape with chunks of at most chunk_limit bytes (0: one slot of the path that
+// takes the least scratch) and the bytes that grid_with_scratch needs to run it.
+struct GridShape {
+  int chunk, lpc, rowv;   // chunk: levels (the pair: slots, of all time levels and eta) per chunk
+};
 int grid_scratch(const swense_modes* md, int32_t n_tl, const double* t, const swense_grid_desc* desc,
-                 float* nodes, float* eta, size_t* bytes);
+                 float* nodes, float* eta, size_t chunk_limit, GridShape* shape, size_t* bytes);
 int grid_with_scratch(const swense_modes* md, int32_t n_tl, const double* t, const swense_grid_desc* desc,
-                      float* nodes, float* eta, void* ws, cudaStream_t stream);
+                      float* nodes, float* eta, const GridShape& shape, void* ws, cudaStream_t stream);
 
 // One gather of a batch (interp.cu): the grid and the points of one instance.
 struct GatherItem {

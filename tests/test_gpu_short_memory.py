@@ -84,3 +84,38 @@ def test_gather_without_planes_keeps_the_workspace(env):
         assert S.swense_workspace_bytes() == held
         for k, v in want.items():
             assert float((out[k] - v).abs().max()) <= 1e-5 * float(v.abs().max()), k
+
+
+@pytest.mark.parametrize("limit", [80 * MB, 30 * MB, 8 * MB])
+def test_batch_with_less_scratch(env, limit):
+    torch, S, api = env
+    rng = np.random.default_rng(5)
+    items = []
+    for nx, ny, n in ((256, 128, 5000), (128, 128, 3000), (64, 32, 900)):
+        sea = seas.linear_sea(nx, ny, nx / 16, ny / 16, seas.random_linear_components(nx, ny, nx / 16, ny / 16, 8, 0.01, rng))
+        pts = np.stack([rng.uniform(0, nx / 16, n), rng.uniform(0, ny / 16, n), rng.uniform(-0.9, 0.0, n)], 1)
+        items.append({"sea": sea, "z_levels": np.linspace(-1.0, 0.05, 40).astype(np.float32), "pad_n": 1,
+                      "t_levels": [0.0, 0.1], "t": 0.04, "pts": pts.astype(np.float32)})
+    b = api.Batch(items)
+    b.run()                                                     # 4 streams' parts of 42 MB
+    want = [{k: v.clone() for k, v in it["out"].items()} for it in b.items]
+    S.swense_release()
+    S.swense_selftest_workspace_limit(limit)
+    held = []
+    for _ in range(3):
+        b.run()
+        held.append(S.swense_workspace_bytes())
+    assert 0 < held[0] <= limit and held == held[:1] * 3
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        b.run()
+    for it in b.items:
+        for v in it["out"].values():
+            v.fill_(float("nan"))
+    graph.replay()
+    torch.cuda.synchronize()
+    # the smallest limit leaves the other transform path: equal to rounding
+    for it, w in zip(b.items, want):
+        for k, v in w.items():
+            assert float((it["out"][k] - v).abs().max()) <= 1e-5 * float(v.abs().max()), k
