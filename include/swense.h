@@ -19,7 +19,9 @@
  *   The library keeps a per-device scratch workspace (allocated with cudaMalloc on first use,
  *   grown on demand, freed by swense_release); entry points that may grow it must not be
  *   called for the first time inside a CUDA stream capture. Where memory is short, calls that take
- *   more scratch only to be faster do with what is held, in a capture as outside one.
+ *   more scratch only to be faster do with what is held, in a capture as outside one. Calls captured
+ *   in a graph use the workspace at every replay: growing it later keeps the one they hold until the graph
+ *   and what was instantiated from it are destroyed; swense_release does not.
  * - `stream` is a cudaStream_t passed as void* (NULL = legacy default stream). All device work
  *   is enqueued on it; calls return before it runs unless documented otherwise.
  * - Calls that overlap on the GPU (different streams, no ordering) race on the library's scratch
@@ -690,10 +692,12 @@ int swense_selftest_tc_gemm(const float* A, const float* B, float* D, int32_t N,
  */
 int swense_selftest_workspace_limit(int64_t bytes);
 
-/* Bytes of scratch workspace currently held on the current device. */
+/* Bytes of scratch workspace currently held on the current device, outgrown ones that captured graphs still
+ * use among them. */
 int64_t swense_workspace_bytes(void);
 
-/* Free the scratch workspace of the current device (synchronises the device). */
+/* Free the scratch workspace of the current device (synchronises the device). Graphs captured before must
+ * not be replayed afterwards. */
 int swense_release(void);
 
 /* One-line description of the calling thread's last error ("" if none). */

@@ -3,8 +3,10 @@
 #include <atomic>
 #include <cmath>
 #include <cstdint>
+#include <memory>
 #include <mutex>
 #include <string>
+#include <vector>
 
 #include "fft.cuh"
 #include "internal.cuh"
@@ -33,9 +35,19 @@ namespace {
 
 constexpr int kMaxDevices = 64;
 
+// A workspace and the captured graphs (and graphs instantiated from them) that hold its address: they use
+// it at every replay, so it lives as long as they do. Counted by user objects of the graphs.
+struct Scratch {
+  void* p = nullptr;
+  size_t bytes = 0;
+  std::shared_ptr<std::atomic<int>> graphs = std::make_shared<std::atomic<int>>(0);
+};
+
 struct DeviceState {
-  void* ws = nullptr;
-  size_t ws_bytes = 0;
+  Scratch ws;
+  // Outgrown while graphs held them; freed by the growth after the last of these is gone, or
+  // swense_release. Each is smaller by a quarter and more than the one after it.
+  std::vector<Scratch> kept;
   bool tw_ready = false;
   // Smallest optional request that could not be had, and how many more of at least its size are answered
   // so without another try: a failing allocation on every call would cost more than the larger scratch
@@ -74,7 +86,25 @@ int current_device(int* dev) {
 
 namespace {
 
-// A new workspace in place of the device's own, which is freed once the new one is there.
+void free_scratch(Scratch& s) {
+  cudaDeviceSynchronize();                       // work in flight may still use it
+  cudaFree(s.p);
+  s = Scratch{};
+}
+
+void free_unheld(DeviceState& d) {
+  for (size_t i = 0; i < d.kept.size();) {
+    if (d.kept[i].graphs->load() > 0) {
+      ++i;
+    } else {
+      free_scratch(d.kept[i]);
+      d.kept.erase(d.kept.begin() + i);
+    }
+  }
+}
+
+// A new workspace in place of the device's own, which is freed (unless a graph holds it) once the new one
+// is there.
 cudaError_t replace_workspace(DeviceState& d, size_t want) {
   void* p = nullptr;
   const cudaError_t e = want > d.limit ? cudaErrorMemoryAllocation : cudaMalloc(&p, want);
@@ -82,14 +112,42 @@ cudaError_t replace_workspace(DeviceState& d, size_t want) {
     cudaGetLastError();
     return e;
   }
-  if (d.ws) {
-    cudaDeviceSynchronize();                     // work in flight may still use the old one
-    cudaFree(d.ws);
+  if (d.ws.p) {
+    if (d.ws.graphs->load() > 0) d.kept.push_back(d.ws);
+    else free_scratch(d.ws);
   }
-  d.ws = p;
-  d.ws_bytes = want;
+  d.ws = Scratch{};
+  d.ws.p = p;
+  d.ws.bytes = want;
   if (want >= d.refused) d.refused = SIZE_MAX;
   return cudaSuccess;
+}
+
+void CUDART_CB drop_graph(void* held) {
+  auto* g = static_cast<std::shared_ptr<std::atomic<int>>*>(held);
+  --**g;
+  delete g;
+}
+
+// The workspace is used by work captured on `stream`: the graph holds it.
+int hold_for_capture(DeviceState& d, cudaStream_t stream) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaGraph_t graph = nullptr;
+  if (cudaStreamGetCaptureInfo(stream, &cap, nullptr, &graph, nullptr, nullptr, nullptr) != cudaSuccess) {
+    cudaGetLastError();                          // (the legacy stream beside a capture: its launch will say so)
+    return SWENSE_OK;
+  }
+  if (cap != cudaStreamCaptureStatusActive) return SWENSE_OK;
+  auto* held = new std::shared_ptr<std::atomic<int>>(d.ws.graphs);
+  ++**held;
+  cudaUserObject_t obj = nullptr;
+  const cudaError_t e = cudaUserObjectCreate(&obj, held, drop_graph, 1, cudaUserObjectNoDestructorSync);
+  if (e != cudaSuccess) {
+    drop_graph(held);
+    return cuda_fail(e, "cudaUserObjectCreate");
+  }
+  SWENSE_CUDA_TRY(cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove));
+  return SWENSE_OK;
 }
 
 int grow(size_t bytes, cudaStream_t stream, void** out, bool optional) {
@@ -99,9 +157,9 @@ int grow(size_t bytes, cudaStream_t stream, void** out, bool optional) {
   std::lock_guard<std::mutex> lock(g_mutex);
   DeviceState& d = g_dev[dev];
   bytes = (bytes + 255) & ~size_t(255);
-  if (bytes <= d.ws_bytes) {
-    *out = d.ws;
-    return SWENSE_OK;
+  if (bytes <= d.ws.bytes) {
+    *out = d.ws.p;
+    return hold_for_capture(d, stream);
   }
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   SWENSE_CUDA_TRY(cudaStreamIsCapturing(stream, &cap));
@@ -110,6 +168,7 @@ int grow(size_t bytes, cudaStream_t stream, void** out, bool optional) {
   if (capturing)
     return fail(SWENSE_ERR_ARG, "scratch workspace must grow, which is not allowed during stream "
                                 "capture; make one call with the same sizes before capturing");
+  free_unheld(d);
   const size_t want = bytes + bytes / 4;         // headroom so small growth does not reallocate
   cudaError_t e = replace_workspace(d, want);
   if (e != cudaSuccess && optional) {
@@ -117,17 +176,15 @@ int grow(size_t bytes, cudaStream_t stream, void** out, bool optional) {
     d.refusals_left = kRefusals;
     return SWENSE_ERR_OOM;
   }
-  if (e != cudaSuccess && d.ws) {                // no room for both: give up the old one first
-    SWENSE_CUDA_TRY(cudaDeviceSynchronize());
-    SWENSE_CUDA_TRY(cudaFree(d.ws));
-    d.ws = nullptr;
-    d.ws_bytes = 0;
+  if (e != cudaSuccess && d.ws.p && d.ws.graphs->load() == 0) {   // no room for both: give up the old one first
+    free_scratch(d.ws);
     e = replace_workspace(d, want);
   }
   if (e != cudaSuccess)
-    return fail(SWENSE_ERR_OOM, "cudaMalloc of the scratch workspace (" + std::to_string(want) +
-                                    " bytes) failed: " + cudaGetErrorString(e));
-  *out = d.ws;
+    return fail(SWENSE_ERR_OOM, "cudaMalloc of the scratch workspace (" + std::to_string(want) + " bytes) failed: " +
+                                    cudaGetErrorString(e) +
+                                    (d.ws.p || !d.kept.empty() ? "; captured graphs hold the present one" : ""));
+  *out = d.ws.p;
   return SWENSE_OK;
 }
 
@@ -170,7 +227,9 @@ int64_t swense_workspace_bytes(void) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= swense::kMaxDevices) return 0;
   std::lock_guard<std::mutex> lock(swense::g_mutex);
-  return int64_t(swense::g_dev[dev].ws_bytes);
+  size_t bytes = swense::g_dev[dev].ws.bytes;
+  for (const swense::Scratch& s : swense::g_dev[dev].kept) bytes += s.bytes;
+  return int64_t(bytes);
 }
 
 int swense_release(void) {
@@ -179,12 +238,10 @@ int swense_release(void) {
   if (dev < 0 || dev >= swense::kMaxDevices) return SWENSE_OK;
   std::lock_guard<std::mutex> lock(swense::g_mutex);
   swense::DeviceState& d = swense::g_dev[dev];
-  if (d.ws) {
-    SWENSE_CUDA_TRY(cudaDeviceSynchronize());
-    SWENSE_CUDA_TRY(cudaFree(d.ws));
-  }
-  d.ws = nullptr;
-  d.ws_bytes = 0;
+  if (d.ws.p) SWENSE_CUDA_TRY(cudaDeviceSynchronize());
+  if (d.ws.p) swense::free_scratch(d.ws);
+  for (swense::Scratch& s : d.kept) swense::free_scratch(s);
+  d.kept.clear();
   d.refused = SIZE_MAX;
   d.refusals_left = 0;
   return SWENSE_OK;

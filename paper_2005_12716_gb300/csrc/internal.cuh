@@ -23,7 +23,8 @@ int cuda_fail(cudaError_t e, const char* what);
 // ---------------------------------------------------------------- per-device scratch
 // Returns a device pointer to at least `bytes` bytes of scratch (256-byte aligned), growing the
 // device's workspace if needed. Growing synchronises the device and is refused during capture. The
-// old workspace is freed after the new one is had, or before it where there is no room for both.
+// old workspace is freed after the new one is had, or before it where there is no room for both; one that
+// captured graphs hold (a capture on `stream` makes its graph hold it) stays until they are gone.
 int workspace(size_t bytes, cudaStream_t stream, void** out);
 // The same for scratch a call can do without: where it cannot be had beside the present workspace, or
 // during a capture that would have to grow it, SWENSE_ERR_OOM and the workspace as it was.

@@ -119,3 +119,39 @@ def test_batch_with_less_scratch(env, limit):
     for it, w in zip(b.items, want):
         for k, v in w.items():
             assert float((it["out"][k] - v).abs().max()) <= 1e-5 * float(v.abs().max()), k
+
+
+def test_growth_keeps_the_workspace_of_a_captured_graph(env):
+    import gc
+    import time
+    torch, S, api = env
+    modes = _modes(api, 64, 32)
+    z = np.linspace(-1.0, 0.08, 12).astype(np.float32)
+    want = api.fields_on_grid(modes, z, 2, [0.0])
+    g = api.alloc_grid(modes, z, 2, [0.0])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        api.fields_on_grid(modes, z, 2, [0.0], out=g)
+    held = S.swense_workspace_bytes()
+    big = _modes(api, 256, 128)
+    api.fields_on_grid(big, z, 1, [0.0])                        # outgrows it
+    grown = S.swense_workspace_bytes()
+    assert grown > 2 * held
+    fill = [torch.full((held // 4,), float("nan"), device="cuda") for _ in range(8)]
+    g.nodes.fill_(float("nan"))
+    g.eta.fill_(float("nan"))
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(g.nodes, want.nodes) and torch.equal(g.eta, want.eta)
+    assert all(bool(torch.isnan(f).all()) for f in fill)
+    del graph
+    gc.collect()
+    torch.cuda.synchronize()
+    time.sleep(0.5)                                             # the graph lets go on a thread of the runtime's
+    api.fields_on_grid(_modes(api, 512, 256), z, 1, [0.0])
+    now = S.swense_workspace_bytes()
+    S.swense_release()
+    assert S.swense_workspace_bytes() == 0
+    api.fields_on_grid(_modes(api, 512, 256), z, 1, [0.0])
+    assert S.swense_workspace_bytes() == now                    # both outgrown ones had been given back
