@@ -175,9 +175,8 @@ int swense_fields_on_grid_noalloc(const swense_modes* modes, int32_t n_tl, const
 /*
  * swense_autotune_grid — choose the launch shape of swense_fields_on_grid for this grid shape
  * (the transform path: the wide-radix transform pair with 1, 2 or 4 levels per column-transform
- * block, or the shared-memory kernels; the level-chunk size among 16, 32, 64, 96, 128 and 256 MB, the
- * last of which stands for the default's chunks of up to 512 MB; and
- * the row pass's form) by
+ * block, or the shared-memory kernels; the level-chunk size among 16, 32, 64, 96, 128 and 256 MB (the
+ * default's chunks of up to 512 MB are not a candidate); and the row pass's form) by
  * timing each candidate five times on `stream` (best of five, each from a cold L2: the
  * workspace, grown to at least 256 MB, is overwritten before each repetition); the choice is
  * cached per (nx, ny, pad_n, nz)
@@ -202,8 +201,8 @@ int swense_autotune_grid(const swense_modes* modes, int32_t n_tl, const double* 
  * (nx, ny, pad_n, nz), e.g. a choice that swense_autotune_grid returned in an earlier process.
  * lpc: -1 (forget any choice: untuned defaults again), 0 (shared-memory path), 1, 2 or 4 levels
  * per column block;
- * chunk_bytes in [1 MiB, 1 GiB] (level chunk; 256 MiB: the default's, up to 512 MiB); row_variant 0..5, or 16 more (see
- * swense_autotune_grid). Results do not depend on the choice beyond FP32 rounding. No
+ * chunk_bytes in [1 MiB, 1 GiB] (level chunk; the untuned default's is 512 MiB); row_variant 0..5, or 16 more
+ * (see swense_autotune_grid). Results do not depend on the choice beyond FP32 rounding. No
  * counterpart in the paper. Errors: SWENSE_ERR_ARG for values outside those sets.
  */
 int swense_set_grid_tune(int32_t nx, int32_t ny, int32_t pad_n, int32_t nz, int32_t lpc,

@@ -327,8 +327,8 @@ constexpr size_t kSmemBudget = 64 * 1024;
 // Level chunks of at most 512 MB, of equal size: each pass pays its first and last wave of blocks (about
 // 20 us) once a chunk, which outweighs an intermediate that stays in L2 (2048 x 1024 modes, 256 levels:
 // 7.44 ms, 7.89 at 256 MB, 9.07 at 64 MB; 512 x 256 modes, 128 levels in one chunk instead of one and a
-// rest of two slots: 13 us less). The largest size a tuned choice names, 256 MB, stands for it too.
-constexpr size_t kChunkBytes = size_t(512) << 20, kChunkNominal = size_t(256) << 20;
+// rest of two slots: 13 us less).
+constexpr size_t kChunkBytes = size_t(512) << 20;
 constexpr int kColLevels = 1;   // levels per column-transform CTA
 
 int set_smem(const void* fn, size_t bytes) {
@@ -943,7 +943,6 @@ int grid_slots(const GridPlan& p, const Shape& s) {
 }
 
 int chunk_slots(const GridPlan& p, const Shape& s, size_t bytes) {
-  if (bytes == kChunkNominal) bytes = kChunkBytes;
   return int(std::max<size_t>(1, std::min<size_t>(size_t(grid_slots(p, s)), bytes / p.per_level)));
 }
 // The same number of chunks, of equal size: no short one at the end.
@@ -1486,7 +1485,7 @@ extern "C" int swense_autotune_grid(const swense_modes* md, int32_t n_tl, const 
     // evicts the grid): the workspace, sized for the largest candidate and at least twice the
     // L2, is overwritten before each repetition (its contents are scratch).
     constexpr size_t kFlushBytes = size_t(256) << 20;
-    const int max_chunk = chunk_slots(p, Shape{0, 1, 0}, kChunkBytes);
+    const int max_chunk = chunk_slots(p, Shape{0, 1, 0}, kFlushBytes);   // the largest candidate: 256 MB
     bool pp = pair_path(p.ny, p.Nxr, p.Nyr);
     size_t ws_all = 0;
     for (;; pp = false) {                        // the pair's candidates only where its scratch can be had
