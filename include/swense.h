@@ -362,7 +362,7 @@ enum swense_direct_precision {
  *   SWENSE_DIRECT_SPLIT_BF16_PAIRWISE: per (point, mode) pair the operand e^{i k.x} f(z) is
  *     generated in registers and split into BF16 hi + lo for legacy mma.sync m16n8k16 products
  *     (the same accuracy; kept for comparison and for tiles the tensor-core path leaves).
- * Uses the scratch workspace (FP32: 48 B per mode slot, rows padded to 64 modes, and at most
+ * Uses the scratch workspace (FP32: 96 B per mode of the rows n >= 0, in whole tiles of 64, and at most
  * 20 B per point and block of modes; SPLIT_BF16: 32 B per mode slot, 20 B
  * per point and 256 KB; PAIRWISE: 80 B per mode). Errors: ARG, SIZE, UNSUPPORTED, OOM, CUDA;
  * the tensor-core kernel's bounded waits report through swense_async_status.

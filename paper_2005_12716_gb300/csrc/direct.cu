@@ -96,20 +96,20 @@ struct PairCoef {
 };
 static_assert(sizeof(PairCoef) == 96, "pair record");
 
-constexpr int kDirTile = 64;    // pairs of one row |n| per tile
+constexpr int kDirTile = 64;    // pairs per tile: a part of one row |n|, or whole rows of fewer modes
 constexpr int kDirAnchor = 16;  // exact phase of theta every this many modes
 
-// Pairs in tiles: entry ((|n| tpr + m / kDirTile) kDirTile + m % kDirTile), zero past nx/2 - 1.
+// Pairs row by row, entry |n| nx/2 + m, zero past the last of them (n: whole tiles).
 __global__ void k_direct_prep(const float2* __restrict__ Ae, const float2* __restrict__ Ap,
                               const float2* __restrict__ At, const double* __restrict__ omega,
-                              double dt, int nx, int ny, float kxs, float kys, float depth, int tpr, int64_t n,
+                              double dt, int nx, int ny, float kxs, float kys, float depth, int64_t n_pairs, int64_t n,
                               PairCoef* __restrict__ out) {
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const int m = int(i % (tpr * kDirTile)), row = int(i / (tpr * kDirTile));
+  const int m = int(i % (nx / 2)), row = int(i / (nx / 2));
   PairCoef pc{};
   pc.invd = 1.f;
-  if (m < nx / 2) {
+  if (i < n_pairs) {
     const int nxh1 = nx / 2 + 1;
     const SlotCoef p = slot_coef(row * nxh1 + m, Ae, Ap, At, omega, dt, nx, ny, kxs, kys, depth);
     SlotCoef o{};                                  // the partner row -n (none for n = 0)
@@ -126,7 +126,8 @@ __global__ void k_direct_prep(const float2* __restrict__ Ae, const float2* __res
 
 struct DirectArgs {
   const PairCoef* pairs;
-  int n_tiles, tpr;          // tiles; tiles per row |n|
+  int n_tiles, rows;         // tiles; rows |n|
+  int mh, log_mh;            // modes per row |n| (a power of two)
   int tps;                   // tiles per split (blockIdx.y)
   const float* pts;
   float *o_eta, *o_u, *o_v, *o_w, *o_p;
@@ -155,6 +156,9 @@ __device__ __forceinline__ void direct_store(const DirectArgs& a, int64_t i, flo
   }
 }
 
+// A tile of 64 pairs holds a part of one row |n| or, where rows are shorter (2 to 32 modes), several whole
+// rows in turn; each took a tile of its own before, and a sea of 8 x 1024 modes 4.04 ms where one mode at a
+// time had taken 1.28 (100,003 points, deep water; 0.40 now).
 // Four points a thread: a pair's 22 coefficients come from shared memory as six 16-byte broadcasts,
 // which occupy the shared-memory port for 24 cycles a warp, against about 31 FP32 operations a point;
 // with one point a thread the port, not the FP32 pipe, would bound the kernel. blockIdx.y takes a
@@ -199,49 +203,55 @@ __global__ void __launch_bounds__(kDirThreads, 4) k_direct_fp32(DirectArgs a) {
       cp_async_wait<0>();
     }
     __syncthreads();
-    const PairCoef* tc = tile[t & 1];
-    const int n = t / a.tpr, m0 = (t - n * a.tpr) * kDirTile;
-    float2 acc[kDirPts][5];                        // (C, S) of each field
-#pragma unroll
-    for (int p = 0; p < kDirPts; ++p)
-#pragma unroll
-      for (int f = 0; f < 5; ++f) acc[p][f] = make_float2(0.f, 0.f);
+    const int seg = min(a.mh, kDirTile);           // the tile's modes of one row
 #pragma unroll 1
-    for (int j0 = 0; j0 < kDirTile; j0 += kDirAnchor) {
+    for (int s0 = 0; s0 < kDirTile; s0 += seg) {
+      const PairCoef* tc = tile[t & 1] + s0;
+      const int64_t e0 = int64_t(t) * kDirTile + s0;
+      const int n = int(e0 >> a.log_mh), m0 = int(e0 & (a.mh - 1));
+      if (n >= a.rows) break;
+      float2 acc[kDirPts][5];                      // (C, S) of each field
 #pragma unroll
-      for (int p = 0; p < kDirPts; ++p)            // exact phase m X (mod 2^32)
-        sincospif(2.f * (float(int(unsigned(m0 + j0) * X[p])) * 2.3283064365386963e-10f), &sn[p], &cs[p]);
+      for (int p = 0; p < kDirPts; ++p)
+#pragma unroll
+        for (int f = 0; f < 5; ++f) acc[p][f] = make_float2(0.f, 0.f);
 #pragma unroll 1
-      for (int j = j0; j < j0 + kDirAnchor; ++j) {
-        const PairCoef& c = tc[j];
-        const float4 qe = c.q[0], qu = c.q[1], qv = c.q[2], qw = c.q[3], qt = c.q[4];
-        const float k = c.k, invd = FINITE ? c.invd : 1.f;
+      for (int j0 = 0; j0 < seg; j0 += kDirAnchor) {
 #pragma unroll
-        for (int p = 0; p < kDirPts; ++p) {
-          float F, S;
-          direct_depth<FINITE>(k, z[p], a.depth, invd, F, S);
-          auto add = [&](float2& s, const float4& q, float cc, float ss) {
-            s = pfma(make_float2(cc, cc), make_float2(q.x, q.y), s);
-            s = pfma(make_float2(ss, ss), make_float2(q.z, q.w), s);
-          };
-          const float fc = F * cs[p], fs = F * sn[p];
-          add(acc[p][0], qe, cs[p], sn[p]);
-          add(acc[p][1], qu, fc, fs);
-          add(acc[p][2], qv, fc, fs);
-          add(acc[p][3], qw, FINITE ? S * cs[p] : fc, FINITE ? S * sn[p] : fs);
-          add(acc[p][4], qt, fc, fs);
-          const float c2 = fmaf(cs[p], cst[p], -sn[p] * sst[p]);
-          sn[p] = fmaf(sn[p], cst[p], cs[p] * sst[p]);
-          cs[p] = c2;
+        for (int p = 0; p < kDirPts; ++p)          // exact phase m X (mod 2^32)
+          sincospif(2.f * (float(int(unsigned(m0 + j0) * X[p])) * 2.3283064365386963e-10f), &sn[p], &cs[p]);
+#pragma unroll 1
+        for (int j = j0; j < min(j0 + kDirAnchor, seg); ++j) {
+          const PairCoef& c = tc[j];
+          const float4 qe = c.q[0], qu = c.q[1], qv = c.q[2], qw = c.q[3], qt = c.q[4];
+          const float k = c.k, invd = FINITE ? c.invd : 1.f;
+#pragma unroll
+          for (int p = 0; p < kDirPts; ++p) {
+            float F, S;
+            direct_depth<FINITE>(k, z[p], a.depth, invd, F, S);
+            auto add = [&](float2& s, const float4& q, float cc, float ss) {
+              s = pfma(make_float2(cc, cc), make_float2(q.x, q.y), s);
+              s = pfma(make_float2(ss, ss), make_float2(q.z, q.w), s);
+            };
+            const float fc = F * cs[p], fs = F * sn[p];
+            add(acc[p][0], qe, cs[p], sn[p]);
+            add(acc[p][1], qu, fc, fs);
+            add(acc[p][2], qv, fc, fs);
+            add(acc[p][3], qw, FINITE ? S * cs[p] : fc, FINITE ? S * sn[p] : fs);
+            add(acc[p][4], qt, fc, fs);
+            const float c2 = fmaf(cs[p], cst[p], -sn[p] * sst[p]);
+            sn[p] = fmaf(sn[p], cst[p], cs[p] * sst[p]);
+            cs[p] = c2;
+          }
         }
       }
-    }
 #pragma unroll
-    for (int p = 0; p < kDirPts; ++p) {
-      float sy, cy;
-      sincospif(2.f * (float(int(unsigned(n) * Y[p])) * 2.3283064365386963e-10f), &sy, &cy);
+      for (int p = 0; p < kDirPts; ++p) {
+        float sy, cy;
+        sincospif(2.f * (float(int(unsigned(n) * Y[p])) * 2.3283064365386963e-10f), &sy, &cy);
 #pragma unroll
-      for (int f = 0; f < 5; ++f) tot[p][f] += fmaf(cy, acc[p][f].x, sy * acc[p][f].y);
+        for (int f = 0; f < 5; ++f) tot[p][f] += fmaf(cy, acc[p][f].x, sy * acc[p][f].y);
+      }
     }
     __syncthreads();                               // tile (t & 1) is reloaded next iteration
   }
@@ -674,8 +684,7 @@ extern "C" int swense_direct(const swense_modes* md, double t, const float* pts,
   if (precision == SWENSE_DIRECT_SPLIT_BF16_PAIRWISE)
     return direct_split_impl(md, t, pts, nullptr, nullptr, 0, np, eta, u, v, w, p, p_mode, rho, grav, stream, 0);
   const int rows = ny > 1 ? ny / 2 : 1;           // |n| = 0 .. ny/2 - 1 (the Nyquist row is ignored)
-  const int tpr = (nx / 2 + kDirTile - 1) / kDirTile;
-  const int64_t n_tiles = int64_t(rows) * tpr, n_pairs = n_tiles * kDirTile;
+  const int64_t n_pairs = int64_t(rows) * (nx / 2), n_tiles = (n_pairs + kDirTile - 1) / kDirTile;
   if (n_tiles >= (int64_t(1) << 31)) return fail(SWENSE_ERR_SIZE, "too many modes for one call");
   const int64_t blocks = (np + kDirThreads * kDirPts - 1) / (kDirThreads * kDirPts);
   if (blocks >= (int64_t(1) << 31)) return fail(SWENSE_ERR_SIZE, "too many points for one call");
@@ -687,24 +696,26 @@ extern "C" int swense_direct(const swense_modes* md, double t, const float* pts,
   const int64_t want = std::max<int64_t>(1, (int64_t(sms) * 12 + blocks - 1) / blocks);
   const int64_t tps = (n_tiles + std::min(want, n_tiles) - 1) / std::min(want, n_tiles);
   const int splits = int((n_tiles + tps - 1) / tps);
-  const size_t b_pairs = (size_t(n_pairs) * sizeof(PairCoef) + 255) & ~size_t(255);
+  const size_t b_pairs = size_t(n_tiles) * kDirTile * sizeof(PairCoef);
   const size_t b_part = splits > 1 ? size_t(splits) * 5 * size_t(np) * sizeof(float) : 0;
   void* ws = nullptr;
   int st = workspace(b_pairs + b_part, stream, &ws);
   if (st) return st;
   PairCoef* pairs = static_cast<PairCoef*>(ws);
   const float depth = md->depth > 0 ? float(md->depth) : 0.f;
-  k_direct_prep<<<unsigned((n_pairs + 255) / 256), 256, 0, stream>>>(
+  k_direct_prep<<<unsigned((n_tiles * kDirTile + 255) / 256), 256, 0, stream>>>(
       reinterpret_cast<const float2*>(md->A_eta), reinterpret_cast<const float2*>(md->A_phi),
       reinterpret_cast<const float2*>(md->A_phit), md->omega, t - md->t_ref, nx, ny,
       float(6.283185307179586476925 / md->Lx), ny > 1 ? float(6.283185307179586476925 / md->Ly) : 0.f,
-      depth, tpr, n_pairs, pairs);
+      depth, n_pairs, n_tiles * kDirTile, pairs);
   SWENSE_CUDA_TRY(cudaGetLastError());
   count_launches(1);
   DirectArgs a{};
   a.pairs = pairs;
   a.n_tiles = int(n_tiles);
-  a.tpr = tpr;
+  a.mh = nx / 2;
+  a.log_mh = ilog2(nx / 2);
+  a.rows = rows;
   a.tps = int(tps);
   a.pts = pts;
   a.o_eta = eta;
