@@ -1454,10 +1454,16 @@ __device__ __forceinline__ void learned_store_a(uint32_t lanes, int hf, const fl
   tc::st_x16(lanes + 32u + 16u * hf, lo);
 }
 
+// PARTS: `parts` blocks a chunk (learned_parts), each with its share of the points and its own tile.
+template <bool PARTS>
 __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_constant__ InterpArgs a, const __grid_constant__ Levels L,
                                                                     const int4* __restrict__ plan,
-                                                                    const PackedFwd* __restrict__ Wg, LearnedWaits waits) {
+                                                                    const PackedFwd* __restrict__ Wg, LearnedWaits waits, int parts) {
   using namespace mlpnet;
+  const int chunk = PARTS ? int(blockIdx.x) / parts : int(blockIdx.x);
+  const int per = BOX_PTS / (LRN_WG * (PARTS ? parts : 1));   // points of a warpgroup
+  const int64_t p0 = int64_t(chunk) * BOX_PTS, pb = PARTS ? p0 + int64_t(int(blockIdx.x) % parts) * (LRN_WG * per) : p0;
+  if (PARTS && pb >= a.np) return;                     // uniform over the block
   extern __shared__ float4 sbox[];
   float* seta = reinterpret_cast<float*>(sbox + BOX_NODES);
   LPoint* recs = reinterpret_cast<LPoint*>(seta + BOX_COLS);
@@ -1487,8 +1493,7 @@ __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_
     tc::alloc(&W.tmem, LRN_WG * LRN_COLS);
     tc::relinquish();
   }
-  const int64_t p0 = int64_t(blockIdx.x) * BOX_PTS;
-  const int4 pl = plan[blockIdx.x];
+  const int4 pl = plan[chunk];
   const BoxPlan bp = decode_plan(pl);
   const int bx = bp.bx, by = bp.by;
   const int sbx = bx + ((4 - bx) & 7);
@@ -1522,7 +1527,7 @@ __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_
   const float* nf = reinterpret_cast<const float*>(boxed ? sbox : own) + f;
   const int SY = boxed ? sbx : 4, SZ = boxed ? zst : 16;
   const int SB = boxed ? LRN_SB : LRN_SB_PP;
-  const int64_t q0 = p0 + int64_t(wg) * (BOX_PTS / LRN_WG);
+  const int64_t q0 = pb + int64_t(wg) * per;
   unsigned ph = 0;
   bool bad = false;
   // every thread of the warpgroup has its share of the operands in place -> the accumulators are ready
@@ -1538,8 +1543,9 @@ __global__ void __launch_bounds__(BOX_THREADS, 2) k_interp_learned(const __grid_
     __syncwarp();
     tc::fence_after();
   };
-  for (int s0 = 0; s0 < BOX_PTS / LRN_WG; s0 += SB) {
-    const int npts = int(a.np - (q0 + s0) < int64_t(SB) ? a.np - (q0 + s0) : int64_t(SB));
+  for (int s0 = 0; s0 < per; s0 += SB) {
+    int npts = int(a.np - (q0 + s0) < int64_t(SB) ? a.np - (q0 + s0) : int64_t(SB));
+    if (PARTS) npts = min(npts, per - s0);
     if (npts <= 0) break;                              // uniform over the warpgroup
     // ---- A
     auto record = [&](LPoint& P, const PointCell& c, float px, float py, float pz, int base, float e) {
@@ -1910,6 +1916,18 @@ namespace {
 std::mutex g_learned_selftest_mutex;
 bool g_learned_selftest[64];      // per device (swense_selftest_learned_wait_timeout)
 
+// Blocks a chunk. A chunk is a chain of sixteen 32-point steps for each warpgroup, 0.19 ms, which a set of few
+// chunks waits for whole (500 points: 191 us, with warp MMAs 150 before; 30 us in 16 parts), and a grid of one
+// wave of blocks and a little takes two. So chunks are split, down to one step a warpgroup, up to five waves
+// of blocks: 400,000 points in two parts 622 -> 485 us, 200,000 in four 346 -> 264. More waves would still
+// help points of their own stencils, but every part stages its chunk's box again (400,000 points on a grid of
+// 64 x 32 nodes: 195 us whole, 197 in two parts, 209 in four).
+int learned_parts(int64_t chunks, int64_t slots) {
+  int parts = 1;
+  while (parts < BOX_PTS / (LRN_WG * 32) && chunks * parts * 2 <= 5 * slots) parts *= 2;
+  return parts;
+}
+
 int learned_waits(LearnedWaits* w) {
   int dev = 0;
   SWENSE_CUDA_TRY(cudaGetDevice(&dev));
@@ -1975,13 +1993,18 @@ extern "C" int swense_interp_learned(const swense_grid* g, double t, const float
     int4* plan = reinterpret_cast<int4*>(static_cast<char*>(ws) + 256);
     k_interp_plan<true><<<unsigned(plan_blocks(np)), BOX_THREADS, 0, stream>>>(a, lev, plan);
     SWENSE_CUDA_TRY(cudaGetLastError());
-    SWENSE_CUDA_TRY(cudaFuncSetAttribute((const void*)k_interp_learned,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, int(LRN_SMEM)));
+    int dev = 0, sms = 0;
+    SWENSE_CUDA_TRY(cudaGetDevice(&dev));
+    SWENSE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int parts = learned_parts(blocks, 2 * sms);
+    const auto kernel = parts > 1 ? k_interp_learned<true> : k_interp_learned<false>;
+    SWENSE_CUDA_TRY(cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         int(LRN_SMEM)));
     LearnedWaits waits;
     st = learned_waits(&waits);
     if (st) return st;
-    k_interp_learned<<<unsigned(blocks), BOX_THREADS, LRN_SMEM, stream>>>(
-        a, lev, plan, static_cast<const PackedFwd*>(packed), waits);
+    kernel<<<unsigned(blocks * parts), BOX_THREADS, LRN_SMEM, stream>>>(
+        a, lev, plan, static_cast<const PackedFwd*>(packed), waits, parts);
     SWENSE_CUDA_TRY(cudaGetLastError());
     count_launches(2);
   }
