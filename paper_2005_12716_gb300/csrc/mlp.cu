@@ -79,7 +79,7 @@ __device__ __forceinline__ void load_x(const float* __restrict__ x, int64_t row0
 // Inference: y[row] = network(x[row])[row % 4] (rows ordered point-major, fields u, v, w, phit).
 __global__ void __launch_bounds__(128) k_mlp_forward(const Packed* __restrict__ P, const float* __restrict__ x,
                                                      int64_t rows, float* __restrict__ y) {
-  __shared__ Packed s;
+  __shared__ __align__(16) Packed s;               // copied and read (ldmatrix) in 16-byte rows
   {
     const uint4* src = reinterpret_cast<const uint4*>(P);
     uint4* dst = reinterpret_cast<uint4*>(&s);
