@@ -847,6 +847,7 @@ __global__ void __launch_bounds__(BOX_THREADS, 5) k_interp_global(const __grid_c
 // their levels and lists the chunks that read planes and those with a staged tile, for persistent
 // kernels, so that an empty list costs a launch; k_interp_global takes the rest in point order.
 // 8.2 M mesh points on the four-fold padded 512 x 256 grid: 1.02 ms straight from the grid, 0.48 ms so (planes 0.13, gather 0.24 of it).
+// 3-D grids only: a 2-D one has too few nodes for the rule.
 constexpr int64_t LAYER_POINTS = int64_t(1) << 21;
 constexpr int PLANE_SLOTS = 4096;                  // planes at most (hash table entries)
 constexpr int PLANE_UNIT = BOX_THREADS;            // a plane's columns are padded to whole units
@@ -907,8 +908,8 @@ __global__ void __launch_bounds__(256) k_gather_register(const __grid_constant__
   int2 sl = make_int2(-1, -1);
   const int bx = pl.w >= 0 ? pl.w & 4095 : pl.w & 16383, by = pl.w >= 0 ? (pl.w >> 12) & 4095 : (pl.w >> 14) & 16383;
   // (a plan of another grid may hold boxes that no stencil of this one fits)
-  if (pl.w != -1 && (pl.z & FLAT_BIT) && bx >= 4 && (a.Nyr > 1 ? by >= 4 : by == 1)) {
-    const int rx = wrap_rel<P2>(pl.x, plan[0].x, a.Nxr), ry = a.Nyr > 1 ? wrap_rel<P2>(pl.y, plan[0].y, a.Nyr) : 0;
+  if (pl.w != -1 && (pl.z & FLAT_BIT) && bx >= 4 && by >= 4) {
+    const int rx = wrap_rel<P2>(pl.x, plan[0].x, a.Nxr), ry = wrap_rel<P2>(pl.y, plan[0].y, a.Nyr);
     const int64_t p0 = int64_t(c) * BOX_PTS, p1 = p0 + BOX_PTS < a.np ? p0 + BOX_PTS : a.np;
     const int n = int(p1 - p0);
     const bool two = pl.z & FLAT2_BIT;
@@ -1102,7 +1103,7 @@ __global__ void __launch_bounds__(BOX_THREADS, 4) k_plane_collapse(const __grid_
     // threads past the box's end repeat its last column and store nothing
     const int ci = (u - e.unit0) * PLANE_UNIT + int(threadIdx.x), c = min(ci, e.bx * e.by - 1);
     const int cy = e.ry + c / e.bx, cx = e.rx + c % e.bx;     // relative to chunk 0's box
-    const size_t col = size_t(a.Nyr > 1 ? wrapi<P2>(ref.y + cy, a.Nyr) : 0) * a.Nxr + wrapi<P2>(ref.x + cx, a.Nxr);
+    const size_t col = size_t(wrapi<P2>(ref.y + cy, a.Nyr)) * a.Nxr + wrapi<P2>(ref.x + cx, a.Nxr);
     PointCell pc;
     point_level(a, T, __uint_as_float(~g.slots[g.members[e.first]].key), pc);
     const float4* src = a.nodes + size_t(pc.j0) * plane + col;
@@ -1162,7 +1163,6 @@ template <bool P2, int WPTS>
 __device__ __forceinline__ void plane_warp(const InterpArgs& a, const Levels& L, const GatherLists& g, int4 ref, int2 sl,
                                            int64_t p0, GatherRec* rec) {
   const int lane = threadIdx.x & 31, k = lane & 3;
-  const bool two_d = a.Nyr == 1;
   const int64_t i = p0 + lane;
   float z = 0.f;
   if (WPTS == 32 || lane < WPTS) {
@@ -1174,7 +1174,7 @@ __device__ __forceinline__ void plane_warp(const InterpArgs& a, const Levels& L,
     int rx, ry, bx, by;
     plane_box(a, s, rx, ry, bx, by);
     const int lx = min(max(wrapi<P2>(c.ix - 1 - (ref.x + rx), a.Nxr), 0), bx - 4);
-    const int ly = two_d ? 0 : min(max(wrapi<P2>(c.iy - 1 - (ref.y + ry), a.Nyr), 0), by - 4);
+    const int ly = min(max(wrapi<P2>(c.iy - 1 - (ref.y + ry), a.Nyr), 0), by - 4);
     GatherRec& r = rec[lane];
     r.cell = make_int4(s.off + ly * bx + lx, bx, 0, 0);
     r.wy = make_float4(c.wy[0], c.wy[1], c.wy[2], c.wy[3]);
@@ -1192,7 +1192,6 @@ __device__ __forceinline__ void plane_warp(const InterpArgs& a, const Levels& L,
     float e = 0.f;
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
-      if (b > 0 && two_d) break;
       const int o = c.x + b * c.y + k;
       const float4 v = __ldg(&g.cols[o]);
       const unsigned long long w2 = pack2(wyb[b], wyb[b]);
@@ -2087,7 +2086,7 @@ int interp_impl(const swense_grid* g, double t, const float* pts, const int32_t*
   // sparse point sets (fewer points than a quarter of a time level's nodes): a chunk's stencils rarely
   // fit a tile
   const bool sparse = double(np) < 0.25 * double(a.Nxr) * double(a.Nyr) * double(a.nz);
-  bool kinds = sparse && np >= LAYER_POINTS && blocks < (int64_t(1) << 31) / (BOX_PTS / GLOBAL_PTS);
+  bool kinds = sparse && a.Nyr > 1 && np >= LAYER_POINTS && blocks < (int64_t(1) << 31) / (BOX_PTS / GLOBAL_PTS);
   void* ws = nullptr;
   st = kinds ? workspace_optional(b_plan + lists_bytes(np, blocks), stream, &ws) : SWENSE_OK;
   if (st || !kinds) {
