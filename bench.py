@@ -299,8 +299,9 @@ def job_throughput(units_per_rank, world, ms_per_step):
     return world * units_per_rank / (ms_per_step * 1e-3)
 
 
-GATHER_SOURCES = ("csrc/interp.cu", "csrc/internal.cuh")
-GRID_SOURCES = ("csrc/grid_ifft.cu", "csrc/fft.cuh", "csrc/internal.cuh")
+GATHER_SOURCES = ("csrc/interp.cu", "csrc/internal.cuh", "csrc/mlp.cuh", "csrc/mma.cuh", "csrc/tcgen05.cuh",
+                  "csrc/tma.cuh")
+GRID_SOURCES = ("csrc/grid_ifft.cu", "csrc/fft.cuh", "csrc/internal.cuh", "csrc/tma.cuh")
 GRID_STAGE = "grid_ifft (stage 1: k_form_modes, k_col_w, k_row_w)"
 
 
@@ -317,9 +318,24 @@ def kernel_source_hash(files=GATHER_SOURCES):
     return h.hexdigest()[:16]
 
 
+# The untuned launch shape of the transform stage.
+DEFAULT_SHAPE = {"lpc": 1, "chunk_bytes": 512 << 20, "row_variant": 0}
+
+
+def captured_traffic(tr, source_hash, workload, shape=None):
+    """Bytes of an NCU_TRAFFIC entry, or None where its kernel sources, workload or (for the transform
+    stage: ``shape``, None if untuned) launch shape are not those of this run."""
+    if not tr or tr.get("hash") != source_hash or tr.get("workload") != workload:
+        return None
+    ran = shape or DEFAULT_SHAPE
+    if "taken_with" in tr and any(ran.get(k) != v for k, v in tr["taken_with"].items()):
+        return None
+    return tr["bytes"]
+
+
 # DRAM bytes per launch from ncu captures (dram__bytes_read.sum + dram__bytes_write.sum), with
-# the hash of the kernel's sources and the workload they were taken on; a changed kernel or
-# workload invalidates them (traffic is then reported as null).
+# the hash of the kernel's sources and the workload they were taken on; a changed kernel,
+# workload or launch shape invalidates them (traffic is then reported as null).
 NCU_TRAFFIC = {
     "k_interp_box": {"bytes": 105900000 + 127300000, "hash": "92ee0328a2d6767e",
                      "workload": "jonswap3d: 512x256 modes, 64 levels, pad 1, 2 time levels, "
@@ -327,14 +343,14 @@ NCU_TRAFFIC = {
     # the three launches of one step, caches kept between them (--cache-control none), untuned launch
     # shape: one chunk of 130 slots, whose intermediate goes through memory
     GRID_STAGE: {"bytes": 6300000 + 266600000 + 527600000, "hash": "1e958107ea5274bd",
-                 "taken_with": {"lpc": 1, "chunk_bytes": 512 << 20, "row_variant": 0},
+                 "taken_with": DEFAULT_SHAPE,
                  "workload": "jonswap3d: 512x256 modes, 64 levels, pad 1, 2 time levels, "
                              "2048000 cell + 6177280 face centres (cylinder O-grid)"},
 }
 
 
 DIRECT_KERNEL = "k_direct_tc"
-DIRECT_SOURCES = ("csrc/direct_tc.cu", "csrc/tcgen05.cuh", "csrc/tma.cuh", "csrc/internal.cuh")
+DIRECT_SOURCES = ("csrc/direct_tc.cu", "csrc/tcgen05.cuh", "csrc/tma.cuh", "csrc/mma.cuh", "csrc/internal.cuh")
 NCU_TRAFFIC[DIRECT_KERNEL] = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum (caches flushed before the launch),
     # one launch: 1,000,000 near-body points x the 2048 x 1024-mode sea (sources since changed
@@ -510,7 +526,7 @@ def run_ours(args, rank, world, emit=True):
         # the stage as a whole (all its launches of one step, one stream or two)
         kname, dom_bytes, dom_ms, dom_hash = GRID_STAGE, k1_bytes, k1_ms, grid_hash
     tr = NCU_TRAFFIC.get(kname)
-    traffic = tr["bytes"] if tr and tr.get("hash") == dom_hash and tr.get("workload") == desc else None
+    traffic = captured_traffic(tr, dom_hash, desc, tune)
     achieved = dom_bytes / (dom_ms * 1e-3) / 1e9
     roofline = {"bound": "hbm", "kernel": kname, "achieved": achieved, "peak": hbm, "unit": "GB/s",
                 "frac": achieved / hbm, "traffic": traffic,
