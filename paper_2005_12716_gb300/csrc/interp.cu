@@ -254,9 +254,15 @@ static_assert(size_t(FLAT2_COLS) * (2 * sizeof(float4) + sizeof(float)) <= BOX_S
 //   two z:    w = bx | by << 12, z = FLAT_BIT | FLAT2_BIT (the z values are those of the chunk's
 //             first and last points; their level windows are looked up by the gather)
 //   neither fits the tile: w < 0 (global gathers): -1, or for one or two z values the extents all the
-//             same, w = 1 << 31 | bx | by << 14, z = FLAT_BIT (| FLAT2_BIT)
+//             same, w = 1 << 31 | bx | by << 14, z = FLAT_BIT (| FLAT2_BIT); ROWS_BIT of z besides where the
+//             points follow one another along the grid's rows
 constexpr int FLAT_BIT = 1 << 30;
 constexpr int FLAT2_BIT = 1 << 29;
+constexpr int ROWS_BIT = 1 << 28;
+// ROWS_BIT: the chunk's box spans half the grid's row length and more, and its first 32 points go ROWS_RATIO times
+// as far along x as along y. So do layers (45 and more), and points binned by rows of tiles (18 and more); points
+// close by in all directions (Morton order, the cells of a mesh) and points in no order do not.
+constexpr int ROWS_RATIO = 6;
 struct BoxPlan {
   int x0, y0, l0, bx, by, bz;
   bool flat;     // z-collapsed plane
@@ -551,6 +557,7 @@ __device__ __forceinline__ void plan_chunk(const InterpArgs& a, const LevelTable
   int two_z = 1;                                    // every point at refz or at the last point's z
   const float lastz = __ldg(&a.pts[3 * ((p0 + BOX_PTS < a.np ? p0 + BOX_PTS : a.np) - 1) + 2]);
   int mn[3] = {1 << 30, 1 << 30, 1 << 30}, mx[3] = {-(1 << 30), -(1 << 30), -(1 << 30)};
+  int first_x = 0, first_y = 0;                     // the lane's point of the chunk's first 32
   // four points per lane per round, their twelve loads issued before any of them is used
   constexpr int PU = 4;
   static_assert((BOX_PTS / 32) % PU == 0, "whole rounds");
@@ -587,9 +594,15 @@ __device__ __forceinline__ void plan_chunk(const InterpArgs& a, const LevelTable
         mx[1] = max(mx[1], ry);
         mn[2] = min(mn[2], c.j0);
         mx[2] = max(mx[2], c.j0);
+        if (k0 == 0 && u == 0) {
+          first_x = rx;
+          first_y = ry;
+        }
       }
     }
   }
+  const int far_x = __reduce_max_sync(0xffffffffu, first_x) - __reduce_min_sync(0xffffffffu, first_x);
+  const int far_y = __reduce_max_sync(0xffffffffu, first_y) - __reduce_min_sync(0xffffffffu, first_y);
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     for (int o = 16; o > 0; o >>= 1) {
@@ -610,14 +623,15 @@ __device__ __forceinline__ void plan_chunk(const InterpArgs& a, const LevelTable
   const bool fits = int64_t(zst) * bz <= NODES && int64_t(sbx) * by <= NODES / 4 && bx < 2048 && by < 2048;
   const bool fits_flat = flat && int64_t(sbx) * by <= FLAT_COLS;
   const bool fits_two = flat2 && int64_t(sbx) * by <= FLAT2_COLS;
+  const int rows = 2 * bx >= a.Nxr && far_x > ROWS_RATIO * far_y ? ROWS_BIT : 0;
   const int x0 = wrapi<P2>(refx + mn[0] - 1, a.Nxr);
   const int y0 = a.Nyr > 1 ? wrapi<P2>(refy + mn[1] - 1, a.Nyr) : 0;
   plan[chunk] = fits_flat  ? make_int4(x0, y0, mn[2] | FLAT_BIT, bx | (by << 12))
               : fits_two   ? make_int4(x0, y0, FLAT_BIT | FLAT2_BIT, bx | (by << 12))
               : fits       ? make_int4(x0, y0, mn[2], bx | (by << 11) | (bz << 22))
               : flat || flat2
-                  ? make_int4(x0, y0, flat ? FLAT_BIT : FLAT_BIT | FLAT2_BIT, int(0x80000000u | unsigned(bx) | unsigned(by) << 14))
-                  : make_int4(x0, y0, mn[2], -1);
+                  ? make_int4(x0, y0, rows | (flat ? FLAT_BIT : FLAT_BIT | FLAT2_BIT), int(0x80000000u | unsigned(bx) | unsigned(by) << 14))
+                  : make_int4(x0, y0, rows | mn[2], -1);
 }
 
 template <bool P2>
@@ -636,6 +650,9 @@ __device__ __forceinline__ bool plan_is_global(const int4 pl, int nz) {
   const BoxPlan bp = decode_plan(pl);
   return bp.l0 + bp.bz > nz;
 }
+
+// Chunks for k_interp_lanes, where that runs.
+__device__ __forceinline__ bool plan_is_lanes(const int4 pl, int nz) { return plan_is_global(pl, nz) && pl.w < 0 && (pl.z & ROWS_BIT); }
 
 // The chunk's points gathered from global memory, 32 at a time by each warp; rec: 32 records per warp.
 static_assert(BOX_THREADS * sizeof(GatherRec) <= BOX_SMEM, "the records fit the tile's shared memory");
@@ -818,7 +835,7 @@ __global__ void __launch_bounds__(BOX_THREADS, 3) k_interp_box(const __grid_cons
 // registers, five CTAs per SM): more of them evict each other's lines from L1 (5.8 ms with sixteen).
 constexpr int GLOBAL_WPTS = 16;
 constexpr int GLOBAL_PTS = GLOBAL_WPTS * (BOX_THREADS / 32);     // points per CTA
-template <bool P2>
+template <bool P2, bool LANES = false>
 __global__ void __launch_bounds__(BOX_THREADS, 5) k_interp_global(const __grid_constant__ InterpArgs a,
                                                                        const __grid_constant__ Levels L,
                                                                        const int4* __restrict__ plan,
@@ -831,10 +848,97 @@ __global__ void __launch_bounds__(BOX_THREADS, 5) k_interp_global(const __grid_c
   // by kinds (NULL otherwise), whose other kernels took the chunks with a plane
   if (n_global && *n_global == 0) return;
   if (p0 >= a.np || (plan && !plan_is_global(plan[p0 / BOX_PTS], a.nz))) return;
+  if (LANES && plan_is_lanes(plan[p0 / BOX_PTS], a.nz)) return;   // k_interp_lanes takes those
   if (chunk_slot && chunk_slot[p0 / BOX_PTS].x >= 0) return;
 #pragma unroll 1
   for (int r = 0; r < rounds && p0 < a.np; ++r, p0 += GLOBAL_PTS)   // within one chunk
     gather_warp<P2, GLOBAL_WPTS>(a, *level_tables(L), p0, rec + warp * GLOBAL_WPTS);
+}
+
+// Untiled chunks whose points follow the grid's rows, on grids whose four levels of all time levels exceed
+// L2: a point a lane. Nothing is met again in L1 or L2 there, so DRAM bounds them, and a lane's load asks
+// for one sector where a quad's asks for the two or three of a stencil row, which L2 fetches in pairs: 77
+// instead of 112 bytes a row (2 M binned points on the four-fold padded 512 x 256 grid: 2.46 against 3.57
+// GB of DRAM reads, 440 against 541 us a time level). Points in no order pay for a lane's 32 pages a load
+// (1.74 ms by quads, 3.27 by lanes, the same grid), points close by in all directions meet in L1 (16 M in
+// Morton order on the large sea: 2.9 against 5.2 ms), and on grids that fit L2 quads win too.
+template <bool P2>
+__device__ __forceinline__ void lane_point(const InterpArgs& a, const LevelTables& T, int64_t i) {
+  const float z = __ldg(&a.pts[3 * i + 2]);
+  const PointCell c = point_cell<P2>(a, T, __ldg(&a.pts[3 * i]), __ldg(&a.pts[3 * i + 1]), z);
+  const size_t plane = size_t(a.Nyr) * a.Nxr;
+  int xi[4], yo[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    xi[q] = wrapi<P2>(c.ix - 1 + q, a.Nxr);
+    yo[q] = wrapi<P2>(c.iy - 1 + q, a.Nyr) * a.Nxr;
+  }
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  float e = 0.f;
+  for (int tl = 0; tl < a.n_tl; ++tl) {
+    const float wtl = a.wt[tl];
+    const float4* base = a.nodes + (size_t(tl) * a.nz + c.j0) * plane;
+    const float* et = a.eta + size_t(tl) * plane;
+#pragma unroll 1
+    for (int q = 0; q < 4; ++q) {
+      const float wq = wtl * (q == 0 ? c.wz[0] : q == 1 ? c.wz[1] : q == 2 ? c.wz[2] : c.wz[3]);
+#pragma unroll 1
+      for (int b = 0; b < 4; ++b) {                // a select, so that the weights stay in registers
+        const float wqy = wq * (b == 0 ? c.wy[0] : b == 1 ? c.wy[1] : b == 2 ? c.wy[2] : c.wy[3]);
+        const float4* row = base + size_t(q) * plane + (b == 0 ? yo[0] : b == 1 ? yo[1] : b == 2 ? yo[2] : yo[3]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float4 g = __ldg(&row[xi[k]]);
+          const float w = wqy * c.wx[k];
+          acc.x = fmaf(w, g.x, acc.x);
+          acc.y = fmaf(w, g.y, acc.y);
+          acc.z = fmaf(w, g.z, acc.z);
+          acc.w = fmaf(w, g.w, acc.w);
+        }
+      }
+    }
+#pragma unroll 1
+    for (int b = 0; b < 4; ++b) {
+      const float wy = wtl * (b == 0 ? c.wy[0] : b == 1 ? c.wy[1] : b == 2 ? c.wy[2] : c.wy[3]);
+      const float* row = et + (b == 0 ? yo[0] : b == 1 ? yo[1] : b == 2 ? yo[2] : yo[3]);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) e = fmaf(wy * c.wx[k], __ldg(&row[xi[k]]), e);
+    }
+  }
+  store_point(a, i, acc, e, z, c.inside);
+}
+
+// A quarter of a chunk a block, in point order: what the points in flight read then spans few enough of them that
+// the next level's, one slab of tiles or layer on, still find it in L2 (the 2 M points above 0.95 ms; whole
+// chunks a block 1.48, quarters by persistent blocks in turn 1.09). list: the gather by kinds, its chunks by
+// ticket, so that an empty list costs a launch; else every chunk, by its plan.
+constexpr int LANE_PARTS = BOX_PTS / BOX_THREADS;
+// Fewer chunks than one wave of blocks (a few whose box happens to span the grid, of points in Morton order) take
+// one chain of loads, 32 us, however few they are.
+constexpr int LANE_FEW = 152;
+template <bool P2>
+__global__ void __launch_bounds__(BOX_THREADS, 4) k_interp_lanes(const __grid_constant__ InterpArgs a,
+                                                                  const __grid_constant__ Levels L,
+                                                                  const int4* __restrict__ plan,
+                                                                  const int* __restrict__ list,
+                                                                  const int* __restrict__ n_list, unsigned* ticket) {
+  if (!list) {
+    const int64_t chunk = blockIdx.x / LANE_PARTS, i = int64_t(blockIdx.x) * BOX_THREADS + threadIdx.x;
+    if (plan_is_lanes(plan[chunk], a.nz) && i < a.np) lane_point<P2>(a, *level_tables(L), i);
+    return;
+  }
+  __shared__ unsigned s_item;
+  const unsigned n = unsigned(*n_list) * LANE_PARTS;
+  if (n == 0) return;
+  for (;;) {
+    __syncthreads();                               // the item before has been read
+    if (threadIdx.x == 0) s_item = atomicAdd(ticket, 1u);
+    __syncthreads();
+    const unsigned item = s_item;
+    if (item >= n) return;                         // uniform over the block
+    const int64_t i = int64_t(list[item / LANE_PARTS]) * BOX_PTS + (item % LANE_PARTS) * BOX_THREADS + threadIdx.x;
+    if (i < a.np) lane_point<P2>(a, *level_tables(L), i);
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -861,7 +965,8 @@ struct PlaneSlot {
 };
 struct GatherCounts {
   unsigned long long oor;
-  int groups, units, n_plane, n_tile, n_global;
+  int groups, units, n_plane, n_tile, n_global, n_lanes;
+  unsigned lane_ticket;
 };
 static_assert(sizeof(GatherCounts) <= 256, "the counters' part of the workspace");
 // Planes whose z has the same four levels and whose boxes lie close (their union no larger than their
@@ -876,7 +981,9 @@ struct GatherLists {
   PlaneGroup* groups;    // [PLANE_SLOTS]
   int* members;          // [PLANE_SLOTS] slots, group by group
   int2* chunk_slot;      // [chunks] slots of the chunk's first and last z, x = -1: not from planes
-  int *l_plane, *l_tile; // [chunks] chunks from planes, and of the others those with a staged tile
+  // [chunks] chunks from planes, and of the others those with a staged tile and those for k_interp_lanes
+  int *l_plane, *l_tile, *l_lanes;
+  int lanes;             // whether that runs
   float4* cols;          // [max_units * PLANE_UNIT]
   float* etas;
   int max_units;
@@ -1050,7 +1157,7 @@ __global__ void __launch_bounds__(1024) k_gather_lists(const __grid_constant__ I
   groups += n_alone;
   __threadfence_block();
   __syncthreads();
-  int np = 0, nt = 0, ng = 0;
+  int np = 0, nt = 0, ng = 0, nl = 0;
   for (int c0 = 0; c0 < chunks; c0 += 1024) {
     const int c = c0 + t;
     int kind = -1;
@@ -1058,15 +1165,26 @@ __global__ void __launch_bounds__(1024) k_gather_lists(const __grid_constant__ I
       const int2 sl = g.chunk_slot[c];
       kind = sl.x >= 0 && sl.y >= 0 && g.slots[sl.x].off >= 0 && g.slots[sl.y].off >= 0 ? 0
              : !plan_is_global(plan[c], a.nz)                                           ? 1
+             : g.lanes && plan_is_lanes(plan[c], a.nz)                                  ? 3
                                                                                         : 2;
-      if (kind != 0) g.chunk_slot[c] = make_int2(-1, -1);
+      // (x >= 0: not for k_interp_global)
+      if (kind != 0) g.chunk_slot[c] = make_int2(kind == 3 ? 0 : -1, -1);
     }
-    const long long pre = block_scan(kind < 0 ? 0 : 1ll << (20 * kind), ws, sum);
-    if (kind == 0) g.l_plane[np + int(pre & 0xfffff)] = c;
-    if (kind == 1) g.l_tile[nt + int(pre >> 20 & 0xfffff)] = c;
-    np += int(sum & 0xfffff);
-    nt += int(sum >> 20 & 0xfffff);
-    ng += int(sum >> 40);
+    const long long pre = block_scan(kind < 0 ? 0 : 1ll << (16 * kind), ws, sum);
+    if (kind == 0) g.l_plane[np + int(pre & 0xffff)] = c;
+    if (kind == 1) g.l_tile[nt + int(pre >> 16 & 0xffff)] = c;
+    if (kind == 3) g.l_lanes[nl + int(pre >> 48 & 0xffff)] = c;
+    np += int(sum & 0xffff);
+    nt += int(sum >> 16 & 0xffff);
+    ng += int(sum >> 32 & 0xffff);
+    nl += int(sum >> 48 & 0xffff);
+  }
+  if (nl < LANE_FEW) {                             // not worth a launch's wait: left to k_interp_global
+    __threadfence_block();
+    __syncthreads();
+    for (int i = t; i < nl; i += 1024) g.chunk_slot[g.l_lanes[i]] = make_int2(-1, -1);
+    ng += nl;
+    nl = 0;
   }
   if (t == 0) {
     g.n->groups = groups;
@@ -1074,6 +1192,8 @@ __global__ void __launch_bounds__(1024) k_gather_lists(const __grid_constant__ I
     g.n->n_plane = np;
     g.n->n_tile = nt;
     g.n->n_global = ng;
+    g.n->n_lanes = nl;
+    g.n->lane_ticket = 0;
   }
 }
 
@@ -2027,9 +2147,9 @@ int plane_units(int64_t np) { return int(std::min<int64_t>(2 * np, int64_t(1) <<
 size_t lists_bytes(int64_t np, int64_t chunks) {
   const size_t cols = size_t(plane_units(np)) * PLANE_UNIT;
   return up256(PLANE_SLOTS * sizeof(PlaneSlot)) + up256(PLANE_SLOTS * sizeof(PlaneGroup)) +
-         up256(PLANE_SLOTS * sizeof(int)) + up256(chunks * sizeof(int2)) + 2 * up256(chunks * sizeof(int)) + up256(cols * sizeof(float4)) + up256(cols * sizeof(float));
+         up256(PLANE_SLOTS * sizeof(int)) + up256(chunks * sizeof(int2)) + 3 * up256(chunks * sizeof(int)) + up256(cols * sizeof(float4)) + up256(cols * sizeof(float));
 }
-GatherLists lists_in(char* c, int64_t np, int64_t chunks, void* counts) {
+GatherLists lists_in(char* c, int64_t np, int64_t chunks, void* counts, bool lanes) {
   const size_t cols = size_t(plane_units(np)) * PLANE_UNIT;
   GatherLists g;
   auto take = [&](size_t b) { char* q = c; c += up256(b); return q; };
@@ -2040,9 +2160,11 @@ GatherLists lists_in(char* c, int64_t np, int64_t chunks, void* counts) {
   g.chunk_slot = reinterpret_cast<int2*>(take(chunks * sizeof(int2)));
   g.l_plane = reinterpret_cast<int*>(take(chunks * sizeof(int)));
   g.l_tile = reinterpret_cast<int*>(take(chunks * sizeof(int)));
+  g.l_lanes = reinterpret_cast<int*>(take(chunks * sizeof(int)));
   g.cols = reinterpret_cast<float4*>(take(cols * sizeof(float4)));
   g.etas = reinterpret_cast<float*>(take(cols * sizeof(float)));
   g.max_units = plane_units(np);
+  g.lanes = lanes;
   return g;
 }
 
@@ -2066,6 +2188,11 @@ int interp_by_kind(const InterpArgs& a, const Levels& lev, const int4* plan, int
       a, lev, plan, &g.n->n_global, g.chunk_slot, 1);
   SWENSE_CUDA_TRY(cudaGetLastError());
   count_launches(6);
+  if (g.lanes) {
+    k_interp_lanes<P2><<<unsigned(sms * 4), BOX_THREADS, 0, stream>>>(a, lev, plan, g.l_lanes, &g.n->n_lanes, &g.n->lane_ticket);
+    SWENSE_CUDA_TRY(cudaGetLastError());
+    count_launches(1);
+  }
   return SWENSE_OK;
 }
 
@@ -2115,6 +2242,16 @@ int interp_impl(const swense_grid* g, double t, const float* pts, const int32_t*
     SWENSE_CUDA_TRY(cudaGetDevice(&dev));
     SWENSE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const bool small = blocks < sms;
+    // Chunks marked ROWS_BIT by lanes: on grids whose four levels of all time levels do not stay in L2 (on others
+    // what a layer or row of tiles reads is still there for the next, and quads are faster), from 2^19 points on
+    // (400,000 binned points on the four-fold padded grid: 355 us either way), and below 2^21, where it is one
+    // more launch for every set, for binned points only (a mesh of a million points would lose 5 of 120 us).
+    bool lanes = sparse && (kinds || perm) && np >= (int64_t(1) << 19) && a.Nyr > 1;
+    if (lanes) {
+      int l2 = 0;
+      SWENSE_CUDA_TRY(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
+      lanes = double(a.Nxr) * a.Nyr * 64 * a.n_tl > 0.75 * double(l2);
+    }
     const int4* plan = small ? nullptr : plan_in;
     if (!plan && !small) {
       int4* pw = reinterpret_cast<int4*>(static_cast<char*>(ws) + 256);
@@ -2125,7 +2262,7 @@ int interp_impl(const swense_grid* g, double t, const float* pts, const int32_t*
       plan = pw;
     }
     if (kinds) {
-      const GatherLists g = lists_in(static_cast<char*>(ws) + b_plan, np, blocks, ws);
+      const GatherLists g = lists_in(static_cast<char*>(ws) + b_plan, np, blocks, ws, lanes);
       st = a.p2 ? interp_by_kind<true>(a, lev, plan, int(blocks), sms, g, stream)
                 : interp_by_kind<false>(a, lev, plan, int(blocks), sms, g, stream);
       if (st) return st;
@@ -2148,9 +2285,16 @@ int interp_impl(const swense_grid* g, double t, const float* pts, const int32_t*
         // (1.5 M mesh points: 81.0 -> 78.1 us); fewer points would leave too few blocks
         const int rounds = np >= (int64_t(1) << 20) && !small ? 2 : 1;
         const unsigned gctas = unsigned((np + rounds * GLOBAL_PTS - 1) / (rounds * GLOBAL_PTS));
-        if (a.p2) k_interp_global<true><<<gctas, BOX_THREADS, 0, stream>>>(a, lev, plan, nullptr, nullptr, rounds);
-        else k_interp_global<false><<<gctas, BOX_THREADS, 0, stream>>>(a, lev, plan, nullptr, nullptr, rounds);
+        const auto kglobal = a.p2 ? (lanes ? k_interp_global<true, true> : k_interp_global<true>)
+                                  : (lanes ? k_interp_global<false, true> : k_interp_global<false>);
+        kglobal<<<gctas, BOX_THREADS, 0, stream>>>(a, lev, plan, nullptr, nullptr, rounds);
         count_launches(1);
+        if (lanes) {
+          const unsigned lctas = unsigned(blocks * LANE_PARTS);
+          if (a.p2) k_interp_lanes<true><<<lctas, BOX_THREADS, 0, stream>>>(a, lev, plan, nullptr, nullptr, nullptr);
+          else k_interp_lanes<false><<<lctas, BOX_THREADS, 0, stream>>>(a, lev, plan, nullptr, nullptr, nullptr);
+          count_launches(1);
+        }
       } else {
         if (a.p2) k_interp_box<true, false><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
         else k_interp_box<false, false><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
