@@ -4,18 +4,20 @@
 // uniformly spaced nodes), the zero-padding refinement (spectrum extended n times with zero
 // modes -> n times finer grid) and the extension of the solution above z = 0.
 //
-// Two passes per level chunk (3-D, ny > 1):
-//   pass A  per (level, block of kx columns): form the four modal fields
-//             U = i kx A^phi F, V = i ky A^phi F, W = |k| A^phi S, T = A^phit F
-//           (depth factors F, S at the level), zero-pad along ky and inverse-transform along y;
-//           writes G[level][field][y][m] (complex, one-sided in m) to the scratch workspace.
-//   pass B  per (level, block of y rows): pack the two real-field pairs into one complex
-//           spectrum each, Z1 = U + iV and Z2 = W + iT (Hermitian extension over m, zero-padded
-//           to nx_r), inverse-transform along x and store float4 (u, v, w, dphi/dt) per node.
-// Level chunks are sized so G stays L2-resident between the passes. eta is one extra transform
-// per time level (pass A on A^eta; pass B packs two grid rows per complex transform).
-// Transforms of 32 to 1024 points along y and 32 points and more along x run as a wide-radix pair over
-// a transposed intermediate instead (k_col_w, k_row_w). 2-D (ny == 1): one kernel (k_line).
+// Columns of 32 to 1024 nodes and rows of 32 and more (3-D): k_form_modes makes the modal fields at z = 0
+//   U = i kx A^phi, V = i ky A^phi, W = |k| A^phi, T = A^phit and A^eta
+// of every time level once; then two passes per chunk of slots (the levels of all time levels, and eta):
+//   columns (k_col_w)  per (slot, block of kx columns): depth factors F and S at the level, zero-padding
+//           along ky, inverse transforms along y; writes G[slot][field][y][m] (complex, one-sided in m) to
+//           the scratch workspace;
+//   rows    (k_row_w; k_row_tb from 4096 nodes on; k_row_tma, an autotuner candidate)  per (slot, block of y
+//           rows): the two real-field pairs packed into one complex spectrum each, Z1 = U + iV and
+//           Z2 = W + iT (Hermitian extension over m, zero-padded to nx_r), inverse transforms along x, one
+//           float4 (u, v, w, dphi/dt) per node.
+// Other sizes, and requests whose scratch cannot be had: the same two passes over one time level's levels,
+// in shared memory, each making its fields itself (k_pass_a, k_pass_b, and k_propagate before them); eta
+// is one extra transform per time level (two grid rows per complex transform).
+// 2-D (ny == 1): one kernel (k_line).
 #include <algorithm>
 #include <array>
 #include <cmath>
