@@ -950,7 +950,9 @@ __global__ void __launch_bounds__(BOX_THREADS, 4) k_interp_lanes(const __grid_co
 // table; k_gather_lists sizes the planes (those that pay, within the scratch given), groups them by
 // their levels and lists the chunks that read planes and those with a staged tile, for persistent
 // kernels, so that an empty list costs a launch; k_interp_global takes the rest in point order.
-// 8.2 M mesh points on the four-fold padded 512 x 256 grid: 1.02 ms straight from the grid, 0.48 ms so (planes 0.13, gather 0.24 of it).
+// 8.2 M mesh points on the four-fold padded 512 x 256 grid: 1.02 ms straight from the grid, 0.46 ms so (planes 0.13, gather 0.22 of it);
+// from 2^21 points on, where the lists' fixed cost pays (2 M mesh points: 178 against 235 us there with one time level,
+// 288 and 300 with two; 4 M: 512 against 428 with two).
 // 3-D grids only: a 2-D one has too few nodes for the rule.
 constexpr int64_t LAYER_POINTS = int64_t(1) << 21;
 constexpr int PLANE_SLOTS = 4096;                  // planes at most (hash table entries)
@@ -2281,9 +2283,11 @@ int interp_impl(const swense_grid* g, double t, const float* pts, const int32_t*
           else k_interp_box<false, true><<<unsigned(blocks), BOX_THREADS, BOX_SMEM, stream>>>(a, lev, plan);
           count_launches(1);
         }
-        // two rounds a block from 2^20 points on: a mesh's blocks with nothing to do are half as many
-        // (1.5 M mesh points: 81.0 -> 78.1 us); fewer points would leave too few blocks
-        const int rounds = np >= (int64_t(1) << 20) && !small ? 2 : 1;
+        // two rounds a block from 2^20 points on: a mesh's blocks with nothing to do are half as many (1.1 to 2 M
+        // mesh points on grids of 1024 x 512 to 2048 x 1024: 2 to 7 % less, 85.4 -> 79.4 us of 2 M, the like or up
+        // to 2 % more with three time levels; points in no order 0.7 % more); not for binned points, which lose by
+        // it (1.1 M on 1024 x 512: 414 against 526 us); fewer points would leave too few blocks
+        const int rounds = !perm && np >= (int64_t(1) << 20) ? 2 : 1;
         const unsigned gctas = unsigned((np + rounds * GLOBAL_PTS - 1) / (rounds * GLOBAL_PTS));
         const auto kglobal = a.p2 ? (lanes ? k_interp_global<true, true> : k_interp_global<true>)
                                   : (lanes ? k_interp_global<false, true> : k_interp_global<false>);
