@@ -499,8 +499,9 @@ __device__ int g_async_timeout;
 // Eight levels of 1024 x 2048 nodes: at padding 1 149 -> 97 us (5.5 TB/s with the
 // intermediate from memory), at padding 4 (a quarter of the input) 76 us; radix-8 passes with
 // straight loads took 124 and 108.
-// TWO: an exchange buffer for each of the two transforms, where the staged rows leave the room.
-template <int N, bool TWO>
+// TWO: an exchange buffer for each of the two transforms, where the staged rows leave the room. SELF: no copy is
+// issued (self-test; its own instance, since the question alone cost 1615 -> 1618 us on the padded grid).
+template <int N, bool TWO, bool SELF = false>
 __global__ void __launch_bounds__(WideRow<N>::T * WideRow<N>::kRows, WideRow<N>::E == 16 ? 4 : 8) k_row_w(RowArgs a, int items) {
   using W = WideRow<N>;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -517,7 +518,7 @@ __global__ void __launch_bounds__(WideRow<N>::T * WideRow<N>::kRows, WideRow<N>:
     const float2* src = a.G + size_t(level) * 4 * fs + size_t(y0) * a.ldG;
     fence_proxy_async();                           // earlier reads of the buffer come first
     mbar_arrive_expect_tx(bar, nf * span);
-    for (int f = 0; f < nf && !a.selftest; ++f) bulk_g2s(stg + size_t(f) * W::kRows * a.ldG, src + f * fs, span, bar);
+    for (int f = 0; f < (SELF ? 0 : nf); ++f) bulk_g2s(stg + size_t(f) * W::kRows * a.ldG, src + f * fs, span, bar);
   };
   int item = blockIdx.x;
   if (item >= items) return;
@@ -789,18 +790,17 @@ int launch_row_w(const RowArgs& r, int nl, cudaStream_t stream) {
   const int per_sm = W::E == 16 ? 4 : 8;
   const size_t stage = size_t(4) * W::kRows * r.ldG * sizeof(float2), buf = size_t(W::kRows) * W::kBuf * sizeof(float2);
   // 227 KB of shared memory per SM, 1 KB of it reserved per block
-  const bool two = (stage + 2 * buf + 1152) * per_sm <= size_t(227) * 1024;
+  const bool two = !r.selftest && (stage + 2 * buf + 1152) * per_sm <= size_t(227) * 1024;
   const size_t smem = stage + (two ? 2 : 1) * buf + sizeof(uint64_t);
-  const void* fn = two ? (const void*)k_row_w<N, true> : (const void*)k_row_w<N, false>;
-  int st = set_smem(fn, smem);
+  const auto kernel = r.selftest ? k_row_w<N, false, true> : (two ? k_row_w<N, true> : k_row_w<N, false>);
+  int st = set_smem((const void*)kernel, smem);
   if (st) return st;
   int dev = 0, sms = 0;
   SWENSE_CUDA_TRY(cudaGetDevice(&dev));
   SWENSE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int items = nl * (r.Nyr / W::kRows);
   const unsigned grid = unsigned(std::min(items, sms * per_sm));
-  if (two) k_row_w<N, true><<<grid, W::T * W::kRows, smem, stream>>>(r, items);
-  else k_row_w<N, false><<<grid, W::T * W::kRows, smem, stream>>>(r, items);
+  kernel<<<grid, W::T * W::kRows, smem, stream>>>(r, items);
   SWENSE_CUDA_TRY(cudaGetLastError());
   count_launches(1);
   return SWENSE_OK;
