@@ -46,7 +46,8 @@ struct Scratch {
 struct DeviceState {
   Scratch ws;
   // Outgrown while graphs held them; freed by the growth after the last of these is gone, or
-  // swense_release. Each is smaller by a quarter and more than the one after it.
+  // swense_release. Each is at most four fifths of the one after it, so together they are at most four times
+  // the present one.
   std::vector<Scratch> kept;
   bool tw_ready = false;
   // Smallest optional request that could not be had, and how many more of at least its size are answered
@@ -141,12 +142,16 @@ int hold_for_capture(DeviceState& d, cudaStream_t stream) {
   auto* held = new std::shared_ptr<std::atomic<int>>(d.ws.graphs);
   ++**held;
   cudaUserObject_t obj = nullptr;
-  const cudaError_t e = cudaUserObjectCreate(&obj, held, drop_graph, 1, cudaUserObjectNoDestructorSync);
+  cudaError_t e = cudaUserObjectCreate(&obj, held, drop_graph, 1, cudaUserObjectNoDestructorSync);
   if (e != cudaSuccess) {
     drop_graph(held);
     return cuda_fail(e, "cudaUserObjectCreate");
   }
-  SWENSE_CUDA_TRY(cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove));
+  e = cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove);
+  if (e != cudaSuccess) {
+    cudaUserObjectRelease(obj, 1);
+    return cuda_fail(e, "cudaGraphRetainUserObject");
+  }
   return SWENSE_OK;
 }
 
