@@ -337,12 +337,12 @@ def captured_traffic(tr, source_hash, workload, shape=None):
 # the hash of the kernel's sources and the workload they were taken on; a changed kernel,
 # workload or launch shape invalidates them (traffic is then reported as null).
 NCU_TRAFFIC = {
-    "k_interp_box": {"bytes": 105900000 + 127300000, "hash": "92ee0328a2d6767e",
+    "k_interp_box": {"bytes": 106200000 + 126900000, "hash": "a6a33ad4b5a12f25",
                      "workload": "jonswap3d: 512x256 modes, 64 levels, pad 1, 2 time levels, "
                                  "2048000 cell + 6177280 face centres (cylinder O-grid)"},
     # the three launches of one step, caches kept between them (--cache-control none), untuned launch
     # shape: one chunk of 130 slots, whose intermediate goes through memory
-    GRID_STAGE: {"bytes": 6300000 + 266600000 + 527600000, "hash": "1e958107ea5274bd",
+    GRID_STAGE: {"bytes": 5700000 + 266500000 + 527200000, "hash": "594599071916006b",
                  "taken_with": DEFAULT_SHAPE,
                  "workload": "jonswap3d: 512x256 modes, 64 levels, pad 1, 2 time levels, "
                              "2048000 cell + 6177280 face centres (cylinder O-grid)"},
@@ -353,9 +353,8 @@ DIRECT_KERNEL = "k_direct_tc"
 DIRECT_SOURCES = ("csrc/direct_tc.cu", "csrc/tcgen05.cuh", "csrc/tma.cuh", "csrc/mma.cuh", "csrc/internal.cuh")
 NCU_TRAFFIC[DIRECT_KERNEL] = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum (caches flushed before the launch),
-    # one launch: 1,000,000 near-body points x the 2048 x 1024-mode sea (sources since changed
-    # only by a compile-time check of the B column slots)
-    "bytes": 59055616 + 9081856, "hash": "f174d5c52843f601",
+    # one launch: 1,000,000 near-body points x the 2048 x 1024-mode sea
+    "bytes": 62016768 + 12850944, "hash": "99498bf2e67d786d",
     "workload": "near-body 1000000 points x 2048x1024 modes"}
 # Algorithmic MMA flops of the split-BF16 direct sum (the per-unit figure of the workload's
 # definition): per (point, mode) pair of the full nx x ny spectrum, u, v, w and dphi/dt each the

@@ -237,7 +237,7 @@ typedef struct swense_grid {
  * and then in x and y per point, which is the same tensor-product sum in another order. Few points
  * (fewer chunks than SMs) are taken straight from the grid. From 2^21 points on, on a grid of more
  * than four times as many nodes, the layers of equal z share such planes in the scratch workspace
- * (40 B per point, at most 1.3 GB, and 32 B per chunk; without it where it cannot be had).
+ * (40 B per point, at most 1.3 GB, and 36 B per chunk; without it where it cannot be had).
  * Errors: ARG, SIZE, LEVELS, CUDA.
  */
 int swense_interp(const swense_grid* grid, double t, const float* pts, int64_t np,
